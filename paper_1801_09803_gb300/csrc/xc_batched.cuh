@@ -36,6 +36,7 @@ struct GeomStats {
     unsigned int nu_bits;      // max nu (float, rounded up)
     unsigned int gref_bits;    // max |gamma_ref|
     unsigned int nT_bits;      // max |n_T|
+    unsigned int acoef_bits;   // max alpha / nu over the conditions (float, rounded up; block-interpolated sweep)
 };
 
 __device__ __forceinline__ float rcp_approx(float x) { return recip(x); }
@@ -171,6 +172,9 @@ cudaError_t launch_fp32_setup(const LinesDev &L, size_t n, const CondDev *conds,
                               double cutoff, int *n_abs, float *f, int *ka, int *kb, GeomStats *gs, CParam *cp,
                               cudaStream_t s);
 xc_status vjp_run(BatchedState *st, const VjpArgs &a, int64_t *launches);
+// the block-interpolated FP32 sweep (xc_tree.cu): whether it takes a call, and the call
+bool tree_takes(const BatchedArgs &a);
+xc_status tree_run(BatchedState *st, const BatchedArgs &a, int64_t *launches);
 // after the stream has synchronised: XC_ETIMEOUT if the tensor-core kernel reported a
 // wait that ran out (its results are then not valid), else XC_OK
 xc_status batched_check(BatchedState *st);

@@ -1,0 +1,82 @@
+"""The block-interpolated FP32 sweep against the general CUDA-core path (a fixed tile shape
+selects it) and the oracle, at the edges of its blocks and over the forms it accepts.
+
+Tolerances: against the oracle those of the FP32 path (2e-4 / band 1e-5); between the two
+FP32 paths 2e-5 relative above 1e-6 of the peak, as between the other FP32 paths (two FP32
+summation orders, interpolation error below 2e-8)."""
+import numpy as np
+import pytest
+
+import xcsynth as xs
+from test_gpu_parity import TOL32, TOL32_BAND, eng, metrics, oracle_sigma, xc  # noqa: F401
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+PROFILES = ["voigt_w4", "lorentz", "doppler", "doppler_binned", "lorentz_binned", "voigt_gh_binned", "voigt_gh_sampled"]
+
+
+def both(eng, conds, grid, opts):  # noqa: F811
+    got = eng.cross_section_batched(conds, grid, opts)
+    assert "block-interpolated" in eng.tuning()
+    eng.set_tile_shape(8, 1)
+    try:
+        ref = eng.cross_section_batched(conds, grid, opts)
+        assert "block-interpolated" not in eng.tuning()
+    finally:
+        eng.set_tile_shape(0, 0)
+    return got, ref
+
+
+def close(got, ref):
+    m = ref > 1e-6 * ref.max(axis=1, keepdims=True)
+    return float(np.max(np.abs(got[m] - ref[m]) / ref[m])) if m.any() else 0.0
+
+
+@pytest.mark.parametrize("n", [1, 31, 33, 64, 65, 127, 513, 4097])
+@pytest.mark.parametrize("profile", PROFILES)
+def test_block_edges(eng, xc, profile, n):  # noqa: F811
+    L = xs.gen_lines(301, 0, 3000, 1000.0, 1060.0)
+    eng.load_lines(L)
+    eng.set_states(*xs.gen_states(301, 500))
+    conds = [xc.make_condition(T, P) for T, P in ((300.0, 1e-3), (900.0, 0.3), (2500.0, 10.0))]
+    for nu_A, step, cut, wm in ((1010.0, 0.01, 25.0, 0.0), (1059.37, 0.0137, 3.0, 0.0), (990.0, 0.01, 25.0, 300.0)):
+        got, ref = both(eng, conds, xc.make_grid(nu_A, step, n), xc.make_opts(profile, "fp32", cut, wm))
+        assert np.all(np.isfinite(got))
+        assert close(got, ref) < 2e-5, (profile, n, nu_A, cut, wm)
+        assert np.all((got == 0) == (ref == 0)) or profile.startswith("doppler") or profile.endswith("binned")
+
+
+@pytest.mark.parametrize("n_cond", [1, 3, 40])
+def test_against_oracle_with_long_cut(eng, xc, oracle_lib, n_cond):  # noqa: F811
+    """2500-step cut, all three block levels, a ragged grid past both ends of the list, threshold
+    and emission; 40 conditions run on the blocks as well (a cut of 1024 steps or more)."""
+    L = xs.gen_lines(302, 0, 20_000, 500.0, 600.0)
+    E, g = xs.gen_states(302, 1000)
+    eng.load_lines(L)
+    eng.set_states(E, g)
+    TP = [(300.0 * 1.06 ** i, 1e-3 * 1.27 ** i) for i in range(n_cond)]
+    nu_A, step, n = 480.03, 0.01, 13_337
+    for quantity, thr in (("absorption", None), ("emission", ("hitran", 550.0, 1e-24))):
+        got = eng.cross_section_batched([xc.make_condition(T, P) for T, P in TP], xc.make_grid(nu_A, step, n),
+                                        xc.make_opts("voigt_w4", "fp32", 25.0, quantity=quantity, threshold=thr))
+        assert "block-interpolated" in eng.tuning()
+        for i in {0, n_cond // 2, n_cond - 1}:
+            ref = oracle_sigma(oracle_lib, L, E, g, *TP[i], nu_A, step, n, "voigt_w4", 25.0, quantity=quantity,
+                               threshold=thr)
+            mr, band = metrics(got[i], ref)
+            assert mr < TOL32 and band < TOL32_BAND, (quantity, i, mr, band)
+
+
+def test_hotter_conditions_after_cooler_ones(eng, xc):  # noqa: F811
+    """The radii follow the call's own conditions: a hot call after a cold one of the same shape."""
+    L = xs.gen_lines(303, 0, 4000, 1000.0, 1030.0)
+    eng.load_lines(L)
+    eng.set_states(*xs.gen_states(303, 500))
+    grid, opts = xc.make_grid(1000.0, 0.01, 3001), xc.make_opts("voigt_w4", "fp32", 25.0)
+    out = torch.zeros((1, 3001), dtype=torch.float64, device="cuda:0")
+    eng.cross_section_batched([xc.make_condition(100.0, 0.01)], grid, opts, out)
+    eng.cross_section_batched([xc.make_condition(3000.0, 0.01)], grid, opts, out)
+    hot = out.cpu().numpy()
+    _, ref = both(eng, [xc.make_condition(3000.0, 0.01)], grid, opts)
+    assert close(hot, ref) < 2e-5
