@@ -277,29 +277,29 @@ __device__ __forceinline__ float contrib_single(float u, float delta, const floa
     }
 }
 
-// Re w in w4's regions III and IV (|x| + y < 5.5), the same forms as w4_eval with only
-// the real part formed: region III the real part of the quotient; region IV needs
-// cos(Im u) of exp(u), u = t^2, and no sine
-__device__ __forceinline__ float w4_region34_re(float x, float y) {
+// Re w in w4's region III (|x| + y < 5.5, y >= 0.195 |x| - 0.176): the real part of the quotient
+__device__ __forceinline__ float w4_region3_re(float x, float y) {
+    // N(t) and D(t) have real coefficients: synthetic division by (z - t)(z - conj t) =
+    // z^2 - r z + s takes two operations per coefficient instead of the four of a complex
+    // Horner step, and is no less accurate here (rms error against FP64 over region III
+    // 2.2e-7, complex Horner 2.4e-7; in region IV it would be 6 times worse, so not there)
+    const float r = y + y, s = fmaf(x, x, y * y);
+    const float n3 = fmaf(0.5642236f, r, 3.778987f);
+    const float n2 = fmaf(r, n3, fmaf(-s, 0.5642236f, 11.96482f));
+    const float n1 = fmaf(r, n2, fmaf(-s, n3, 20.20933f));
+    const float d4 = r + 6.699398f;
+    const float d3 = fmaf(r, d4, 21.69274f - s);
+    const float d2 = fmaf(r, d3, fmaf(-s, d4, 39.27121f));
+    const float d1 = fmaf(r, d2, fmaf(-s, d3, 38.82363f));
+    const float Nr = fmaf(y, n1, fmaf(-s, n2, 16.4955f)), Dr = fmaf(y, d1, fmaf(-s, d2, 16.4955f));
+    const float Ni = x * n1, Di = x * d1;   // both imaginary parts with the sign of conj t
+    return fmaf(Nr, Dr, Ni * Di) * recip(fmaf(Dr, Dr, Di * Di));
+}
+
+// Re w in w4's region IV (|x| + y < 5.5, y < 0.195 |x| - 0.176): cos(Im u) of exp(u), u = t^2,
+// and no sine
+__device__ __forceinline__ float w4_region4_re(float x, float y) {
     const Cx<float> t = cx<float>(y, -x);
-    const float ax = fabsf(x);
-    if (y >= 0.195f * ax - 0.176f) {
-        // N(t) and D(t) have real coefficients: synthetic division by (z - t)(z - conj t) =
-        // z^2 - r z + s takes two operations per coefficient instead of the four of a complex
-        // Horner step, and is no less accurate here (rms error against FP64 over region III
-        // 2.2e-7, complex Horner 2.4e-7; in region IV it would be 6 times worse, so not there)
-        const float r = y + y, s = fmaf(x, x, y * y);
-        const float n3 = fmaf(0.5642236f, r, 3.778987f);
-        const float n2 = fmaf(r, n3, fmaf(-s, 0.5642236f, 11.96482f));
-        const float n1 = fmaf(r, n2, fmaf(-s, n3, 20.20933f));
-        const float d4 = r + 6.699398f;
-        const float d3 = fmaf(r, d4, 21.69274f - s);
-        const float d2 = fmaf(r, d3, fmaf(-s, d4, 39.27121f));
-        const float d1 = fmaf(r, d2, fmaf(-s, d3, 38.82363f));
-        const float Nr = fmaf(y, n1, fmaf(-s, n2, 16.4955f)), Dr = fmaf(y, d1, fmaf(-s, d2, 16.4955f));
-        const float Ni = x * n1, Di = x * d1;   // both imaginary parts with the sign of conj t
-        return fmaf(Nr, Dr, Ni * Di) * recip(fmaf(Dr, Dr, Di * Di));
-    }
     const Cx<float> u = t * t;
     const Cx<float> m = cx<float>(-u.re, -u.im);
     const Cx<float> N = 36183.31f + m * (3321.9905f + m * (1540.787f + m * (219.0313f +
@@ -308,6 +308,10 @@ __device__ __forceinline__ float w4_region34_re(float x, float y) {
                         m * (364.2191f + m * (61.57037f + m * (1.841439f + m))))));
     const Cx<float> r = cdiv(N, D);
     return expf(u.re) * cosf(u.im) - (t.re * r.re - t.im * r.im);
+}
+
+__device__ __forceinline__ float w4_region34_re(float x, float y) {
+    return y >= 0.195f * fabsf(x) - 0.176f ? w4_region3_re(x, y) : w4_region4_re(x, y);
 }
 
 // width of a condition's profiles at a representative line (nu = 5000 cm^-1, n = 0.6):

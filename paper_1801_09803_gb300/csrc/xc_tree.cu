@@ -30,138 +30,13 @@
 
 #include "xc_batched.cuh"
 #include "xc_f32.cuh"
+#include "xc_tree.cuh"
 
 namespace xc {
 
-constexpr int TR_M = 16;                    // nodes per block
-constexpr int TR_LEVELS = 3;
-__device__ __host__ constexpr int tr_block(int lev) { return lev == 0 ? 64 : (lev == 1 ? 128 : 512); }
-__device__ __host__ constexpr int tr_gap(int lev) { return lev == 0 ? 36 : (lev == 1 ? 72 : 284); }   // 0.55 B
-constexpr int TR_T = 256;                   // threads per CTA
-constexpr int TR_W = TR_T / 32;
 constexpr int TR_FOLD = 4;                  // scanned chunks (32 lines) per FP32 partial sum at the nodes
                                             // (each chunk at the points, where one strong line can
                                             // dominate: 512 lines in one sum left 6e-7 of rounding)
-constexpr int TR_CELL = 64;                 // grid steps per entry of the line index
-
-struct TreeParams {
-    LinesDev L;
-    const int4 *geo;             // per line: integer grid position n, cut range ka..kb (inclusive), fraction f (bits)
-    const float4 *recA, *recB;   // per (condition, line): profile constants (see line_consts); B: Voigt w4 only
-    const CParam *cp;
-    const GeomStats *gs;
-    const unsigned *cell;        // cell[j]: first line with n >= cell0 + 64 j, j = 0..ncell
-    int cell0, ncell;
-    double *nodes;               // per condition: node sums of levels 0, 1, 2
-    int nblk[TR_LEVELS], node_off[TR_LEVELS], nodes_per_cond;
-    const double *mat;           // interpolation matrices (see TR_MAT_*)
-    int c0, n_cond;              // conditions c0 .. c0 + n_cond - 1 of the call are in recA / recB
-    size_t n;                    // lines
-    int n_pts;
-    int reach;                   // no line reaches a point farther than this many steps from its n
-    int cover;                   // every line covers the points within this many steps (0: not known)
-    int far;                     // 0: no blocks (profiles without far wings)
-    int wpt;                     // warps per task
-    double nu_A, step, cutoff;
-    float inv_h, ext;            // ext: real distance of the outermost pole from the centre, per alpha (grid steps)
-    int ext0;                    // ... plus this many steps
-    float core;                  // radius of the points that need the full profile, per alpha
-    const double *ghx, *ghw;
-    int ngh;
-    double *sigma;               // [n_cond rows of the call][n_pts]
-};
-
-// interpolation matrices, destination index fastest: nodes of a 512-point block -> nodes of its
-// eight 64-point blocks, of a 128-point block -> its two, of a 64-point block -> its points
-constexpr int TR_MAT_512 = 0;                              // [8][16 source][16]
-constexpr int TR_MAT_128 = 8 * TR_M * TR_M;                // [2][16 source][16]
-constexpr int TR_MAT_PT = TR_MAT_128 + 2 * TR_M * TR_M;    // [16 source][64]
-constexpr int TR_MAT = TR_MAT_PT + TR_M * 64;
-
-// node m of a block of B points, in grid steps from its first point: Chebyshev nodes of
-// [0, B - 1] rounded to 1/128, so that node - n is exact in FP32
-__device__ __forceinline__ float tr_node(int B, int m) {
-    return rintf(64.f * (float)(B - 1) * (1.f - cospif((float)(2 * m + 1) * (1.f / (2 * TR_M))))) * (1.f / 128.f);
-}
-
-// Gap (grid steps) beyond which a block ending at b1 takes a line: the same for all lines
-// (alpha from an upper bound of the wavenumbers that reach the block), growing with the
-// level and with the block's position, so a line taken by a block is taken by its children
-__device__ __forceinline__ int tr_radius(const TreeParams &p, int lev, int b1) {
-    const float nu = fmaxf(__double2float_ru(__dadd_rn(grid_x(p.nu_A, p.step, b1), p.cutoff)), 0.f);
-    const float ah = __fmul_ru(__fmul_ru(__uint_as_float(p.gs->acoef_bits), nu), p.inv_h);
-    const int a = tr_gap(lev) + p.ext0 + (int)ceilf(__fmul_ru(fminf(ah, 1e6f), p.ext));
-    const int b = (int)ceilf(__fmul_ru(fminf(ah, 1e6f), p.core)) + 2;
-    return max(a, b);
-}
-
-// a block [b0, b1] (b1c: clipped to the grid) with radius D takes a line
-__device__ __forceinline__ bool tr_takes(const int4 &g, int b0, int b1, int b1c, int D) {
-    return g.y <= b0 && g.z >= b1c && (g.x < b0 - D || g.x > b1 + D);
-}
-
-__device__ __forceinline__ unsigned tr_lower(const TreeParams &p, int v) {   // <= first line with n >= v
-    return p.cell[min(max((v - p.cell0) >> 6, 0), p.ncell)];
-}
-__device__ __forceinline__ unsigned tr_upper(const TreeParams &p, int v) {   // >= first line with n >= v
-    return p.cell[min(max((v - p.cell0 + (TR_CELL - 1)) >> 6, 0), p.ncell)];
-}
-
-struct Segs {
-    unsigned s[4], e[4];
-};
-
-// Candidate lines of a block of a far level: positions that can cover it, outside its radius,
-// without those its parent takes for certain.  Ranges are rounded outwards to index cells and
-// kept disjoint; tr_takes decides per line.
-__device__ __forceinline__ Segs tr_far_segs(const TreeParams &p, int b0, int b1, int D, bool has_parent, int p0,
-                                            int p1, int Dp) {
-    const int b1c = min(b1, p.n_pts - 1);
-    const int a = b1c - p.reach, z = b0 - D;
-    int e1 = z, s2 = z;
-    if (has_parent) {
-        e1 = min(z, max(a, p1 - p.cover));
-        s2 = min(z, max(e1, p0 - Dp));
-    }
-    const int a2 = b1 + D + 1, z2 = b0 + p.reach + 1;
-    int e3 = z2, s4 = z2;
-    if (has_parent) {
-        e3 = min(z2, p1 + Dp + 1);
-        s4 = min(z2, max(e3, p0 + p.cover));
-    }
-    Segs g;
-    g.s[0] = tr_lower(p, a);
-    g.e[0] = max(g.s[0], a < e1 ? tr_upper(p, e1) : 0u);
-    g.s[1] = max(g.e[0], tr_lower(p, s2));
-    g.e[1] = max(g.s[1], s2 < z ? tr_upper(p, z) : 0u);
-    g.s[2] = max(g.e[1], tr_lower(p, a2));
-    g.e[2] = max(g.s[2], a2 < e3 ? tr_upper(p, e3) : 0u);
-    g.s[3] = max(g.e[2], tr_lower(p, s4));
-    g.e[3] = max(g.s[3], s4 < z2 ? tr_upper(p, z2) : 0u);
-    return g;
-}
-
-// Candidate lines of the points s0..s1 inside the level-0 block [p0, p1] of radius Dp
-__device__ __forceinline__ Segs tr_point_segs(const TreeParams &p, int s0, int s1, int p0, int p1, int Dp) {
-    const int a = s0 - p.reach, z = s1 + p.reach + 1;
-    int e1 = a, s2 = a, e2 = z, s3 = z;
-    if (p.far) {
-        e1 = max(a, min(p0 - Dp, p1 - p.cover));
-        s2 = max(e1, p0 - Dp);
-        e2 = min(z, p1 + Dp + 1);
-        s3 = min(z, max(e2, p0 + p.cover));
-    }
-    Segs g;
-    g.s[0] = tr_lower(p, a);
-    g.e[0] = max(g.s[0], a < e1 ? tr_upper(p, e1) : 0u);
-    g.s[1] = max(g.e[0], tr_lower(p, s2));
-    g.e[1] = max(g.s[1], s2 < e2 ? tr_upper(p, e2) : 0u);
-    g.s[2] = max(g.e[1], tr_lower(p, s3));
-    g.e[2] = max(g.s[2], s3 < z ? tr_upper(p, z) : 0u);
-    g.s[3] = g.e[3] = g.e[2];
-    return g;
-}
-
 template <int PROF>
 __device__ __forceinline__ float tr_amplitude(const float4 &A) {
     return (PROF == XC_VOIGT_W4 || PROF == XC_VOIGT_GH_SAMPLED || PROF == XC_LORENTZ_BINNED) ? A.z
@@ -171,11 +46,24 @@ __device__ __forceinline__ float tr_amplitude(const float4 &A) {
 template <int PROF>
 constexpr bool tr_pairs() { return PROF == XC_VOIGT_W4 || PROF == XC_LORENTZ; }
 
-// two lines at one position per packed operation: region I of w4, or the Lorentzian
-template <int PROF>
-__device__ __forceinline__ f32x2 tr_pair_value(f32x2 u, const ulonglong2 &c0, const ulonglong2 &c1) {
-    if (PROF == XC_VOIGT_W4) return mul2(fma2(c1.x, u, c1.y), rcp2(fma2(u, add2(u, c0.x), c0.y)));
-    return mul2(c0.y, rcp2(add2(u, c0.x)));
+// w4's region II (see w4_region2_re) of two lines: X = x^2, Y = y^2, yP = y times the amplitude
+__device__ __forceinline__ f32x2 w4_region2_pair(f32x2 X, f32x2 Y, f32x2 yP) {
+    constexpr double a = 1.410474, b = 0.5641896, s6 = 2.449489742783178098;
+    constexpr float Q1 = (float)((3.0 - s6) / 2.0), Q2 = (float)((3.0 + s6) / 2.0);
+    constexpr float A1 = (float)((a - b * ((3.0 - s6) / 2.0)) / s6);
+    constexpr float A2 = (float)(-(a - b * ((3.0 + s6) / 2.0)) / s6);
+    const f32x2 Z = add2(X, Y);
+    const f32x2 t1 = add2(Z, pk2(-Q1, -Q1)), t2 = add2(Z, pk2(-Q2, -Q2));
+    const f32x2 D1 = fma2(t1, t1, mul2(Y, pk2(4.f * Q1, 4.f * Q1)));
+    const f32x2 D2 = fma2(t2, t2, mul2(Y, pk2(4.f * Q2, 4.f * Q2)));
+    const f32x2 N1 = mul2(pk2(A1, A1), add2(Z, pk2(Q1, Q1))), N2 = mul2(pk2(A2, A2), add2(Z, pk2(Q2, Q2)));
+    return mul2(mul2(yP, fma2(N1, D2, mul2(N2, D1))), rcp2(mul2(D1, D2)));
+}
+
+__device__ __forceinline__ float sum2(f32x2 v) {
+    float a, b;
+    upk2(v, a, b);
+    return a + b;
 }
 
 // sum += acc, compensated
@@ -201,6 +89,11 @@ __global__ void k_tree_prep(const CondDev *conds, int n_cond, GeomStats *gs) {
         *gs = GeomStats{};
         gs->acoef_bits = __float_as_uint(a);
     }
+}
+
+cudaError_t launch_tree_prep(const CondDev *conds, int n_cond, GeomStats *gs, cudaStream_t s) {
+    k_tree_prep<<<1, 32, 0, s>>>(conds, n_cond, gs);
+    return cudaGetLastError();
 }
 
 // Line geometry in grid steps and the intensity statistics.  width_mult > 0: the cut of
@@ -277,6 +170,20 @@ __device__ double tr_basis(int B, int m, double x) {
     return num / den;
 }
 
+// entry k of the interpolation matrices
+__device__ double tr_mat_entry(int k) {
+    if (k < TR_MAT_128) {
+        const int j = k / (TR_M * TR_M), s = (k / TR_M) % TR_M, d = k % TR_M;
+        return tr_basis(512, s, (double)(64 * j) + (double)tr_node(64, d));
+    }
+    if (k < TR_MAT_PT) {
+        const int q = k - TR_MAT_128, j = q / (TR_M * TR_M), s = (q / TR_M) % TR_M, d = q % TR_M;
+        return tr_basis(128, s, (double)(64 * j) + (double)tr_node(64, d));
+    }
+    const int q = k - TR_MAT_PT;
+    return tr_basis(64, q / 64, (double)(q % 64));
+}
+
 // block 0: per-condition constants; block 1..: line index, then the interpolation matrices
 __global__ void __launch_bounds__(256) k_tree_setup(TreeParams p, const CondDev *conds, int n_cond, CParam *cp,
                                                     int quantity, const unsigned *gmax, unsigned *cell, double *mat) {
@@ -296,17 +203,17 @@ __global__ void __launch_bounds__(256) k_tree_setup(TreeParams p, const CondDev 
         cell[i] = (unsigned)a;
     }
     const int k = i - (p.ncell + 1);
-    if (!p.far || k < 0 || k >= TR_MAT) return;
-    if (k < TR_MAT_128) {
-        const int j = k / (TR_M * TR_M), s = (k / TR_M) % TR_M, d = k % TR_M;
-        mat[k] = tr_basis(512, s, (double)(64 * j) + (double)tr_node(64, d));
-    } else if (k < TR_MAT_PT) {
-        const int q = k - TR_MAT_128, j = q / (TR_M * TR_M), s = (q / TR_M) % TR_M, d = q % TR_M;
-        mat[k] = tr_basis(128, s, (double)(64 * j) + (double)tr_node(64, d));
-    } else {
-        const int q = k - TR_MAT_PT;
-        mat[k] = tr_basis(64, q / 64, (double)(q % 64));
-    }
+    if (p.far && k >= 0 && k < TR_MAT) mat[k] = tr_mat_entry(k);
+}
+
+__global__ void __launch_bounds__(256) k_tree_mat(double *mat) {
+    const int k = blockIdx.x * 256 + threadIdx.x;
+    if (k < TR_MAT) mat[k] = tr_mat_entry(k);
+}
+
+cudaError_t launch_tree_mat(double *mat, cudaStream_t s) {
+    k_tree_mat<<<(TR_MAT + 255) / 256, 256, 0, s>>>(mat);
+    return cudaGetLastError();
 }
 
 // profile constants of every (condition, line) of the group
@@ -325,17 +232,19 @@ __global__ void __launch_bounds__(256) k_tree_recs(TreeParams p, float4 *recA, f
 }
 
 // ---------------------------------------------------------------------------
-// far levels: sums at the nodes.  A warp holds 16 nodes twice: its half-warps take different
-// lines.  Per 32 scanned lines the accepted ones are compacted into shared memory, pairs of
-// lines interleaved for the packed arithmetic; one iteration of the loop takes 4 lines.
+// far levels: sums at the nodes.  A lane holds two of the block's 16 nodes, and the four
+// quarter-warps take different lines.  Per 32 scanned lines the accepted ones are compacted
+// into shared memory, pairs of lines interleaved for the packed arithmetic; one iteration
+// takes 8 lines.  (With one node per lane and two line streams the loop was bound by the
+// shared-memory reads: 81 % of their rate at the 1e7-line list on 2e6 points, 1.65 ms.)
 // ---------------------------------------------------------------------------
 template <int PROF>
 __global__ void __launch_bounds__(TR_T) k_tree_nodes(TreeParams p) {
     constexpr int PAIR = tr_pairs<PROF>() ? (PROF == XC_VOIGT_W4 ? 3 : 2) : 2;   // 16-byte words per pair
     __shared__ float4 sL[TR_W][tr_pairs<PROF>() ? 16 * PAIR : 48];   // non-pairs: 24 bytes a line
     __shared__ float sX[64], sW[64];
-    __shared__ float2 sRed[TR_W][32];
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, half = lane >> 4;
+    __shared__ double sRed[TR_W][TR_M];
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, strm = lane >> 3;
     if (p.ngh > 0) {
         if (threadIdx.x < p.ngh) {
             sX[threadIdx.x] = (float)p.ghx[threadIdx.x];
@@ -356,21 +265,22 @@ __global__ void __launch_bounds__(TR_T) k_tree_nodes(TreeParams p) {
         }
     }
     const bool live = task < p.nblk[lev];
-    float hi = 0.f, lo = 0.f;
+    float hi[2] = {0.f, 0.f}, lo[2] = {0.f, 0.f};
     if (live) {
+        const float ac = p.cp[p.c0 + c].acoef;
         const int B = tr_block(lev), b0 = task * B, b1 = b0 + B - 1, b1c = min(b1, p.n_pts - 1);
-        const int D = tr_radius(p, lev, b1);
+        const int D = tr_radius(p, ac, tr_gap(lev), b1);
         const bool up = lev < 2;
         const int PB = up ? tr_block(lev + 1) : 1;
         const int p0 = up ? b0 / PB * PB : 0, p1 = p0 + PB - 1, p1c = min(p1, p.n_pts - 1);
-        const int Dp = up ? tr_radius(p, lev + 1, p1) : 0;
+        const int Dp = up ? tr_radius(p, ac, tr_gap(lev + 1), p1) : 0;
         const Segs sg = tr_far_segs(p, b0, b1, D, up, p0, p1, Dp);
-        const float x = tr_node(B, lane & 15);
-        const f32x2 x2 = pk2(x, x);
+        const float x[2] = {tr_node(B, 2 * (lane & 7)), tr_node(B, 2 * (lane & 7) + 1)};
+        const f32x2 xa = pk2(x[0], x[0]), xb = pk2(x[1], x[1]);
         const float4 *recA = p.recA + (size_t)c * p.n;
         float4 *buf = sL[warp];
-        f32x2 acc2 = 0ull;
-        float acc = 0.f;
+        f32x2 acca = 0ull, accb = 0ull;
+        float acc[2] = {0.f, 0.f};
         int in_fold = 0;
 #pragma unroll 1
         for (int k = 0; k < 4; ++k) {
@@ -392,7 +302,7 @@ __global__ void __launch_bounds__(TR_T) k_tree_nodes(TreeParams p) {
                 const unsigned m = __ballot_sync(0xffffffffu, ok);
                 const int cnt = __popc(m);
                 if (cnt) {
-                    const int pad = tr_pairs<PROF>() ? 4 : 2;
+                    const int pad = tr_pairs<PROF>() ? 8 : 4;
                     int slot = __popc(m & ((1u << lane) - 1u));
                     float n = (float)(g.x - b0), f = __int_as_float(g.w);
                     bool put = ok;
@@ -428,213 +338,89 @@ __global__ void __launch_bounds__(TR_T) k_tree_nodes(TreeParams p) {
                     }
                     __syncwarp();
                     if (tr_pairs<PROF>()) {
-#pragma unroll 2
-                        for (int j = half; 2 * j < cnt; j += 2) {
+                        for (int j = strm; 2 * j < cnt; j += 4) {
                             const ulonglong2 *q = reinterpret_cast<const ulonglong2 *>(buf + j * PAIR);
                             const ulonglong2 nf = q[0], c0 = q[1];
                             ulonglong2 c1 = c0;
                             if (PROF == XC_VOIGT_W4) c1 = q[2];
-                            const f32x2 d = sub2(sub2(x2, nf.x), nf.y);
-                            const f32x2 u = mul2(d, d);
-                            if (PROF == XC_VOIGT_W4)
-                                acc2 = fma2(fma2(c1.x, u, c1.y), rcp2(fma2(u, add2(u, c0.x), c0.y)), acc2);
-                            else
-                                acc2 = fma2(c0.y, rcp2(add2(u, c0.x)), acc2);
+                            const f32x2 da = sub2(sub2(xa, nf.x), nf.y), db = sub2(sub2(xb, nf.x), nf.y);
+                            const f32x2 ua = mul2(da, da), ub = mul2(db, db);
+                            if (PROF == XC_VOIGT_W4) {
+                                acca = fma2(fma2(c1.x, ua, c1.y), rcp2(fma2(ua, add2(ua, c0.x), c0.y)), acca);
+                                accb = fma2(fma2(c1.x, ub, c1.y), rcp2(fma2(ub, add2(ub, c0.x), c0.y)), accb);
+                            } else {
+                                acca = fma2(c0.y, rcp2(add2(ua, c0.x)), acca);
+                                accb = fma2(c0.y, rcp2(add2(ub, c0.x)), accb);
+                            }
                         }
                     } else {
-                        for (int j = half; j < cnt; j += 2) {
+                        for (int j = strm; j < cnt; j += 4) {
                             const float2 *q = reinterpret_cast<const float2 *>(buf) + j * 3;
                             const float2 nf = q[0], a01 = q[1], a23 = q[2];
-                            const float d = (x - nf.x) - nf.y;
-                            acc += contrib_single<PROF>(d * d, d, make_float4(a01.x, a01.y, a23.x, a23.y),
-                                                        make_float4(0.f, 0.f, 0.f, -1.f), sX, sW, p.ngh);
+                            const float4 Ac = make_float4(a01.x, a01.y, a23.x, a23.y);
+#pragma unroll
+                            for (int r = 0; r < 2; ++r) {
+                                const float d = (x[r] - nf.x) - nf.y;
+                                acc[r] += contrib_single<PROF>(d * d, d, Ac, make_float4(0.f, 0.f, 0.f, -1.f), sX, sW,
+                                                               p.ngh);
+                            }
                         }
                     }
                     __syncwarp();
                     if (++in_fold == TR_FOLD) {
                         if (tr_pairs<PROF>()) {
-                            acc = lo2(acc2) + lo2((acc2 >> 32) | (acc2 << 32));
-                            acc2 = 0ull;
+                            acc[0] = sum2(acca);
+                            acc[1] = sum2(accb);
+                            acca = accb = 0ull;
                         }
-                        tr_fold(hi, lo, acc);
+                        tr_fold(hi[0], lo[0], acc[0]);
+                        tr_fold(hi[1], lo[1], acc[1]);
                         in_fold = 0;
                     }
                 }
                 g = gn;
             }
         }
-        if (tr_pairs<PROF>()) acc = lo2(acc2) + lo2((acc2 >> 32) | (acc2 << 32));
-        tr_fold(hi, lo, acc);
+        if (tr_pairs<PROF>()) {
+            acc[0] = sum2(acca);
+            acc[1] = sum2(accb);
+        }
+        tr_fold(hi[0], lo[0], acc[0]);
+        tr_fold(hi[1], lo[1], acc[1]);
     }
-    // the half-warps' (and the task's warps') sums, in a fixed order
-    double v = (double)hi + (double)lo;
-    v += __shfl_xor_sync(0xffffffffu, v, 16);
+    // the line streams' (and the task's warps') sums, in a fixed order
+    double v[2];
+#pragma unroll
+    for (int r = 0; r < 2; ++r) {
+        v[r] = (double)hi[r] + (double)lo[r];
+        v[r] += __shfl_xor_sync(0xffffffffu, v[r], 8);
+        v[r] += __shfl_xor_sync(0xffffffffu, v[r], 16);
+    }
     if (wpt > 1) {
-        double *red = reinterpret_cast<double *>(sRed);
         __syncthreads();
-        red[warp * 32 + lane] = v;
+        if (lane < 8) {
+            sRed[warp][2 * lane] = v[0];
+            sRed[warp][2 * lane + 1] = v[1];
+        }
         __syncthreads();
-        if (part == 0)
-            for (int w = 1; w < wpt; ++w) v += red[(warp + w) * 32 + lane];
+        if (part == 0 && lane < 8)
+            for (int w = 1; w < wpt; ++w) {
+                v[0] += sRed[warp + w][2 * lane];
+                v[1] += sRed[warp + w][2 * lane + 1];
+            }
     }
-    if (live && part == 0 && half == 0)
-        p.nodes[(size_t)c * p.nodes_per_cond + p.node_off[lev] + task * TR_M + lane] = v;
+    if (live && part == 0 && lane < 8)
+        reinterpret_cast<double2 *>(p.nodes + (size_t)c * p.nodes_per_cond + p.node_off[lev] + task * TR_M)[lane] =
+            make_double2(v[0], v[1]);
 }
 
 // ---------------------------------------------------------------------------
-// points: the pairs no block takes, plus the interpolated sums.  A warp owns 32 points.  Lines
-// whose full-profile zone cannot reach the points go in packed pairs (region I, masked by the
-// cut), the others one by one with w4's regions per point.
+// points: the pairs no block takes, plus the interpolated sums.  A warp owns 32 points.
+// This kernel takes every profile but w4: Lorentzians in packed pairs of lines, masked by
+// the cut, the other profiles one line at a time.
 // ---------------------------------------------------------------------------
-template <int PROF>
-__global__ void __launch_bounds__(TR_T) k_tree_points(TreeParams p) {
-    constexpr bool W4 = PROF == XC_VOIGT_W4;
-    __shared__ float4 sF[TR_W][tr_pairs<PROF>() ? 16 * 4 : 1];   // pairs: n, f | cut ranges | constants
-    __shared__ float4 sC[TR_W][32 * (W4 ? 3 : 2)];               // singles: n, f, ka, kb | A | B
-    __shared__ float sX[64], sW[64];
-    __shared__ double sRed[TR_W][32];
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    if (p.ngh > 0) {
-        if (threadIdx.x < p.ngh) {
-            sX[threadIdx.x] = (float)p.ghx[threadIdx.x];
-            sW[threadIdx.x] = (float)p.ghw[threadIdx.x];
-        }
-        __syncthreads();
-    }
-    const int wpt = p.wpt, part = warp % wpt;
-    const int task = blockIdx.x * (TR_W / wpt) + warp / wpt;
-    const int c = blockIdx.y;
-    const int s0 = task * 32, s1 = s0 + 31;
-    const bool live = s0 < p.n_pts;
-    float hi = 0.f, lo = 0.f;
-    if (live) {
-        const int p0 = s0 & ~63, p1 = p0 + 63, p1c = min(p1, p.n_pts - 1);
-        const int Dp = p.far ? tr_radius(p, 0, p1) : 0;
-        // points within this of a line may need its full profile (w4's regions II to IV)
-        int core = 0;
-        if (W4) {
-            const float nu = fmaxf(__double2float_ru(__dadd_rn(grid_x(p.nu_A, p.step, p1), p.cutoff)), 0.f);
-            core = (int)ceilf(__fmul_ru(fminf(__fmul_ru(__fmul_ru(__uint_as_float(p.gs->acoef_bits), nu), p.inv_h), 1e6f),
-                                        p.core)) + 2;
-        }
-        const Segs sg = tr_point_segs(p, s0, s1, p0, p1, Dp);
-        const float x = (float)lane;
-        const f32x2 x2 = pk2(x, x);
-        const float4 *recA = p.recA + (size_t)c * p.n;
-        const float4 *recB = p.recB + (size_t)c * p.n;
-        float4 *bufF = sF[warp], *bufC = sC[warp];
-        f32x2 acc2 = 0ull;
-        float acc = 0.f;
-#pragma unroll 1
-        for (int k = 0; k < 3; ++k) {
-            const unsigned e = sg.e[k];
-            unsigned i = sg.s[k] + 32u * part;
-            int4 g = make_int4(0, 1, 0, 0);
-            if (i + lane < e) g = p.geo[i + lane];
-#pragma unroll 1
-            for (; i < e; i += 32u * wpt) {
-                const unsigned l = i + lane;
-                int4 gn = make_int4(0, 1, 0, 0);
-                if (l + 32u * wpt < e) gn = p.geo[l + 32u * wpt];
-                bool ok = l < e && g.y <= s1 && g.z >= s0 && g.y <= g.z &&
-                          !(p.far && tr_takes(g, p0, p1, p1c, Dp));
-                const bool cen = !tr_pairs<PROF>() || (W4 && g.x >= s0 - core && g.x <= s1 + core);
-                float4 A = make_float4(0.f, 0.f, 0.f, 0.f), Bv = make_float4(0.f, 0.f, 0.f, -1.f);
-                if (ok) {
-                    A = recA[l];
-                    if (W4 && cen) Bv = recB[l];
-                    ok = W4 && cen ? Bv.z != 0.f : tr_amplitude<PROF>(A) != 0.f;
-                }
-                const unsigned mc = __ballot_sync(0xffffffffu, ok && cen);
-                const unsigned mf = tr_pairs<PROF>() ? __ballot_sync(0xffffffffu, ok && !cen) : 0u;
-                if (mc | mf) {
-                    const unsigned below = (1u << lane) - 1u;
-                    const float n = (float)(g.x - s0), f = __int_as_float(g.w);
-                    const int ka = max(g.y - s0, 0), kb = min(g.z - s0, 31);
-                    if (ok && cen) {
-                        float4 *q = bufC + __popc(mc & below) * (W4 ? 3 : 2);
-                        q[0] = make_float4(n, f, __int_as_float(ka), __int_as_float(kb));
-                        q[1] = A;
-                        if (W4) q[2] = Bv;
-                    }
-                    if (tr_pairs<PROF>()) {
-                        const int cnt = __popc(mf);
-                        const bool fill = !(ok && !cen) && (cnt & 1) && __popc(~mf & below) == 0;
-                        if ((ok && !cen) || fill) {
-                            const int slot = fill ? cnt : __popc(mf & below);
-                            float *q = reinterpret_cast<float *>(bufF) + (slot >> 1) * 16 + (slot & 1);
-                            q[0] = fill ? -1e4f : n;
-                            q[2] = fill ? 0.f : f;
-                            q[4] = __int_as_float(fill ? 0 : ka);
-                            q[6] = __int_as_float(fill ? -1 : kb - ka);
-                            q[8] = fill ? 0.f : A.x;
-                            q[10] = fill ? 0.f : A.y;
-                            if (W4) {
-                                q[12] = fill ? 0.f : A.z;
-                                q[14] = fill ? 0.f : A.w;
-                            }
-                        }
-                    }
-                    __syncwarp();
-                    if (tr_pairs<PROF>()) {
-                        const int cnt = __popc(mf);
-#pragma unroll 2
-                        for (int j = 0; 2 * j < cnt; ++j) {
-                            const ulonglong2 *q = reinterpret_cast<const ulonglong2 *>(bufF + j * 4);
-                            const ulonglong2 nf = q[0], c0 = q[2];
-                            ulonglong2 c1 = c0;
-                            if (W4) c1 = q[3];
-                            const int4 kk = reinterpret_cast<const int4 *>(bufF + j * 4)[1];   // ka1 ka2 w1 w2
-                            const f32x2 d = sub2(sub2(x2, nf.x), nf.y);
-                            const f32x2 v = tr_pair_value<PROF>(mul2(d, d), c0, c1);
-                            float v1, v2;
-                            upk2(v, v1, v2);
-                            v1 = lane - kk.x >= 0 && lane - kk.x <= kk.z ? v1 : 0.f;
-                            v2 = lane - kk.y >= 0 && lane - kk.y <= kk.w ? v2 : 0.f;
-                            acc2 = add2(acc2, pk2(v1, v2));
-                        }
-                    }
-                    const int cnt = __popc(mc);
-                    for (int j = 0; j < cnt; ++j) {
-                        // a strong line's value in the sum makes the next ones' rounding: 16 a sum
-                        if ((j & 15) == 15) tr_fold(hi, lo, acc);
-                        const float4 *q = bufC + j * (W4 ? 3 : 2);
-                        const float4 t = q[0], a = q[1];
-                        const float d = (x - t.x) - t.y, u = d * d;
-                        if (lane < __float_as_int(t.z) || lane > __float_as_int(t.w)) continue;
-                        if (W4) {
-                            const float4 b = q[2];
-                            const float xx = b.x * fabsf(d), s = xx + b.y;
-                            if (u >= b.w)
-                                acc = fmaf(fmaf(a.z, u, a.w), rcp_approx(fmaf(u, u + a.x, a.y)), acc);
-                            else
-                                acc = fmaf(b.z, s >= 15.f ? w4_region1_re(xx, b.y)
-                                                          : (s >= 5.5f ? w4_region2_re(xx, b.y) : w4_region34_re(xx, b.y)),
-                                           acc);
-                        } else {
-                            acc += contrib_single<PROF>(u, d, a, make_float4(0.f, 0.f, 0.f, -1.f), sX, sW, p.ngh);
-                        }
-                    }
-                    __syncwarp();
-                    if (tr_pairs<PROF>()) {
-                        acc += lo2(acc2) + lo2((acc2 >> 32) | (acc2 << 32));
-                        acc2 = 0ull;
-                    }
-                    tr_fold(hi, lo, acc);
-                }
-                g = gn;
-            }
-        }
-    }
-    double v = (double)hi + (double)lo;
-    if (wpt > 1) {
-        __syncthreads();
-        sRed[warp][lane] = v;
-        __syncthreads();
-        if (part == 0)
-            for (int w = 1; w < wpt; ++w) v += sRed[warp + w][lane];
-    }
-    if (!live || part != 0) return;
+// the interpolated far field at the warp's 32 points (from s0) added to v, and the output
+__device__ __forceinline__ void tr_finish(const TreeParams &p, int c, int s0, int lane, double v) {
     if (p.far) {
         // node sums of the enclosing blocks, brought down to the level-0 block and to the points
         const double *nd = p.nodes + (size_t)c * p.nodes_per_cond;
@@ -660,6 +446,349 @@ __global__ void __launch_bounds__(TR_T) k_tree_points(TreeParams p) {
         const CParam &cp = p.cp[p.c0 + c];
         p.sigma[(size_t)cp.row * (size_t)p.n_pts + k] = v * cp.inv_scale;
     }
+}
+
+template <int PROF>
+__global__ void __launch_bounds__(TR_T) k_tree_points(TreeParams p) {
+    constexpr bool PAIRS = tr_pairs<PROF>();
+    __shared__ float4 sL[TR_W][PAIRS ? 16 * 3 : 32 * 2];   // pairs: n, f | cut ranges | constants; singles: n, f, ka, kb | A
+    __shared__ float sX[64], sW[64];
+    __shared__ double sRed[TR_W][32];
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    if (p.ngh > 0) {
+        if (threadIdx.x < p.ngh) {
+            sX[threadIdx.x] = (float)p.ghx[threadIdx.x];
+            sW[threadIdx.x] = (float)p.ghw[threadIdx.x];
+        }
+        __syncthreads();
+    }
+    const int wpt = p.wpt, part = warp % wpt;
+    const int task = blockIdx.x * (TR_W / wpt) + warp / wpt;
+    const int c = blockIdx.y;
+    const int s0 = task * 32, s1 = s0 + 31;
+    const bool live = s0 < p.n_pts;
+    float hi = 0.f, lo = 0.f;
+    if (live) {
+        const int p0 = s0 & ~63, p1 = p0 + 63, p1c = min(p1, p.n_pts - 1);
+        const int Dp = p.far ? tr_radius(p, p.cp[p.c0 + c].acoef, tr_gap(0), p1) : 0;
+        const Segs sg = tr_point_segs(p, s0, s1, p0, p1, Dp);
+        const float x = (float)lane;
+        const f32x2 x2 = pk2(x, x);
+        const float4 *recA = p.recA + (size_t)c * p.n;
+        float4 *buf = sL[warp];
+#pragma unroll 1
+        for (int k = 0; k < 3; ++k) {
+            const unsigned e = sg.e[k];
+            unsigned i = sg.s[k] + 32u * part;
+            int4 g = make_int4(0, 1, 0, 0);
+            if (i + lane < e) g = p.geo[i + lane];
+#pragma unroll 1
+            for (; i < e; i += 32u * wpt) {
+                const unsigned l = i + lane;
+                int4 gn = make_int4(0, 1, 0, 0);
+                if (l + 32u * wpt < e) gn = p.geo[l + 32u * wpt];
+                bool ok = l < e && g.y <= s1 && g.z >= s0 && g.y <= g.z &&
+                          !(p.far && tr_takes(g, p0, p1, p1c, Dp));
+                float4 A = make_float4(0.f, 0.f, 0.f, 0.f);
+                if (ok) {
+                    A = recA[l];
+                    ok = tr_amplitude<PROF>(A) != 0.f;
+                }
+                const unsigned m = __ballot_sync(0xffffffffu, ok);
+                if (m) {
+                    const unsigned below = (1u << lane) - 1u;
+                    const int cnt = __popc(m);
+                    const float n = (float)(g.x - s0), f = __int_as_float(g.w);
+                    const int ka = max(g.y - s0, 0), kb = min(g.z - s0, 31);
+                    float acc = 0.f;
+                    if (PAIRS) {
+                        const bool fill = !ok && (cnt & 1) && __popc(~m & below) == 0;   // completes the last pair
+                        if (ok || fill) {
+                            const int slot = fill ? cnt : __popc(m & below);
+                            float *q = reinterpret_cast<float *>(buf) + (slot >> 1) * 12 + (slot & 1);
+                            q[0] = fill ? -1e4f : n;
+                            q[2] = fill ? 0.f : f;
+                            q[4] = __int_as_float(fill ? 0 : ka);
+                            q[6] = __int_as_float(fill ? -1 : kb - ka);
+                            q[8] = fill ? 0.f : A.x;
+                            q[10] = fill ? 0.f : A.y;
+                        }
+                        __syncwarp();
+                        f32x2 acc2 = 0ull;
+#pragma unroll 2
+                        for (int j = 0; 2 * j < cnt; ++j) {
+                            const ulonglong2 *q = reinterpret_cast<const ulonglong2 *>(buf + j * 3);
+                            const ulonglong2 nf = q[0], c0 = q[2];
+                            const int4 kk = reinterpret_cast<const int4 *>(buf + j * 3)[1];   // ka1 ka2 w1 w2
+                            const f32x2 d = sub2(sub2(x2, nf.x), nf.y);
+                            float v1, v2;
+                            upk2(mul2(c0.y, rcp2(add2(mul2(d, d), c0.x))), v1, v2);
+                            v1 = lane - kk.x >= 0 && lane - kk.x <= kk.z ? v1 : 0.f;
+                            v2 = lane - kk.y >= 0 && lane - kk.y <= kk.w ? v2 : 0.f;
+                            acc2 = add2(acc2, pk2(v1, v2));
+                        }
+                        acc = sum2(acc2);
+                    } else {
+                        if (ok) {
+                            float4 *q = buf + __popc(m & below) * 2;
+                            q[0] = make_float4(n, f, __int_as_float(ka), __int_as_float(kb));
+                            q[1] = A;
+                        }
+                        __syncwarp();
+                        for (int j = 0; j < cnt; ++j) {
+                            // a strong line's value in the sum makes the next ones' rounding: 16 a sum
+                            if ((j & 15) == 15) tr_fold(hi, lo, acc);
+                            const float4 t = buf[2 * j], a = buf[2 * j + 1];
+                            const float d = (x - t.x) - t.y;
+                            if (lane >= __float_as_int(t.z) && lane <= __float_as_int(t.w))
+                                acc += contrib_single<PROF>(d * d, d, a, make_float4(0.f, 0.f, 0.f, -1.f), sX, sW, p.ngh);
+                        }
+                    }
+                    __syncwarp();
+                    tr_fold(hi, lo, acc);
+                }
+                g = gn;
+            }
+        }
+    }
+    double v = (double)hi + (double)lo;
+    if (wpt > 1) {
+        __syncthreads();
+        sRed[warp][lane] = v;
+        __syncthreads();
+        if (part == 0)
+            for (int w = 1; w < wpt; ++w) v += sRed[warp + w][lane];
+    }
+    if (live && part == 0) tr_finish(p, c, s0, lane, v);
+}
+
+// Voigt w4 at the points.  Per 32 scanned lines, each lane classifies its line for the warp's
+// 32 points and the lines go three ways:
+//   F  region I at every point of the warp: packed pairs of lines, masked by the cut;
+//   Z  the zone |x| + y < 15 reaches the points: packed pairs that evaluate regions I and II
+//      and select per point (region I is skipped where no point needs it);
+//   items  the points in regions III and IV, which are few per line and costly: numbered line
+//      after line, region by region, and evaluated 32 at a time with one region per warp
+//      instruction; their owner lanes then add them in line order.
+// One line at a time with a branch per region left 22 of 32 lanes active and paid for up to
+// four regions per line: 6.4 ms at the 1e7-line list on 2e6 points.
+struct W4Buf {
+    float4 F[16 * 4];       // per pair: n, f | E, F | P, PC | masks
+    float4 Z[16 * 6];       // per pair: n, f | E, F | P, PC | a^2, y^2 | y Pv, t2 | masks
+    float4 I[2][32];        // per line with items of region III / IV: n, f, a, y
+    int4 R[2][32];          // first item, first point, points of the left run, Pv (bits)
+    int2 S[2][32];          // first point of the right run, number of items
+};
+
+
+__global__ void __launch_bounds__(TR_T) k_tree_points_w4(TreeParams p) {
+    __shared__ W4Buf sBuf[TR_W];
+    __shared__ double sRed[TR_W][32];
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int wpt = p.wpt, part = warp % wpt;
+    const int task = blockIdx.x * (TR_W / wpt) + warp / wpt;
+    const int c = blockIdx.y;
+    const int s0 = task * 32, s1 = s0 + 31;
+    const bool live = s0 < p.n_pts;
+    float hi = 0.f, lo = 0.f;
+    if (live) {
+        const int p0 = s0 & ~63, p1 = p0 + 63, p1c = min(p1, p.n_pts - 1);
+        const int Dp = tr_radius(p, p.cp[p.c0 + c].acoef, tr_gap(0), p1);
+        const Segs sg = tr_point_segs(p, s0, s1, p0, p1, Dp);
+        const float x = (float)lane;
+        const f32x2 x2 = pk2(x, x);
+        const unsigned below = (1u << lane) - 1u;
+        const float4 *recA = p.recA + (size_t)c * p.n;
+        const float4 *recB = p.recB + (size_t)c * p.n;
+        W4Buf &buf = sBuf[warp];
+#pragma unroll 1
+        for (int k = 0; k < 3; ++k) {
+            const unsigned e = sg.e[k];
+            unsigned i = sg.s[k] + 32u * part;
+            int4 g = make_int4(0, 1, 0, 0);
+            if (i + lane < e) g = p.geo[i + lane];
+#pragma unroll 1
+            for (; i < e; i += 32u * wpt) {
+                const unsigned l = i + lane;
+                int4 gn = make_int4(0, 1, 0, 0);
+                if (l + 32u * wpt < e) gn = p.geo[l + 32u * wpt];
+                const bool ok = l < e && g.y <= s1 && g.z >= s0 && g.y <= g.z && !tr_takes(g, p0, p1, p1c, Dp);
+                if (!__any_sync(0xffffffffu, ok)) {
+                    g = gn;
+                    continue;
+                }
+                float4 A = make_float4(0.f, 0.f, 0.f, 0.f), B = make_float4(1.f, 1.f, 0.f, -1.f);
+                if (ok) {
+                    A = recA[l];
+                    B = recB[l];
+                }
+                const float n = (float)(g.x - s0), f = __int_as_float(g.w), pos = n + f;
+                const int ka = max(g.y - s0, 0), kb = min(g.z - s0, 31);
+                const unsigned cut = ok ? lanes_of(ka, kb) : 0u;
+                // zone |x| + y < 15 (with a margin: the points decide by u < t2 themselves)
+                const float rz = sqrtf(fmaxf(B.w, 0.f)) + 0.1f;
+                const bool zone = ok && B.w > 0.f && pos + rz >= 0.f && pos - rz <= 31.f;
+                // points of regions III and IV, |x| + y < 5.5: runs of lanes around the centre
+                unsigned m3 = 0u, m34 = 0u;
+                int k0 = 0, k1 = -1, k30 = 0, k31 = -1;
+                if (zone && B.y < 5.5f && B.z != 0.f) {
+                    const float ra = rcp_approx(B.x);
+                    const float r34 = (5.5f - B.y) * ra, r3 = fminf(r34, (B.y + 0.176f) * (1.f / 0.195f) * ra);
+                    k0 = max((int)ceilf(fmaxf(pos - r34, -1.f)), ka);
+                    k1 = min((int)floorf(fminf(pos + r34, 32.f)), kb);
+                    k30 = max((int)ceilf(fmaxf(pos - r3, -1.f)), k0);
+                    k31 = min((int)floorf(fminf(pos + r3, 32.f)), k1);
+                    m34 = lanes_of(k0, k1);
+                    m3 = lanes_of(k30, k31);
+                }
+                const unsigned m4 = m34 & ~m3, m12 = cut & ~m34;
+                const bool isZ = zone && m12 != 0u && A.z != 0.f, isF = ok && !zone && A.z != 0.f;
+                const unsigned bF = __ballot_sync(0xffffffffu, isF), bZ = __ballot_sync(0xffffffffu, isZ);
+                const unsigned b3 = __ballot_sync(0xffffffffu, m3 != 0u), b4 = __ballot_sync(0xffffffffu, m4 != 0u);
+                const int nF = __popc(bF), nZ = __popc(bZ);
+                if (isF) {
+                    const int slot = __popc(bF & below);
+                    float *q = reinterpret_cast<float *>(buf.F) + (slot >> 1) * 16 + (slot & 1);
+                    q[0] = n;
+                    q[2] = f;
+                    q[4] = A.x;
+                    q[6] = A.y;
+                    q[8] = A.z;
+                    q[10] = A.w;
+                    q[12] = __uint_as_float(cut);
+                }
+                if (isZ) {
+                    const int slot = __popc(bZ & below);
+                    float *q = reinterpret_cast<float *>(buf.Z) + (slot >> 1) * 24 + (slot & 1);
+                    q[0] = n;
+                    q[2] = f;
+                    q[4] = A.x;
+                    q[6] = A.y;
+                    q[8] = A.z;
+                    q[10] = A.w;
+                    q[12] = B.x * B.x;
+                    q[14] = B.y * B.y;
+                    q[16] = B.y * B.z;
+                    q[18] = B.w;
+                    q[20] = __uint_as_float(m12);
+                }
+                // a pair without a second line: nothing of it is selected
+                if (lane == 0 && (nF & 1)) reinterpret_cast<float *>(buf.F)[(nF >> 1) * 16 + 13] = 0.f;
+                if (lane == 1 && (nZ & 1)) reinterpret_cast<float *>(buf.Z)[(nZ >> 1) * 24 + 21] = 0.f;
+                int tot[2];
+#pragma unroll
+                for (int t = 0; t < 2; ++t) {   // III, IV
+                    const unsigned m = t == 0 ? m3 : m4;
+                    tot[t] = 0;
+                    if ((t == 0 ? b3 : b4) == 0u) continue;
+                    const int ni = __popc(m);
+                    int off = ni;
+#pragma unroll
+                    for (int o = 1; o < 32; o <<= 1) {
+                        const int v = __shfl_up_sync(0xffffffffu, off, o);
+                        if (lane >= o) off += v;
+                    }
+                    tot[t] = __shfl_sync(0xffffffffu, off, 31);
+                    if (ni > 0) {
+                        const int slot = __popc((t == 0 ? b3 : b4) & below);
+                        buf.I[t][slot] = make_float4(n, f, B.x, B.y);
+                        const bool split = t == 1 && m3 != 0u;
+                        const int left = t == 0 ? ni : (split ? k30 - k0 : ni);
+                        buf.R[t][slot] = make_int4(off - ni, t == 0 ? k30 : k0, left, __float_as_int(B.z));
+                        buf.S[t][slot] = make_int2(k31 + 1, ni);
+                    }
+                }
+                __syncwarp();
+                float acc = 0.f;
+                {
+                    f32x2 acc2 = 0ull;
+#pragma unroll 2
+                    for (int j = 0; 2 * j < nF; ++j) {
+                        const ulonglong2 *q = reinterpret_cast<const ulonglong2 *>(buf.F + j * 4);
+                        const ulonglong2 nf = q[0], c0 = q[1], c1 = q[2];
+                        const uint2 mk = *reinterpret_cast<const uint2 *>(buf.F + j * 4 + 3);
+                        const f32x2 d = sub2(sub2(x2, nf.x), nf.y), u = mul2(d, d);
+                        float v1, v2;
+                        upk2(mul2(fma2(c1.x, u, c1.y), rcp2(fma2(u, add2(u, c0.x), c0.y))), v1, v2);
+                        v1 = (mk.x >> lane) & 1u ? v1 : 0.f;
+                        v2 = (mk.y >> lane) & 1u ? v2 : 0.f;
+                        acc2 = add2(acc2, pk2(v1, v2));
+                    }
+                    acc = sum2(acc2);
+                    tr_fold(hi, lo, acc);
+                }
+                if (nZ) {
+                    f32x2 acc2 = 0ull;
+                    for (int j = 0; 2 * j < nZ; ++j) {
+                        const ulonglong2 *q = reinterpret_cast<const ulonglong2 *>(buf.Z + j * 6);
+                        const ulonglong2 nf = q[0], c0 = q[1], c1 = q[2], ay = q[3], pt = q[4];
+                        const uint2 mk = *reinterpret_cast<const uint2 *>(buf.Z + j * 6 + 5);
+                        const f32x2 d = sub2(sub2(x2, nf.x), nf.y), u = mul2(d, d);
+                        float u1, u2, t1, t2, v1, v2;
+                        upk2(u, u1, u2);
+                        upk2(pt.y, t1, t2);
+                        upk2(w4_region2_pair(mul2(u, ay.x), ay.y, pt.x), v1, v2);
+                        const bool r1 = u1 >= t1, r2 = u2 >= t2;
+                        if (__any_sync(0xffffffffu, r1 || r2)) {
+                            float w1, w2;
+                            upk2(mul2(fma2(c1.x, u, c1.y), rcp2(fma2(u, add2(u, c0.x), c0.y))), w1, w2);
+                            v1 = r1 ? w1 : v1;
+                            v2 = r2 ? w2 : v2;
+                        }
+                        v1 = (mk.x >> lane) & 1u ? v1 : 0.f;
+                        v2 = (mk.y >> lane) & 1u ? v2 : 0.f;
+                        acc2 = add2(acc2, pk2(v1, v2));
+                    }
+                    acc = sum2(acc2);
+                    tr_fold(hi, lo, acc);
+                }
+#pragma unroll
+                for (int t = 0; t < 2; ++t) {
+                    int line0 = 0;                      // lines whose items start before this batch
+                    for (int b = 0; b < tot[t]; b += 32) {
+                        // lines whose first item lies in this batch: a bit at that item
+                        int first = -1;
+                        if (lane < __popc(t == 0 ? b3 : b4)) first = buf.R[t][lane].x - b;
+                        const unsigned starts = __reduce_or_sync(0xffffffffu, first >= 0 && first < 32 ? 1u << first : 0u);
+                        const int line = line0 + __popc(starts & (below | (1u << lane))) - 1;
+                        float v = 0.f;
+                        if (b + lane < tot[t]) {
+                            const float4 q = buf.I[t][line];
+                            const int4 r = buf.R[t][line];
+                            const int o = b + lane - r.x;
+                            const int kp = o < r.z ? r.y + o : buf.S[t][line].x + o - r.z;
+                            const float xx = q.z * fabsf(((float)kp - q.x) - q.y);
+                            v = __int_as_float(r.w) * (t == 0 ? w4_region3_re(xx, q.w) : w4_region4_re(xx, q.w));
+                        }
+                        // owners add their points' values, line after line
+                        const int jl = __shfl_sync(0xffffffffu, line, min(31, tot[t] - 1 - b));
+                        for (int j = __shfl_sync(0xffffffffu, line, 0); j <= jl; ++j) {
+                            const int4 r = buf.R[t][j];
+                            const int2 s2 = buf.S[t][j];
+                            int o = lane - r.y;
+                            if (o >= r.z) o = lane - s2.x >= 0 ? lane - s2.x + r.z : -1;
+                            const int it = r.x + o - b;
+                            const float w = __shfl_sync(0xffffffffu, v, it & 31);
+                            if (o >= 0 && o < s2.y && it >= 0 && it < 32) acc += w;
+                        }
+                        tr_fold(hi, lo, acc);
+                        line0 += __popc(starts);
+                    }
+                }
+                __syncwarp();
+                g = gn;
+            }
+        }
+    }
+    double v = (double)hi + (double)lo;
+    if (wpt > 1) {
+        __syncthreads();
+        sRed[warp][lane] = v;
+        __syncthreads();
+        if (part == 0)
+            for (int w = 1; w < wpt; ++w) v += sRed[warp + w][lane];
+    }
+    if (live && part == 0) tr_finish(p, c, s0, lane, v);
 }
 
 // ---------------------------------------------------------------------------
@@ -693,7 +822,9 @@ bool fns_of(int profile, ProfFns *f) {
     switch (profile) {
     case XC_DOPPLER: *f = ProfFns TR_FNS(XC_DOPPLER); return true;
     case XC_LORENTZ: *f = ProfFns TR_FNS(XC_LORENTZ); return true;
-    case XC_VOIGT_W4: *f = ProfFns TR_FNS(XC_VOIGT_W4); return true;
+    case XC_VOIGT_W4:
+        *f = ProfFns{k_tree_recs<XC_VOIGT_W4, false>, k_tree_recs<XC_VOIGT_W4, true>, k_tree_nodes<XC_VOIGT_W4>, k_tree_points_w4};
+        return true;
     case XC_VOIGT_GH_BINNED: *f = ProfFns TR_FNS(XC_VOIGT_GH_BINNED); return true;
     case XC_VOIGT_GH_SAMPLED: *f = ProfFns TR_FNS(XC_VOIGT_GH_SAMPLED); return true;
     case XC_DOPPLER_BINNED: *f = ProfFns TR_FNS(XC_DOPPLER_BINNED); return true;
@@ -819,7 +950,7 @@ xc_status tree_run(BatchedState *st, const BatchedArgs &a, int64_t *launches) {
         p.sigma = a.sigma + (size_t)pass * (size_t)a.grid.n;
         p.L = a.L;
         unsigned *gmax = nullptr;
-        k_tree_prep<<<1, 32, 0, s>>>(conds, nc_pass, gs);
+        TR_TRY(launch_tree_prep(conds, nc_pass, gs, s));
         if (a.L.n_broad > 0) {
             gmax = (unsigned *)(b + o_gmax);
             TR_TRY(cudaMemsetAsync(gmax, 0, (size_t)nc_pass * 4, s));
