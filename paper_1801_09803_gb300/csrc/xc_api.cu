@@ -315,7 +315,14 @@ xc_status cross_section_f64(xc_handle *h, const CondDev *dcond, const xc_grid *g
         return XC_OK;
     }
     XC_TRY_MEM(h->params.ensure(n * 4 * sizeof(double)));
-    XC_TRY_MEM(h->ranges.ensure(n_win * 2 * sizeof(int64_t)));
+    // the block-interpolated form (the Vectorized Voigt is not smooth at its split: direct sum),
+    // unless its 16 bytes per line do not fit next to a very large list
+    bool tree = tree64_takes(o->profile, *g, o->cutoff, n);
+    if (tree && h->ranges.ensure(tree64_scratch(*g, o->cutoff, n)) != cudaSuccess) {
+        cudaGetLastError();
+        tree = false;
+    }
+    if (!tree) XC_TRY_MEM(h->ranges.ensure(n_win * 2 * sizeof(int64_t)));
     double *I = h->params.as<double>(), *al = I + n, *ga = al + n, *cut = ga + n;
     int64_t *lo = h->ranges.as<int64_t>(), *hi = lo + n_win;
     stage_begin(h, ST_PARAMS, s);
@@ -323,7 +330,7 @@ xc_status cross_section_f64(xc_handle *h, const CondDev *dcond, const xc_grid *g
                                 ga, cut, s, strength_sel(*o)));
     stage_end(h, ST_PARAMS, s);
     stage_begin(h, ST_RANGES, s);
-    XC_TRY(launch_window_ranges(h->nu, n, g->nu_A, g->step, g->n, W, o->cutoff, n_win, lo, hi, s));
+    if (!tree) XC_TRY(launch_window_ranges(h->nu, n, g->nu_A, g->step, g->n, W, o->cutoff, n_win, lo, hi, s));
     stage_end(h, ST_RANGES, s);
     const double *ghx = nullptr, *ghw = nullptr;
     if (o->profile == XC_VOIGT_GH_BINNED || o->profile == XC_VOIGT_GH_SAMPLED) {
@@ -339,6 +346,13 @@ xc_status cross_section_f64(xc_handle *h, const CondDev *dcond, const xc_grid *g
         h->launches += 1;
     }
     stage_begin(h, ST_PROFILE, s);
+    if (tree) {
+        XC_TRY(launch_tree64(o->profile, h->nu, I, al, ga, cut, n, dcond, *g, o->cutoff, o->width_mult <= 0.0, ghx, ghw,
+                             ghx ? o->n_gh : 0, h->ranges.p, sig, &h->launches, s));
+        stage_end(h, ST_PROFILE, s);
+        h->launches += 1;
+        return XC_OK;
+    }
     XC_TRY(launch_gather_f64(o->profile, h->nu, I, al, ga, cut, lo, hi, n_win, g->nu_A, g->step, g->n, ghx, ghw,
                              ghx ? o->n_gh : 0, sig, s, vv_split, vv_beta));
     stage_end(h, ST_PROFILE, s);
