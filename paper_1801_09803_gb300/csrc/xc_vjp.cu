@@ -44,6 +44,7 @@
 #include <algorithm>
 
 #include "xc_batched.cuh"
+#include "xc_tree.cuh"
 
 namespace xc {
 
@@ -243,20 +244,24 @@ __global__ void __launch_bounds__(VT) k_vjp_lines(LinesDev L, size_t n, const Co
     }
 }
 
-// sum block partials in block order: quantity q of this chunk's condition c (values
+// sum the block partials in a fixed order: quantity q of this chunk's condition c (values
 // [blk][nc][NQ]) -> its output row (rows[c], or c0 + c when rows is null).  acc holds per
 // row: gamma_scale and n_shift sums, then 2 nb per-broadener sums.
-__global__ void k_vjp_finish(const double *block_part, int n_blocks, int nc, int NQ, int c0, const CParam *rows,
-                             double *dT, double *dP, double *acc) {
-    for (int i = threadIdx.x; i < nc * NQ; i += blockDim.x) {
-        const int c = i / NQ, q = i % NQ;
-        double s = 0.0;
-        for (int b = 0; b < n_blocks; ++b) s += block_part[((size_t)b * nc + c) * NQ + q];
-        const int r = rows ? rows[c].row : c0 + c;
-        if (q == 0) dT[r] = s;
-        else if (q == 1) dP[r] = s;
-        else acc[(size_t)r * (NQ - 2) + (q - 2)] = s;
-    }
+__global__ void __launch_bounds__(128) k_vjp_finish(const double *block_part, int n_blocks, int nc, int NQ, int c0,
+                                                    const CParam *rows, double *dT, double *dP, double *acc) {
+    // one warp per sum: lane j takes blocks j, j + 32, ..., then a fixed butterfly
+    const int lane = threadIdx.x & 31;
+    const int i = blockIdx.x * 4 + (threadIdx.x >> 5);
+    if (i >= nc * NQ) return;
+    const int c = i / NQ, q = i % NQ;
+    double s = 0.0;
+    for (int b = lane; b < n_blocks; b += 32) s += block_part[((size_t)b * nc + c) * NQ + q];
+    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+    if (lane) return;
+    const int r = rows ? rows[c].row : c0 + c;
+    if (q == 0) dT[r] = s;
+    else if (q == 1) dP[r] = s;
+    else acc[(size_t)r * (NQ - 2) + (q - 2)] = s;
 }
 
 // global scalars and per-broadener sums: sums over conditions in order
@@ -397,6 +402,76 @@ __device__ __forceinline__ F2 f2_warp_sum(F2 v) {
     return v;
 }
 
+__device__ __forceinline__ F2 f2_scale(F2 a, float k) {
+    const float h = __fmul_rn(a.hi, k);
+    return F2{h, fmaf(a.lo, k, fmaf(a.hi, k, -h))};
+}
+__device__ __forceinline__ F2 f2_of(const KahanF &k) { return F2{k.s, -k.c}; }
+
+// Sums of one line and condition over grid points or block nodes, without their constant
+// factors, and the profile's constants in grid units.
+template <int PROF>
+struct VjpLine {
+    float a_h, g_h, g2, C, g4, asc, y, thr2, ia2;
+    const float *gx, *gw;
+    int ngh;
+    __device__ __forceinline__ VjpLine(float a, float g, const float *sx, const float *sw, int n)
+        : a_h(a), g_h(g), gx(sx), gw(sw), ngh(n) {
+        g2 = g * g;
+        if (PROF == XC_VOIGT_W4) {
+            asc = kSqrtLn2f * rcp_approx(a);                 // x = asc |delta|
+            y = asc * g;
+            C = a * a * (float)(0.5 / 0.6931471805599453) + g2;
+            g4 = 4.f * g2;
+            const float thr = (15.f - y) * rcp_approx(asc);
+            thr2 = y < 15.f ? thr * thr : -1.f;              // region I iff u >= thr2
+        } else if (PROF == XC_DOPPLER) {
+            ia2 = rcp_approx(a * a);
+        }
+    }
+    // one point (or node) at offset dl with weight gk
+    __device__ __forceinline__ void add(float dl, float gk, float &q0, float &q1, float &q2) const {
+        const float u = dl * dl;
+        if (PROF == XC_VOIGT_W4) {
+            const float t = C - u;
+            const float rD = rcp_approx(fmaf(t, t, g4 * u));
+            const float w = (u + C) * rD;
+            q0 = fmaf(gk, w, q0);
+            q1 = fmaf(gk, rD * fmaf(-2.f * t, w, 1.f), q1);
+            q2 = fmaf(gk, u * w * rD, q2);
+        } else if (PROF == XC_VOIGT_GH_BINNED) {
+            // bin average of the Gauss-Hermite Voigt (Eq. e:sigma:quad), grid units (bin width 1):
+            // per node j, s+ = delta + 1/2 - a x_j/sqrt(ln2), s- = s+ - 1, Q+- = s+-^2 + g^2,
+            //   V = pi^(-3/2) sum_j w_j atan2(g, g^2 + s+ s-),
+            //   dV/dg = pi^(-3/2) sum_j w_j (s+ s- - g^2)/(Q+ Q-),
+            //   dV/da = pi^(-3/2) sum_j w_j (x_j/sqrt(ln2)) g (s+ + s-)/(Q+ Q-)
+            const float d = dl + 0.5f;
+            float v = 0.f, da = 0.f, dg = 0.f;
+            for (int m = 0; m < ngh; ++m) {
+                const float sp = fmaf(-a_h, gx[m], d), sm = sp - 1.f;
+                const float iQ = rcp_approx(fmaf(sp, sp, g2) * fmaf(sm, sm, g2));
+                v = fmaf(gw[m], atan2_ypos(g_h, fmaf(sp, sm, g2)), v);
+                dg = fmaf(gw[m], fmaf(sp, sm, -g2) * iQ, dg);
+                da = fmaf(gw[m] * gx[m], (sp + sm) * iQ, da);
+            }
+            q0 = fmaf(gk, v, q0);
+            q1 = fmaf(gk, da, q1);
+            q2 = fmaf(gk, dg, q2);
+        } else if (PROF == XC_DOPPLER) {
+            // V = sqrt(ln2/pi)/a 2^(-u/a^2): sums of g 2^(-u/a^2) and g u 2^(-u/a^2)
+            const float e = ex2_approx(-u * ia2) * gk;
+            q0 += e;
+            q1 = fmaf(e, u, q1);
+        } else {
+            // Lorentz: V = (1/pi) g/(u + g^2), dV/dg = (1/pi)(u - g^2)/(u + g^2)^2
+            const float r = rcp_approx(u + g2);
+            const float gr = gk * r;
+            q0 += gr;
+            q2 = fmaf(gr, (u - g2) * r, q2);
+        }
+    }
+};
+
 struct Vjp32Params {
     LinesDev L;
     size_t n;
@@ -413,7 +488,43 @@ struct Vjp32Params {
     int accumulate;                       // add to the per-line outputs (later condition chunks)
     const double *ghx, *ghw;              // Gauss-Hermite nodes and weights (binned GH), device
     int ngh;
+    const float *gnode;                   // dL/dsigma projected on the block nodes (see k_vjp_nodes), or nullptr
+    int node_off[TR_LEVELS], nodes_per_cond;   // [caller row][nodes_per_cond], level l from node_off[l]
 };
+
+// dL/dsigma projected on the nodes of the blocks of xc_tree.cu: with V(k) = sum_m L_m(k) V(m)
+// on a block, sum_k g_k V(k) = sum_m V(m) g(m), g(m) = sum_k L_m(k) g_k.  One CTA per
+// 512-point block and condition: its eight 64-point blocks from the points, then the 128- and
+// 512-point ones from those (the transposes of the sweep's matrices), in FP64.
+__global__ void __launch_bounds__(128) k_vjp_nodes(const double *__restrict__ g, int64_t n_pts,
+                                                   const double *__restrict__ mat, float *gnode, int off0, int off1,
+                                                   int off2, int per_cond) {
+    __shared__ double sG[512], s0[128];
+    const int j = blockIdx.x, t = threadIdx.x;
+    const double *gc = g + (size_t)blockIdx.y * (size_t)n_pts;
+    float *out = gnode + (size_t)blockIdx.y * per_cond;
+    for (int i = t; i < 512; i += 128) sG[i] = 512 * (int64_t)j + i < n_pts ? gc[512 * (int64_t)j + i] : 0.0;
+    __syncthreads();
+    {
+        const int b = t >> 4, m = t & 15;
+        double s = 0.0;
+        for (int k = 0; k < 64; ++k) s = fma(mat[TR_MAT_PT + m * 64 + k], sG[64 * b + k], s);
+        s0[t] = s;
+        out[off0 + j * 128 + t] = (float)s;
+    }
+    __syncthreads();
+    if (t < 64) {
+        const int b = t >> 4, m = t & 15;
+        double s = 0.0;
+        for (int i = 0; i < 32; ++i) s = fma(mat[TR_MAT_128 + ((i >> 4) * TR_M + m) * TR_M + (i & 15)], s0[32 * b + i], s);
+        out[off1 + j * 64 + t] = (float)s;
+    } else if (t < 80) {
+        const int m = t - 64;
+        double s = 0.0;
+        for (int i = 0; i < 128; ++i) s = fma(mat[TR_MAT_512 + ((i >> 4) * TR_M + m) * TR_M + (i & 15)], s0[i], s);
+        out[off2 + j * 16 + m] = (float)s;
+    }
+}
 
 // MIX: the Lorentz widths come from the handle's mixture of broadeners (per broadener
 // and line rho_i gamma_0,i and n_i): gamma = gamma_scale P/P_ref sum_i rho_i gamma_0,i
@@ -425,6 +536,12 @@ __global__ void __launch_bounds__(VT) k_vjp32(Vjp32Params p) {
     __shared__ double s_part[VW][VMAXC][4];
     __shared__ double s_broad[VW][VMAXC][MIX ? 2 * VMAXB : 1];
     __shared__ float s_gx[PROF == XC_VOIGT_GH_BINNED ? 64 : 1], s_gw[PROF == XC_VOIGT_GH_BINNED ? 64 : 1];
+    __shared__ float s_node[TR_LEVELS][TR_M];
+    // the outermost Gauss-Hermite node lies within sqrt(2 n + 2) (a_h / sqrt(ln 2)) of the centre
+    const float s_ext = sqrtf(2.f * (float)p.ngh + 2.f) * 1.203f;
+    if (threadIdx.x < TR_LEVELS * TR_M)
+        s_node[threadIdx.x / TR_M][threadIdx.x % TR_M] = tr_node(tr_block(threadIdx.x / TR_M), threadIdx.x % TR_M);
+    __syncthreads();
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     if (PROF == XC_VOIGT_GH_BINNED) {
         // the node shifts x_j / sqrt(ln2) (in units of the Doppler width) and the weights
@@ -509,149 +626,151 @@ __global__ void __launch_bounds__(VT) k_vjp32(Vjp32Params p) {
             }
             const float *gc = p.g32 + (size_t)__shfl_sync(0xffffffffu, cc.row, c) * (size_t)p.n_pts;
             KahanF K0, K1, K2, B0, B1, B2;
-            if (PROF == XC_VOIGT_W4) {
-                const float asc = kSqrtLn2f * rcp_approx(a_h);   // x = asc |delta|
-                const float y = asc * g_h;
-                const float bb = a_h * a_h * (float)(0.5 / 0.6931471805599453), g2 = g_h * g_h;
-                const float C = bb + g2, g4 = 4.f * g2;
-                const float thr = (15.f - y) * rcp_approx(asc);
-                const float thr2 = y < 15.f ? thr * thr : -1.f;   // region I iff u >= thr2
-                for (int k8 = ka + lane; k8 <= kb; k8 += 32 * 8) {
-                    float q0 = 0.f, q1 = 0.f, q2 = 0.f;
-#pragma unroll
-                    for (int j = 0; j < 8; ++j) {
-                        const int k = k8 + 32 * j;
-                        if (k <= kb) {
-                            const float d = (float)(k - na) - ff;
-                            const float u = d * d;
-                            const float gk = gc[k];
-                            if (u >= thr2) {
-                                const float t = C - u;
-                                const float Dn = fmaf(t, t, g4 * u);
-                                const float rD = rcp_approx(Dn);
-                                const float w = (u + C) * rD;
-                                q0 = fmaf(gk, w, q0);
-                                q1 = fmaf(gk, rD * fmaf(-2.f * t, w, 1.f), q1);
-                                q2 = fmaf(gk, u * w * rD, q2);
-                            } else {
-                                const float3 r = w4_band_f32(asc * fabsf(d), y);
-                                B0.add(gk * r.x);
-                                B1.add(gk * r.z);   // Re(F + t F')
-                                B2.add(gk * r.y);   // Re F'
-                            }
-                        }
-                    }
-                    K0.add(q0);
-                    K1.add(q1);
-                    K2.add(q2);
-                }
-                const F2 s0 = f2_warp_sum(F2{K0.s, -K0.c}), s1 = f2_warp_sum(F2{K1.s, -K1.c});
-                const F2 s2 = f2_warp_sum(F2{K2.s, -K2.c});
-                const F2 b0 = f2_warp_sum(F2{B0.s, -B0.c}), b1 = f2_warp_sum(F2{B1.s, -B1.c});
-                const F2 b2 = f2_warp_sum(F2{B2.s, -B2.c});
-                if (lane == c) {
-                    const float S0 = s0.hi + s0.lo, S1 = s1.hi + s1.lo, S2 = s2.hi + s2.lo;
-                    const float ia = rcp_approx(a_h);
-                    const float kd = kSqrtLn2OverPi * ia;                        // sqrt(ln2/pi)/a
-                    const float kg = (float)(0.6931471805599453 / 1.772453850905516027) * ia * ia;
-                    SIm = kKappa * g_h * S0 + kd * (b0.hi + b0.lo);
-                    Sam = kKappa * g_h * (a_h * (float)(1.0 / 0.6931471805599453)) * S1 - kd * ia * (b1.hi + b1.lo);
-                    Sgm = kKappa * (S0 + 2.f * g2 * (S1 - 4.f * S2)) + kg * (b2.hi + b2.lo);
-                }
-            } else if (PROF == XC_VOIGT_GH_BINNED) {
-                // bin average of the Gauss-Hermite Voigt (Eq. e:sigma:quad), grid units (bin width 1):
-                // per node j, s+ = delta + 1/2 - a x_j/sqrt(ln2), s- = s+ - 1, Q+- = s+-^2 + g^2,
-                //   V = pi^(-3/2) sum_j w_j atan2(g, g^2 + s+ s-),
-                //   dV/dg = pi^(-3/2) sum_j w_j (s+ s- - g^2)/(Q+ Q-),
-                //   dV/da = pi^(-3/2) sum_j w_j (x_j/sqrt(ln2)) g (s+ + s-)/(Q+ Q-)
-                const float g2 = g_h * g_h;
-                const int ngh = p.ngh;
-                for (int k8 = ka + lane; k8 <= kb; k8 += 32 * 8) {
+            const VjpLine<PROF> ln_c(a_h, g_h, s_gx, s_gw, p.ngh);
+            // grid points k0..k1, all in w4's region I
+            auto points = [&](int k0, int k1) {
+                for (int k8 = k0 + lane; k8 <= k1; k8 += 32 * 8) {
                     float q0 = 0.f, q1 = 0.f, q2 = 0.f;
 #pragma unroll 2
                     for (int j = 0; j < 8; ++j) {
                         const int k = k8 + 32 * j;
-                        if (k <= kb) {
-                            const float d = (float)(k - na) - ff + 0.5f;
-                            float v = 0.f, da = 0.f, dg = 0.f;
-                            for (int m = 0; m < ngh; ++m) {
-                                const float sp = fmaf(-a_h, s_gx[m], d), sm = sp - 1.f;
-                                const float iQ = rcp_approx(fmaf(sp, sp, g2) * fmaf(sm, sm, g2));
-                                v = fmaf(s_gw[m], atan2_ypos(g_h, fmaf(sp, sm, g2)), v);
-                                dg = fmaf(s_gw[m], fmaf(sp, sm, -g2) * iQ, dg);
-                                da = fmaf(s_gw[m] * s_gx[m], (sp + sm) * iQ, da);
-                            }
+                        if (k > k1) break;
+                        ln_c.add((float)(k - na) - ff, gc[k], q0, q1, q2);
+                    }
+                    K0.add(q0);
+                    K1.add(q1);
+                    K2.add(q2);
+                }
+            };
+            int c0 = ka, c1 = kb;   // the points around the centre
+            if (PROF == XC_DOPPLER) {
+                // 2^(-u / a^2) is exactly 0 in FP32 beyond 11.3 a
+                const int r = (int)fminf(ceilf(11.3f * a_h) + 2.f, 1e9f);
+                c0 = max(c0, na - r);
+                c1 = min(c1, na + r);
+            } else if (p.gnode) {
+                // the far points on both sides by the nodes of the blocks they fill: a block of
+                // level l when it lies inside the cut and beyond the level's radius (xc_tree.cu)
+                const float *gn = p.gnode + (size_t)__shfl_sync(0xffffffffu, cc.row, c) * (size_t)p.nodes_per_cond;
+                const float am = fminf(a_h, 1e6f);
+                const int e = PROF == XC_VOIGT_W4 ? 2 + (int)ceilf(0.86f * am)
+                              : PROF == XC_VOIGT_GH_BINNED ? 3 + (int)ceilf(am * s_ext)
+                                                           : 1;
+                const int core = PROF == XC_VOIGT_W4 ? 2 + (int)ceilf(18.05f * am) : 0;
+                int D[TR_LEVELS];
+#pragma unroll
+                for (int l = 0; l < TR_LEVELS; ++l) D[l] = max(tr_gap(l) + e, core);
+                auto nodes = [&](int lev, int j0, int j1) {
+                    const int B = tr_block(lev);
+                    float q0 = 0.f, q1 = 0.f, q2 = 0.f;
+                    for (int i = j0 * TR_M + lane; i < j1 * TR_M; i += 32) {
+                        const float dl = ((float)((i >> 4) * B - na) + s_node[lev][i & 15]) - ff;
+                        ln_c.add(dl, gn[p.node_off[lev] + i], q0, q1, q2);
+                    }
+                    K0.add(q0);
+                    K1.add(q1);
+                    K2.add(q2);
+                };
+                // points lo[l]..hi[l] may be taken by level l; returns the points taken
+                auto side = [&](int lo0, int hi0, int lo1, int hi1, int lo2, int hi2, int *t0, int *t1) {
+                    const int a0 = (lo0 + 63) >> 6, b0 = (hi0 + 1) >> 6;
+                    const int a1 = (lo1 + 127) >> 7, b1 = (hi1 + 1) >> 7;
+                    const int a2 = (lo2 + 511) >> 9, b2 = (hi2 + 1) >> 9;
+                    *t0 = *t1 = 0;
+                    if (b0 <= a0) return;
+                    *t0 = 64 * a0;
+                    *t1 = 64 * b0;
+                    if (b1 <= a1) {
+                        nodes(0, a0, b0);
+                        return;
+                    }
+                    if (a0 < 2 * a1) nodes(0, a0, 2 * a1);
+                    if (2 * b1 < b0) nodes(0, 2 * b1, b0);
+                    if (b2 <= a2) {
+                        nodes(1, a1, b1);
+                        return;
+                    }
+                    if (a1 < 4 * a2) nodes(1, a1, 4 * a2);
+                    if (4 * b2 < b1) nodes(1, 4 * b2, b1);
+                    nodes(2, a2, b2);
+                };
+                int t0, t1;
+                side(ka, min(kb, na - D[0] - 1), ka, min(kb, na - D[1] - 1), ka, min(kb, na - D[2] - 1), &t0, &t1);
+                if (t1 > t0) {
+                    points(ka, t0 - 1);
+                    c0 = t1;
+                }
+                side(max(ka, na + D[0] + 1), kb, max(ka, na + D[1] + 1), kb, max(ka, na + D[2] + 1), kb, &t0, &t1);
+                if (t1 > t0) {
+                    points(t1, kb);
+                    c1 = t0 - 1;
+                }
+            }
+            if (PROF != XC_VOIGT_W4) {
+                points(c0, c1);
+            } else {
+                for (int k8 = c0 + lane; k8 <= c1; k8 += 32 * 8) {
+                    float q0 = 0.f, q1 = 0.f, q2 = 0.f;
+#pragma unroll 2
+                    for (int j = 0; j < 8; ++j) {
+                        const int k = k8 + 32 * j;
+                        if (k > c1) break;
+                        const float d = (float)(k - na) - ff;
+                        if (d * d >= ln_c.thr2) {
+                            ln_c.add(d, gc[k], q0, q1, q2);
+                        } else {
                             const float gk = gc[k];
-                            q0 = fmaf(gk, v, q0);
-                            q1 = fmaf(gk, da, q1);
-                            q2 = fmaf(gk, dg, q2);
+                            const float3 r = w4_band_f32(ln_c.asc * fabsf(d), ln_c.y);
+                            B0.add(gk * r.x);
+                            B1.add(gk * r.z);   // Re(F + t F')
+                            B2.add(gk * r.y);   // Re F'
                         }
                     }
                     K0.add(q0);
                     K1.add(q1);
                     K2.add(q2);
                 }
-                const F2 s0 = f2_warp_sum(F2{K0.s, -K0.c}), s1 = f2_warp_sum(F2{K1.s, -K1.c});
-                const F2 s2 = f2_warp_sum(F2{K2.s, -K2.c});
-                if (lane == c) {
+            }
+            // the lanes' sums to the three derivative sums, each reduced over the warp
+            F2 vI, va, vg;
+            if (PROF == XC_VOIGT_W4) {
+                const float ia = rcp_approx(a_h), g2 = g_h * g_h;
+                const float kd = kSqrtLn2OverPi * ia;                        // sqrt(ln2/pi)/a
+                const float kg = (float)(0.6931471805599453 / 1.772453850905516027) * ia * ia;
+                vI = f2_add(f2_scale(f2_of(K0), kKappa * g_h), f2_scale(f2_of(B0), kd));
+                va = f2_add(f2_scale(f2_of(K1), kKappa * g_h * (a_h * (float)(1.0 / 0.6931471805599453))),
+                            f2_scale(f2_of(B1), -kd * ia));
+                const F2 t = f2_add(f2_of(K1), f2_scale(f2_of(K2), -4.f));
+                vg = f2_add(f2_add(f2_scale(f2_of(K0), kKappa), f2_scale(t, 2.f * kKappa * g2)), f2_scale(f2_of(B2), kg));
+            } else {
+                vI = f2_of(K0);
+                va = f2_of(K1);
+                vg = f2_of(K2);
+            }
+            vI = f2_warp_sum(vI);
+            if (PROF != XC_LORENTZ) va = f2_warp_sum(va);
+            if (PROF != XC_DOPPLER) vg = f2_warp_sum(vg);
+            if (lane == c) {
+                const float S0 = vI.hi + vI.lo, S1 = va.hi + va.lo, S2 = vg.hi + vg.lo;
+                if (PROF == XC_VOIGT_W4) {
+                    SIm = S0;
+                    Sam = S1;
+                    Sgm = S2;
+                } else if (PROF == XC_VOIGT_GH_BINNED) {
                     constexpr float kpi = (float)(1.0 / (3.141592653589793 * 1.772453850905516));   // pi^(-3/2)
-                    SIm = kpi * (s0.hi + s0.lo);
-                    Sam = kpi * g_h * (s1.hi + s1.lo);
-                    Sgm = kpi * (s2.hi + s2.lo);
-                }
-            } else if (PROF == XC_DOPPLER) {
-                // V = sqrt(ln2/pi)/a 2^(-u/a^2): sums of g 2^(-u/a^2) and g u 2^(-u/a^2)
-                const float ia2 = rcp_approx(a_h * a_h);
-                for (int k8 = ka + lane; k8 <= kb; k8 += 32 * 8) {
-                    float q0 = 0.f, q1 = 0.f;
-#pragma unroll
-                    for (int j = 0; j < 8; ++j) {
-                        const int k = k8 + 32 * j;
-                        if (k <= kb) {
-                            const float d = (float)(k - na) - ff;
-                            const float u = d * d;
-                            const float e = ex2_approx(-u * ia2) * gc[k];
-                            q0 += e;
-                            q1 = fmaf(e, u, q1);
-                        }
-                    }
-                    K0.add(q0);
-                    K1.add(q1);
-                }
-                const F2 s0 = f2_warp_sum(F2{K0.s, -K0.c}), s1 = f2_warp_sum(F2{K1.s, -K1.c});
-                if (lane == c) {
+                    SIm = kpi * S0;
+                    Sam = kpi * g_h * S1;
+                    Sgm = kpi * S2;
+                } else if (PROF == XC_DOPPLER) {
                     const float ia = rcp_approx(a_h);
                     const float pd = kSqrtLn2OverPi * ia;
-                    const float S0 = s0.hi + s0.lo, S1 = s1.hi + s1.lo;
                     SIm = pd * S0;
-                    Sam = pd * (-S0 * ia + (float)(2.0 * 0.6931471805599453) * ia2 * ia * S1);
+                    Sam = pd * (-S0 * ia + (float)(2.0 * 0.6931471805599453) * rcp_approx(a_h * a_h) * ia * S1);
                     Sgm = 0.f;
-                }
-            } else {
-                // Lorentz: V = (1/pi) g/(u + g^2), dV/dg = (1/pi)(u - g^2)/(u + g^2)^2
-                const float g2 = g_h * g_h;
-                for (int k8 = ka + lane; k8 <= kb; k8 += 32 * 8) {
-                    float q0 = 0.f, q2 = 0.f;
-#pragma unroll
-                    for (int j = 0; j < 8; ++j) {
-                        const int k = k8 + 32 * j;
-                        if (k <= kb) {
-                            const float d = (float)(k - na) - ff;
-                            const float u = d * d;
-                            const float r = rcp_approx(u + g2);
-                            const float gr = gc[k] * r;
-                            q0 += gr;
-                            q2 = fmaf(gr, (u - g2) * r, q2);
-                        }
-                    }
-                    K0.add(q0);
-                    K2.add(q2);
-                }
-                const F2 s0 = f2_warp_sum(F2{K0.s, -K0.c}), s2 = f2_warp_sum(F2{K2.s, -K2.c});
-                if (lane == c) {
-                    SIm = g_h * (float)(1.0 / kPi) * (s0.hi + s0.lo);
+                } else {
+                    SIm = g_h * (float)(1.0 / kPi) * S0;
                     Sam = 0.f;
-                    Sgm = (float)(1.0 / kPi) * (s2.hi + s2.lo);
+                    Sgm = (float)(1.0 / kPi) * S2;
                 }
             }
         }
@@ -758,6 +877,11 @@ xc_status vjp_run(BatchedState *st, const VjpArgs &a, int64_t *launches) {
     size_t o_geo = f64 ? 0 : carve(n * 16);
     size_t o_gs = f64 ? 0 : carve(sizeof(GeomStats));
     size_t o_cp = f64 ? 0 : carve((size_t)nc * sizeof(CParam));
+    // block nodes of the far field (FP32, profiles with far wings): 28 floats per 64 points
+    const bool far = !f64 && a.opts.profile != XC_DOPPLER && a.grid.n < ((int64_t)1 << 30);
+    const int nblk512 = far ? (int)((a.grid.n + 511) / 512) : 0;
+    const size_t per_cond = (size_t)nblk512 * (128 + 64 + 16);
+    size_t o_gn = far ? carve((size_t)nc * per_cond * 4) : 0, o_mat = far ? carve(TR_MAT * 8) : 0;
     VJ_TRY(st->vjp_buf.ensure(off + 256));
     char *base = st->vjp_buf.as<char>();
     const double *g64 = a.grad_sigma;
@@ -802,7 +926,7 @@ xc_status vjp_run(BatchedState *st, const VjpArgs &a, int64_t *launches) {
             fn<<<blocks, VT, 0, s>>>(a.L, n, a.conds_dev + c0, cc, a.grid.nu_A, a.grid.step, a.grid.n, a.opts.cutoff,
                                      a.opts.width_mult, g64 + (size_t)c0 * N, bp, dgl, dnl, c0 > 0 ? 1 : 0, a.ghx,
                                      a.ghw, a.opts.n_gh);
-            k_vjp_finish<<<1, 128, 0, s>>>(bp, blocks, cc, NQ, c0, nullptr, dT, dP, acc);
+            k_vjp_finish<<<(cc * NQ + 3) / 4, 128, 0, s>>>(bp, blocks, cc, NQ, c0, nullptr, dT, dP, acc);
             *launches += 2;
         }
         k_vjp_scalars<<<1, 32, 0, s>>>(acc, nc, nb, ds, dn, dg0b, dnb);
@@ -818,6 +942,13 @@ xc_status vjp_run(BatchedState *st, const VjpArgs &a, int64_t *launches) {
         if (N) {
             k_to_f32<<<nsm * 4, 256, 0, s>>>(g64, g32, (size_t)nc * N);
             ++*launches;
+        }
+        if (far && N) {
+            double *mat = (double *)(base + o_mat);
+            VJ_TRY(launch_tree_mat(mat, s));
+            k_vjp_nodes<<<dim3(nblk512, nc), 128, 0, s>>>(g64, a.grid.n, mat, (float *)(base + o_gn), 0, nblk512 * 128,
+                                                          nblk512 * 192, (int)per_cond);
+            *launches += 2;
         }
         VJ_TRY(launch_fp32_setup(a.L, n, a.conds_dev, nc, a.grid, a.opts.cutoff, n_abs, ffr, ka, kb, gs, cp, s));
         *launches += 2;
@@ -845,6 +976,11 @@ xc_status vjp_run(BatchedState *st, const VjpArgs &a, int64_t *launches) {
             vp.ghx = a.ghx;
             vp.ghw = a.ghw;
             vp.ngh = a.opts.n_gh;
+            vp.gnode = far && N ? (const float *)(base + o_gn) : nullptr;
+            vp.node_off[0] = 0;
+            vp.node_off[1] = nblk512 * 128;
+            vp.node_off[2] = nblk512 * 192;
+            vp.nodes_per_cond = (int)per_cond;
             const bool mix = nb > 0;
             switch (a.opts.profile) {
             case XC_DOPPLER:
@@ -864,7 +1000,7 @@ xc_status vjp_run(BatchedState *st, const VjpArgs &a, int64_t *launches) {
                 else k_vjp32<XC_VOIGT_W4, false><<<blocks, VT, 0, s>>>(vp);
                 break;
             }
-            k_vjp_finish<<<1, 128, 0, s>>>(bp, blocks, vp.nc, NQ, 0, cp + c0, dT, dP, acc);
+            k_vjp_finish<<<(vp.nc * NQ + 3) / 4, 128, 0, s>>>(bp, blocks, vp.nc, NQ, 0, cp + c0, dT, dP, acc);
             *launches += 2;
         }
         k_vjp_scalars<<<1, 32, 0, s>>>(acc, nc, nb, ds, dn, dg0b, dnb);
