@@ -64,7 +64,7 @@ struct xc_handle {
     int32_t *st_g = nullptr;
     size_t n_states = 0;
     int *d_flag = nullptr;
-    DevBuf sort_tmp[5];
+    DevBuf sort_tmp[6];
     DevBuf stage_in;         // unsorted host lines copied to the device
     DevBuf params;           // FP64 per-line I, alpha, gamma, cut
     DevBuf ranges;           // window line ranges

@@ -119,3 +119,28 @@ def test_adjoint_on_blocks_against_fp64(eng, xc, profile, n):  # noqa: F811
         for k in ("dT", "dP", "d_gamma_ref_line", "d_n_line"):
             a, b = np.asarray(r32[k]), np.asarray(r64[k])
             assert np.max(np.abs(a - b)) <= 1e-4 * max(np.max(np.abs(b)), 1e-300), (k, profile, n, nu_A)
+
+
+# ------------------------------------------------------------------ sort
+@pytest.mark.parametrize("case", ["dense", "runs", "long_run", "two", "narrow"])
+def test_sort_of_lines_that_agree_in_their_high_digits(eng, xc, case):  # noqa: F811
+    """The in-place finish of the sort: many short runs of nearly equal wavenumbers, a run that is
+    too long for it, equal wavenumbers (input order), and keys whose low digits alone differ."""
+    rng = np.random.default_rng(7)
+    n = {"two": 2}.get(case, 50_000)
+    L = xs.gen_lines(306, 0, n, 1.0, 9000.0)
+    base = L["nu"].copy()
+    if case in ("runs", "long_run"):
+        L["nu"] = np.repeat(base[::10], 10)[:n] * (1.0 + rng.integers(0, 40, n) * 2.0 ** -50)
+    if case == "long_run":
+        L["nu"][1000:2000] = 5000.0 + rng.integers(0, 300, 1000) * 2.0 ** -40
+    if case == "narrow":
+        L["nu"] = 4000.0 + rng.integers(0, 5000, n) * 2.0 ** -40
+    p = rng.permutation(n)
+    L = {k: v[p] for k, v in L.items()}
+    eng.load_lines(L)
+    order = np.argsort(L["nu"], kind="stable")
+    assert np.array_equal(eng.get_permutation(), order.astype(np.uint32))
+    got = eng.get_lines()
+    for k in L:
+        assert np.array_equal(got[k], L[k][order]), (case, k)
