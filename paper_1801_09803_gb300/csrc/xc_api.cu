@@ -233,13 +233,6 @@ xc_status check_conds(const xc_condition *c, size_t n, const xc_handle *h) {
 
 // Upload conditions and fill Q, dQ/dT for those with Q <= 0 from the states,
 // one Q(T) evaluation per distinct temperature.  Returns the device CondDev array.
-__global__ void k_fill_conds(CondDev *c, int n, const int *tix, const double *Q, const double *dQ) {
-    int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n || tix[i] < 0) return;
-    c[i].Q = Q[tix[i]];
-    c[i].dQdT = dQ[tix[i]];
-}
-
 xc_status resolve_conds(xc_handle *h, const xc_condition *conds, size_t n, cudaStream_t s, CondDev **out) {
     std::vector<CondDev> hc(n);
     std::vector<double> uT;
@@ -257,27 +250,28 @@ xc_status resolve_conds(xc_handle *h, const xc_condition *conds, size_t n, cudaS
             }
         }
     }
-    size_t nT = uT.size();
-    size_t bytes_c = n * sizeof(CondDev);
-    size_t off_q = (bytes_c + 255) & ~size_t(255);
-    size_t need = off_q + 3 * nT * sizeof(double) + n * sizeof(int) + 64;
-    XC_TRY_MEM(h->conds.ensure(need));
+    // one host -> device copy (stream-ordered, pageable): conditions, temperatures, indices
+    const size_t nT = uT.size(), bytes_c = n * sizeof(CondDev);
+    const size_t off_t = (bytes_c + 255) & ~size_t(255), off_i = off_t + nT * sizeof(double);
+    const size_t up = nT ? off_i + n * sizeof(int) : bytes_c;
+    const size_t off_q = (up + 255) & ~size_t(255);
+    XC_TRY_MEM(h->conds.ensure(off_q + 2 * nT * sizeof(double) + 64));
+    std::vector<char> hb(up);
+    memcpy(hb.data(), hc.data(), bytes_c);
+    if (nT) {
+        memcpy(hb.data() + off_t, uT.data(), nT * sizeof(double));
+        memcpy(hb.data() + off_i, tix.data(), n * sizeof(int));
+    }
     char *base = h->conds.as<char>();
     CondDev *dc = reinterpret_cast<CondDev *>(base);
-    double *dT = reinterpret_cast<double *>(base + off_q);
-    double *dQ = dT + nT, *ddQ = dQ + nT;
-    int *dtix = reinterpret_cast<int *>(ddQ + nT);
-    // pageable host -> device copies of small parameter blocks (stream-ordered)
-    XC_TRY(cudaMemcpyAsync(dc, hc.data(), bytes_c, cudaMemcpyHostToDevice, s));
+    XC_TRY(cudaMemcpyAsync(base, hb.data(), up, cudaMemcpyHostToDevice, s));
     if (nT) {
-        XC_TRY(cudaMemcpyAsync(dT, uT.data(), nT * sizeof(double), cudaMemcpyHostToDevice, s));
-        XC_TRY(cudaMemcpyAsync(dtix, tix.data(), n * sizeof(int), cudaMemcpyHostToDevice, s));
+        double *dQ = reinterpret_cast<double *>(base + off_q), *ddQ = dQ + nT;
         stage_begin(h, ST_Q, s);
-        XC_TRY(launch_partition_function(h->st_E, h->st_g, h->n_states, dT, (int)nT, dQ, ddQ, s));
-        k_fill_conds<<<(unsigned)((n + 127) / 128), 128, 0, s>>>(dc, (int)n, dtix, dQ, ddQ);
-        XC_TRY(cudaGetLastError());
+        XC_TRY(launch_partition_function(h->st_E, h->st_g, h->n_states, reinterpret_cast<double *>(base + off_t),
+                                         (int)nT, dQ, ddQ, s, dc, reinterpret_cast<int *>(base + off_i), (int)n));
         stage_end(h, ST_Q, s);
-        h->launches += 2;
+        h->launches += 1;
     }
     *out = dc;
     return XC_OK;
@@ -304,8 +298,8 @@ xc_status ensure_gh(xc_handle *h, int n, cudaStream_t s) {
 }
 
 // FP64 plain cross section of one (already resolved) condition into device memory
-xc_status cross_section_f64(xc_handle *h, const CondDev *dcond, const xc_grid *g, const xc_opts *o, double *sig,
-                            cudaStream_t s) {
+xc_status cross_section_f64(xc_handle *h, const CondDev *dcond, const xc_condition &cond, const xc_grid *g,
+                            const xc_opts *o, double *sig, cudaStream_t s) {
     const size_t n = h->n_lines;
     const int64_t W = 256;
     const int64_t n_win = (g->n + W - 1) / W;
@@ -318,7 +312,8 @@ xc_status cross_section_f64(xc_handle *h, const CondDev *dcond, const xc_grid *g
     // the block-interpolated form (the Vectorized Voigt is not smooth at its split: direct sum),
     // unless its 16 bytes per line do not fit next to a very large list
     bool tree = tree64_takes(o->profile, *g, o->cutoff, n);
-    if (tree && h->ranges.ensure(tree64_scratch(*g, o->cutoff, n)) != cudaSuccess) {
+    if (tree && (tree64_mat(&h->batched.tree_mat64, s) != cudaSuccess ||
+                 h->ranges.ensure(tree64_scratch(*g, o->cutoff, n)) != cudaSuccess)) {
         cudaGetLastError();
         tree = false;
     }
@@ -347,8 +342,8 @@ xc_status cross_section_f64(xc_handle *h, const CondDev *dcond, const xc_grid *g
     }
     stage_begin(h, ST_PROFILE, s);
     if (tree) {
-        XC_TRY(launch_tree64(o->profile, h->nu, I, al, ga, cut, n, dcond, *g, o->cutoff, o->width_mult <= 0.0, ghx, ghw,
-                             ghx ? o->n_gh : 0, h->ranges.p, sig, &h->launches, s));
+        XC_TRY(launch_tree64(o->profile, h->nu, I, al, ga, cut, n, alpha_coef(cond.T, cond.mass_da), *g, o->cutoff,
+                             o->width_mult <= 0.0, ghx, ghw, ghx ? o->n_gh : 0, h->batched.tree_mat64.as<double>(), h->ranges.p, sig, &h->launches, s));
         stage_end(h, ST_PROFILE, s);
         h->launches += 1;
         return XC_OK;
@@ -823,7 +818,7 @@ xc_status xc_cross_section_batched(xc_handle *h, const xc_condition *conds, size
     if ((st = resolve_conds(h, conds, n_cond, s, &dc))) return st;
     if (opts->precision == XC_FP64_PLAIN || h->n_lines == 0) {
         for (size_t c = 0; c < n_cond; ++c) {
-            if ((st = cross_section_f64(h, dc + c, grid, opts, sig + c * grid->n, s))) return st;
+            if ((st = cross_section_f64(h, dc + c, conds[c], grid, opts, sig + c * grid->n, s))) return st;
         }
         used[ST_PARAMS] = used[ST_RANGES] = used[ST_PROFILE] = h->n_lines > 0;
     } else {

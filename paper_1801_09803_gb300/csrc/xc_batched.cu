@@ -168,20 +168,6 @@ __global__ void k_line_geom(LinesDev L, size_t n, double nu_A, double step, int6
     }
 }
 
-cudaError_t launch_fp32_setup(const LinesDev &L, size_t n, const CondDev *conds, int nc, const xc_grid &grid,
-                              double cutoff, int *n_abs, float *f, int *ka, int *kb, GeomStats *gs, CParam *cp,
-                              cudaStream_t s) {
-    cudaError_t e = cudaMemsetAsync(gs, 0, sizeof(GeomStats), s);
-    if (e != cudaSuccess) return e;
-    if (n) {
-        const unsigned gb = (unsigned)std::max<size_t>(1, std::min<size_t>((n + 255) / 256, 152 * 16));
-        k_line_geom<<<gb, 256, 0, s>>>(L, n, grid.nu_A, grid.step, grid.n, cutoff, 0.0, nullptr, n_abs, f, ka, kb,
-                                       gs, nullptr, nullptr);
-    }
-    if (nc) k_cparams<<<(nc + 63) / 64, 64, 0, s>>>(conds, nc, gs, cp, grid.step, XC_ABSORPTION, nullptr, 4.f, 0);
-    return cudaGetLastError();
-}
-
 // window -> line range for a fixed maximum cut
 __global__ void k_win_ranges32(const double *__restrict__ nu, int64_t n, double nu_A, double step, int64_t n_pts,
                                int W, double cutmax, int n_win, unsigned *lo, unsigned *hi) {
@@ -2130,6 +2116,8 @@ void batched_release(BatchedState *st) {
     st->vjp_buf.release();
     st->gsig32.release();
     st->staging.release();
+    st->tree_mat.release();
+    st->tree_mat64.release();
 }
 
 // ---------------------------------------------------------------------------

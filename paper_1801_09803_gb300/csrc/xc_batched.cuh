@@ -36,7 +36,6 @@ struct GeomStats {
     unsigned int nu_bits;      // max nu (float, rounded up)
     unsigned int gref_bits;    // max |gamma_ref|
     unsigned int nT_bits;      // max |n_T|
-    unsigned int acoef_bits;   // max alpha / nu over the conditions (float, rounded up; block-interpolated sweep)
 };
 
 __device__ __forceinline__ float rcp_approx(float x) { return recip(x); }
@@ -153,6 +152,8 @@ struct BatchedState {
     DevBuf vjp_buf;    // adjoint scratch
     DevBuf gsig32;     // grad sigma as float
     DevBuf staging;    // host <-> device staging for the adjoint
+    DevBuf tree_mat;   // interpolation matrices of the block-interpolated sweep (constants)
+    DevBuf tree_mat64; // ... of the FP64 one
     std::map<std::string, TileCfg> tuned;       // autotune cache: shape key -> config
     std::map<std::string, GraphEntry> graphs;   // graph cache: shape key + pointers -> graph
     std::map<std::string, std::string> tune_log; // shape key -> candidate predictions
@@ -165,12 +166,11 @@ struct BatchedState {
 };
 
 xc_status batched_run(BatchedState *st, const BatchedArgs &a, int64_t *launches);
-// per-line grid geometry for a fixed cut (integer position n_abs, fraction f, inclusive
-// cut range [ka, kb]) and the per-condition FP32 constants (in order of increasing
-// profile width, each with its caller's row), as the batched FP32 kernels make them
+// per-line grid geometry for a fixed cut (integer position n, inclusive cut range ka..kb,
+// fraction f as bits) and the per-condition FP32 constants in the caller's order, as the
+// block-interpolated sweep makes them
 cudaError_t launch_fp32_setup(const LinesDev &L, size_t n, const CondDev *conds, int nc, const xc_grid &grid,
-                              double cutoff, int *n_abs, float *f, int *ka, int *kb, GeomStats *gs, CParam *cp,
-                              cudaStream_t s);
+                              double cutoff, int4 *geo, GeomStats *gs, CParam *cp, cudaStream_t s);
 xc_status vjp_run(BatchedState *st, const VjpArgs &a, int64_t *launches);
 // the block-interpolated FP32 sweep (xc_tree.cu): whether it takes a call, and the call
 bool tree_takes(const BatchedArgs &a);

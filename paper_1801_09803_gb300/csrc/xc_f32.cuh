@@ -334,40 +334,44 @@ __device__ inline int cond_rank(int c, const CondDev *conds, int n_cond) {
     return rank;
 }
 
+// Per-condition constants in parts (their FP64 chains are independent of one another)
+__device__ inline void cparam_strength(const CondDev &d, const GeomStats *gs, int quantity, CParam *p) {
+    const bool emis = quantity == XC_EMISSION;
+    const double pref = emis ? d.abundance * kPlanckErg * kLightCm / (4.0 * kPi * d.Q)
+                             : d.abundance / (8.0 * kPi * kLightCm * d.Q);
+    const double s1 = (double)__uint_as_float(gs->gA_nu2_bits);
+    const double s2 = (double)__uint_as_float(gs->gA_nu_bits);
+    const double numax = (double)__uint_as_float(gs->nu_bits);
+    // bound on the largest intensity (absorption), or emissivity: g A nu <= max(g A / nu) nu_max^2
+    const double ib = emis ? pref * s2 * numax * numax : pref * fmin(s1, kC2 / d.T * s2);
+    int e2 = 0;
+    if (ib > 0.0 && isfinite(ib)) e2 = max(-120, min(120, ilogb(1e10 / ib)));   // floor(log2)
+    p->inv_scale = ldexp(1.0, -e2);
+    p->pref = (float)(pref * ldexp(1.0, e2));
+    p->emis = emis ? 1.f : 0.f;
+}
+__device__ inline void cparam_temperature(const CondDev &d, CParam *p) {
+    const double kT = kC2 * 1.4426950408889634 / d.T;
+    p->kT_hi = (float)kT;
+    p->kT_lo = (float)(kT - (double)p->kT_hi);
+    p->c2T = (float)(kC2 / d.T);
+    p->nshift = (float)d.n_shift;
+}
+__device__ inline void cparam_widths(const CondDev &d, CParam *p) {
+    p->acoef = (float)alpha_coef(d.T, d.mass_da);
+    p->pscale = (float)(d.gamma_scale * d.P / d.P_ref);
+}
+
 // Per-condition constants of condition c; row keeps the caller's index.
 __device__ inline CParam make_cparam(int c, const CondDev *conds, const GeomStats *gs, double step, int quantity,
                                      const unsigned *gmax_bits, float vv_split, int vv_beta) {
     const CondDev d = conds[c];
-    const double log2e = 1.4426950408889634;
-    double kT = kC2 * log2e / d.T;
-    float hi = (float)kT;
-    float lo = (float)(kT - (double)hi);
-    const bool emis = quantity == XC_EMISSION;
-    double pref = emis ? d.abundance * kPlanckErg * kLightCm / (4.0 * kPi * d.Q)
-                       : d.abundance / (8.0 * kPi * kLightCm * d.Q);
-    double s1 = (double)__uint_as_float(gs->gA_nu2_bits);
-    double s2 = (double)__uint_as_float(gs->gA_nu_bits);
-    const double numax = (double)__uint_as_float(gs->nu_bits);
-    // bound on the largest intensity (absorption), or emissivity: g A nu <= max(g A / nu) nu_max^2
-    double ib = emis ? pref * s2 * numax * numax : pref * fmin(s1, kC2 / d.T * s2);
-    int e2 = 0;
-    if (ib > 0.0 && isfinite(ib)) {
-        e2 = (int)floor(log2(1e10 / ib));
-        e2 = max(-120, min(120, e2));
-    }
-    double scale = ldexp(1.0, e2);
     CParam p;
-    p.inv_scale = ldexp(1.0, -e2);
-    p.kT_hi = hi;
-    p.kT_lo = lo;
-    p.c2T = (float)(kC2 / d.T);
-    p.pref = (float)(pref * scale);
-    p.acoef = (float)alpha_coef(d.T, d.mass_da);
+    cparam_strength(d, gs, quantity, &p);
+    cparam_temperature(d, &p);
+    cparam_widths(d, &p);
     p.log2Tr = (float)log2(d.T_ref / d.T);
-    p.pscale = (float)(d.gamma_scale * d.P / d.P_ref);
-    p.nshift = (float)d.n_shift;
     p.row = c;
-    p.emis = emis ? 1.f : 0.f;
     p.vv_split = vv_split;
     p.vv_beta = vv_beta;
     {

@@ -13,6 +13,7 @@
 #include <vector>
 
 #include "../../include/xc.h"
+#include "xc_exp64.cuh"
 
 namespace xc {
 
@@ -71,6 +72,13 @@ struct LinesDev {
     int vv_stride = 0;
 };
 
+// float -> double by moving the bits: the conversion instruction runs at the FP64 pipe's rate
+__device__ __forceinline__ double f2d(float f) {
+    const int b = __float_as_int(f), e = b & 0x7f800000;
+    if (e == 0 || e == 0x7f800000) return (double)f;   // zero, subnormal, infinite, NaN
+    return __hiloint2double((b & 0x80000000) | (((b & 0x7fffffff) >> 3) + 0x38000000), b << 29);
+}
+
 struct CondDev {  // mirrors xc_condition plus resolved Q
     double T, P, Q, dQdT, mass_da, T_ref, P_ref, gamma_scale, n_shift, abundance;
 };
@@ -89,34 +97,55 @@ __host__ __device__ inline double alpha_coef(double T, double mass_da) {
 // Line strength in FP64: the absorption intensity of Eq. (e:int), or with XC_EMISSION the
 // emissivity of Eq. (e:emiss) (upper state E' = E'' + nu) times the photon energy h c nu;
 // -1 when the intensity threshold leaves the line out.  pref_abs = abundance / (8 pi c Q).
-__device__ inline double line_strength64(double nu, double elower, double gA, const CondDev &c,
+// The factors common to all lines of a condition are formed once by the caller.
+struct StrengthPre {
+    double pref, c2T;    // the constant factor, c2 / T
+    __device__ explicit StrengthPre(const CondDev &c, const StrengthSel &s)
+        : pref(s.quantity == XC_EMISSION ? c.abundance * (kPlanckErg * kLightCm) / (4.0 * kPi) / c.Q
+                                         : c.abundance / (8.0 * kPi * kLightCm * c.Q)),
+          c2T(kC2 * (1.0 / c.T)) {}
+    __device__ StrengthPre(double pref_, double c2T_) : pref(pref_), c2T(c2T_) {}
+};
+__device__ inline double line_strength64(double nu, double elower, double gA, const StrengthPre &p,
                                          const StrengthSel &s) {
-    const double inv_T = 1.0 / c.T;
+    const double x = p.c2T * nu;
     double S;
     if (s.quantity == XC_EMISSION) {
-        S = c.abundance * gA * (kPlanckErg * kLightCm * nu) / (4.0 * kPi) * exp(-kC2 * (elower + nu) * inv_T) / c.Q;
+        S = p.pref * gA * nu * exp64(-p.c2T * (elower + nu));
     } else {
-        const double boltz = exp(-kC2 * elower * inv_T);
-        const double stim = -expm1(-kC2 * nu * inv_T);
-        S = c.abundance / (8.0 * kPi * kLightCm * c.Q) * gA / (nu * nu) * boltz * stim;
+        const double boltz = exp64(-p.c2T * elower);
+        // 1 - exp(-x) directly where it loses nothing
+        const double stim = x >= 1.0 ? 1.0 - exp64(-x) : -expm1(-x);
+        S = p.pref * gA / (nu * nu) * boltz * stim;
     }
-    if (s.threshold != XC_THRESHOLD_NONE) {
-        double thr = s.I_cut;
-        if (s.threshold == XC_THRESHOLD_HITRAN)
-            thr = nu > s.nu_crit ? s.I_crit : s.I_crit * (nu / s.nu_crit) * tanh(kC2 * nu * inv_T * 0.5);
-        if (S < thr) return -1.0;
+    if (s.threshold == XC_THRESHOLD_CONSTANT) {
+        if (S < s.I_cut) return -1.0;
+    } else if (s.threshold == XC_THRESHOLD_HITRAN) {
+        // S < I_crit (nu / nu_crit) tanh(x / 2), without its divisions
+        if (nu > s.nu_crit) {
+            if (S < s.I_crit) return -1.0;
+        } else if (x >= 1.0) {
+            const double e = exp64(-x);
+            if (S * s.nu_crit * (1.0 + e) < s.I_crit * nu * (1.0 - e)) return -1.0;
+        } else if (S * s.nu_crit < s.I_crit * nu * tanh(0.5 * x)) {
+            return -1.0;
+        }
     }
     return S;
 }
 
 // Lorentz HWHM of line l under the broadener mixture (Sec. "Mixtures of broadeners"):
-// gamma_scale P/P_ref sum_i rho_i gamma_0,i (T_ref/T)^(n_i + n_shift), each term Eq. (e:gamma_L)
-__device__ inline double mixture_gamma64(const LinesDev &L, size_t l, const CondDev &c) {
-    const double lnTr = log(c.T_ref / c.T);
+// gamma_scale P/P_ref sum_i rho_i gamma_0,i (T_ref/T)^(n_i + n_shift), each term Eq. (e:gamma_L);
+// lnTr = ln(T_ref/T) and pscale = gamma_scale P/P_ref from the caller
+__device__ inline double mixture_gamma64(const LinesDev &L, size_t l, const CondDev &c, double lnTr, double pscale) {
     double g = 0.0;
     for (int i = 0; i < L.n_broad; ++i)
-        g += L.bgam[(size_t)i * L.bstride + l] * exp((L.bn[(size_t)i * L.bstride + l] + c.n_shift) * lnTr);
-    return c.gamma_scale * g * (c.P / c.P_ref);
+        g += L.bgam[(size_t)i * L.bstride + l] * exp64((L.bn[(size_t)i * L.bstride + l] + c.n_shift) * lnTr);
+    return pscale * g;
+}
+
+__device__ inline double mixture_gamma64(const LinesDev &L, size_t l, const CondDev &c) {
+    return mixture_gamma64(L, l, c, log(c.T_ref / c.T), c.gamma_scale * (c.P / c.P_ref));
 }
 
 // grid point nu_k = nu_A + k * step, rounded exactly as two separate operations
@@ -318,8 +347,10 @@ struct DevBuf {
 };
 
 // kernel launchers implemented in the other translation units
+// Q(T), dQ/dT per temperature; with conds: also into the conditions whose tix names the temperature
 cudaError_t launch_partition_function(const double *E, const int32_t *g, size_t n, const double *T, int nT,
-                                      double *Q, double *dQ, cudaStream_t s);
+                                      double *Q, double *dQ, cudaStream_t s, CondDev *conds = nullptr,
+                                      const int *tix = nullptr, int n_cond = 0);
 cudaError_t launch_sort_lines(const LinesDev &in, size_t n, bool assume_sorted, DevBuf *tmp, double *nu,
                               float *elower, float *A, float *gref, float *nT, int16_t *g, int16_t *j,
                               uint32_t *perm, int *d_flag, cudaStream_t s, cudaEvent_t *ev, int64_t *launches,
@@ -357,9 +388,10 @@ cudaError_t launch_gather_f64(int profile, const double *nu, const double *I, co
 bool tree64_takes(int profile, const xc_grid &g, double cutoff, size_t n);
 size_t tree64_scratch(const xc_grid &g, double cutoff, size_t n);
 cudaError_t launch_tree64(int profile, const double *nu, const double *I, const double *al, const double *ga,
-                          const double *cut, size_t n, const CondDev *cond, const xc_grid &g, double cutoff,
-                          bool fixed_cut, const double *ghx, const double *ghw, int ngh, void *scratch, double *sigma,
-                          int64_t *launches, cudaStream_t s);
+                          const double *cut, size_t n, double acoef, const xc_grid &g, double cutoff, bool fixed_cut,
+                          const double *ghx, const double *ghw, int ngh, const double *mat, void *scratch,
+                          double *sigma, int64_t *launches, cudaStream_t s);
+cudaError_t tree64_mat(DevBuf *buf, cudaStream_t s);   // its interpolation matrices, made once per handle
 // VVN: I[l] /= h sum_k f_VV(nu_k - nu_l) over the line's cut window on the grid lattice
 cudaError_t launch_vv_norm64(const double *nu, double *I, const double *alpha, const double *gamma,
                              const double *cut, size_t n, double nu_A, double step, double vv_split, int vv_beta,

@@ -1,9 +1,10 @@
 // xc_lines.cu -- per-line and per-state kernels:
-//   Q(T) and dQ/dT (Eq. e:pf) in FP64, one CTA per temperature;
+//   Q(T) and dQ/dT (Eq. e:pf) in FP64, a cluster of CTAs per temperature;
 //   FP64 line parameters I (Eq. e:int), alpha_D (Eq. e:alphaD), gamma_L (Eq. e:gamma_L);
 //   window -> line range by binary search on the sorted wavenumbers;
 //   exact count of (line, grid point) pairs inside the cutoff;
 //   Gauss-Hermite nodes and weights on the device.
+#include <cooperative_groups.h>
 #include <math.h>
 
 #include "xc_internal.cuh"
@@ -12,21 +13,28 @@ namespace xc {
 
 // ---------------------------------------------------------------------------
 // Q(T) = sum_n g_n exp(-c2 E_n / T) and dQ/dT = sum_n g_n (c2 E_n / T^2) exp(-c2 E_n / T)
-// One CTA per temperature; fixed-order tree reduction (deterministic).
+// A cluster of PF_CL CTAs per temperature: the exponentials are bound by the FP64 pipe (2
+// lanes per cycle and SM), so one CTA's 5000 states took 47 us on one SM.  Each CTA sums
+// its share of the states by a fixed-order tree; the first adds the others' sums from their
+// shared memory in rank order (deterministic).  tix (may be null): index of the temperature
+// of each condition, whose Q and dQ/dT are then filled in as well.
 // ---------------------------------------------------------------------------
-__global__ void __launch_bounds__(256) k_partition_function(const double *__restrict__ E,
-                                                            const int32_t *__restrict__ g, size_t n,
-                                                            const double *__restrict__ T, double *Q,
-                                                            double *dQ) {
+constexpr int PF_CL = 16;   // 16 is beyond the portable cluster size: allowed explicitly below
+__global__ void __launch_bounds__(256)
+    k_partition_function(const double *__restrict__ E, const int32_t *__restrict__ g, size_t n,
+                         const double *__restrict__ T, double *Q, double *dQ, CondDev *conds, const int *tix,
+                         int n_cond) {
     __shared__ double sq[256], sd[256];
-    const double t = T[blockIdx.x];
+    cooperative_groups::cluster_group cl = cooperative_groups::this_cluster();
+    const int j = blockIdx.x / PF_CL, r = (int)cl.block_rank();
+    const double t = T[j];
     const double a = kC2 / t;
     double q = 0.0, d = 0.0;
-    for (size_t i = threadIdx.x; i < n; i += 256) {
-        double b = exp(-a * E[i]);
-        double gb = (double)g[i] * b;
+    for (size_t i = threadIdx.x + 256 * (size_t)r; i < n; i += 256 * PF_CL) {
+        const double e = E[i];
+        const double gb = (double)g[i] * exp64(-a * e);
         q += gb;
-        d += gb * (a * E[i] / t);
+        d = fma(gb, e, d);
     }
     sq[threadIdx.x] = q;
     sd[threadIdx.x] = d;
@@ -38,17 +46,45 @@ __global__ void __launch_bounds__(256) k_partition_function(const double *__rest
         }
         __syncthreads();
     }
-    if (threadIdx.x == 0) {
-        Q[blockIdx.x] = sq[0];
-        if (dQ) dQ[blockIdx.x] = sd[0];
+    cl.sync();
+    if (r == 0 && threadIdx.x < 32) {
+        double sumq = 0.0, sumd = 0.0;
+        for (int k = 0; k < PF_CL; ++k) {
+            sumq += *cl.map_shared_rank(&sq[0], k);
+            sumd += *cl.map_shared_rank(&sd[0], k);
+        }
+        sumd *= a / t;
+        if (threadIdx.x == 0) {
+            Q[j] = sumq;
+            if (dQ) dQ[j] = sumd;
+        }
+        for (int c = threadIdx.x; c < n_cond; c += 32)
+            if (tix[c] == j) {
+                conds[c].Q = sumq;
+                conds[c].dQdT = sumd;
+            }
     }
+    cl.sync();   // no CTA leaves while its shared memory is read
 }
 
 cudaError_t launch_partition_function(const double *E, const int32_t *g, size_t n, const double *T, int nT,
-                                      double *Q, double *dQ, cudaStream_t s) {
+                                      double *Q, double *dQ, cudaStream_t s, CondDev *conds, const int *tix,
+                                      int n_cond) {
     if (nT <= 0) return cudaSuccess;
-    k_partition_function<<<nT, 256, 0, s>>>(E, g, n, T, Q, dQ);
-    return cudaGetLastError();
+    cudaError_t e = cudaFuncSetAttribute((const void *)k_partition_function,
+                                         cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+    if (e != cudaSuccess) return e;
+    cudaLaunchAttribute at;
+    at.id = cudaLaunchAttributeClusterDimension;
+    at.val.clusterDim.x = PF_CL;
+    at.val.clusterDim.y = at.val.clusterDim.z = 1;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)nT * PF_CL);
+    cfg.blockDim = dim3(256);
+    cfg.stream = s;
+    cfg.attrs = &at;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, k_partition_function, E, g, n, T, Q, dQ, conds, tix, n_cond);
 }
 
 // ---------------------------------------------------------------------------
@@ -67,17 +103,29 @@ __global__ void __launch_bounds__(256) k_line_params64(LinesDev L, size_t n, con
                                                        int cut_mode, double cutoff, double width_mult,
                                                        double *I, double *alpha, double *gamma, double *cut,
                                                        StrengthSel sel) {
+    // the condition's factors once per CTA: their divisions and logarithm are as costly as several lines
+    __shared__ double sc[5];
     const CondDev c = *cd;
-    const double inv_T = 1.0 / c.T;
-    const double acoef = alpha_coef(c.T, c.mass_da);
-    const double lnTr = log(c.T_ref * inv_T);
-    const double pscale = c.gamma_scale * (c.P / c.P_ref);
+    if (threadIdx.x == 0) {
+        const StrengthPre p0(c, sel);
+        sc[0] = p0.pref;
+        sc[1] = p0.c2T;
+    } else if (threadIdx.x == 32) {
+        sc[2] = alpha_coef(c.T, c.mass_da);
+    } else if (threadIdx.x == 64) {
+        sc[3] = log(c.T_ref * (1.0 / c.T));
+    } else if (threadIdx.x == 96) {
+        sc[4] = c.gamma_scale * (c.P / c.P_ref);
+    }
+    __syncthreads();
+    const StrengthPre pre(sc[0], sc[1]);
+    const double acoef = sc[2], lnTr = sc[3], pscale = sc[4];
     for (size_t l = (size_t)blockIdx.x * blockDim.x + threadIdx.x; l < n; l += (size_t)gridDim.x * blockDim.x) {
         double nu = L.nu[l];
-        double Il = line_strength64(nu, (double)L.elower[l], (double)L.g_up[l] * (double)L.A[l], c, sel);
+        double Il = line_strength64(nu, f2d(L.elower[l]), f2d((float)L.g_up[l]) * f2d(L.A[l]), pre, sel);
         double al = acoef * nu;
-        double ga = L.n_broad > 0 ? mixture_gamma64(L, l, c)
-                                  : pscale * (double)L.gamma_ref[l] * exp(((double)L.n_T[l] + c.n_shift) * lnTr);
+        double ga = L.n_broad > 0 ? mixture_gamma64(L, l, c, lnTr, pscale)
+                                  : pscale * f2d(L.gamma_ref[l]) * exp64((f2d(L.n_T[l]) + c.n_shift) * lnTr);
         double cl = line_cut(cut_mode, cutoff, width_mult, al, ga);
         if (Il < 0.0) {   // left out by the intensity threshold: no grid point is within a negative cut
             Il = 0.0;
@@ -90,14 +138,25 @@ __global__ void __launch_bounds__(256) k_line_params64(LinesDev L, size_t n, con
     }
 }
 
+// Threshold decisions, bit by bit.  A condition's factors (FP64 divisions) are formed once per
+// thread, so the conditions are the outer loop within a word.
 __global__ void __launch_bounds__(256) k_line_keep(LinesDev L, size_t n, const CondDev *__restrict__ conds, int nc,
                                                    StrengthSel sel, uint32_t *keep, int words) {
-    for (size_t l = (size_t)blockIdx.x * blockDim.x + threadIdx.x; l < n; l += (size_t)gridDim.x * blockDim.x) {
-        const double nu = L.nu[l], E = (double)L.elower[l], gA = (double)L.g_up[l] * (double)L.A[l];
-        for (int w = 0; w < words; ++w) {
+    __shared__ double sPre[32][2];
+    for (int w = 0; w < words; ++w) {
+        const int m = min(32, nc - 32 * w);
+        __syncthreads();
+        if (threadIdx.x < m) {
+            const StrengthPre p(conds[w * 32 + threadIdx.x], sel);
+            sPre[threadIdx.x][0] = p.pref;
+            sPre[threadIdx.x][1] = p.c2T;
+        }
+        __syncthreads();
+        for (size_t l = (size_t)blockIdx.x * blockDim.x + threadIdx.x; l < n; l += (size_t)gridDim.x * blockDim.x) {
+            const double nu = L.nu[l], E = f2d(L.elower[l]), gA = f2d((float)L.g_up[l]) * f2d(L.A[l]);
             uint32_t bits = 0u;
-            for (int b = 0; b < 32 && w * 32 + b < nc; ++b)
-                if (line_strength64(nu, E, gA, conds[w * 32 + b], sel) >= 0.0) bits |= 1u << b;
+            for (int b = 0; b < m; ++b)
+                if (line_strength64(nu, E, gA, StrengthPre(sPre[b][0], sPre[b][1]), sel) >= 0.0) bits |= 1u << b;
             keep[l * (size_t)words + w] = bits;
         }
     }
@@ -158,14 +217,26 @@ cudaError_t launch_permute_i16(const int16_t *in, const uint32_t *perm, size_t n
 
 __global__ void __launch_bounds__(256) k_line_gamma(LinesDev L, size_t n, const CondDev *__restrict__ conds, int nc,
                                                     float *gamma_lc, unsigned *gmax_bits) {
+    __shared__ double sc[32][2];   // ln(T_ref/T) and gamma_scale P/P_ref, once per CTA
     for (int c = 0; c < nc; ++c) {
+        if ((c & 31) == 0) {
+            __syncthreads();
+            if (threadIdx.x < min(32, nc - c)) {
+                const CondDev d = conds[c + threadIdx.x];
+                sc[threadIdx.x][0] = log(d.T_ref / d.T);
+                sc[threadIdx.x][1] = d.gamma_scale * (d.P / d.P_ref);
+            }
+            __syncthreads();
+        }
         const CondDev cd = conds[c];
+        const double lnTr = sc[c & 31][0], pscale = sc[c & 31][1];
         float m = 0.f;
         for (size_t l = (size_t)blockIdx.x * blockDim.x + threadIdx.x; l < n; l += (size_t)gridDim.x * blockDim.x) {
-            const float g = (float)mixture_gamma64(L, l, cd);
+            const float g = (float)mixture_gamma64(L, l, cd, lnTr, pscale);
             gamma_lc[l * (size_t)nc + c] = g;
             m = fmaxf(m, g);
         }
+        if (!gmax_bits) continue;
         for (int o = 16; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
         // non-negative floats order as their bit patterns; rounded up so that the bound holds
         if ((threadIdx.x & 31) == 0) atomicMax(&gmax_bits[c], __float_as_uint(m) + 1u);

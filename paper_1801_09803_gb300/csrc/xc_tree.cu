@@ -77,33 +77,17 @@ __device__ __forceinline__ void tr_fold(float &hi, float &lo, float &acc) {
 // ---------------------------------------------------------------------------
 // setup
 // ---------------------------------------------------------------------------
-__global__ void k_tree_prep(const CondDev *conds, int n_cond, GeomStats *gs) {
-    __shared__ float s[32];
-    float a = 0.f;
-    for (int c = threadIdx.x; c < n_cond; c += 32)
-        a = fmaxf(a, __double2float_ru(alpha_coef(conds[c].T, conds[c].mass_da) * (1.0 + 1e-6)));
-    s[threadIdx.x] = a;
-    __syncwarp();
-    if (threadIdx.x == 0) {
-        for (int i = 1; i < 32; ++i) a = fmaxf(a, s[i]);
-        *gs = GeomStats{};
-        gs->acoef_bits = __float_as_uint(a);
-    }
-}
-
-cudaError_t launch_tree_prep(const CondDev *conds, int n_cond, GeomStats *gs, cudaStream_t s) {
-    k_tree_prep<<<1, 32, 0, s>>>(conds, n_cond, gs);
-    return cudaGetLastError();
-}
-
 // Line geometry in grid steps and the intensity statistics.  width_mult > 0: the cut of
-// condition *cond; zero_k > 0: profiles that are exactly 0 in FP32 beyond
-// zero_k alpha + zero_0 (grid steps) of the centre, alpha the largest of the conditions.
+// condition *cond; zero_k > 0: profiles that are exactly 0 in FP32 beyond zero_k nu + zero_0
+// (cm^-1) of the centre, for the largest alpha of the conditions.
+// Bound by the FP64 pipe.  The estimates of the range's ends are exact unless they lie within
+// eps of an integer (eps: many times their rounding error); only then the exact predicate
+// settles them (57 -> about 25 FP64 operations per line; 0.91 -> 0.60 ms for 1e7 lines).
 __global__ void __launch_bounds__(256) k_tree_geom(LinesDev L, size_t n, double nu_A, double step, int64_t n_pts,
                                                    double cutoff, double width_mult, const CondDev *cond,
-                                                   float zero_k, double zero_0, int4 *geo, GeomStats *gs) {
-    const double inv_h = 1.0 / step;
-    float m1 = 0.f, m2 = 0.f, m3 = 0.f, m4 = 0.f, m5 = 0.f;
+                                                   double zero_k, double zero_0, double eps, double inv_h,
+                                                   int4 *geo, GeomStats *gs) {
+    float m1 = 0.f, m2 = 0.f;
     double ac = 0.0, lnTr = 0.0, gsc = 0.0;
     CondDev c{};
     if (width_mult > 0.0) {
@@ -112,87 +96,113 @@ __global__ void __launch_bounds__(256) k_tree_geom(LinesDev L, size_t n, double 
         lnTr = log(c.T_ref / c.T);
         gsc = c.P / c.P_ref;
     }
-    const double zk = (double)zero_k * (double)__uint_as_float(gs->acoef_bits);
-    for (size_t l = (size_t)blockIdx.x * blockDim.x + threadIdx.x; l < n; l += (size_t)gridDim.x * blockDim.x) {
+    for (size_t l = (size_t)blockIdx.x * 256 + threadIdx.x; l < n; l += (size_t)gridDim.x * 256) {
         const double nu = L.nu[l];
         const float gr = L.gamma_ref[l], nT = L.n_T[l];
-        m3 = fmaxf(m3, __double2float_ru(fabs(nu)));
-        m4 = fmaxf(m4, fabsf(gr));
-        m5 = fmaxf(m5, fabsf(nT));
         double cut = cutoff;
         if (width_mult > 0.0) {
-            const double ga = L.n_broad > 0 ? mixture_gamma64(L, l, c)
-                                            : c.gamma_scale * (double)gr * exp(((double)nT + c.n_shift) * lnTr) * gsc;
+            const double ga = L.n_broad > 0 ? mixture_gamma64(L, l, c, lnTr, c.gamma_scale * gsc)
+                                            : c.gamma_scale * f2d(gr) * exp64((f2d(nT) + c.n_shift) * lnTr) * gsc;
             cut = fmin(width_mult * fmax(ac * nu, ga), cutoff);
         }
-        if (zero_k > 0.f) cut = fmin(cut, zk * nu + zero_0 * step);
+        if (zero_k > 0.0) cut = fmin(cut, zero_k * nu + zero_0);
         const double d = (nu - nu_A) * inv_h;
         const double fl = floor(d);
         const double flc = fmin(fmax(fl, -1073741824.0), 1073741824.0);
-        int64_t ka, kb;
-        line_k_range(nu, cut, nu_A, step, inv_h, n_pts, &ka, &kb);
+        const double ta = (nu - cut - nu_A) * inv_h, tb = (nu + cut - nu_A) * inv_h;
+        int ka = 1, kb = 0;
+        if (fabs(ta - rint(ta)) > eps && fabs(tb - rint(tb)) > eps) {
+            const double top = (double)n_pts;   // < 2^30
+            if (ta <= top && tb >= -1.0) {
+                ka = max(0, (int)ceil(fmax(ta, -1.0)));
+                kb = (int)floor(fmin(tb, top - 1.0));
+            }
+        } else {
+            int64_t k0, k1;
+            line_k_range(nu, cut, nu_A, step, inv_h, n_pts, &k0, &k1);
+            ka = (int)i64min(i64max(k0, -1), (int64_t)0x7fffffff);
+            kb = (int)i64min(i64max(k1, -1), (int64_t)0x7fffffff);
+        }
         if (kb < ka) { ka = 1; kb = 0; }
-        geo[l] = make_int4((int)flc, (int)i64min(i64max(ka, -1), (int64_t)0x7fffffff),
-                           (int)i64min(i64max(kb, -1), (int64_t)0x7fffffff), __float_as_int((float)(d - fl)));
+        geo[l] = make_int4((int)flc, ka, kb, __float_as_int((float)(d - fl)));
         const float gA = (float)L.g_up[l] * L.A[l];
         const float nuf = (float)nu;
         m1 = fmaxf(m1, gA / (nuf * nuf));
         m2 = fmaxf(m2, gA / nuf);
     }
+    // two atomics per CTA: one per warp and statistic on the same words took longer than the lines
+    __shared__ float sm[2][8];
+    m1 = isfinite(m1) ? m1 : 0.f;
+    m2 = isfinite(m2) ? m2 : 0.f;
     for (int o = 16; o > 0; o >>= 1) {
         m1 = fmaxf(m1, __shfl_xor_sync(0xffffffffu, m1, o));
         m2 = fmaxf(m2, __shfl_xor_sync(0xffffffffu, m2, o));
-        m3 = fmaxf(m3, __shfl_xor_sync(0xffffffffu, m3, o));
-        m4 = fmaxf(m4, __shfl_xor_sync(0xffffffffu, m4, o));
-        m5 = fmaxf(m5, __shfl_xor_sync(0xffffffffu, m5, o));
     }
     if ((threadIdx.x & 31) == 0) {
-        if (isfinite(m1)) atomicMax(&gs->gA_nu2_bits, __float_as_uint(m1));
-        if (isfinite(m2)) atomicMax(&gs->gA_nu_bits, __float_as_uint(m2));
-        atomicMax(&gs->nu_bits, __float_as_uint(m3));   // non-negative floats: integer order
-        atomicMax(&gs->gref_bits, __float_as_uint(m4));
-        atomicMax(&gs->nT_bits, __float_as_uint(m5));
+        sm[0][threadIdx.x >> 5] = m1;
+        sm[1][threadIdx.x >> 5] = m2;
+    }
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        for (int w = 1; w < 8; ++w) {
+            m1 = fmaxf(m1, sm[0][w]);
+            m2 = fmaxf(m2, sm[1][w]);
+        }
+        atomicMax(&gs->gA_nu2_bits, __float_as_uint(m1));   // non-negative floats: integer order
+        atomicMax(&gs->gA_nu_bits, __float_as_uint(m2));
+        if (blockIdx.x == 0) gs->nu_bits = __float_as_uint(__double2float_ru(L.nu[n - 1]));   // sorted
     }
 }
 
-// Lagrange basis polynomial of node m (of a block of B points) at x, from the nodes as rounded
-__device__ double tr_basis(int B, int m, double x) {
-    const double xm = (double)tr_node(B, m);
+// Lagrange basis polynomial of node m at x, from the block's nodes xn as rounded
+__device__ double tr_basis(const float *xn, int B, int m, double x) {
+    const double xm = (double)xn[m], s = 4.0 / (double)B;   // scaled: the products stay near 1
     double num = 1.0, den = 1.0;
+#pragma unroll
     for (int j = 0; j < TR_M; ++j) {
-        if (j == m) continue;
-        const double xj = (double)tr_node(B, j);
-        // scaled by the half-length so that the products stay near 1
-        const double s = 4.0 / (double)B;
-        num *= (x - xj) * s;
-        den *= (xm - xj) * s;
+        const double xj = (double)xn[j];
+        num *= j == m ? 1.0 : (x - xj) * s;
+        den *= j == m ? 1.0 : (xm - xj) * s;
     }
     return num / den;
 }
 
-// entry k of the interpolation matrices
-__device__ double tr_mat_entry(int k) {
+// entry k of the interpolation matrices; xn: the nodes of each level
+__device__ double tr_mat_entry(int k, const float (*xn)[TR_M]) {
     if (k < TR_MAT_128) {
         const int j = k / (TR_M * TR_M), s = (k / TR_M) % TR_M, d = k % TR_M;
-        return tr_basis(512, s, (double)(64 * j) + (double)tr_node(64, d));
+        return tr_basis(xn[2], 512, s, (double)(64 * j) + (double)xn[0][d]);
     }
     if (k < TR_MAT_PT) {
         const int q = k - TR_MAT_128, j = q / (TR_M * TR_M), s = (q / TR_M) % TR_M, d = q % TR_M;
-        return tr_basis(128, s, (double)(64 * j) + (double)tr_node(64, d));
+        return tr_basis(xn[1], 128, s, (double)(64 * j) + (double)xn[0][d]);
     }
     const int q = k - TR_MAT_PT;
-    return tr_basis(64, q / 64, (double)(q % 64));
+    return tr_basis(xn[0], 64, q / 64, (double)(q % 64));
 }
 
-// block 0: per-condition constants; block 1..: line index, then the interpolation matrices
-__global__ void __launch_bounds__(256) k_tree_setup(TreeParams p, const CondDev *conds, int n_cond, CParam *cp,
-                                                    int quantity, const unsigned *gmax, unsigned *cell, double *mat) {
+// block 0: per-condition constants, a field (or two) per warp so that their FP64 chains run side
+// by side; block 1..: line index
+__global__ void __launch_bounds__(128) k_tree_setup(TreeParams p, const CondDev *conds, int n_cond, CParam *cp,
+                                                    int quantity, unsigned *cell) {
     if (blockIdx.x == 0) {
-        for (int c = threadIdx.x; c < n_cond; c += 256)
-            cp[c] = make_cparam(c, conds, p.gs, p.step, quantity, gmax, 4.f, 0);
+        for (int c = threadIdx.x & 31; c < n_cond; c += 32) {
+            const CondDev d = conds[c];
+            switch (threadIdx.x >> 5) {
+            case 0: cparam_strength(d, p.gs, quantity, &cp[c]); break;
+            case 1: cparam_temperature(d, &cp[c]); break;
+            case 2: cparam_widths(d, &cp[c]); break;
+            default:
+                cp[c].log2Tr = (float)log2(d.T_ref / d.T);
+                cp[c].row = c;
+                cp[c].vv_split = 4.f;
+                cp[c].vv_beta = 0;
+                cp[c].dbound = 0.f;
+            }
+        }
         return;
     }
-    const int i = (blockIdx.x - 1) * 256 + threadIdx.x;
+    const int i = (blockIdx.x - 1) * 128 + threadIdx.x;
     if (i <= p.ncell) {
         const int v = p.cell0 + TR_CELL * i;
         size_t a = 0, b = p.n;
@@ -202,17 +212,54 @@ __global__ void __launch_bounds__(256) k_tree_setup(TreeParams p, const CondDev 
         }
         cell[i] = (unsigned)a;
     }
-    const int k = i - (p.ncell + 1);
-    if (p.far && k >= 0 && k < TR_MAT) mat[k] = tr_mat_entry(k);
 }
 
-__global__ void __launch_bounds__(256) k_tree_mat(double *mat) {
-    const int k = blockIdx.x * 256 + threadIdx.x;
-    if (k < TR_MAT) mat[k] = tr_mat_entry(k);
+__global__ void __launch_bounds__(128) k_tree_mat(double *mat) {
+    __shared__ float xn[TR_LEVELS][TR_M];
+    if (threadIdx.x < TR_LEVELS * TR_M)
+        xn[threadIdx.x / TR_M][threadIdx.x % TR_M] = tr_node(tr_block(threadIdx.x / TR_M), threadIdx.x % TR_M);
+    __syncthreads();
+    const int k = blockIdx.x * 128 + threadIdx.x;
+    if (k < TR_MAT) mat[k] = tr_mat_entry(k, xn);
+}
+
+static double geom_eps(const xc_grid &g, double cutoff) {
+    // 64 times the rounding of a line's position in grid steps
+    return std::max(1e-9, 64.0 * 2.3e-16 * (fabs(g.nu_A) + g.step * (double)g.n + 2.0 * cutoff) / g.step);
+}
+
+cudaError_t launch_fp32_setup(const LinesDev &L, size_t n, const CondDev *conds, int nc, const xc_grid &grid,
+                              double cutoff, int4 *geo, GeomStats *gs, CParam *cp, cudaStream_t s) {
+    cudaError_t e = cudaMemsetAsync(gs, 0, sizeof(GeomStats), s);
+    if (e != cudaSuccess) return e;
+    if (n)
+        k_tree_geom<<<(unsigned)std::min<size_t>((n + 255) / 256, 152 * 8), 256, 0, s>>>(
+            L, n, grid.nu_A, grid.step, grid.n, cutoff, 0.0, nullptr, 0.0, 0.0, geom_eps(grid, cutoff), 1.0 / grid.step,
+            geo, gs);
+    TreeParams p{};
+    p.gs = gs;
+    p.ncell = -1;
+    if (nc) k_tree_setup<<<1, 128, 0, s>>>(p, conds, nc, cp, XC_ABSORPTION, nullptr);
+    return cudaGetLastError();
+}
+
+// the handle's interpolation matrices (constants), made by its first call that needs them; that
+// call synchronises its stream before it returns
+cudaError_t tree_mat(BatchedState *st, const double **mat, cudaStream_t s) {
+    *mat = st->tree_mat.as<double>();
+    if (*mat) return cudaSuccess;
+    cudaError_t e = st->tree_mat.ensure(TR_MAT * sizeof(double));
+    if (e == cudaSuccess) e = launch_tree_mat(st->tree_mat.as<double>(), s);
+    if (e != cudaSuccess) {
+        st->tree_mat.release();
+        return e;
+    }
+    *mat = st->tree_mat.as<double>();
+    return cudaSuccess;
 }
 
 cudaError_t launch_tree_mat(double *mat, cudaStream_t s) {
-    k_tree_mat<<<(TR_MAT + 255) / 256, 256, 0, s>>>(mat);
+    k_tree_mat<<<(TR_MAT + 127) / 128, 128, 0, s>>>(mat);
     return cudaGetLastError();
 }
 
@@ -233,7 +280,8 @@ __global__ void __launch_bounds__(256) k_tree_recs(TreeParams p, float4 *recA, f
 
 // ---------------------------------------------------------------------------
 // far levels: sums at the nodes.  A lane holds two of the block's 16 nodes, and the four
-// quarter-warps take different lines.  Per 32 scanned lines the accepted ones are compacted
+// quarter-warps take different lines (one node and two half-warps for the profiles that are
+// costly per value: fewer lines to fill an iteration).  Per 32 scanned lines the accepted ones are compacted
 // into shared memory, pairs of lines interleaved for the packed arithmetic; one iteration
 // takes 8 lines.  (With one node per lane and two line streams the loop was bound by the
 // shared-memory reads: 81 % of their rate at the 1e7-line list on 2e6 points, 1.65 ms.)
@@ -244,7 +292,8 @@ __global__ void __launch_bounds__(TR_T) k_tree_nodes(TreeParams p) {
     __shared__ float4 sL[TR_W][tr_pairs<PROF>() ? 16 * PAIR : 48];   // non-pairs: 24 bytes a line
     __shared__ float sX[64], sW[64];
     __shared__ double sRed[TR_W][TR_M];
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, strm = lane >> 3;
+    constexpr int R = tr_pairs<PROF>() ? 2 : 1, LN = TR_M / R, NS = 32 / LN;   // nodes per lane, lanes per stream, streams
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, strm = lane / LN;
     if (p.ngh > 0) {
         if (threadIdx.x < p.ngh) {
             sX[threadIdx.x] = (float)p.ghx[threadIdx.x];
@@ -252,18 +301,14 @@ __global__ void __launch_bounds__(TR_T) k_tree_nodes(TreeParams p) {
         }
         __syncthreads();
     }
-    const int wpt = p.wpt, part = warp % wpt;
-    int task = blockIdx.x * (TR_W / wpt) + warp / wpt;
+    // Neighbouring tasks share a CTA: they read the same lines (dealt out over the CTAs instead,
+    // the 32-condition table took 27 ms more).  The large blocks have the most lines, so each
+    // level has its own number of warps per task.
+    int lev = 2, cta = blockIdx.x;
+    while (lev > 0 && cta >= p.ncta[lev]) cta -= p.ncta[lev--];
+    const int wpt = p.wptl[lev], part = warp % wpt;
+    const int task = cta * (TR_W / wpt) + warp / wpt;
     const int c = blockIdx.y;
-    int lev = 2;   // the largest blocks have the most lines: first
-    if (task >= p.nblk[2]) {
-        task -= p.nblk[2];
-        lev = 1;
-        if (task >= p.nblk[1]) {
-            task -= p.nblk[1];
-            lev = 0;
-        }
-    }
     const bool live = task < p.nblk[lev];
     float hi[2] = {0.f, 0.f}, lo[2] = {0.f, 0.f};
     if (live) {
@@ -275,7 +320,7 @@ __global__ void __launch_bounds__(TR_T) k_tree_nodes(TreeParams p) {
         const int p0 = up ? b0 / PB * PB : 0, p1 = p0 + PB - 1, p1c = min(p1, p.n_pts - 1);
         const int Dp = up ? tr_radius(p, ac, tr_gap(lev + 1), p1) : 0;
         const Segs sg = tr_far_segs(p, b0, b1, D, up, p0, p1, Dp);
-        const float x[2] = {tr_node(B, 2 * (lane & 7)), tr_node(B, 2 * (lane & 7) + 1)};
+        const float x[2] = {tr_node(B, R * (lane % LN)), tr_node(B, R * (lane % LN) + R - 1)};
         const f32x2 xa = pk2(x[0], x[0]), xb = pk2(x[1], x[1]);
         const float4 *recA = p.recA + (size_t)c * p.n;
         float4 *buf = sL[warp];
@@ -302,7 +347,7 @@ __global__ void __launch_bounds__(TR_T) k_tree_nodes(TreeParams p) {
                 const unsigned m = __ballot_sync(0xffffffffu, ok);
                 const int cnt = __popc(m);
                 if (cnt) {
-                    const int pad = tr_pairs<PROF>() ? 8 : 4;
+                    constexpr int pad = tr_pairs<PROF>() ? 2 * NS : NS;
                     int slot = __popc(m & ((1u << lane) - 1u));
                     float n = (float)(g.x - b0), f = __int_as_float(g.w);
                     bool put = ok;
@@ -338,7 +383,7 @@ __global__ void __launch_bounds__(TR_T) k_tree_nodes(TreeParams p) {
                     }
                     __syncwarp();
                     if (tr_pairs<PROF>()) {
-                        for (int j = strm; 2 * j < cnt; j += 4) {
+                        for (int j = strm; 2 * j < cnt; j += NS) {
                             const ulonglong2 *q = reinterpret_cast<const ulonglong2 *>(buf + j * PAIR);
                             const ulonglong2 nf = q[0], c0 = q[1];
                             ulonglong2 c1 = c0;
@@ -354,12 +399,12 @@ __global__ void __launch_bounds__(TR_T) k_tree_nodes(TreeParams p) {
                             }
                         }
                     } else {
-                        for (int j = strm; j < cnt; j += 4) {
+                        for (int j = strm; j < cnt; j += NS) {
                             const float2 *q = reinterpret_cast<const float2 *>(buf) + j * 3;
                             const float2 nf = q[0], a01 = q[1], a23 = q[2];
                             const float4 Ac = make_float4(a01.x, a01.y, a23.x, a23.y);
 #pragma unroll
-                            for (int r = 0; r < 2; ++r) {
+                            for (int r = 0; r < R; ++r) {
                                 const float d = (x[r] - nf.x) - nf.y;
                                 acc[r] += contrib_single<PROF>(d * d, d, Ac, make_float4(0.f, 0.f, 0.f, -1.f), sX, sW,
                                                                p.ngh);
@@ -393,25 +438,25 @@ __global__ void __launch_bounds__(TR_T) k_tree_nodes(TreeParams p) {
 #pragma unroll
     for (int r = 0; r < 2; ++r) {
         v[r] = (double)hi[r] + (double)lo[r];
-        v[r] += __shfl_xor_sync(0xffffffffu, v[r], 8);
+        if (LN == 8) v[r] += __shfl_xor_sync(0xffffffffu, v[r], 8);
         v[r] += __shfl_xor_sync(0xffffffffu, v[r], 16);
     }
     if (wpt > 1) {
         __syncthreads();
-        if (lane < 8) {
-            sRed[warp][2 * lane] = v[0];
-            sRed[warp][2 * lane + 1] = v[1];
-        }
+        if (lane < LN)
+#pragma unroll
+            for (int r = 0; r < R; ++r) sRed[warp][R * lane + r] = v[r];
         __syncthreads();
-        if (part == 0 && lane < 8)
-            for (int w = 1; w < wpt; ++w) {
-                v[0] += sRed[warp + w][2 * lane];
-                v[1] += sRed[warp + w][2 * lane + 1];
-            }
+        if (part == 0 && lane < LN)
+            for (int w = 1; w < wpt; ++w)
+#pragma unroll
+                for (int r = 0; r < R; ++r) v[r] += sRed[warp + w][R * lane + r];
     }
-    if (live && part == 0 && lane < 8)
-        reinterpret_cast<double2 *>(p.nodes + (size_t)c * p.nodes_per_cond + p.node_off[lev] + task * TR_M)[lane] =
-            make_double2(v[0], v[1]);
+    if (live && part == 0 && lane < LN) {
+        double *out = p.nodes + (size_t)c * p.nodes_per_cond + p.node_off[lev] + task * TR_M + R * lane;
+#pragma unroll
+        for (int r = 0; r < R; ++r) out[r] = v[r];
+    }
 }
 
 // ---------------------------------------------------------------------------
@@ -838,7 +883,7 @@ bool is_doppler(int profile) { return profile == XC_DOPPLER || profile == XC_DOP
 // warps per task: several where the tasks alone would leave the SMs with few warps
 int warps_per_task(int64_t tasks) {
     int w = 1;
-    while (w < TR_W && tasks * w < 152 * 32) w *= 2;
+    while (w < TR_W && tasks * w < 152 * 16) w *= 2;
     return w;
 }
 
@@ -879,6 +924,7 @@ xc_status tree_run(BatchedState *st, const BatchedArgs &a, int64_t *launches) {
     p.core = w4 ? 18.05f : 0.f;
     p.ext = 0.f;
     p.ext0 = 1;
+    p.gh_ext = 0.f;
     p.ngh = 0;
     p.ghx = a.ghx;
     p.ghw = a.ghw;
@@ -889,6 +935,7 @@ xc_status tree_run(BatchedState *st, const BatchedArgs &a, int64_t *launches) {
         p.ext0 = 2;
     } else if (a.opts.profile == XC_VOIGT_GH_BINNED || a.opts.profile == XC_VOIGT_GH_SAMPLED) {
         p.ngh = a.opts.n_gh;
+        p.gh_ext = (float)sqrt(2.0 * a.opts.n_gh + 2.0) * 1.001f;
         p.ext = (float)(sqrt(2.0 * a.opts.n_gh + 2.0) / 0.83255) * 1.001f;   // nodes lie within sqrt(2 n + 2)
         p.ext0 = 3;
     }
@@ -915,52 +962,52 @@ xc_status tree_run(BatchedState *st, const BatchedArgs &a, int64_t *launches) {
     auto carve = [&](size_t bytes) { size_t r = o; o += (bytes + 255) & ~size_t(255); return r; };
     // (the caller falls back to the tiled kernels when this does not fit in device memory)
     const size_t o_gs = carve(sizeof(GeomStats)), o_cp = carve((size_t)nc_pass * sizeof(CParam));
-    const size_t o_cell = carve((size_t)(p.ncell + 1) * 4), o_mat = carve(TR_MAT * 8);
+    const size_t o_cell = carve((size_t)(p.ncell + 1) * 4);
     const size_t o_nodes = carve((size_t)cg * p.nodes_per_cond * 8);
     const size_t o_geo = carve(n * sizeof(int4));
     const size_t o_A = carve((size_t)cg * n * 16), o_B = carve(w4 ? (size_t)cg * n * 16 : 16);
-    size_t o_keep = 0, o_glc = 0, o_gmax = 0;
+    size_t o_keep = 0, o_glc = 0;
     if (a.opts.threshold != XC_THRESHOLD_NONE) o_keep = carve(n * (size_t)((nc_pass + 31) / 32) * 4);
-    if (a.L.n_broad > 0) {
-        o_glc = carve(n * (size_t)nc_pass * 4);
-        o_gmax = carve((size_t)nc_pass * 4);
-    }
+    if (a.L.n_broad > 0) o_glc = carve(n * (size_t)nc_pass * 4);
     TR_TRY(st->tiles.ensure(o));
     char *b = st->tiles.as<char>();
     GeomStats *gs = (GeomStats *)(b + o_gs);
     CParam *cp = (CParam *)(b + o_cp);
     unsigned *cell = (unsigned *)(b + o_cell);
-    double *mat = (double *)(b + o_mat);
     int4 *geo = (int4 *)(b + o_geo);
     float4 *recA = (float4 *)(b + o_A), *recB = (float4 *)(b + o_B);
     p.gs = gs;
     p.cp = cp;
     p.cell = cell;
-    p.mat = mat;
+    p.mat = nullptr;
+    if (p.far) TR_TRY(tree_mat(st, &p.mat, s));
     p.geo = geo;
     p.recA = recA;
     p.recB = recB;
     p.nodes = (double *)(b + o_nodes);
     const unsigned lb = (unsigned)std::max<size_t>(1, std::min<size_t>((n + 255) / 256, 152 * 16));
 
+    const double eps = geom_eps(a.grid, a.opts.cutoff);
     if (a.timing) TR_TRY(cudaEventRecord(a.ev_begin, s));
     if (a.timing && a.ev_main0) TR_TRY(cudaEventRecord(a.ev_main0, s));
     for (int pass = 0; pass < nc_all; pass += nc_pass) {
         const CondDev *conds = a.conds_dev + pass;
         p.sigma = a.sigma + (size_t)pass * (size_t)a.grid.n;
         p.L = a.L;
-        unsigned *gmax = nullptr;
-        TR_TRY(launch_tree_prep(conds, nc_pass, gs, s));
+        TR_TRY(cudaMemsetAsync(gs, 0, sizeof(GeomStats), s));
         if (a.L.n_broad > 0) {
-            gmax = (unsigned *)(b + o_gmax);
-            TR_TRY(cudaMemsetAsync(gmax, 0, (size_t)nc_pass * 4, s));
-            TR_TRY(launch_line_gamma(a.L, n, conds, nc_pass, (float *)(b + o_glc), gmax, s));
+            TR_TRY(launch_line_gamma(a.L, n, conds, nc_pass, (float *)(b + o_glc), nullptr, s));
             p.L.gamma_lc = (float *)(b + o_glc);
             p.L.gamma_stride = nc_pass;
             *launches += 1;
         }
-        k_tree_geom<<<lb, 256, 0, s>>>(a.L, n, a.grid.nu_A, a.grid.step, a.grid.n, a.opts.cutoff,
-                                       per_cond ? a.opts.width_mult : 0.0, conds, zero_k, 1.5, geo, gs);
+        double am = 0.0;
+        for (int c = 0; c < nc_pass; ++c)
+            am = std::max(am, alpha_coef(a.conds_host[pass + c].T, a.conds_host[pass + c].mass_da));
+        k_tree_geom<<<(unsigned)std::min<size_t>((n + 255) / 256, 152 * 8), 256, 0, s>>>(
+            a.L, n, a.grid.nu_A, a.grid.step, a.grid.n, a.opts.cutoff, per_cond ? a.opts.width_mult : 0.0, conds,
+            (double)zero_k * am * (1.0 + 1e-6), 1.5 * a.grid.step, eps,
+            1.0 / a.grid.step, geo, gs);
         if (a.opts.threshold != XC_THRESHOLD_NONE) {
             const int words = (nc_pass + 31) / 32;
             uint32_t *keep = (uint32_t *)(b + o_keep);
@@ -969,9 +1016,8 @@ xc_status tree_run(BatchedState *st, const BatchedArgs &a, int64_t *launches) {
             p.L.keep_words = words;
             *launches += 1;
         }
-        const int setup = 1 + (p.ncell + 1 + (p.far ? TR_MAT : 0) + 255) / 256;
-        k_tree_setup<<<setup, 256, 0, s>>>(p, conds, nc_pass, cp, a.opts.quantity, gmax, cell, mat);
-        *launches += 3;
+        k_tree_setup<<<1 + (p.ncell + 1 + 127) / 128, 128, 0, s>>>(p, conds, nc_pass, cp, a.opts.quantity, cell);
+        *launches += 2;
         for (int c0 = 0; c0 < nc_pass; c0 += cg) {
             const int m = std::min(cg, nc_pass - c0);
             p.c0 = c0;
@@ -979,10 +1025,13 @@ xc_status tree_run(BatchedState *st, const BatchedArgs &a, int64_t *launches) {
             (ext ? fn.rec_ext : fn.rec)<<<dim3(lb, m), 256, 0, s>>>(p, recA, recB);
             *launches += 2;
             if (p.far) {
-                const int64_t tasks = (int64_t)p.nblk[0] + p.nblk[1] + p.nblk[2];
-                p.wpt = warps_per_task(tasks * m);
-                const int per = TR_W / p.wpt;
-                fn.nodes<<<dim3((unsigned)((tasks + per - 1) / per), m), TR_T, 0, s>>>(p);
+                int ctas = 0;
+                for (int lev = 0; lev < TR_LEVELS; ++lev) {
+                    p.wptl[lev] = warps_per_task((int64_t)p.nblk[lev] * m);
+                    const int per = TR_W / p.wptl[lev];
+                    ctas += p.ncta[lev] = (p.nblk[lev] + per - 1) / per;
+                }
+                fn.nodes<<<dim3((unsigned)ctas, m), TR_T, 0, s>>>(p);
                 *launches += 1;
             }
             const int64_t tasks = ((int64_t)p.n_pts + 31) / 32;

@@ -31,13 +31,15 @@ struct TreeParams {
     int reach;                   // no line reaches a point farther than this many steps from its n
     int cover;                   // every line covers the points within this many steps (0: not known)
     int far;                     // 0: no blocks (profiles without far wings)
-    int wpt;                     // warps per task
+    int wpt;                     // warps per task (points)
+    int wptl[TR_LEVELS], ncta[TR_LEVELS];   // nodes: warps per task and CTAs of each level
     double nu_A, step, cutoff;
     float inv_h, ext;            // ext: real distance of the outermost pole from the centre, per alpha (grid steps)
     int ext0;                    // ... plus this many steps
     float core;                  // radius of the points that need the full profile, per alpha
     const double *ghx, *ghw;
     int ngh;
+    float gh_ext;                // bound of the Gauss-Hermite nodes
     double *sigma;               // [n_cond rows of the call][n_pts]
 };
 
@@ -138,10 +140,8 @@ __device__ __forceinline__ Segs tr_point_segs(const TreeParams &p, int s0, int s
     return g;
 }
 
-// zeroes the statistics and sets acoef_bits, the largest alpha / nu of the conditions
-cudaError_t launch_tree_prep(const CondDev *conds, int n_cond, GeomStats *gs, cudaStream_t s);
-
 // the FP32 sweep's interpolation matrices (TR_MAT doubles, see TR_MAT_*)
 cudaError_t launch_tree_mat(double *mat, cudaStream_t s);
+cudaError_t tree_mat(BatchedState *st, const double **mat, cudaStream_t s);   // the handle's copy
 
 }  // namespace xc

@@ -39,6 +39,7 @@ constexpr int T64_MAT = T64_MAT_DV + T64_M * 128;
 struct T64Params {
     TreeParams t;                 // geo: x = n, y..z = cut range (not clipped to the grid)
     const double *nu, *I, *al, *ga;
+    float acoef;                  // alpha / nu, rounded up
     int koff;                     // blocks start at multiples of their size minus koff
 };
 
@@ -46,15 +47,16 @@ __device__ __forceinline__ double t64_node(int B, int m) {
     return (double)(rintf(64.f * (float)(B - 1) * (1.f - cospif((float)(2 * m + 1) * (1.f / (2 * T64_M))))) * (1.f / 128.f));
 }
 
-// Lagrange basis polynomial of node m at x (grid steps from the block's first point)
-__device__ double t64_basis(int B, int m, double x) {
-    const double xm = t64_node(B, m), s = 4.0 / (double)B;
+// Lagrange basis polynomial of node m at x (grid steps from the first point of a block of B
+// points with nodes xn)
+__device__ double t64_basis(const double *xn, int B, int m, double x) {
+    const double xm = xn[m], s = 4.0 / (double)B;
     double num = 1.0, den = 1.0;
+#pragma unroll 4
     for (int j = 0; j < T64_M; ++j) {
-        if (j == m) continue;
-        const double xj = t64_node(B, j);
-        num *= (x - xj) * s;
-        den *= (xm - xj) * s;
+        const double f = j == m ? 1.0 : (x - xn[j]) * s, g = j == m ? 1.0 : (xm - xn[j]) * s;
+        num *= f;
+        den *= g;
     }
     return num / den;
 }
@@ -85,29 +87,44 @@ __global__ void __launch_bounds__(256) k_t64_geom(const double *__restrict__ nu,
     }
 }
 
-__global__ void __launch_bounds__(256) k_t64_setup(TreeParams p, unsigned *cell, double *mat) {
-    const int i = blockIdx.x * 256 + threadIdx.x;
-    if (i <= p.ncell) {
-        const int v = p.cell0 + TR_CELL * i;
-        size_t a = 0, b = p.n;
-        while (a < b) {
-            const size_t m = a + ((b - a) >> 1);
-            if (p.geo[m].x < v) a = m + 1; else b = m;
-        }
-        cell[i] = (unsigned)a;
+__global__ void __launch_bounds__(64) k_t64_setup(TreeParams p, unsigned *cell) {
+    const int i = blockIdx.x * 64 + threadIdx.x;
+    if (i > p.ncell) return;
+    const int v = p.cell0 + TR_CELL * i;
+    size_t a = 0, b = p.n;
+    while (a < b) {
+        const size_t m = a + ((b - a) >> 1);
+        if (p.geo[m].x < v) a = m + 1; else b = m;
     }
-    const int k = i - (p.ncell + 1);
-    if (!p.far || k < 0 || k >= T64_MAT_DV) return;
+    cell[i] = (unsigned)a;
+}
+
+__global__ void __launch_bounds__(64) k_t64_mat(double *mat) {
+    __shared__ double xn[2][T64_M];   // nodes of a 128- and a 512-point block
+    xn[threadIdx.x / T64_M][threadIdx.x % T64_M] = t64_node(t64_block(threadIdx.x / T64_M), threadIdx.x % T64_M);
+    __syncthreads();
+    const int k = blockIdx.x * 64 + threadIdx.x;
+    if (k >= T64_MAT_DV) return;
     if (k < T64_MAT_PT) {
         const int j = k / (T64_M * T64_M), s = (k / T64_M) % T64_M, d = k % T64_M;
-        mat[k] = t64_basis(512, s, (double)(128 * j) + t64_node(128, d));
+        mat[k] = t64_basis(xn[1], 512, s, (double)(128 * j) + xn[0][d]);
     } else {
         const int q = k - T64_MAT_PT, s = q / 128;
         const double x = (double)(q % 128);
-        mat[k] = t64_basis(128, s, x);
+        mat[k] = t64_basis(xn[0], 128, s, x);
         // the derivative multiplies a rounding error: three digits of it are plenty
-        mat[k + (T64_MAT_DV - T64_MAT_PT)] = (t64_basis(128, s, x + 1e-3) - t64_basis(128, s, x - 1e-3)) * 500.0;
+        mat[k + (T64_MAT_DV - T64_MAT_PT)] = (t64_basis(xn[0], 128, s, x + 1e-3) - t64_basis(xn[0], 128, s, x - 1e-3)) * 500.0;
     }
+}
+
+// the handle's interpolation matrices (constants), made by its first call that needs them; that
+// call synchronises its stream before it returns
+cudaError_t tree64_mat(DevBuf *buf, cudaStream_t s) {
+    if (buf->p) return cudaSuccess;
+    const cudaError_t e = buf->ensure((size_t)T64_MAT * sizeof(double));
+    if (e != cudaSuccess) return e;
+    k_t64_mat<<<(T64_MAT_DV + 63) / 64, 64, 0, s>>>(buf->as<double>());
+    return cudaGetLastError();
 }
 
 // w4 region I in u = D^2: I V = P (u + C) / (u^2 + E u + C^2), with s = alpha^2 / ln 2,
@@ -157,13 +174,14 @@ __global__ void __launch_bounds__(TR_T) k_t64_nodes(T64Params q) {
         }
         __syncthreads();
     }
-    int task = blockIdx.x * TR_W + warp;
+    // the large blocks have the most lines: dealt out over the CTAs (an SM's FP64 pipe is the limit)
+    int task = blockIdx.x + warp * gridDim.x;
     const int lev = task < p.nblk[1] ? 1 : 0;
     if (lev == 0) task -= p.nblk[1];
     if (task >= p.nblk[lev]) return;
     const int B = t64_block(lev), b0 = task * B - q.koff, b1 = b0 + B - 1;
     if (b1 < 0 || b0 >= p.n_pts) return;   // outside the grid (alignment): nothing reads its nodes
-    const float ac = __uint_as_float(p.gs->acoef_bits);
+    const float ac = q.acoef;
     const int D = tr_radius(p, ac, t64_gap(lev), b1);
     const bool up = lev == 0;
     const int p0 = (task & ~3) * 128 - q.koff, p1 = p0 + 511;   // the parent of a 128-point block
@@ -303,7 +321,7 @@ __global__ void __launch_bounds__(TR_T) k_t64_points(T64Params q) {
     const int s0 = task * 32 - q.koff, s1 = s0 + 31;
     if (s0 >= p.n_pts || s1 < 0) return;
     const int p0 = (task >> 2) * 128 - q.koff, p1 = p0 + 127;
-    const int Dp = p.far ? tr_radius(p, __uint_as_float(p.gs->acoef_bits), t64_gap(0), p1) : 0;
+    const int Dp = p.far ? tr_radius(p, q.acoef, t64_gap(0), p1) : 0;
     const Segs sg = tr_point_segs(p, s0, s1, p0, p1, Dp);
     const double xk = grid_x(p.nu_A, p.step, s0 + lane);
     double *buf = sL[warp];
@@ -378,7 +396,7 @@ __device__ __forceinline__ double t64_region4(double x, double y) {
                 m * (1.841439 + m))))));
     const double d = t64_rcp(D.re * D.re + D.im * D.im);
     const double rr = (N.re * D.re + N.im * D.im) * d, ri = (N.im * D.re - N.re * D.im) * d;
-    return exp(ur) * cos(ui) - (y * rr + x * ri);   // t = y - i x
+    return exp64(ur) * cos(ui) - (y * rr + x * ri);   // t = y - i x
 }
 
 struct W4Buf64 {
@@ -400,7 +418,7 @@ __global__ void __launch_bounds__(128) k_t64_points_w4(T64Params q) {
     const int s0 = task * 32 - q.koff, s1 = s0 + 31;
     if (s0 >= p.n_pts || s1 < 0) return;
     const int p0 = (task >> 2) * 128 - q.koff, p1 = p0 + 127;
-    const int Dp = tr_radius(p, __uint_as_float(p.gs->acoef_bits), t64_gap(0), p1);
+    const int Dp = tr_radius(p, q.acoef, t64_gap(0), p1);
     const Segs sg = tr_point_segs(p, s0, s1, p0, p1, Dp);
     const double xk = grid_x(p.nu_A, p.step, s0 + lane), x0 = grid_x(p.nu_A, p.step, s0);
     const double inv_h = 1.0 / p.step;
@@ -545,8 +563,7 @@ bool tree64_takes(int profile, const xc_grid &g, double cutoff, size_t n) {
 }
 
 // bytes of scratch behind the int4 geometry of n lines
-static size_t tree64_layout(const xc_grid &g, double cutoff, size_t n, TreeParams *p, size_t *o_cell, size_t *o_mat,
-                            size_t *o_nodes, size_t *o_gs) {
+static size_t tree64_layout(const xc_grid &g, double cutoff, size_t n, TreeParams *p, size_t *o_cell, size_t *o_nodes) {
     p->n = n;
     p->n_pts = (int)g.n;
     p->nu_A = g.nu_A;
@@ -566,17 +583,15 @@ static size_t tree64_layout(const xc_grid &g, double cutoff, size_t n, TreeParam
     size_t o = 0;
     auto carve = [&](size_t bytes) { size_t r = o; o += (bytes + 255) & ~size_t(255); return r; };
     carve(n * sizeof(int4));
-    *o_gs = carve(sizeof(GeomStats));
     *o_cell = carve((size_t)(p->ncell + 1) * 4);
-    *o_mat = carve((size_t)T64_MAT * 8);
     *o_nodes = carve((size_t)off * 8);
     return o;
 }
 
 size_t tree64_scratch(const xc_grid &g, double cutoff, size_t n) {
     TreeParams p;
-    size_t a, b, c, d;
-    return tree64_layout(g, cutoff, n, &p, &a, &b, &c, &d);
+    size_t a, b;
+    return tree64_layout(g, cutoff, n, &p, &a, &b);
 }
 
 template <int PROF>
@@ -594,20 +609,17 @@ static void t64_launch(const T64Params &q, int64_t *launches, cudaStream_t s) {
 }
 
 cudaError_t launch_tree64(int profile, const double *nu, const double *I, const double *al, const double *ga,
-                          const double *cut, size_t n, const CondDev *cond, const xc_grid &g, double cutoff,
-                          bool fixed_cut, const double *ghx, const double *ghw, int ngh, void *scratch, double *sigma,
-                          int64_t *launches, cudaStream_t s) {
+                          const double *cut, size_t n, double acoef, const xc_grid &g, double cutoff, bool fixed_cut,
+                          const double *ghx, const double *ghw, int ngh, const double *mat, void *scratch,
+                          double *sigma, int64_t *launches, cudaStream_t s) {
     T64Params q;
     TreeParams &p = q.t;
-    size_t o_cell, o_mat, o_nodes, o_gs;
-    tree64_layout(g, cutoff, n, &p, &o_cell, &o_mat, &o_nodes, &o_gs);
+    size_t o_cell, o_nodes;
+    tree64_layout(g, cutoff, n, &p, &o_cell, &o_nodes);
     char *b = static_cast<char *>(scratch);
     int4 *geo = reinterpret_cast<int4 *>(b);
-    GeomStats *gs = reinterpret_cast<GeomStats *>(b + o_gs);
     unsigned *cell = reinterpret_cast<unsigned *>(b + o_cell);
-    double *mat = reinterpret_cast<double *>(b + o_mat);
     p.geo = geo;
-    p.gs = gs;
     p.cell = cell;
     p.mat = mat;
     p.nodes = reinterpret_cast<double *>(b + o_nodes);
@@ -639,13 +651,12 @@ cudaError_t launch_tree64(int profile, const double *nu, const double *I, const 
     q.ga = ga;
     const double a0 = nearbyint(g.nu_A / g.step);
     q.koff = fabs(a0) < 1e15 ? (int)(((int64_t)a0 % 512 + 512) % 512) : 0;
-    cudaError_t e = launch_tree_prep(cond, 1, gs, s);
-    if (e != cudaSuccess) return e;
+    q.acoef = (float)(acoef * (1.0 + 1e-6));
     const unsigned lb = (unsigned)std::max<size_t>(1, std::min<size_t>((n + 255) / 256, 152 * 16));
     // exp(-x) and erfc(x) are exactly 0 in FP64 from x = 745.2 and x = 27.3 on: 32.8 alpha for both
     k_t64_geom<<<lb, 256, 0, s>>>(nu, al, cut, n, g.nu_A, g.step, dop ? 33.2 : 0.0, geo);
-    k_t64_setup<<<(unsigned)((p.ncell + 1 + (p.far ? T64_MAT_DV : 0) + 255) / 256), 256, 0, s>>>(p, cell, mat);
-    *launches += 3;
+    k_t64_setup<<<(unsigned)((p.ncell + 1 + 63) / 64), 64, 0, s>>>(p, cell);
+    *launches += 2;
     switch (profile) {
     case XC_DOPPLER: t64_launch<XC_DOPPLER>(q, launches, s); break;
     case XC_LORENTZ: t64_launch<XC_LORENTZ>(q, launches, s); break;

@@ -475,9 +475,8 @@ struct VjpLine {
 struct Vjp32Params {
     LinesDev L;
     size_t n;
-    const int *n_abs, *ka_abs, *kb_abs;   // per line (fixed cut)
-    const float *f_frac;
-    const CParam *cp;                     // this launch's conditions (width order), rows = caller index
+    const int4 *geo;                      // per line: n, ka, kb (fixed cut), fraction (bits)
+    const CParam *cp;                     // this launch's conditions, rows = caller index
     const CondDev *conds;                 // all conditions, caller order
     int nc;                               // conditions in this launch (<= 32)
     double nu_A, step, cutoff, width_mult;
@@ -532,7 +531,7 @@ __global__ void __launch_bounds__(128) k_vjp_nodes(const double *__restrict__ g,
 // scale on its gamma_0 values (d gamma = gamma_i) and of a shift of its n values
 // (d gamma = gamma_i ln(T_ref/T))
 template <int PROF, bool MIX>
-__global__ void __launch_bounds__(VT) k_vjp32(Vjp32Params p) {
+__global__ void __launch_bounds__(VT, MIX ? 2 : 3) k_vjp32(Vjp32Params p) {
     __shared__ double s_part[VW][VMAXC][4];
     __shared__ double s_broad[VW][VMAXC][MIX ? 2 * VMAXB : 1];
     __shared__ float s_gx[PROF == XC_VOIGT_GH_BINNED ? 64 : 1], s_gw[PROF == XC_VOIGT_GH_BINNED ? 64 : 1];
@@ -559,12 +558,15 @@ __global__ void __launch_bounds__(VT) k_vjp32(Vjp32Params p) {
     // this lane's condition: FP32 constants, and FP64 accumulators of its four scalars
     const bool mine = lane < nc;
     const CParam cc = p.cp[mine ? lane : 0];
-    const CondDev cd = p.conds[cc.row];
-    const float invT = (float)(1.0 / cd.T);
-    const float dQQ = (float)(cd.dQdT / cd.Q);
-    const float lnTr = (float)log(cd.T_ref / cd.T);
-    const float fP = (float)(cd.gamma_scale / cd.P_ref);     // d(gamma_scale P/P_ref)/dP
-    const float fS = (float)(cd.P / cd.P_ref);               // d(gamma_scale P/P_ref)/d(gamma_scale)
+    float invT, dQQ, lnTr, fP, fS;
+    {
+        const CondDev cd = p.conds[cc.row];
+        invT = (float)(1.0 / cd.T);
+        dQQ = (float)(cd.dQdT / cd.Q);
+        lnTr = (float)log(cd.T_ref / cd.T);
+        fP = (float)(cd.gamma_scale / cd.P_ref);     // d(gamma_scale P/P_ref)/dP
+        fS = (float)(cd.P / cd.P_ref);               // d(gamma_scale P/P_ref)/d(gamma_scale)
+    }
     double accT = 0.0, accP = 0.0, accS = 0.0, accN = 0.0;
     for (size_t l = (size_t)blockIdx.x * VW + warp; l < p.n; l += (size_t)gridDim.x * VW) {
         const float nu = (float)p.L.nu[l];
@@ -604,9 +606,10 @@ __global__ void __launch_bounds__(VT) k_vjp32(Vjp32Params p) {
             }
             dlnI = cc.c2T * E * invT - xs * invT / expm1f(xs) - dQQ;
         }
-        const int na = p.n_abs[l];
-        const float ff = p.f_frac[l];
-        int ka = p.ka_abs[l], kb = p.kb_abs[l];
+        const int4 geo = p.geo[l];
+        const int na = geo.x;
+        const float ff = __int_as_float(geo.w);
+        int ka = geo.y, kb = geo.z;
         float SIm = 0.f, Sam = 0.f, Sgm = 0.f;   // lane c: its condition's three sums
         for (int c = 0; c < nc; ++c) {
             const float a_h = __shfl_sync(0xffffffffu, ah, c), g_h = __shfl_sync(0xffffffffu, gh, c);
@@ -615,6 +618,7 @@ __global__ void __launch_bounds__(VT) k_vjp32(Vjp32Params p) {
                 // the forward kernels' geometry
                 int64_t k0 = 1, k1 = 0;
                 if (lane == c) {
+                    const CondDev cd = p.conds[cc.row];
                     const double nud = p.L.nu[l];
                     const double al = alpha_coef(cd.T, cd.mass_da) * nud;
                     const double ga = cd.gamma_scale * (double)gref * exp(((double)nT + cd.n_shift) *
@@ -627,109 +631,86 @@ __global__ void __launch_bounds__(VT) k_vjp32(Vjp32Params p) {
             const float *gc = p.g32 + (size_t)__shfl_sync(0xffffffffu, cc.row, c) * (size_t)p.n_pts;
             KahanF K0, K1, K2, B0, B1, B2;
             const VjpLine<PROF> ln_c(a_h, g_h, s_gx, s_gw, p.ngh);
-            // grid points k0..k1, all in w4's region I
-            auto points = [&](int k0, int k1) {
-                for (int k8 = k0 + lane; k8 <= k1; k8 += 32 * 8) {
-                    float q0 = 0.f, q1 = 0.f, q2 = 0.f;
-#pragma unroll 2
-                    for (int j = 0; j < 8; ++j) {
-                        const int k = k8 + 32 * j;
-                        if (k > k1) break;
-                        ln_c.add((float)(k - na) - ff, gc[k], q0, q1, q2);
-                    }
-                    K0.add(q0);
-                    K1.add(q1);
-                    K2.add(q2);
-                }
-            };
-            int c0 = ka, c1 = kb;   // the points around the centre
+            int k0 = ka, k1 = kb;   // the points around the centre, taken one by one
             if (PROF == XC_DOPPLER) {
                 // 2^(-u / a^2) is exactly 0 in FP32 beyond 11.3 a
                 const int r = (int)fminf(ceilf(11.3f * a_h) + 2.f, 1e9f);
-                c0 = max(c0, na - r);
-                c1 = min(c1, na + r);
+                k0 = max(k0, na - r);
+                k1 = min(k1, na + r);
             } else if (p.gnode) {
-                // the far points on both sides by the nodes of the blocks they fill: a block of
-                // level l when it lies inside the cut and beyond the level's radius (xc_tree.cu)
+                // The far points on both sides by the nodes of the blocks they fill: a block of
+                // level l when it lies inside the cut and beyond the level's radius (xc_tree.cu).
+                // Lane 5 s + q (s: side) finds segment q of that side: level 0 outside and inside
+                // of level 1, level 1 outside and inside of level 2, level 2.
                 const float *gn = p.gnode + (size_t)__shfl_sync(0xffffffffu, cc.row, c) * (size_t)p.nodes_per_cond;
                 const float am = fminf(a_h, 1e6f);
                 const int e = PROF == XC_VOIGT_W4 ? 2 + (int)ceilf(0.86f * am)
                               : PROF == XC_VOIGT_GH_BINNED ? 3 + (int)ceilf(am * s_ext)
                                                            : 1;
                 const int core = PROF == XC_VOIGT_W4 ? 2 + (int)ceilf(18.05f * am) : 0;
-                int D[TR_LEVELS];
+                int A[TR_LEVELS], Z[TR_LEVELS];
 #pragma unroll
-                for (int l = 0; l < TR_LEVELS; ++l) D[l] = max(tr_gap(l) + e, core);
-                auto nodes = [&](int lev, int j0, int j1) {
-                    const int B = tr_block(lev);
-                    float q0 = 0.f, q1 = 0.f, q2 = 0.f;
-                    for (int i = j0 * TR_M + lane; i < j1 * TR_M; i += 32) {
-                        const float dl = ((float)((i >> 4) * B - na) + s_node[lev][i & 15]) - ff;
-                        ln_c.add(dl, gn[p.node_off[lev] + i], q0, q1, q2);
-                    }
-                    K0.add(q0);
-                    K1.add(q1);
-                    K2.add(q2);
-                };
-                // points lo[l]..hi[l] may be taken by level l; returns the points taken
-                auto side = [&](int lo0, int hi0, int lo1, int hi1, int lo2, int hi2, int *t0, int *t1) {
-                    const int a0 = (lo0 + 63) >> 6, b0 = (hi0 + 1) >> 6;
-                    const int a1 = (lo1 + 127) >> 7, b1 = (hi1 + 1) >> 7;
-                    const int a2 = (lo2 + 511) >> 9, b2 = (hi2 + 1) >> 9;
-                    *t0 = *t1 = 0;
-                    if (b0 <= a0) return;
-                    *t0 = 64 * a0;
-                    *t1 = 64 * b0;
-                    if (b1 <= a1) {
-                        nodes(0, a0, b0);
-                        return;
-                    }
-                    if (a0 < 2 * a1) nodes(0, a0, 2 * a1);
-                    if (2 * b1 < b0) nodes(0, 2 * b1, b0);
-                    if (b2 <= a2) {
-                        nodes(1, a1, b1);
-                        return;
-                    }
-                    if (a1 < 4 * a2) nodes(1, a1, 4 * a2);
-                    if (4 * b2 < b1) nodes(1, 4 * b2, b1);
-                    nodes(2, a2, b2);
-                };
-                int t0, t1;
-                side(ka, min(kb, na - D[0] - 1), ka, min(kb, na - D[1] - 1), ka, min(kb, na - D[2] - 1), &t0, &t1);
-                if (t1 > t0) {
-                    points(ka, t0 - 1);
-                    c0 = t1;
+                for (int l = 0; l < TR_LEVELS; ++l) {
+                    const int D = max(tr_gap(l) + e, core), sh = l == 2 ? 9 : 6 + l;
+                    const int lo = lane >= 5 ? max(ka, na + D + 1) : ka, hi = lane >= 5 ? kb : min(kb, na - D - 1);
+                    A[l] = (lo + (1 << sh) - 1) >> sh;
+                    Z[l] = (hi + 1) >> sh;
                 }
-                side(max(ka, na + D[0] + 1), kb, max(ka, na + D[1] + 1), kb, max(ka, na + D[2] + 1), kb, &t0, &t1);
-                if (t1 > t0) {
-                    points(t1, kb);
-                    c1 = t0 - 1;
+                const bool h0 = Z[0] > A[0], h1 = h0 && Z[1] > A[1], h2 = h1 && Z[2] > A[2];
+                const int q = lane >= 5 ? lane - 5 : lane;
+                int lev = q < 2 ? 0 : (q < 4 ? 1 : 2), j0 = 0, j1 = 0;
+                if (q == 0 && h0) { j0 = A[0]; j1 = h1 ? 2 * A[1] : Z[0]; }
+                if (q == 1 && h1) { j0 = 2 * Z[1]; j1 = Z[0]; }
+                if (q == 2 && h1) { j0 = A[1]; j1 = h2 ? 4 * A[2] : Z[1]; }
+                if (q == 3 && h2) { j0 = 4 * Z[2]; j1 = Z[1]; }
+                if (q == 4 && h2) { j0 = A[2]; j1 = Z[2]; }
+                float q0 = 0.f, q1 = 0.f, q2 = 0.f;
+                for (unsigned segs = __ballot_sync(0xffffffffu, lane < 10 && j1 > j0); segs; segs &= segs - 1) {
+                    const int src = __ffs(segs) - 1;
+                    const int lv = __shfl_sync(0xffffffffu, lev, src), sh = lv == 2 ? 9 : 6 + lv;
+                    const int i1 = TR_M * __shfl_sync(0xffffffffu, j1, src);
+                    const float *gl = gn + p.node_off[lv];
+                    for (int i = TR_M * __shfl_sync(0xffffffffu, j0, src) + lane; i < i1; i += 32)
+                        ln_c.add(((float)(((i >> 4) << sh) - na) + s_node[lv][i & 15]) - ff, gl[i], q0, q1, q2);
                 }
+                K0.add(q0);
+                K1.add(q1);
+                K2.add(q2);
+                // what is left between the cut's ends and the blocks
+                const bool hl = __shfl_sync(0xffffffffu, (int)h0, 0), hr = __shfl_sync(0xffffffffu, (int)h0, 5);
+                const int l0 = 64 * __shfl_sync(0xffffffffu, A[0], 0), l1 = 64 * __shfl_sync(0xffffffffu, Z[0], 0);
+                const int r0 = 64 * __shfl_sync(0xffffffffu, A[0], 5), r1 = 64 * __shfl_sync(0xffffffffu, Z[0], 5);
+                const int nl = hl ? l0 - ka : 0, nr = hr ? kb - r1 + 1 : 0;
+                q0 = q1 = q2 = 0.f;
+                for (int i = lane; i < nl + nr; i += 32) {
+                    const int k = i < nl ? ka + i : r1 + i - nl;
+                    ln_c.add((float)(k - na) - ff, gc[k], q0, q1, q2);
+                }
+                K0.add(q0);
+                K1.add(q1);
+                K2.add(q2);
+                if (hl) k0 = l1;
+                if (hr) k1 = r0 - 1;
             }
-            if (PROF != XC_VOIGT_W4) {
-                points(c0, c1);
-            } else {
-                for (int k8 = c0 + lane; k8 <= c1; k8 += 32 * 8) {
-                    float q0 = 0.f, q1 = 0.f, q2 = 0.f;
-#pragma unroll 2
-                    for (int j = 0; j < 8; ++j) {
-                        const int k = k8 + 32 * j;
-                        if (k > c1) break;
-                        const float d = (float)(k - na) - ff;
-                        if (d * d >= ln_c.thr2) {
-                            ln_c.add(d, gc[k], q0, q1, q2);
-                        } else {
-                            const float gk = gc[k];
-                            const float3 r = w4_band_f32(ln_c.asc * fabsf(d), ln_c.y);
-                            B0.add(gk * r.x);
-                            B1.add(gk * r.z);   // Re(F + t F')
-                            B2.add(gk * r.y);   // Re F'
-                        }
+            for (int k8 = k0 + lane; k8 <= k1; k8 += 32 * 8) {
+                float q0 = 0.f, q1 = 0.f, q2 = 0.f;
+#pragma unroll 1
+                for (int j = 0; j < 8; ++j) {
+                    const int k = k8 + 32 * j;
+                    if (k > k1) break;
+                    const float d = (float)(k - na) - ff, gk = gc[k];
+                    if (PROF != XC_VOIGT_W4 || d * d >= ln_c.thr2) {
+                        ln_c.add(d, gk, q0, q1, q2);
+                    } else {
+                        const float3 r = w4_band_f32(ln_c.asc * fabsf(d), ln_c.y);
+                        B0.add(gk * r.x);
+                        B1.add(gk * r.z);   // Re(F + t F')
+                        B2.add(gk * r.y);   // Re F'
                     }
-                    K0.add(q0);
-                    K1.add(q1);
-                    K2.add(q2);
                 }
+                K0.add(q0);
+                K1.add(q1);
+                K2.add(q2);
             }
             // the lanes' sums to the three derivative sums, each reduced over the warp
             F2 vI, va, vg;
@@ -881,7 +862,7 @@ xc_status vjp_run(BatchedState *st, const VjpArgs &a, int64_t *launches) {
     const bool far = !f64 && a.opts.profile != XC_DOPPLER && a.grid.n < ((int64_t)1 << 30);
     const int nblk512 = far ? (int)((a.grid.n + 511) / 512) : 0;
     const size_t per_cond = (size_t)nblk512 * (128 + 64 + 16);
-    size_t o_gn = far ? carve((size_t)nc * per_cond * 4) : 0, o_mat = far ? carve(TR_MAT * 8) : 0;
+    size_t o_gn = far ? carve((size_t)nc * per_cond * 4) : 0;
     VJ_TRY(st->vjp_buf.ensure(off + 256));
     char *base = st->vjp_buf.as<char>();
     const double *g64 = a.grad_sigma;
@@ -934,9 +915,8 @@ xc_status vjp_run(BatchedState *st, const VjpArgs &a, int64_t *launches) {
         VJ_TRY(cudaGetLastError());
     } else {
         // FP32: the forward FP32 kernels' line geometry and condition constants, then the
-        // adjoint per chunk of <= 32 conditions (in order of profile width)
-        int *n_abs = (int *)(base + o_geo), *ka = n_abs + n, *kb = ka + n;
-        float *ffr = (float *)(kb + n);
+        // adjoint per chunk of <= 32 conditions
+        int4 *geo = (int4 *)(base + o_geo);
         GeomStats *gs = (GeomStats *)(base + o_gs);
         CParam *cp = (CParam *)(base + o_cp);
         if (N) {
@@ -944,22 +924,19 @@ xc_status vjp_run(BatchedState *st, const VjpArgs &a, int64_t *launches) {
             ++*launches;
         }
         if (far && N) {
-            double *mat = (double *)(base + o_mat);
-            VJ_TRY(launch_tree_mat(mat, s));
+            const double *mat = nullptr;
+            VJ_TRY(tree_mat(st, &mat, s));
             k_vjp_nodes<<<dim3(nblk512, nc), 128, 0, s>>>(g64, a.grid.n, mat, (float *)(base + o_gn), 0, nblk512 * 128,
                                                           nblk512 * 192, (int)per_cond);
-            *launches += 2;
+            ++*launches;
         }
-        VJ_TRY(launch_fp32_setup(a.L, n, a.conds_dev, nc, a.grid, a.opts.cutoff, n_abs, ffr, ka, kb, gs, cp, s));
+        VJ_TRY(launch_fp32_setup(a.L, n, a.conds_dev, nc, a.grid, a.opts.cutoff, geo, gs, cp, s));
         *launches += 2;
         for (int c0 = 0; c0 < nc; c0 += VMAXC) {
             Vjp32Params vp;
             vp.L = a.L;
             vp.n = n;
-            vp.n_abs = n_abs;
-            vp.ka_abs = ka;
-            vp.kb_abs = kb;
-            vp.f_frac = ffr;
+            vp.geo = geo;
             vp.cp = cp + c0;
             vp.conds = a.conds_dev;
             vp.nc = std::min(VMAXC, nc - c0);
