@@ -399,6 +399,9 @@ __global__ void __launch_bounds__(TR_T) k_tree_nodes(TreeParams p) {
                             }
                         }
                     } else {
+                        // binned Gauss-Hermite: the short arctangent when all the chunk's lines allow it
+                        const bool far = PROF == XC_VOIGT_GH_BINNED &&
+                                         __all_sync(0xffffffffu, !ok || gh_far(A.y, (float)D, A.x * p.gh_ext));
                         for (int j = strm; j < cnt; j += NS) {
                             const float2 *q = reinterpret_cast<const float2 *>(buf) + j * 3;
                             const float2 nf = q[0], a01 = q[1], a23 = q[2];
@@ -406,8 +409,9 @@ __global__ void __launch_bounds__(TR_T) k_tree_nodes(TreeParams p) {
 #pragma unroll
                             for (int r = 0; r < R; ++r) {
                                 const float d = (x[r] - nf.x) - nf.y;
-                                acc[r] += contrib_single<PROF>(d * d, d, Ac, make_float4(0.f, 0.f, 0.f, -1.f), sX, sW,
-                                                               p.ngh);
+                                acc[r] += far ? gh_far_value(d, Ac, sX, sW, p.ngh)
+                                              : contrib_single<PROF>(d * d, d, Ac, make_float4(0.f, 0.f, 0.f, -1.f), sX, sW,
+                                                                     p.ngh);
                             }
                         }
                     }
@@ -576,7 +580,9 @@ __global__ void __launch_bounds__(TR_T) k_tree_points(TreeParams p) {
                     } else {
                         if (ok) {
                             float4 *q = buf + __popc(m & below) * 2;
-                            q[0] = make_float4(n, f, __int_as_float(ka), __int_as_float(kb));
+                            const bool far = PROF == XC_VOIGT_GH_BINNED &&
+                                             gh_far(A.y, (float)max(s0 - g.x, g.x - s1), A.x * p.gh_ext);
+                            q[0] = make_float4(n, f, __int_as_float(ka), __int_as_float(far ? kb + 64 : kb));
                             q[1] = A;
                         }
                         __syncwarp();
@@ -585,8 +591,13 @@ __global__ void __launch_bounds__(TR_T) k_tree_points(TreeParams p) {
                             if ((j & 15) == 15) tr_fold(hi, lo, acc);
                             const float4 t = buf[2 * j], a = buf[2 * j + 1];
                             const float d = (x - t.x) - t.y;
-                            if (lane >= __float_as_int(t.z) && lane <= __float_as_int(t.w))
+                            const int ka1 = __float_as_int(t.z), kb1 = __float_as_int(t.w);
+                            if (PROF == XC_VOIGT_GH_BINNED && kb1 >= 64) {
+                                const float v = gh_far_value(d, a, sX, sW, p.ngh);
+                                acc += lane >= ka1 && lane <= kb1 - 64 ? v : 0.f;
+                            } else if (lane >= ka1 && lane <= kb1) {
                                 acc += contrib_single<PROF>(d * d, d, a, make_float4(0.f, 0.f, 0.f, -1.f), sX, sW, p.ngh);
+                            }
                         }
                     }
                     __syncwarp();
