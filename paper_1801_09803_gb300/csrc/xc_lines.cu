@@ -308,7 +308,7 @@ cudaError_t launch_line_params64(const LinesDev &L, size_t n, const CondDev *con
                                  double *cut, cudaStream_t s, const StrengthSel &sel) {
     if (n == 0) return cudaSuccess;
     size_t blocks = (n + 255) / 256;
-    if (blocks > 152 * 32) blocks = 152 * 32;
+    if (blocks > 152 * 8) blocks = 152 * 8;
     k_line_params64<<<(unsigned)blocks, 256, 0, s>>>(L, n, cond_dev, cut_mode, cutoff, width_mult, I, alpha,
                                                      gamma, cut, sel);
     return cudaGetLastError();

@@ -160,10 +160,13 @@ __device__ __forceinline__ double t64_rcp(double d) {
 // ---------------------------------------------------------------------------
 constexpr int T64_RING = 36;   // accepted lines held: up to 3 left over and 32 new ones
 
+// Two warps per CTA and the large blocks first: an SM's FP64 pipe is the limit, so the blocks
+// (a 512-point one has five times the lines of a 128-point one) are spread in small pieces.
+constexpr int T64_NW = 2;
 template <int PROF>
-__global__ void __launch_bounds__(TR_T) k_t64_nodes(T64Params q) {
+__global__ void __launch_bounds__(32 * T64_NW) k_t64_nodes(T64Params q) {
     constexpr bool W4 = PROF == XC_VOIGT_W4;
-    __shared__ double sL[TR_W][T64_RING * (W4 ? 5 : 4)];
+    __shared__ double sL[T64_NW][T64_RING * (W4 ? 5 : 4)];
     __shared__ double sX[64], sW[64];
     const TreeParams &p = q.t;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -174,8 +177,7 @@ __global__ void __launch_bounds__(TR_T) k_t64_nodes(T64Params q) {
         }
         __syncthreads();
     }
-    // the large blocks have the most lines: dealt out over the CTAs (an SM's FP64 pipe is the limit)
-    int task = blockIdx.x + warp * gridDim.x;
+    int task = blockIdx.x * T64_NW + warp;
     const int lev = task < p.nblk[1] ? 1 : 0;
     if (lev == 0) task -= p.nblk[1];
     if (task >= p.nblk[lev]) return;
@@ -400,16 +402,18 @@ __device__ __forceinline__ double t64_region4(double x, double y) {
 }
 
 struct W4Buf64 {
-    double L[32 * 9];       // lines with points in regions I, II: nu, E, F, P, PC, a, y, y amp, zone?
-    unsigned m12[32];
+    double F[T64_RING * 5]; // lines in region I at all the warp's points, inside the cut: nu, E, F, P, PC
+    double Z[32 * 8];       // lines whose zone |x| + y < 15 or an end of whose cut lies there: ..., a, y, amplitude
+    unsigned m12[32];       // ... their points in regions I and II
     double I[2][32 * 4];    // lines with items of region III / IV: nu, a, y, amplitude
     int4 R[2][32];          // first item, first point, points of the left run, first point of the right run
     int cnt[2][32];
 };
 
-// w4: lines with points in regions I and II one after the other (region II only where the line's
-// zone reaches the points), items of III and IV as in k_tree_points_w4.  One sum for each of
-// the three, in line order.
+// w4.  Lines that cover the warp's points in region I go four to a reciprocal (8.5 FP64 operations
+// a value, against 11 one by one), lines with a zone or an end of their cut there one by one, items of regions III and IV
+// as in xc_tree.cu.  One sum for each, in line order; groups of four are counted from the
+// warp's first line.  Only lines near the points are classified in FP64.
 __global__ void __launch_bounds__(128) k_t64_points_w4(T64Params q) {
     __shared__ W4Buf64 sBuf[4];
     const TreeParams &p = q.t;
@@ -419,12 +423,21 @@ __global__ void __launch_bounds__(128) k_t64_points_w4(T64Params q) {
     if (s0 >= p.n_pts || s1 < 0) return;
     const int p0 = (task >> 2) * 128 - q.koff, p1 = p0 + 127;
     const int Dp = tr_radius(p, q.acoef, t64_gap(0), p1);
+    const int core = tr_radius(p, q.acoef, -(1 << 28), p1) + 1;   // the zones' radius alone
     const Segs sg = tr_point_segs(p, s0, s1, p0, p1, Dp);
     const double xk = grid_x(p.nu_A, p.step, s0 + lane), x0 = grid_x(p.nu_A, p.step, s0);
     const double inv_h = 1.0 / p.step;
     const unsigned below = (1u << lane) - 1u;
     W4Buf64 &buf = sBuf[warp];
-    double acc = 0.0, acc34[2] = {0.0, 0.0};
+    double accF = 0.0, accZ = 0.0, acc34[2] = {0.0, 0.0};
+    int held = 0;
+    // the numerator and denominator of region I of list line j at this lane's point
+    auto one = [&](int j, double &N, double &Dn) {
+        const double *w = buf.F + 5 * j;
+        const double d = __dsub_rn(xk, w[0]), u = d * d;
+        Dn = fma(u, u + w[1], w[2]);
+        N = fma(w[3], u, w[4]);
+    };
 #pragma unroll 1
     for (int k = 0; k < 3; ++k) {
         const unsigned e = sg.e[k];
@@ -437,32 +450,46 @@ __global__ void __launch_bounds__(128) k_t64_points_w4(T64Params q) {
             if (!__any_sync(0xffffffffu, ok)) continue;
             W4Line w{};
             bool zone = false;
-            unsigned m12 = 0u, m3 = 0u, m34 = 0u;
+            unsigned cut = 0u, m3 = 0u, m34 = 0u;
             int k0 = 0, k1 = -1, k30 = 0, k31 = -1;
             if (ok) {
                 w = t64_line(q, l);
                 const int ka = max(g.y - s0, 0), kb = min(g.z - s0, 31);
-                m12 = lanes_of(ka, kb);
-                const double pos = (w.nu - x0) * inv_h, ra = q.al[l] * (1.0 / kSqrtLn2) * inv_h;   // 1/a in grid steps
-                const double rz = (15.0 - w.y) * ra + 1e-3;
-                zone = w.y < 15.0 && pos + rz >= 0.0 && pos - rz <= 31.0;
-                if (zone && w.y < 5.5) {
-                    const double r34 = (5.5 - w.y) * ra, r3 = fmin(r34, (w.y + 0.176) * (1.0 / 0.195) * ra);
-                    k0 = max((int)ceil(fmax(pos - r34, -1.0)), ka);
-                    k1 = min((int)floor(fmin(pos + r34, 32.0)), kb);
-                    k30 = max((int)ceil(fmax(pos - r3, -1.0)), k0);
-                    k31 = min((int)floor(fmin(pos + r3, 32.0)), k1);
-                    m34 = lanes_of(k0, k1);
-                    m3 = lanes_of(k30, k31);
-                    m12 &= ~m34;
+                cut = lanes_of(ka, kb);
+                if (g.x >= s0 - core && g.x <= s1 + core && w.y < 15.0) {
+                    const double pos = (w.nu - x0) * inv_h, ra = q.al[l] * (1.0 / kSqrtLn2) * inv_h;   // 1/a in grid steps
+                    const double rz = (15.0 - w.y) * ra + 1e-3;
+                    zone = pos + rz >= 0.0 && pos - rz <= 31.0;
+                    if (zone && w.y < 5.5) {
+                        const double r34 = (5.5 - w.y) * ra, r3 = fmin(r34, (w.y + 0.176) * (1.0 / 0.195) * ra);
+                        k0 = max((int)ceil(fmax(pos - r34, -1.0)), ka);
+                        k1 = min((int)floor(fmin(pos + r34, 32.0)), kb);
+                        k30 = max((int)ceil(fmax(pos - r3, -1.0)), k0);
+                        k31 = min((int)floor(fmin(pos + r3, 32.0)), k1);
+                        m34 = lanes_of(k0, k1);
+                        m3 = lanes_of(k30, k31);
+                    }
                 }
             }
-            const unsigned m4 = m34 & ~m3;
-            const unsigned bL = __ballot_sync(0xffffffffu, m12 != 0u);
+            const unsigned m4 = m34 & ~m3, m12 = cut & ~m34;
+            // groups of four only of lines that cover all 32 points: a grid shard, which holds the lines
+            // that reach its own points, then forms the same groups
+            const bool isF = ok && !zone && cut == 0xffffffffu, isZ = ok && !isF && m12 != 0u;
+            const unsigned bF = __ballot_sync(0xffffffffu, isF), bZ = __ballot_sync(0xffffffffu, isZ);
             const unsigned b34[2] = {__ballot_sync(0xffffffffu, m3 != 0u), __ballot_sync(0xffffffffu, m4 != 0u)};
-            if (m12) {
-                const int slot = __popc(bL & below);
-                double *b = buf.L + 9 * slot;
+            if (isF) {
+                const int slot = held + __popc(bF & below);
+                double *b = buf.F + 5 * slot;
+                b[0] = w.nu;
+                b[1] = w.E;
+                b[2] = w.F;
+                b[3] = w.P;
+                b[4] = w.PC;
+            }
+            held += __popc(bF);
+            if (isZ) {
+                const int slot = __popc(bZ & below);
+                double *b = buf.Z + 8 * slot;
                 b[0] = w.nu;
                 b[1] = w.E;
                 b[2] = w.F;
@@ -471,7 +498,6 @@ __global__ void __launch_bounds__(128) k_t64_points_w4(T64Params q) {
                 b[5] = w.ia;
                 b[6] = w.y;
                 b[7] = w.amp;
-                b[8] = zone ? 1.0 : 0.0;
                 buf.m12[slot] = m12;
             }
             int tot[2];
@@ -501,23 +527,37 @@ __global__ void __launch_bounds__(128) k_t64_points_w4(T64Params q) {
                 }
             }
             __syncwarp();
-            const int nL = __popc(bL);
-            for (int j = 0; j < nL; ++j) {
-                const double *b = buf.L + 9 * j;
+            int j4 = 0;
+            for (; j4 + 4 <= held; j4 += 4) {
+                double N[4], Dn[4];
+#pragma unroll
+                for (int j = 0; j < 4; ++j) one(j4 + j, N[j], Dn[j]);
+                const double D01 = Dn[0] * Dn[1], D23 = Dn[2] * Dn[3];
+                const double N01 = fma(N[0], Dn[1], N[1] * Dn[0]), N23 = fma(N[2], Dn[3], N[3] * Dn[2]);
+                accF = fma(fma(N01, D23, N23 * D01), t64_rcp(D01 * D23), accF);
+            }
+            if (j4) {   // the lines left over move to the front
+                const int rest = held - j4;
+                double keep = 0.0;
+                if (lane < 5 * rest) keep = buf.F[5 * j4 + lane];
+                __syncwarp();
+                if (lane < 5 * rest) buf.F[lane] = keep;
+                held = rest;
+            }
+            const int nZ = __popc(bZ);
+            for (int j = 0; j < nZ; ++j) {
+                const double *b = buf.Z + 8 * j;
                 const bool in = (buf.m12[j] >> lane) & 1u;
                 const double d = __dsub_rn(xk, b[0]), u = d * d;
-                bool one = true;
+                const double x = fabs(d) * b[5], y = b[6];
+                const bool first = x + y >= 15.0;
                 double v = 0.0;
-                if (b[8] != 0.0) {
-                    const double x = fabs(d) * b[5], y = b[6];
-                    one = x + y >= 15.0;
-                    if (__any_sync(0xffffffffu, in && !one)) v = b[7] * t64_region2(x * x, y, y * y);
-                }
-                if (__any_sync(0xffffffffu, in && one)) {
+                if (__any_sync(0xffffffffu, in && !first)) v = b[7] * t64_region2(x * x, y, y * y);
+                if (__any_sync(0xffffffffu, in && first)) {
                     const double v1 = fma(b[3], u, b[4]) * t64_rcp(fma(u, u + b[1], b[2]));
-                    v = one ? v1 : v;
+                    v = first ? v1 : v;
                 }
-                if (in) acc += v;
+                if (in) accZ += v;
             }
 #pragma unroll
             for (int t = 0; t < 2; ++t) {
@@ -551,7 +591,12 @@ __global__ void __launch_bounds__(128) k_t64_points_w4(T64Params q) {
             __syncwarp();
         }
     }
-    t64_finish(q, task >> 2, (task & 3) * 32 + lane, s0 + lane, lane, acc + (acc34[0] + acc34[1]));
+    for (int j = 0; j < held; ++j) {
+        double N, Dn;
+        one(j, N, Dn);
+        accF = fma(N, t64_rcp(Dn), accF);
+    }
+    t64_finish(q, task >> 2, (task & 3) * 32 + lane, s0 + lane, lane, (accF + accZ) + (acc34[0] + acc34[1]));
 }
 
 // ---------------------------------------------------------------------------
@@ -597,7 +642,7 @@ size_t tree64_scratch(const xc_grid &g, double cutoff, size_t n) {
 template <int PROF>
 static void t64_launch(const T64Params &q, int64_t *launches, cudaStream_t s) {
     if (q.t.far) {
-        k_t64_nodes<PROF><<<(q.t.nblk[0] + q.t.nblk[1] + TR_W - 1) / TR_W, TR_T, 0, s>>>(q);
+        k_t64_nodes<PROF><<<(q.t.nblk[0] + q.t.nblk[1] + T64_NW - 1) / T64_NW, 32 * T64_NW, 0, s>>>(q);
         *launches += 1;
     }
     const int64_t tasks = ((int64_t)q.t.n_pts + q.koff + 31) / 32;
