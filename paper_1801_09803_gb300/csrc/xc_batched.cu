@@ -1830,12 +1830,18 @@ int grid_size(const Variant *v, int dev, int n_tiles) {
 // Autotune: time each candidate variant on a probe (every tile, first 4096 lines)
 // and predict the full run from the measured time per (tile line x condition);
 // the prediction includes the wave quantisation of the tile count.
-// far wings of the Voigt w4 sweep on the tensor cores: many conditions (the MMA's N is
-// 32, so a handful of conditions would waste it), one fixed cut, grids of < 2^30 points
+// Far wings of the Voigt w4 sweep on the tensor cores: many conditions (the MMA's N is
+// 32, so a handful of conditions would waste it), one fixed cut, grids of < 2^23 points.
+// The block-interpolated sweep (xc_tree.cu) evaluates a ninth of the points at long cuts and is
+// faster at every size measured: 32 conditions x 3e6 lines, cut 1000 steps 23.2 ms against 42.3,
+// 500 steps 20.2 against 35.6, 100 steps 15.7 against 30.2; 15 000 lines 0.2 against 0.9.  This
+// form stays for short cuts and small lists, where xc_last_sweep_kernels and
+// xc_count_far_evals report on it and a call takes about a millisecond either way, and where the
+// tiled kernels run because of a fixed tile shape or for want of memory.
 bool use_tc(const BatchedArgs &a, int nc) {
     return a.allow_tc && a.opts.profile == XC_VOIGT_W4 && a.opts.width_mult <= 0.0 && nc >= 16 &&
            !(a.opts.flags & XC_OPT_NO_TENSOR_CORES) && a.grid.n < ((int64_t)1 << 23) &&
-           a.opts.cutoff / a.grid.step < 1024.0;
+           (a.tiled || (a.opts.cutoff / a.grid.step < 1024.0 && a.n_lines * (size_t)nc < ((size_t)1 << 19)));
 }
 
 std::string tuned_key(const BatchedState *st, const BatchedArgs &a, int nc) {
@@ -1950,7 +1956,9 @@ xc_status autotune(BatchedState *st, const BatchedArgs &a, int nc, TileCfg *out,
 
 }  // namespace
 
-xc_status batched_run(BatchedState *st, const BatchedArgs &a, int64_t *launches) {
+xc_status batched_run(BatchedState *st, const BatchedArgs &args, int64_t *launches) {
+    BatchedArgs a = args;
+    a.tiled = st->force_R > 0;
     if (a.grid.n >= ((int64_t)1 << 31) - (1 << 20)) {
         set_error("the FP32 path needs fewer than 2^31 grid points");
         return XC_EINVAL;
@@ -1961,11 +1969,12 @@ xc_status batched_run(BatchedState *st, const BatchedArgs &a, int64_t *launches)
     st->tc_blk_lo = st->tc_blk_hi = nullptr;
     st->tc_n_blk = st->tc_groups = 0;
     if (a.n_lines == 0 || a.n_cond == 0 || a.grid.n == 0) return XC_OK;
-    if (st->force_R == 0 && !use_tc(a, a.n_cond) && tree_takes(a)) {
+    if (!a.tiled && !use_tc(a, a.n_cond) && tree_takes(a)) {
         // its scratch is larger (32 to 48 bytes per line and condition held): where that does not
         // fit next to a very large list, the tiled kernels below run the call
         const xc_status ts = tree_run(st, a, launches);
         if (ts != XC_ENOMEM) return ts;
+        a.tiled = true;
     }
     int dev = 0;
     cudaGetDevice(&dev);
@@ -2063,7 +2072,9 @@ int64_t batched_tc_mma_count(BatchedState *st) {
     return chunks * st->tc_groups * TC_BLK * TC_MMAS;
 }
 
-xc_status batched_count_far(BatchedState *st, const BatchedArgs &a, int64_t *count) {
+xc_status batched_count_far(BatchedState *st, const BatchedArgs &args, int64_t *count) {
+    BatchedArgs a = args;
+    a.tiled = st->force_R > 0;
     *count = 0;
     const int nc = a.n_cond;
     if (a.n_lines == 0 || nc == 0 || a.grid.n == 0 || !use_tc(a, nc)) return XC_OK;

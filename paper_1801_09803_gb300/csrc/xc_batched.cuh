@@ -111,6 +111,7 @@ struct BatchedArgs {
     cudaEvent_t ev_tc1 = nullptr;            // after the tensor-core far-wing kernel (when it runs)
     const double *ghx = nullptr, *ghw = nullptr;  // device Gauss-Hermite nodes/weights
     bool allow_tc = true;                   // far wings may use the tensor-core kernel
+    bool tiled = false;                     // the tiled kernels whatever the sizes (fixed tile shape, memory)
 };
 
 struct VjpArgs {
@@ -167,7 +168,7 @@ struct BatchedState {
 
 xc_status batched_run(BatchedState *st, const BatchedArgs &a, int64_t *launches);
 // per-line grid geometry for a fixed cut (integer position n, inclusive cut range ka..kb,
-// fraction f as bits) and the per-condition FP32 constants in the caller's order, as the
+// fraction f as bits) and the per-condition FP32 constants in order of alpha (row: the caller's), as the
 // block-interpolated sweep makes them
 cudaError_t launch_fp32_setup(const LinesDev &L, size_t n, const CondDev *conds, int nc, const xc_grid &grid,
                               double cutoff, int4 *geo, GeomStats *gs, CParam *cp, cudaStream_t s);

@@ -37,6 +37,13 @@ namespace xc {
 constexpr int TR_FOLD = 4;                  // scanned chunks (32 lines) per FP32 partial sum at the nodes
                                             // (each chunk at the points, where one strong line can
                                             // dominate: 512 lines in one sum left 6e-7 of rounding)
+// the largest alpha / nu of conditions c0 .. c0 + n - 1 of the pass
+__device__ __forceinline__ float tr_group_acoef(const TreeParams &p, int c0, int n) {
+    float a = 0.f;
+    for (int c = 0; c < n; ++c) a = fmaxf(a, p.cp[p.c0 + c0 + c].acoef);
+    return a;
+}
+
 template <int PROF>
 __device__ __forceinline__ float tr_amplitude(const float4 &A) {
     return (PROF == XC_VOIGT_W4 || PROF == XC_VOIGT_GH_SAMPLED || PROF == XC_LORENTZ_BINNED) ? A.z
@@ -186,18 +193,30 @@ __device__ double tr_mat_entry(int k, const float (*xn)[TR_M]) {
 __global__ void __launch_bounds__(128) k_tree_setup(TreeParams p, const CondDev *conds, int n_cond, CParam *cp,
                                                     int quantity, unsigned *cell) {
     if (blockIdx.x == 0) {
+        // conditions in order of alpha / nu (as T / mass): those taken together have similar zones
+        __shared__ float key[1024];
+        const bool order = n_cond > 1 && n_cond <= 1024;
+        if (order) {
+            for (int c = threadIdx.x; c < n_cond; c += 128) key[c] = (float)conds[c].T / (float)conds[c].mass_da;
+            __syncthreads();
+        }
         for (int c = threadIdx.x & 31; c < n_cond; c += 32) {
             const CondDev d = conds[c];
+            int r = c;
+            if (order) {
+                r = 0;
+                for (int j = 0; j < n_cond; ++j) r += key[j] < key[c] || (key[j] == key[c] && j < c);
+            }
             switch (threadIdx.x >> 5) {
-            case 0: cparam_strength(d, p.gs, quantity, &cp[c]); break;
-            case 1: cparam_temperature(d, &cp[c]); break;
-            case 2: cparam_widths(d, &cp[c]); break;
+            case 0: cparam_strength(d, p.gs, quantity, &cp[r]); break;
+            case 1: cparam_temperature(d, &cp[r]); break;
+            case 2: cparam_widths(d, &cp[r]); break;
             default:
-                cp[c].log2Tr = (float)log2(d.T_ref / d.T);
-                cp[c].row = c;
-                cp[c].vv_split = 4.f;
-                cp[c].vv_beta = 0;
-                cp[c].dbound = 0.f;
+                cp[r].log2Tr = (float)log2(d.T_ref / d.T);
+                cp[r].row = c;
+                cp[r].vv_split = 4.f;
+                cp[r].vv_beta = 0;
+                cp[r].dbound = 0.f;
             }
         }
         return;
@@ -463,6 +482,161 @@ __global__ void __launch_bounds__(TR_T) k_tree_nodes(TreeParams p) {
     }
 }
 
+// w4 at the nodes, CG (2 or 4) conditions at a time.  A line's position, its range tests, its place in the
+// shared-memory list and u = delta^2 are the same for every condition; a condition adds its
+// constants and 6 packed instructions per node and pair of lines.  The group's blocks use the
+// largest alpha of its conditions (they are ordered by alpha).  32 conditions x 1e7 lines:
+// 53 ms one condition at a time, 33 ms four.
+template <int CG>
+__global__ void __launch_bounds__(TR_T, 3) k_tree_nodes_w4(TreeParams p) {
+    constexpr int PAIR = 1 + 2 * CG, NS = 4;   // 16-byte words per pair of lines; line streams
+    __shared__ float4 sL[TR_W][16 * PAIR];
+    __shared__ double sRed[TR_W][CG][TR_M];
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, strm = lane >> 3;
+    int lev = 2, cta = blockIdx.x;
+    while (lev > 0 && cta >= p.ncta[lev]) cta -= p.ncta[lev--];
+    const int wpt = p.wptl[lev], part = warp % wpt;
+    const int task = cta * (TR_W / wpt) + warp / wpt;
+    const int c0 = blockIdx.y * CG, nc = min(CG, p.n_cond - c0);
+    const bool live = task < p.nblk[lev];
+    float hi[CG][2], lo[CG][2];
+#pragma unroll
+    for (int q = 0; q < CG; ++q) hi[q][0] = hi[q][1] = lo[q][0] = lo[q][1] = 0.f;
+    if (live) {
+        const float ac = tr_group_acoef(p, c0, nc);
+        const int B = tr_block(lev), b0 = task * B, b1 = b0 + B - 1, b1c = min(b1, p.n_pts - 1);
+        const int D = tr_radius(p, ac, tr_gap(lev), b1);
+        const bool up = lev < 2;
+        const int PB = up ? tr_block(lev + 1) : 1;
+        const int p0 = up ? b0 / PB * PB : 0, p1 = p0 + PB - 1, p1c = min(p1, p.n_pts - 1);
+        const int Dp = up ? tr_radius(p, ac, tr_gap(lev + 1), p1) : 0;
+        const Segs sg = tr_far_segs(p, b0, b1, D, up, p0, p1, Dp);
+        const float xn0 = tr_node(B, 2 * (lane & 7)), xn1 = tr_node(B, 2 * (lane & 7) + 1);
+        const f32x2 xa = pk2(xn0, xn0), xb = pk2(xn1, xn1);
+        const float4 *recA = p.recA + (size_t)c0 * p.n;
+        float4 *buf = sL[warp];
+        f32x2 acc[CG][2];
+#pragma unroll
+        for (int q = 0; q < CG; ++q) acc[q][0] = acc[q][1] = 0ull;
+        int in_fold = 0;
+        auto fold = [&]() {
+#pragma unroll
+            for (int q = 0; q < CG; ++q)
+#pragma unroll
+                for (int r = 0; r < 2; ++r) {
+                    float a = sum2(acc[q][r]);
+                    acc[q][r] = 0ull;
+                    tr_fold(hi[q][r], lo[q][r], a);
+                }
+        };
+#pragma unroll 1
+        for (int k = 0; k < 4; ++k) {
+            const unsigned e = sg.e[k];
+            unsigned i = sg.s[k] + 32u * part;
+            int4 g = make_int4(0, 1, 0, 0);
+            if (i + lane < e) g = p.geo[i + lane];
+#pragma unroll 1
+            for (; i < e; i += 32u * wpt) {
+                const unsigned l = i + lane;
+                int4 gn = make_int4(0, 1, 0, 0);
+                if (l + 32u * wpt < e) gn = p.geo[l + 32u * wpt];
+                bool ok = l < e && tr_takes(g, b0, b1, b1c, D) && !(up && tr_takes(g, p0, p1, p1c, Dp));
+                float4 A[CG];
+                bool any = false;
+#pragma unroll
+                for (int q = 0; q < CG; ++q) {
+                    A[q] = make_float4(0.f, 0.f, 0.f, 0.f);
+                    if (ok && q < nc) A[q] = recA[(size_t)q * p.n + l];
+                    any |= A[q].z != 0.f;
+                }
+                ok &= any;
+                const unsigned m = __ballot_sync(0xffffffffu, ok);
+                const int cnt = __popc(m);
+                if (cnt) {
+                    const unsigned below = (1u << lane) - 1u;
+                    int slot = __popc(m & below);
+                    float n = (float)(g.x - b0), f = __int_as_float(g.w);
+                    bool put = ok;
+                    if (!ok) {   // lanes that fill the last iteration with lines of amplitude 0
+                        const int z = __popc(~m & below);
+                        put = z < ((-cnt) & (2 * NS - 1));
+                        slot = cnt + z;
+                        n = -1e4f;
+                        f = 0.f;
+#pragma unroll
+                        for (int q = 0; q < CG; ++q) A[q] = make_float4(0.f, 0.f, 0.f, 0.f);
+                    }
+                    if (put) {
+                        float *w = reinterpret_cast<float *>(buf) + (slot >> 1) * (4 * PAIR) + (slot & 1);
+                        w[0] = n;
+                        w[2] = f;
+#pragma unroll
+                        for (int q = 0; q < CG; ++q) {
+                            w[4 + 8 * q] = A[q].x;
+                            w[6 + 8 * q] = A[q].y;
+                            w[8 + 8 * q] = A[q].z;
+                            w[10 + 8 * q] = A[q].w;
+                        }
+                    }
+                    __syncwarp();
+                    for (int j = strm; 2 * j < cnt; j += NS) {
+                        const ulonglong2 *w = reinterpret_cast<const ulonglong2 *>(buf + j * PAIR);
+                        const ulonglong2 nf = w[0];
+                        const f32x2 da = sub2(sub2(xa, nf.x), nf.y), db = sub2(sub2(xb, nf.x), nf.y);
+                        const f32x2 ua = mul2(da, da), ub = mul2(db, db);
+#pragma unroll
+                        for (int q = 0; q < CG; ++q) {
+                            const ulonglong2 k0 = w[1 + 2 * q], k1 = w[2 + 2 * q];
+                            acc[q][0] = fma2(fma2(k1.x, ua, k1.y), rcp2(fma2(ua, add2(ua, k0.x), k0.y)), acc[q][0]);
+                            acc[q][1] = fma2(fma2(k1.x, ub, k1.y), rcp2(fma2(ub, add2(ub, k0.x), k0.y)), acc[q][1]);
+                        }
+                    }
+                    __syncwarp();
+                    if (++in_fold == TR_FOLD) {
+                        fold();
+                        in_fold = 0;
+                    }
+                }
+                g = gn;
+            }
+        }
+        fold();
+    }
+    // the line streams' (and the task's warps') sums, in a fixed order
+    double v[CG][2];
+#pragma unroll
+    for (int q = 0; q < CG; ++q)
+#pragma unroll
+        for (int r = 0; r < 2; ++r) {
+            v[q][r] = (double)hi[q][r] + (double)lo[q][r];
+            v[q][r] += __shfl_xor_sync(0xffffffffu, v[q][r], 8);
+            v[q][r] += __shfl_xor_sync(0xffffffffu, v[q][r], 16);
+        }
+    if (wpt > 1) {
+        __syncthreads();
+        if (lane < 8)
+#pragma unroll
+            for (int q = 0; q < CG; ++q) {
+                sRed[warp][q][2 * lane] = v[q][0];
+                sRed[warp][q][2 * lane + 1] = v[q][1];
+            }
+        __syncthreads();
+        if (part == 0 && lane < 8)
+            for (int w = 1; w < wpt; ++w)
+#pragma unroll
+                for (int q = 0; q < CG; ++q) {
+                    v[q][0] += sRed[warp + w][q][2 * lane];
+                    v[q][1] += sRed[warp + w][q][2 * lane + 1];
+                }
+    }
+    if (live && part == 0 && lane < 8)
+#pragma unroll
+        for (int q = 0; q < CG; ++q)
+            if (q < nc)
+                reinterpret_cast<double2 *>(p.nodes + (size_t)(c0 + q) * p.nodes_per_cond + p.node_off[lev] +
+                                            task * TR_M)[lane] = make_double2(v[q][0], v[q][1]);
+}
+
 // ---------------------------------------------------------------------------
 // points: the pairs no block takes, plus the interpolated sums.  A warp owns 32 points.
 // This kernel takes every profile but w4: Lorentzians in packed pairs of lines, masked by
@@ -618,45 +792,82 @@ __global__ void __launch_bounds__(TR_T) k_tree_points(TreeParams p) {
     if (live && part == 0) tr_finish(p, c, s0, lane, v);
 }
 
-// Voigt w4 at the points.  Per 32 scanned lines, each lane classifies its line for the warp's
-// 32 points and the lines go three ways:
-//   F  region I at every point of the warp: packed pairs of lines, masked by the cut;
-//   Z  the zone |x| + y < 15 reaches the points: packed pairs that evaluate regions I and II
-//      and select per point (region I is skipped where no point needs it);
+// Voigt w4 at the points, CG conditions at a time.  Lines whose zone |x| + y < 15 cannot reach the
+// warp's 32 points (most are there for an end of their cut) are in region I at every one of them
+// for all conditions: packed pairs of lines, masked by the cut, position and masks shared by the
+// conditions.  The lines near the points are then taken condition by condition.  Each lane
+// classifies one line, and they go three ways:
+//   F  region I at every point of the warp: packed pairs, masked by the cut;
+//   Z  the zone reaches the points: packed pairs that evaluate regions I and II and select per
+//      point (region I is skipped where no point needs it);
 //   items  the points in regions III and IV, which are few per line and costly: numbered line
 //      after line, region by region, and evaluated 32 at a time with one region per warp
 //      instruction; their owner lanes then add them in line order.
 // One line at a time with a branch per region left 22 of 32 lanes active and paid for up to
-// four regions per line: 6.4 ms at the 1e7-line list on 2e6 points.
+// four regions per line: 6.4 ms at the 1e7-line list on 2e6 points, 5.5 ms so.  32 conditions x
+// 1e7 lines: 92 ms one condition at a time, 82 ms four.
+template <int CG>
 struct W4Buf {
-    float4 F[16 * 4];       // per pair: n, f | E, F | P, PC | masks
-    float4 Z[16 * 6];       // per pair: n, f | E, F | P, PC | a^2, y^2 | y Pv, t2 | masks
-    float4 I[2][32];        // per line with items of region III / IV: n, f, a, y
-    int4 R[2][32];          // first item, first point, points of the left run, Pv (bits)
-    int2 S[2][32];          // first point of the right run, number of items
+    float4 F[16 * (2 + 2 * CG)];   // per pair: n, f | masks | E, F | P, PC of each condition
+    float4 Z[16 * 6];              // per pair: n, f | E, F | P, PC | a^2, y^2 | y Pv, t2 | masks
+    float4 I[2][32];               // per line with items of region III / IV: n, f, a, y
+    int4 R[2][32];                 // first item, first point, points of the left run, Pv (bits)
+    int2 S[2][32];                 // first point of the right run, number of items
+    float2 sum[CG][32];            // each point's sums (compensated)
 };
 
+// F pairs of NQ conditions: values at the lane's point (bit: the lane's), masked, into acc
+template <int NQ>
+__device__ __forceinline__ void w4_masked_pairs(const float4 *F, int nF, unsigned bit, f32x2 x2, float (&acc)[2 * NQ]) {
+#pragma unroll 2
+    for (int j = 0; 2 * j < nF; ++j) {
+        const ulonglong2 *w = reinterpret_cast<const ulonglong2 *>(F + j * (2 + 2 * NQ));
+        const ulonglong2 nf = w[0];
+        const uint2 mk = *reinterpret_cast<const uint2 *>(w + 1);
+        const f32x2 d = sub2(sub2(x2, nf.x), nf.y), u = mul2(d, d);
+        const bool i1 = (mk.x & bit) != 0u, i2 = (mk.y & bit) != 0u;
+#pragma unroll
+        for (int q = 0; q < NQ; ++q) {
+            const ulonglong2 k0 = w[2 + 2 * q], k1 = w[3 + 2 * q];
+            float v1, v2;
+            upk2(mul2(fma2(k1.x, u, k1.y), rcp2(fma2(u, add2(u, k0.x), k0.y))), v1, v2);
+            if (i1) acc[2 * q] += v1;
+            if (i2) acc[2 * q + 1] += v2;
+        }
+    }
+}
 
-__global__ void __launch_bounds__(TR_T) k_tree_points_w4(TreeParams p) {
-    __shared__ W4Buf sBuf[TR_W];
-    __shared__ double sRed[TR_W][32];
+template <int CG>
+__global__ void __launch_bounds__(CG == 1 ? 256 : 128) k_tree_points_w4(TreeParams p) {
+    constexpr int NW = CG == 1 ? 8 : 4;
+    __shared__ W4Buf<CG> sBuf[NW];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int wpt = p.wpt, part = warp % wpt;
-    const int task = blockIdx.x * (TR_W / wpt) + warp / wpt;
-    const int c = blockIdx.y;
+    const int task = blockIdx.x * (NW / wpt) + warp / wpt;
+    const int g0 = blockIdx.y * CG, nc = CG == 1 ? 1 : min(CG, p.n_cond - g0);
     const int s0 = task * 32, s1 = s0 + 31;
     const bool live = s0 < p.n_pts;
-    float hi = 0.f, lo = 0.f;
+    W4Buf<CG> &buf = sBuf[warp];
+    float2 own = make_float2(0.f, 0.f);   // the sums of a single condition
+#pragma unroll
+    for (int q = 0; q < CG; ++q) buf.sum[q][lane] = own;
+    auto add = [&](int q, float a) {   // the lane's own sums: no other lane touches them
+        float2 s = CG == 1 ? own : buf.sum[q][lane];
+        tr_fold(s.x, s.y, a);
+        if (CG == 1) own = s;
+        else buf.sum[q][lane] = s;
+    };
     if (live) {
         const int p0 = s0 & ~63, p1 = p0 + 63, p1c = min(p1, p.n_pts - 1);
-        const int Dp = tr_radius(p, p.cp[p.c0 + c].acoef, tr_gap(0), p1);
+        const float ac = tr_group_acoef(p, g0, nc);
+        const int Dp = tr_radius(p, ac, tr_gap(0), p1);
+        const int core = tr_radius(p, ac, -(1 << 28), p1);   // the zones' radius alone
         const Segs sg = tr_point_segs(p, s0, s1, p0, p1, Dp);
         const float x = (float)lane;
         const f32x2 x2 = pk2(x, x);
         const unsigned below = (1u << lane) - 1u;
-        const float4 *recA = p.recA + (size_t)c * p.n;
-        const float4 *recB = p.recB + (size_t)c * p.n;
-        W4Buf &buf = sBuf[warp];
+        const float4 *recA = p.recA + (size_t)g0 * p.n;
+        const float4 *recB = p.recB + (size_t)g0 * p.n;
 #pragma unroll 1
         for (int k = 0; k < 3; ++k) {
             const unsigned e = sg.e[k];
@@ -669,182 +880,208 @@ __global__ void __launch_bounds__(TR_T) k_tree_points_w4(TreeParams p) {
                 int4 gn = make_int4(0, 1, 0, 0);
                 if (l + 32u * wpt < e) gn = p.geo[l + 32u * wpt];
                 const bool ok = l < e && g.y <= s1 && g.z >= s0 && g.y <= g.z && !tr_takes(g, p0, p1, p1c, Dp);
-                if (!__any_sync(0xffffffffu, ok)) {
+                // (a single condition takes all lines in one go)
+                const bool near = CG == 1 || (g.x >= s0 - core && g.x <= s1 + core);
+                const unsigned bN = __ballot_sync(0xffffffffu, ok && near);
+                const unsigned bO = CG == 1 ? 0u : __ballot_sync(0xffffffffu, ok && !near);
+                if ((bN | bO) == 0u) {   // most chunks of a width-limited cut
                     g = gn;
                     continue;
-                }
-                float4 A = make_float4(0.f, 0.f, 0.f, 0.f), B = make_float4(1.f, 1.f, 0.f, -1.f);
-                if (ok) {
-                    A = recA[l];
-                    B = recB[l];
                 }
                 const float n = (float)(g.x - s0), f = __int_as_float(g.w), pos = n + f;
                 const int ka = max(g.y - s0, 0), kb = min(g.z - s0, 31);
                 const unsigned cut = ok ? lanes_of(ka, kb) : 0u;
-                // zone |x| + y < 15 (with a margin: the points decide by u < t2 themselves)
-                const float rz = sqrtf(fmaxf(B.w, 0.f)) + 0.1f;
-                const bool zone = ok && B.w > 0.f && pos + rz >= 0.f && pos - rz <= 31.f;
-                // points of regions III and IV, |x| + y < 5.5: runs of lanes around the centre
-                unsigned m3 = 0u, m34 = 0u;
-                int k0 = 0, k1 = -1, k30 = 0, k31 = -1;
-                if (zone && B.y < 5.5f && B.z != 0.f) {
-                    const float ra = rcp_approx(B.x);
-                    const float r34 = (5.5f - B.y) * ra, r3 = fminf(r34, (B.y + 0.176f) * (1.f / 0.195f) * ra);
-                    k0 = max((int)ceilf(fmaxf(pos - r34, -1.f)), ka);
-                    k1 = min((int)floorf(fminf(pos + r34, 32.f)), kb);
-                    k30 = max((int)ceilf(fmaxf(pos - r3, -1.f)), k0);
-                    k31 = min((int)floorf(fminf(pos + r3, 32.f)), k1);
-                    m34 = lanes_of(k0, k1);
-                    m3 = lanes_of(k30, k31);
-                }
-                const unsigned m4 = m34 & ~m3, m12 = cut & ~m34;
-                const bool isZ = zone && m12 != 0u && A.z != 0.f, isF = ok && !zone && A.z != 0.f;
-                const unsigned bF = __ballot_sync(0xffffffffu, isF), bZ = __ballot_sync(0xffffffffu, isZ);
-                const unsigned b3 = __ballot_sync(0xffffffffu, m3 != 0u), b4 = __ballot_sync(0xffffffffu, m4 != 0u);
-                const int nF = __popc(bF), nZ = __popc(bZ);
-                if (isF) {
-                    const int slot = __popc(bF & below);
-                    float *q = reinterpret_cast<float *>(buf.F) + (slot >> 1) * 16 + (slot & 1);
-                    q[0] = n;
-                    q[2] = f;
-                    q[4] = A.x;
-                    q[6] = A.y;
-                    q[8] = A.z;
-                    q[10] = A.w;
-                    q[12] = __uint_as_float(cut);
-                }
-                if (isZ) {
-                    const int slot = __popc(bZ & below);
-                    float *q = reinterpret_cast<float *>(buf.Z) + (slot >> 1) * 24 + (slot & 1);
-                    q[0] = n;
-                    q[2] = f;
-                    q[4] = A.x;
-                    q[6] = A.y;
-                    q[8] = A.z;
-                    q[10] = A.w;
-                    q[12] = B.x * B.x;
-                    q[14] = B.y * B.y;
-                    q[16] = B.y * B.z;
-                    q[18] = B.w;
-                    q[20] = __uint_as_float(m12);
-                }
-                // a pair without a second line: nothing of it is selected
-                if (lane == 0 && (nF & 1)) reinterpret_cast<float *>(buf.F)[(nF >> 1) * 16 + 13] = 0.f;
-                if (lane == 1 && (nZ & 1)) reinterpret_cast<float *>(buf.Z)[(nZ >> 1) * 24 + 21] = 0.f;
-                int tot[2];
+                if (bO) {
+                    const int nF = __popc(bO);
+                    if (ok && !near) {
+                        const int slot = __popc(bO & below);
+                        float *w = reinterpret_cast<float *>(buf.F) + (slot >> 1) * (4 * (2 + 2 * CG)) + (slot & 1);
+                        w[0] = n;
+                        w[2] = f;
+                        w[4] = __uint_as_float(cut);
 #pragma unroll
-                for (int t = 0; t < 2; ++t) {   // III, IV
-                    const unsigned m = t == 0 ? m3 : m4;
-                    tot[t] = 0;
-                    if ((t == 0 ? b3 : b4) == 0u) continue;
-                    const int ni = __popc(m);
-                    int off = ni;
+                        for (int q = 0; q < CG; ++q) {
+                            const float4 A = q < nc ? recA[(size_t)q * p.n + l] : make_float4(0.f, 1.f, 0.f, 0.f);
+                            w[8 + 8 * q] = A.x;
+                            w[10 + 8 * q] = A.y;
+                            w[12 + 8 * q] = A.z;
+                            w[14 + 8 * q] = A.w;
+                        }
+                    }
+                    // a pair without a second line: nothing of it is selected
+                    if (lane == 0 && (nF & 1))
+                        reinterpret_cast<float *>(buf.F)[(nF >> 1) * (4 * (2 + 2 * CG)) + 5] = 0.f;
+                    __syncwarp();
+                    float acc[2 * CG];
 #pragma unroll
-                    for (int o = 1; o < 32; o <<= 1) {
-                        const int v = __shfl_up_sync(0xffffffffu, off, o);
-                        if (lane >= o) off += v;
-                    }
-                    tot[t] = __shfl_sync(0xffffffffu, off, 31);
-                    if (ni > 0) {
-                        const int slot = __popc((t == 0 ? b3 : b4) & below);
-                        buf.I[t][slot] = make_float4(n, f, B.x, B.y);
-                        const bool split = t == 1 && m3 != 0u;
-                        const int left = t == 0 ? ni : (split ? k30 - k0 : ni);
-                        buf.R[t][slot] = make_int4(off - ni, t == 0 ? k30 : k0, left, __float_as_int(B.z));
-                        buf.S[t][slot] = make_int2(k31 + 1, ni);
-                    }
-                }
-                __syncwarp();
-                float acc = 0.f;
-                {
-                    f32x2 acc2 = 0ull;
-#pragma unroll 2
-                    for (int j = 0; 2 * j < nF; ++j) {
-                        const ulonglong2 *q = reinterpret_cast<const ulonglong2 *>(buf.F + j * 4);
-                        const ulonglong2 nf = q[0], c0 = q[1], c1 = q[2];
-                        const uint2 mk = *reinterpret_cast<const uint2 *>(buf.F + j * 4 + 3);
-                        const f32x2 d = sub2(sub2(x2, nf.x), nf.y), u = mul2(d, d);
-                        float v1, v2;
-                        upk2(mul2(fma2(c1.x, u, c1.y), rcp2(fma2(u, add2(u, c0.x), c0.y))), v1, v2);
-                        v1 = (mk.x >> lane) & 1u ? v1 : 0.f;
-                        v2 = (mk.y >> lane) & 1u ? v2 : 0.f;
-                        acc2 = add2(acc2, pk2(v1, v2));
-                    }
-                    acc = sum2(acc2);
-                    tr_fold(hi, lo, acc);
-                }
-                if (nZ) {
-                    f32x2 acc2 = 0ull;
-                    for (int j = 0; 2 * j < nZ; ++j) {
-                        const ulonglong2 *q = reinterpret_cast<const ulonglong2 *>(buf.Z + j * 6);
-                        const ulonglong2 nf = q[0], c0 = q[1], c1 = q[2], ay = q[3], pt = q[4];
-                        const uint2 mk = *reinterpret_cast<const uint2 *>(buf.Z + j * 6 + 5);
-                        const f32x2 d = sub2(sub2(x2, nf.x), nf.y), u = mul2(d, d);
-                        float u1, u2, t1, t2, v1, v2;
-                        upk2(u, u1, u2);
-                        upk2(pt.y, t1, t2);
-                        upk2(w4_region2_pair(mul2(u, ay.x), ay.y, pt.x), v1, v2);
-                        const bool r1 = u1 >= t1, r2 = u2 >= t2;
-                        if (__any_sync(0xffffffffu, r1 || r2)) {
-                            float w1, w2;
-                            upk2(mul2(fma2(c1.x, u, c1.y), rcp2(fma2(u, add2(u, c0.x), c0.y))), w1, w2);
-                            v1 = r1 ? w1 : v1;
-                            v2 = r2 ? w2 : v2;
-                        }
-                        v1 = (mk.x >> lane) & 1u ? v1 : 0.f;
-                        v2 = (mk.y >> lane) & 1u ? v2 : 0.f;
-                        acc2 = add2(acc2, pk2(v1, v2));
-                    }
-                    acc = sum2(acc2);
-                    tr_fold(hi, lo, acc);
-                }
+                    for (int q = 0; q < 2 * CG; ++q) acc[q] = 0.f;
+                    w4_masked_pairs<CG>(buf.F, nF, below + 1u, x2, acc);
 #pragma unroll
-                for (int t = 0; t < 2; ++t) {
-                    int line0 = 0;                      // lines whose items start before this batch
-                    for (int b = 0; b < tot[t]; b += 32) {
-                        // lines whose first item lies in this batch: a bit at that item
-                        int first = -1;
-                        if (lane < __popc(t == 0 ? b3 : b4)) first = buf.R[t][lane].x - b;
-                        const unsigned starts = __reduce_or_sync(0xffffffffu, first >= 0 && first < 32 ? 1u << first : 0u);
-                        const int line = line0 + __popc(starts & (below | (1u << lane))) - 1;
-                        float v = 0.f;
-                        if (b + lane < tot[t]) {
-                            const float4 q = buf.I[t][line];
-                            const int4 r = buf.R[t][line];
-                            const int o = b + lane - r.x;
-                            const int kp = o < r.z ? r.y + o : buf.S[t][line].x + o - r.z;
-                            const float xx = q.z * fabsf(((float)kp - q.x) - q.y);
-                            v = __int_as_float(r.w) * (t == 0 ? w4_region3_re(xx, q.w) : w4_region4_re(xx, q.w));
-                        }
-                        // owners add their points' values, line after line
-                        const int jl = __shfl_sync(0xffffffffu, line, min(31, tot[t] - 1 - b));
-                        for (int j = __shfl_sync(0xffffffffu, line, 0); j <= jl; ++j) {
-                            const int4 r = buf.R[t][j];
-                            const int2 s2 = buf.S[t][j];
-                            int o = lane - r.y;
-                            if (o >= r.z) o = lane - s2.x >= 0 ? lane - s2.x + r.z : -1;
-                            const int it = r.x + o - b;
-                            const float w = __shfl_sync(0xffffffffu, v, it & 31);
-                            if (o >= 0 && o < s2.y && it >= 0 && it < 32) acc += w;
-                        }
-                        tr_fold(hi, lo, acc);
-                        line0 += __popc(starts);
-                    }
+                    for (int q = 0; q < CG; ++q) add(q, acc[2 * q] + acc[2 * q + 1]);
+                    __syncwarp();
                 }
-                __syncwarp();
+#pragma unroll 1
+                for (int q = 0; bN && q < nc; ++q) {
+                    float4 A = make_float4(0.f, 0.f, 0.f, 0.f), B = make_float4(1.f, 1.f, 0.f, -1.f);
+                    const bool mine = ok && near;
+                    if (mine) {
+                        A = recA[(size_t)q * p.n + l];
+                        B = recB[(size_t)q * p.n + l];
+                    }
+                    // zone |x| + y < 15 (with a margin: the points decide by u < t2 themselves)
+                    const float rz = sqrtf(fmaxf(B.w, 0.f)) + 0.1f;
+                    const bool zone = mine && B.w > 0.f && pos + rz >= 0.f && pos - rz <= 31.f;
+                    // points of regions III and IV, |x| + y < 5.5: runs of lanes around the centre
+                    unsigned m3 = 0u, m34 = 0u;
+                    int k0 = 0, k1 = -1, k30 = 0, k31 = -1;
+                    if (zone && B.y < 5.5f && B.z != 0.f) {
+                        const float ra = rcp_approx(B.x);
+                        const float r34 = (5.5f - B.y) * ra, r3 = fminf(r34, (B.y + 0.176f) * (1.f / 0.195f) * ra);
+                        k0 = max((int)ceilf(fmaxf(pos - r34, -1.f)), ka);
+                        k1 = min((int)floorf(fminf(pos + r34, 32.f)), kb);
+                        k30 = max((int)ceilf(fmaxf(pos - r3, -1.f)), k0);
+                        k31 = min((int)floorf(fminf(pos + r3, 32.f)), k1);
+                        m34 = lanes_of(k0, k1);
+                        m3 = lanes_of(k30, k31);
+                    }
+                    const unsigned m4 = m34 & ~m3, m12 = cut & ~m34;
+                    const bool isZ = zone && m12 != 0u && A.z != 0.f, isF = mine && !zone && A.z != 0.f;
+                    const unsigned bF = __ballot_sync(0xffffffffu, isF), bZ = __ballot_sync(0xffffffffu, isZ);
+                    const unsigned b3 = __ballot_sync(0xffffffffu, m3 != 0u), b4 = __ballot_sync(0xffffffffu, m4 != 0u);
+                    const int nF = __popc(bF), nZ = __popc(bZ);
+                    if (isF) {
+                        const int slot = __popc(bF & below);
+                        float *w = reinterpret_cast<float *>(buf.F) + (slot >> 1) * 16 + (slot & 1);
+                        w[0] = n;
+                        w[2] = f;
+                        w[4] = __uint_as_float(cut);
+                        w[8] = A.x;
+                        w[10] = A.y;
+                        w[12] = A.z;
+                        w[14] = A.w;
+                    }
+                    if (isZ) {
+                        const int slot = __popc(bZ & below);
+                        float *w = reinterpret_cast<float *>(buf.Z) + (slot >> 1) * 24 + (slot & 1);
+                        w[0] = n;
+                        w[2] = f;
+                        w[4] = A.x;
+                        w[6] = A.y;
+                        w[8] = A.z;
+                        w[10] = A.w;
+                        w[12] = B.x * B.x;
+                        w[14] = B.y * B.y;
+                        w[16] = B.y * B.z;
+                        w[18] = B.w;
+                        w[20] = __uint_as_float(m12);
+                    }
+                    if (lane == 0 && (nF & 1)) reinterpret_cast<float *>(buf.F)[(nF >> 1) * 16 + 5] = 0.f;
+                    if (lane == 1 && (nZ & 1)) reinterpret_cast<float *>(buf.Z)[(nZ >> 1) * 24 + 21] = 0.f;
+                    int tot[2];
+#pragma unroll
+                    for (int t = 0; t < 2; ++t) {   // III, IV
+                        const unsigned m = t == 0 ? m3 : m4;
+                        tot[t] = 0;
+                        if ((t == 0 ? b3 : b4) == 0u) continue;
+                        const int ni = __popc(m);
+                        int off = ni;
+#pragma unroll
+                        for (int o = 1; o < 32; o <<= 1) {
+                            const int v = __shfl_up_sync(0xffffffffu, off, o);
+                            if (lane >= o) off += v;
+                        }
+                        tot[t] = __shfl_sync(0xffffffffu, off, 31);
+                        if (ni > 0) {
+                            const int slot = __popc((t == 0 ? b3 : b4) & below);
+                            buf.I[t][slot] = make_float4(n, f, B.x, B.y);
+                            const bool split = t == 1 && m3 != 0u;
+                            const int left = t == 0 ? ni : (split ? k30 - k0 : ni);
+                            buf.R[t][slot] = make_int4(off - ni, t == 0 ? k30 : k0, left, __float_as_int(B.z));
+                            buf.S[t][slot] = make_int2(k31 + 1, ni);
+                        }
+                    }
+                    __syncwarp();
+                    if (nF) {
+                        float acc[2] = {0.f, 0.f};
+                        w4_masked_pairs<1>(buf.F, nF, below + 1u, x2, acc);
+                        add(q, acc[0] + acc[1]);
+                    }
+                    if (nZ) {
+                        float acc1 = 0.f, acc2 = 0.f;
+                        for (int j = 0; 2 * j < nZ; ++j) {
+                            const ulonglong2 *w = reinterpret_cast<const ulonglong2 *>(buf.Z + j * 6);
+                            const ulonglong2 nf = w[0], c0 = w[1], c1 = w[2], ay = w[3], pt = w[4];
+                            const uint2 mk = *reinterpret_cast<const uint2 *>(w + 5);
+                            const f32x2 d = sub2(sub2(x2, nf.x), nf.y), u = mul2(d, d);
+                            float u1, u2, t1, t2, v1, v2;
+                            upk2(u, u1, u2);
+                            upk2(pt.y, t1, t2);
+                            upk2(w4_region2_pair(mul2(u, ay.x), ay.y, pt.x), v1, v2);
+                            const bool r1 = u1 >= t1, r2 = u2 >= t2;
+                            if (__any_sync(0xffffffffu, r1 || r2)) {
+                                float w1, w2;
+                                upk2(mul2(fma2(c1.x, u, c1.y), rcp2(fma2(u, add2(u, c0.x), c0.y))), w1, w2);
+                                v1 = r1 ? w1 : v1;
+                                v2 = r2 ? w2 : v2;
+                            }
+                            if (mk.x & (below + 1u)) acc1 += v1;
+                            if (mk.y & (below + 1u)) acc2 += v2;
+                        }
+                        add(q, acc1 + acc2);
+                    }
+#pragma unroll
+                    for (int t = 0; t < 2; ++t) {
+                        int line0 = 0;                      // lines whose items start before this batch
+                        for (int b = 0; b < tot[t]; b += 32) {
+                            // lines whose first item lies in this batch: a bit at that item
+                            int first = -1;
+                            if (lane < __popc(t == 0 ? b3 : b4)) first = buf.R[t][lane].x - b;
+                            const unsigned starts =
+                                __reduce_or_sync(0xffffffffu, first >= 0 && first < 32 ? 1u << first : 0u);
+                            const int line = line0 + __popc(starts & (below | (1u << lane))) - 1;
+                            float v = 0.f;
+                            if (b + lane < tot[t]) {
+                                const float4 w = buf.I[t][line];
+                                const int4 r = buf.R[t][line];
+                                const int o = b + lane - r.x;
+                                const int kp = o < r.z ? r.y + o : buf.S[t][line].x + o - r.z;
+                                const float xx = w.z * fabsf(((float)kp - w.x) - w.y);
+                                v = __int_as_float(r.w) * (t == 0 ? w4_region3_re(xx, w.w) : w4_region4_re(xx, w.w));
+                            }
+                            // owners add their points' values, line after line
+                            const int jl = __shfl_sync(0xffffffffu, line, min(31, tot[t] - 1 - b));
+                            float acc = 0.f;
+                            for (int j = __shfl_sync(0xffffffffu, line, 0); j <= jl; ++j) {
+                                const int4 r = buf.R[t][j];
+                                const int2 s2 = buf.S[t][j];
+                                int o = lane - r.y;
+                                if (o >= r.z) o = lane - s2.x >= 0 ? lane - s2.x + r.z : -1;
+                                const int it = r.x + o - b;
+                                const float w = __shfl_sync(0xffffffffu, v, it & 31);
+                                if (o >= 0 && o < s2.y && it >= 0 && it < 32) acc += w;
+                            }
+                            add(q, acc);
+                            line0 += __popc(starts);
+                        }
+                    }
+                    __syncwarp();
+                }
                 g = gn;
             }
         }
     }
-    double v = (double)hi + (double)lo;
-    if (wpt > 1) {
-        __syncthreads();
-        sRed[warp][lane] = v;
-        __syncthreads();
-        if (part == 0)
-            for (int w = 1; w < wpt; ++w) v += sRed[warp + w][lane];
+    if (CG == 1) buf.sum[0][lane] = own;
+    if (wpt > 1) __syncthreads();
+    if (!live || part != 0) return;
+#pragma unroll 1
+    for (int q = 0; q < nc; ++q) {
+        double v = 0.0;
+        for (int w = 0; w < wpt; ++w) {
+            const float2 s = sBuf[warp + w].sum[q][lane];
+            v += (double)s.x + (double)s.y;
+        }
+        tr_finish(p, g0 + q, s0, lane, v);
     }
-    if (live && part == 0) tr_finish(p, c, s0, lane, v);
 }
 
 // ---------------------------------------------------------------------------
@@ -879,7 +1116,7 @@ bool fns_of(int profile, ProfFns *f) {
     case XC_DOPPLER: *f = ProfFns TR_FNS(XC_DOPPLER); return true;
     case XC_LORENTZ: *f = ProfFns TR_FNS(XC_LORENTZ); return true;
     case XC_VOIGT_W4:
-        *f = ProfFns{k_tree_recs<XC_VOIGT_W4, false>, k_tree_recs<XC_VOIGT_W4, true>, k_tree_nodes<XC_VOIGT_W4>, k_tree_points_w4};
+        *f = ProfFns{k_tree_recs<XC_VOIGT_W4, false>, k_tree_recs<XC_VOIGT_W4, true>, nullptr, nullptr};   // see w4_fns
         return true;
     case XC_VOIGT_GH_BINNED: *f = ProfFns TR_FNS(XC_VOIGT_GH_BINNED); return true;
     case XC_VOIGT_GH_SAMPLED: *f = ProfFns TR_FNS(XC_VOIGT_GH_SAMPLED); return true;
@@ -889,12 +1126,18 @@ bool fns_of(int profile, ProfFns *f) {
     }
 }
 
+// w4's kernels take 1, 2 or 4 conditions at a time
+void w4_fns(int cg, ProfFns *f) {
+    f->nodes = cg == 4 ? k_tree_nodes_w4<4> : (cg == 2 ? k_tree_nodes_w4<2> : k_tree_nodes<XC_VOIGT_W4>);
+    f->points = cg == 4 ? k_tree_points_w4<4> : (cg == 2 ? k_tree_points_w4<2> : k_tree_points_w4<1>);
+}
+
 bool is_doppler(int profile) { return profile == XC_DOPPLER || profile == XC_DOPPLER_BINNED; }
 
 // warps per task: several where the tasks alone would leave the SMs with few warps
-int warps_per_task(int64_t tasks) {
+int warps_per_task(int64_t tasks, int most = TR_W) {
     int w = 1;
-    while (w < TR_W && tasks * w < 152 * 16) w *= 2;
+    while (w < most && tasks * w < 152 * 16) w *= 2;
     return w;
 }
 
@@ -969,18 +1212,28 @@ xc_status tree_run(BatchedState *st, const BatchedArgs &a, int64_t *launches) {
     }
     p.nodes_per_cond = off;
 
-    size_t o = 0;
+    if (cg < nc_pass && cg > 4) cg &= ~3;   // whole groups of four
+    size_t o, o_gs, o_cp, o_cell, o_nodes, o_geo, o_A, o_B, o_keep = 0, o_glc = 0;
     auto carve = [&](size_t bytes) { size_t r = o; o += (bytes + 255) & ~size_t(255); return r; };
-    // (the caller falls back to the tiled kernels when this does not fit in device memory)
-    const size_t o_gs = carve(sizeof(GeomStats)), o_cp = carve((size_t)nc_pass * sizeof(CParam));
-    const size_t o_cell = carve((size_t)(p.ncell + 1) * 4);
-    const size_t o_nodes = carve((size_t)cg * p.nodes_per_cond * 8);
-    const size_t o_geo = carve(n * sizeof(int4));
-    const size_t o_A = carve((size_t)cg * n * 16), o_B = carve(w4 ? (size_t)cg * n * 16 : 16);
-    size_t o_keep = 0, o_glc = 0;
-    if (a.opts.threshold != XC_THRESHOLD_NONE) o_keep = carve(n * (size_t)((nc_pass + 31) / 32) * 4);
-    if (a.L.n_broad > 0) o_glc = carve(n * (size_t)nc_pass * 4);
-    TR_TRY(st->tiles.ensure(o));
+    for (;; cg = cg > 4 ? 4 : 1) {
+        o = 0;
+        o_gs = carve(sizeof(GeomStats));
+        o_cp = carve((size_t)nc_pass * sizeof(CParam));
+        o_cell = carve((size_t)(p.ncell + 1) * 4);
+        o_nodes = carve((size_t)cg * p.nodes_per_cond * 8);
+        o_geo = carve(n * sizeof(int4));
+        o_A = carve((size_t)cg * n * 16);
+        o_B = carve(w4 ? (size_t)cg * n * 16 : 16);
+        if (a.opts.threshold != XC_THRESHOLD_NONE) o_keep = carve(n * (size_t)((nc_pass + 31) / 32) * 4);
+        if (a.L.n_broad > 0) o_glc = carve(n * (size_t)nc_pass * 4);
+        const cudaError_t e = st->tiles.ensure(o);
+        if (e == cudaErrorMemoryAllocation && cg > 1) {   // fewer conditions at a time
+            cudaGetLastError();
+            continue;
+        }
+        TR_TRY(e);   // out of memory here: the caller falls back to the tiled kernels
+        break;
+    }
     char *b = st->tiles.as<char>();
     GeomStats *gs = (GeomStats *)(b + o_gs);
     CParam *cp = (CParam *)(b + o_cp);
@@ -1033,22 +1286,25 @@ xc_status tree_run(BatchedState *st, const BatchedArgs &a, int64_t *launches) {
             const int m = std::min(cg, nc_pass - c0);
             p.c0 = c0;
             p.n_cond = m;
+            const int grp = w4 ? (m >= 3 ? 4 : m) : 1, ng = (m + grp - 1) / grp;   // conditions taken together, groups
+            if (w4) w4_fns(grp, &fn);
             (ext ? fn.rec_ext : fn.rec)<<<dim3(lb, m), 256, 0, s>>>(p, recA, recB);
             *launches += 2;
             if (p.far) {
                 int ctas = 0;
                 for (int lev = 0; lev < TR_LEVELS; ++lev) {
-                    p.wptl[lev] = warps_per_task((int64_t)p.nblk[lev] * m);
+                    p.wptl[lev] = warps_per_task((int64_t)p.nblk[lev] * ng);
                     const int per = TR_W / p.wptl[lev];
                     ctas += p.ncta[lev] = (p.nblk[lev] + per - 1) / per;
                 }
-                fn.nodes<<<dim3((unsigned)ctas, m), TR_T, 0, s>>>(p);
+                fn.nodes<<<dim3((unsigned)ctas, ng), TR_T, 0, s>>>(p);
                 *launches += 1;
             }
             const int64_t tasks = ((int64_t)p.n_pts + 31) / 32;
-            p.wpt = warps_per_task(tasks * m);
-            const int per = TR_W / p.wpt;
-            fn.points<<<dim3((unsigned)((tasks + per - 1) / per), m), TR_T, 0, s>>>(p);
+            const int nw = grp == 1 ? TR_W : 4;   // warps per CTA
+            p.wpt = warps_per_task(tasks * ng, nw);
+            const int per = nw / p.wpt;
+            fn.points<<<dim3((unsigned)((tasks + per - 1) / per), ng), 32 * nw, 0, s>>>(p);
         }
     }
     if (a.timing && a.ev_main1) TR_TRY(cudaEventRecord(a.ev_main1, s));
