@@ -1380,9 +1380,13 @@ __global__ void __launch_bounds__(CORE_T) k_core_w4_f32(CoreParams p) {
 
 // window -> line range for the centre zone: |nu - x| < K nu with K = 18.02 alpha_max/nu
 __global__ void k_core_ranges(const double *__restrict__ nu, int64_t n, double nu_A, double step, int64_t n_pts,
-                              double K, int n_win, unsigned *lo, unsigned *hi) {
+                              const CParam *cp, int nc, int n_win, unsigned *lo, unsigned *hi) {
     int w = blockIdx.x * blockDim.x + threadIdx.x;
     if (w >= n_win) return;
+    // from the call's own conditions: a launch argument would be frozen in a captured graph
+    float am = 0.f;
+    for (int c = 0; c < nc; ++c) am = fmaxf(am, cp[c].acoef);
+    const double K = 18.05 * (double)am * (1.0 + 1e-6);
     int64_t k0 = (int64_t)w * CORE_T;
     int64_t k1 = i64min(k0 + CORE_T, n_pts) - 1;
     double x0 = grid_x(nu_A, step, k0), x1 = grid_x(nu_A, step, k1);
@@ -1688,12 +1692,8 @@ xc_status enqueue(const BatchedArgs &a, const Plan &pl, int c0, int nc, int grid
     *launches += 1;
     if (a.opts.profile == XC_VOIGT_W4 && max_lines == 0) {
         // centre zone: |x| + y < 15, |nu - x| < 18.02 alpha <= K nu
-        double amax = 0.0;
-        for (int c = 0; c < nc; ++c)
-            amax = std::max(amax, alpha_coef(a.conds_host[c0 + c].T, a.conds_host[c0 + c].mass_da));
-        const double K = 18.05 * amax;
         k_core_ranges<<<(pl.n_win_core + 127) / 128, 128, 0, s>>>(a.L.nu, (int64_t)n, a.grid.nu_A, a.grid.step,
-                                                                   a.grid.n, K, pl.n_win_core, pl.core_lo,
+                                                                   a.grid.n, pl.cp, nc, pl.n_win_core, pl.core_lo,
                                                                    pl.core_hi);
         CoreParams cp;
         cp.L = L;

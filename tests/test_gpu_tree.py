@@ -82,6 +82,23 @@ def test_hotter_conditions_after_cooler_ones(eng, xc):  # noqa: F811
     assert close(hot, ref) < 2e-5
 
 
+def test_hotter_conditions_in_a_replayed_graph(eng, xc):  # noqa: F811
+    """The tiled sweep's centre zones in a graph captured for a cold call and replayed for a hot one."""
+    L = xs.gen_lines(303, 0, 4000, 1000.0, 1030.0)
+    eng.load_lines(L)
+    eng.set_states(*xs.gen_states(303, 500))
+    grid, opts = xc.make_grid(1000.0, 0.01, 3001), xc.make_opts("voigt_w4", "fp32", 25.0)
+    out = torch.zeros((1, 3001), dtype=torch.float64, device="cuda:0")
+    eng.set_tile_shape(8, 1)
+    try:
+        eng.cross_section_batched([xc.make_condition(100.0, 0.01)], grid, opts, out)
+        eng.cross_section_batched([xc.make_condition(3000.0, 0.01)], grid, opts, out)
+    finally:
+        eng.set_tile_shape(0, 0)
+    ref = eng.cross_section_batched([xc.make_condition(3000.0, 0.01)], grid, opts)
+    assert close(out.cpu().numpy(), ref) < 2e-5
+
+
 # ------------------------------------------------------------------ FP64
 def binned64(L, Q, T, P, x, step, cut, wm, profile):
     """Binned profiles with one arctangent per node.  (The oracle takes the difference of two, which
