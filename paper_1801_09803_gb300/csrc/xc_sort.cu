@@ -481,6 +481,8 @@ cudaError_t launch_sort_lines(const LinesDev &in, size_t n, bool assume_sorted, 
     int h_flag = 0;
     if ((e = cudaMemcpyAsync(&h_flag, d_flag, sizeof(int), cudaMemcpyDeviceToHost, s)) != cudaSuccess) return e;
     if ((e = cudaStreamSynchronize(s)) != cudaSuccess) return e;
+    // the packed records of a very large list are given back
+    if (tmp[5].bytes > ((size_t)4 << 30)) tmp[5].release();
     *bad_input = (h_flag & 1) != 0;
     *unsorted = (h_flag & 2) != 0;
     return cudaSuccess;
