@@ -804,15 +804,18 @@ __global__ void __launch_bounds__(TR_T) k_tree_points(TreeParams p) {
 //      after line, region by region, and evaluated 32 at a time with one region per warp
 //      instruction; their owner lanes then add them in line order.
 // One line at a time with a branch per region left 22 of 32 lanes active and paid for up to
-// four regions per line: 6.4 ms at the 1e7-line list on 2e6 points, 5.5 ms so.  32 conditions x
-// 1e7 lines: 92 ms one condition at a time, 82 ms four.
+// four regions per line: 6.4 ms at the 1e7-line list on 2e6 points, 5.5 ms so, 5.1 ms with each
+// line's points kept as a bit per lane (an owner's item is the count of the bits below its own;
+// from the runs' ends it took a dozen instructions per line).  32 conditions x 1e7 lines: 92 ms
+// one condition at a time, 82 ms four, 76 ms with the bits.
 template <int CG>
 struct W4Buf {
     float4 F[16 * (2 + 2 * CG)];   // per pair: n, f | masks | E, F | P, PC of each condition
     float4 Z[16 * 6];              // per pair: n, f | E, F | P, PC | a^2, y^2 | y Pv, t2 | masks
     float4 I[2][32];               // per line with items of region III / IV: n, f, a, y
     int4 R[2][32];                 // first item, first point, points of the left run, Pv (bits)
-    int2 S[2][32];                 // first point of the right run, number of items
+    int S[2][32];                  // first point of the right run
+    uint2 M[2][32];                // first item, points (a bit per lane)
     float2 sum[CG][32];            // each point's sums (compensated)
 };
 
@@ -997,7 +1000,8 @@ __global__ void __launch_bounds__(CG == 1 ? 256 : 128) k_tree_points_w4(TreePara
                             const bool split = t == 1 && m3 != 0u;
                             const int left = t == 0 ? ni : (split ? k30 - k0 : ni);
                             buf.R[t][slot] = make_int4(off - ni, t == 0 ? k30 : k0, left, __float_as_int(B.z));
-                            buf.S[t][slot] = make_int2(k31 + 1, ni);
+                            buf.S[t][slot] = k31 + 1;
+                            buf.M[t][slot] = make_uint2((unsigned)(off - ni), m);
                         }
                     }
                     __syncwarp();
@@ -1044,7 +1048,7 @@ __global__ void __launch_bounds__(CG == 1 ? 256 : 128) k_tree_points_w4(TreePara
                                 const float4 w = buf.I[t][line];
                                 const int4 r = buf.R[t][line];
                                 const int o = b + lane - r.x;
-                                const int kp = o < r.z ? r.y + o : buf.S[t][line].x + o - r.z;
+                                const int kp = o < r.z ? r.y + o : buf.S[t][line] + o - r.z;
                                 const float xx = w.z * fabsf(((float)kp - w.x) - w.y);
                                 v = __int_as_float(r.w) * (t == 0 ? w4_region3_re(xx, w.w) : w4_region4_re(xx, w.w));
                             }
@@ -1052,13 +1056,10 @@ __global__ void __launch_bounds__(CG == 1 ? 256 : 128) k_tree_points_w4(TreePara
                             const int jl = __shfl_sync(0xffffffffu, line, min(31, tot[t] - 1 - b));
                             float acc = 0.f;
                             for (int j = __shfl_sync(0xffffffffu, line, 0); j <= jl; ++j) {
-                                const int4 r = buf.R[t][j];
-                                const int2 s2 = buf.S[t][j];
-                                int o = lane - r.y;
-                                if (o >= r.z) o = lane - s2.x >= 0 ? lane - s2.x + r.z : -1;
-                                const int it = r.x + o - b;
+                                const uint2 r = buf.M[t][j];
+                                const int it = (int)r.x + __popc(r.y & below) - b;
                                 const float w = __shfl_sync(0xffffffffu, v, it & 31);
-                                if (o >= 0 && o < s2.y && it >= 0 && it < 32) acc += w;
+                                if ((r.y & (below + 1u)) != 0u && (unsigned)it < 32u) acc += w;
                             }
                             add(q, acc);
                             line0 += __popc(starts);
@@ -1213,7 +1214,7 @@ xc_status tree_run(BatchedState *st, const BatchedArgs &a, int64_t *launches) {
     p.nodes_per_cond = off;
 
     if (cg < nc_pass && cg > 4) cg &= ~3;   // whole groups of four
-    size_t o, o_gs, o_cp, o_cell, o_nodes, o_geo, o_A, o_B, o_keep = 0, o_glc = 0;
+    size_t o = 0, o_gs, o_cp, o_cell, o_nodes, o_geo, o_A, o_B, o_keep = 0, o_glc = 0;
     auto carve = [&](size_t bytes) { size_t r = o; o += (bytes + 255) & ~size_t(255); return r; };
     for (;; cg = cg > 4 ? 4 : 1) {
         o = 0;
