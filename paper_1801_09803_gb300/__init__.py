@@ -443,32 +443,43 @@ class Engine:
 
 
 # ---------------------------------------------------------------------------- autograd
+_Function = None
+
+
+def _autograd_function():
+    """The torch.autograd.Function, made once: building the class takes a tenth of a small
+    forward and backward pass."""
+    global _Function
+    if _Function is None:
+        import torch
+
+        class _CrossSection(torch.autograd.Function):
+            @staticmethod
+            def forward(ctx, T, P, s, n, engine, grid, opts, mass_da, T_ref, P_ref):
+                sv, nv = float(s), float(n)
+                conds = [make_condition(t, p, mass_da=mass_da, T_ref=T_ref, P_ref=P_ref, gamma_scale=sv, n_shift=nv)
+                         for t, p in zip(T.detach().cpu().tolist(), P.detach().cpu().tolist())]
+                ctx.call = (engine, conds, grid, opts)
+                ctx.devices = [torch.as_tensor(v).device for v in (T, P, s, n)]
+                out = torch.empty((len(conds), grid.n), dtype=torch.float64, device=f"cuda:{engine.device}")
+                engine.cross_section_batched(conds, grid, opts, out)
+                return out
+
+            @staticmethod
+            def backward(ctx, g):
+                engine, conds, grid, opts = ctx.call
+                r = engine.cross_section_vjp(conds, grid, opts, g.contiguous().to(torch.float64), per_line=False)
+                d = ctx.devices
+                return (r["dT"].to(d[0]), r["dP"].to(d[1]), r["d_gamma_scale"].reshape(()).to(d[2]),
+                        r["d_n_shift"].reshape(()).to(d[3]), None, None, None, None, None, None)
+
+        _Function = _CrossSection
+    return _Function
+
+
 def cross_section_autograd(engine: "Engine", T, P, gamma_scale, n_shift, grid: XcGrid, opts: XcOpts,
                            mass_da: float = 18.0, T_ref: float = 296.0, P_ref: float = 1.0):
     """Differentiable batched cross section: sigma[C][N] as a function of the tensors
     T[C], P[C] and the scalars gamma_scale, n_shift (float64 tensors).  The backward
     pass calls the library's adjoint (xc_cross_section_vjp)."""
-    import torch
-
-    class _CrossSection(torch.autograd.Function):
-        @staticmethod
-        def forward(ctx, T_, P_, s_, n_):
-            conds = [make_condition(float(t), float(p), mass_da=mass_da, T_ref=T_ref, P_ref=P_ref,
-                                    gamma_scale=float(s_), n_shift=float(n_))
-                     for t, p in zip(T_.detach().cpu().tolist(), P_.detach().cpu().tolist())]
-            ctx.conds = conds
-            out = torch.empty((len(conds), grid.n), dtype=torch.float64, device=f"cuda:{engine.device}")
-            engine.cross_section_batched(conds, grid, opts, out)
-            return out
-
-        @staticmethod
-        def backward(ctx, g):
-            r = engine.cross_section_vjp(ctx.conds, grid, opts, g.contiguous().to(torch.float64),
-                                         per_line=False)
-            dT = r["dT"].to(T.device)
-            dP = r["dP"].to(P.device)
-            ds = r["d_gamma_scale"].reshape(()).to(torch.as_tensor(gamma_scale).device)
-            dn = r["d_n_shift"].reshape(()).to(torch.as_tensor(n_shift).device)
-            return dT, dP, ds, dn
-
-    return _CrossSection.apply(T, P, gamma_scale, n_shift)
+    return _autograd_function().apply(T, P, gamma_scale, n_shift, engine, grid, opts, mass_da, T_ref, P_ref)
