@@ -819,6 +819,19 @@ struct W4Buf {
     float2 sum[CG][32];            // each point's sums (compensated)
 };
 
+// inclusive sum over the warp's lanes: the shuffle's own predicate selects the lanes that add
+__device__ __forceinline__ unsigned tr_scan(unsigned v) {
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1)
+        asm volatile(
+            "{\n\t.reg .pred p;\n\t.reg .u32 t;\n\t"
+            "shfl.sync.up.b32 t|p, %0, %1, 0, 0xffffffff;\n\t"
+            "@p add.u32 %0, %0, t;\n\t}"
+            : "+r"(v)
+            : "r"(o));
+    return v;
+}
+
 // F pairs of NQ conditions: values at the lane's point (bit: the lane's), masked, into acc
 template <int NQ>
 __device__ __forceinline__ void w4_masked_pairs(const float4 *F, int nF, unsigned bit, f32x2 x2, float (&acc)[2 * NQ]) {
@@ -894,6 +907,8 @@ __global__ void __launch_bounds__(CG == 1 ? 256 : 128) k_tree_points_w4(TreePara
                 const float n = (float)(g.x - s0), f = __int_as_float(g.w), pos = n + f;
                 const int ka = max(g.y - s0, 0), kb = min(g.z - s0, 31);
                 const unsigned cut = ok ? lanes_of(ka, kb) : 0u;
+                // (distance to the warp's points less a margin)^2: against a zone's radius^2
+                const float dist = fmaxf(fmaxf(-pos, pos - 31.f) - 0.1f, 0.f), dist2 = dist * dist;
                 if (bO) {
                     const int nF = __popc(bO);
                     if (ok && !near) {
@@ -932,18 +947,17 @@ __global__ void __launch_bounds__(CG == 1 ? 256 : 128) k_tree_points_w4(TreePara
                         B = recB[(size_t)q * p.n + l];
                     }
                     // zone |x| + y < 15 (with a margin: the points decide by u < t2 themselves)
-                    const float rz = sqrtf(fmaxf(B.w, 0.f)) + 0.1f;
-                    const bool zone = mine && B.w > 0.f && pos + rz >= 0.f && pos - rz <= 31.f;
+                    const bool zone = dist2 <= B.w;
                     // points of regions III and IV, |x| + y < 5.5: runs of lanes around the centre
                     unsigned m3 = 0u, m34 = 0u;
                     int k0 = 0, k1 = -1, k30 = 0, k31 = -1;
                     if (zone && B.y < 5.5f && B.z != 0.f) {
                         const float ra = rcp_approx(B.x);
                         const float r34 = (5.5f - B.y) * ra, r3 = fminf(r34, (B.y + 0.176f) * (1.f / 0.195f) * ra);
-                        k0 = max((int)ceilf(fmaxf(pos - r34, -1.f)), ka);
-                        k1 = min((int)floorf(fminf(pos + r34, 32.f)), kb);
-                        k30 = max((int)ceilf(fmaxf(pos - r3, -1.f)), k0);
-                        k31 = min((int)floorf(fminf(pos + r3, 32.f)), k1);
+                        k0 = max(__float2int_ru(fmaxf(pos - r34, -1.f)), ka);
+                        k1 = min(__float2int_rd(fminf(pos + r34, 32.f)), kb);
+                        k30 = max(__float2int_ru(fmaxf(pos - r3, -1.f)), k0);
+                        k31 = min(__float2int_rd(fminf(pos + r3, 32.f)), k1);
                         m34 = lanes_of(k0, k1);
                         m3 = lanes_of(k30, k31);
                     }
@@ -980,21 +994,18 @@ __global__ void __launch_bounds__(CG == 1 ? 256 : 128) k_tree_points_w4(TreePara
                     }
                     if (lane == 0 && (nF & 1)) reinterpret_cast<float *>(buf.F)[(nF >> 1) * 16 + 5] = 0.f;
                     if (lane == 1 && (nZ & 1)) reinterpret_cast<float *>(buf.Z)[(nZ >> 1) * 24 + 21] = 0.f;
-                    int tot[2];
+                    // III (low half) and IV (high half): both counts are summed in one scan
+                    unsigned ends = 0u, all = 0u;
+                    if ((b3 | b4) != 0u) {
+                        ends = tr_scan((unsigned)__popc(m3) | (unsigned)__popc(m4) << 16);
+                        all = __shfl_sync(0xffffffffu, ends, 31);
+                    }
+                    const int tot[2] = {(int)(all & 0xffffu), (int)(all >> 16)};
 #pragma unroll
-                    for (int t = 0; t < 2; ++t) {   // III, IV
+                    for (int t = 0; t < 2; ++t) {
                         const unsigned m = t == 0 ? m3 : m4;
-                        tot[t] = 0;
-                        if ((t == 0 ? b3 : b4) == 0u) continue;
-                        const int ni = __popc(m);
-                        int off = ni;
-#pragma unroll
-                        for (int o = 1; o < 32; o <<= 1) {
-                            const int v = __shfl_up_sync(0xffffffffu, off, o);
-                            if (lane >= o) off += v;
-                        }
-                        tot[t] = __shfl_sync(0xffffffffu, off, 31);
-                        if (ni > 0) {
+                        if (m != 0u) {
+                            const int ni = __popc(m), off = t == 0 ? (int)(ends & 0xffffu) : (int)(ends >> 16);
                             const int slot = __popc((t == 0 ? b3 : b4) & below);
                             buf.I[t][slot] = make_float4(n, f, B.x, B.y);
                             const bool split = t == 1 && m3 != 0u;
@@ -1039,7 +1050,7 @@ __global__ void __launch_bounds__(CG == 1 ? 256 : 128) k_tree_points_w4(TreePara
                         for (int b = 0; b < tot[t]; b += 32) {
                             // lines whose first item lies in this batch: a bit at that item
                             int first = -1;
-                            if (lane < __popc(t == 0 ? b3 : b4)) first = buf.R[t][lane].x - b;
+                            if (lane < __popc(t == 0 ? b3 : b4)) first = (int)buf.M[t][lane].x - b;
                             const unsigned starts =
                                 __reduce_or_sync(0xffffffffu, first >= 0 && first < 32 ? 1u << first : 0u);
                             const int line = line0 + __popc(starts & (below | (1u << lane))) - 1;
