@@ -807,11 +807,17 @@ __global__ void __launch_bounds__(TR_T) k_tree_points(TreeParams p) {
 // four regions per line: 6.4 ms at the 1e7-line list on 2e6 points, 5.5 ms so, 5.1 ms with each
 // line's points kept as a bit per lane (an owner's item is the count of the bits below its own;
 // from the runs' ends it took a dozen instructions per line).  32 conditions x 1e7 lines: 92 ms
-// one condition at a time, 82 ms four, 76 ms with the bits.
+// one condition at a time, 82 ms four, 76 ms with the bits, 73 ms with the odd spacing below.
+// Pairs of lines lie an odd number of 16-byte words apart (the last word is not used), so that
+// the lanes that write a pair each meet in the same bank two at a time instead of eight.
+constexpr int w4_words_f(int nq) { return 3 + 2 * nq; }   // n, f | masks | E, F | P, PC of each condition
+constexpr int W4_WORDS_Z = 7;                             // n, f | E, F | P, PC | a^2, y^2 | y Pv, t2 | masks
 template <int CG>
 struct W4Buf {
-    float4 F[16 * (2 + 2 * CG)];   // per pair: n, f | masks | E, F | P, PC of each condition
-    float4 Z[16 * 6];              // per pair: n, f | E, F | P, PC | a^2, y^2 | y Pv, t2 | masks
+    static_assert(w4_words_f(CG) <= w4_words_f(1) + W4_WORDS_Z, "F of all conditions fits");
+    // F of CG conditions, or F of one condition followed by Z
+    float4 F[16 * (w4_words_f(1) + W4_WORDS_Z)];
+    __device__ __forceinline__ float4 *Z() { return F + 16 * w4_words_f(1); }
     float4 I[2][32];               // per line with items of region III / IV: n, f, a, y
     int4 R[2][32];                 // first item, first point, points of the left run, Pv (bits)
     int S[2][32];                  // first point of the right run
@@ -837,7 +843,7 @@ template <int NQ>
 __device__ __forceinline__ void w4_masked_pairs(const float4 *F, int nF, unsigned bit, f32x2 x2, float (&acc)[2 * NQ]) {
 #pragma unroll 2
     for (int j = 0; 2 * j < nF; ++j) {
-        const ulonglong2 *w = reinterpret_cast<const ulonglong2 *>(F + j * (2 + 2 * NQ));
+        const ulonglong2 *w = reinterpret_cast<const ulonglong2 *>(F + j * w4_words_f(NQ));
         const ulonglong2 nf = w[0];
         const uint2 mk = *reinterpret_cast<const uint2 *>(w + 1);
         const f32x2 d = sub2(sub2(x2, nf.x), nf.y), u = mul2(d, d);
@@ -913,7 +919,7 @@ __global__ void __launch_bounds__(CG == 1 ? 256 : 128) k_tree_points_w4(TreePara
                     const int nF = __popc(bO);
                     if (ok && !near) {
                         const int slot = __popc(bO & below);
-                        float *w = reinterpret_cast<float *>(buf.F) + (slot >> 1) * (4 * (2 + 2 * CG)) + (slot & 1);
+                        float *w = reinterpret_cast<float *>(buf.F) + (slot >> 1) * (4 * w4_words_f(CG)) + (slot & 1);
                         w[0] = n;
                         w[2] = f;
                         w[4] = __uint_as_float(cut);
@@ -928,7 +934,7 @@ __global__ void __launch_bounds__(CG == 1 ? 256 : 128) k_tree_points_w4(TreePara
                     }
                     // a pair without a second line: nothing of it is selected
                     if (lane == 0 && (nF & 1))
-                        reinterpret_cast<float *>(buf.F)[(nF >> 1) * (4 * (2 + 2 * CG)) + 5] = 0.f;
+                        reinterpret_cast<float *>(buf.F)[(nF >> 1) * (4 * w4_words_f(CG)) + 5] = 0.f;
                     __syncwarp();
                     float acc[2 * CG];
 #pragma unroll
@@ -968,7 +974,7 @@ __global__ void __launch_bounds__(CG == 1 ? 256 : 128) k_tree_points_w4(TreePara
                     const int nF = __popc(bF), nZ = __popc(bZ);
                     if (isF) {
                         const int slot = __popc(bF & below);
-                        float *w = reinterpret_cast<float *>(buf.F) + (slot >> 1) * 16 + (slot & 1);
+                        float *w = reinterpret_cast<float *>(buf.F) + (slot >> 1) * (4 * w4_words_f(1)) + (slot & 1);
                         w[0] = n;
                         w[2] = f;
                         w[4] = __uint_as_float(cut);
@@ -979,7 +985,7 @@ __global__ void __launch_bounds__(CG == 1 ? 256 : 128) k_tree_points_w4(TreePara
                     }
                     if (isZ) {
                         const int slot = __popc(bZ & below);
-                        float *w = reinterpret_cast<float *>(buf.Z) + (slot >> 1) * 24 + (slot & 1);
+                        float *w = reinterpret_cast<float *>(buf.Z()) + (slot >> 1) * (4 * W4_WORDS_Z) + (slot & 1);
                         w[0] = n;
                         w[2] = f;
                         w[4] = A.x;
@@ -992,8 +998,8 @@ __global__ void __launch_bounds__(CG == 1 ? 256 : 128) k_tree_points_w4(TreePara
                         w[18] = B.w;
                         w[20] = __uint_as_float(m12);
                     }
-                    if (lane == 0 && (nF & 1)) reinterpret_cast<float *>(buf.F)[(nF >> 1) * 16 + 5] = 0.f;
-                    if (lane == 1 && (nZ & 1)) reinterpret_cast<float *>(buf.Z)[(nZ >> 1) * 24 + 21] = 0.f;
+                    if (lane == 0 && (nF & 1)) reinterpret_cast<float *>(buf.F)[(nF >> 1) * (4 * w4_words_f(1)) + 5] = 0.f;
+                    if (lane == 1 && (nZ & 1)) reinterpret_cast<float *>(buf.Z())[(nZ >> 1) * (4 * W4_WORDS_Z) + 21] = 0.f;
                     // III (low half) and IV (high half): both counts are summed in one scan
                     unsigned ends = 0u, all = 0u;
                     if ((b3 | b4) != 0u) {
@@ -1024,7 +1030,7 @@ __global__ void __launch_bounds__(CG == 1 ? 256 : 128) k_tree_points_w4(TreePara
                     if (nZ) {
                         float acc1 = 0.f, acc2 = 0.f;
                         for (int j = 0; 2 * j < nZ; ++j) {
-                            const ulonglong2 *w = reinterpret_cast<const ulonglong2 *>(buf.Z + j * 6);
+                            const ulonglong2 *w = reinterpret_cast<const ulonglong2 *>(buf.Z() + j * W4_WORDS_Z);
                             const ulonglong2 nf = w[0], c0 = w[1], c1 = w[2], ay = w[3], pt = w[4];
                             const uint2 mk = *reinterpret_cast<const uint2 *>(w + 5);
                             const f32x2 d = sub2(sub2(x2, nf.x), nf.y), u = mul2(d, d);
