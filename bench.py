@@ -211,10 +211,11 @@ def cpu_oracle_rate(W, lines, E, g, conds, budget_s=12.0, threads=None):
                       f"full grid ({best[2]:.3g} evals in {best[3]:.1f} s)"}
 
 
-# Modelled HBM traffic of the line-list sort (bytes per line): key making (read nu 8 B,
-# write key 8 + index 4), one histogram pass over the keys (8), 8 LSD digit passes
-# (tile histogram 8 + scatter read 12 + write 12), gather (index 4 + 28 read + 28 write).
-SORT_BYTES_PER_LINE = 20 + 8 + 8 * 32 + 60
+# Modelled HBM traffic of the line-list sort (bytes per line): key making (read the 28 B
+# record, write key 8 + index 4 + packed record 32), one histogram pass over the keys (8), 5
+# LSD digit passes (tile histogram 8 + scatter read 12 + write 12), the finish of short runs
+# (key 8), gather (index 4 + key 8 + record 32 read, 28 written).
+SORT_BYTES_PER_LINE = 72 + 8 + 5 * 32 + 8 + 72
 # Standalone FP64 line parameters: read nu, E'', A, g', gamma_ref, n (26 B), write I, alpha, gamma (24 B).
 PARAMS_BYTES_PER_LINE = 26 + 24
 
@@ -229,7 +230,8 @@ def hbm_stages(eng, xc, torch, dev, n, cond, sort_ms, gather_ms):
     out["sort_gather"] = {"ms": sort_ms + gather_ms, "modelled_bytes": sb,
                           "gbs": sb / ((sort_ms + gather_ms) / 1e3) / 1e9,
                           "frac": sb / ((sort_ms + gather_ms) / 1e3) / 1e9 / pk["hbm_gbs"],
-                          "model": "20 + 8 + 8 x 32 + 60 B per line (keys, histogram, 8 digit passes, gather)"}
+                          "model": "72 + 8 + 5 x 32 + 8 + 72 B per line (keys and records, histogram, 5 digit "
+                                   "passes, short runs, gather)"}
     I = torch.empty(n, dtype=torch.float64, device=dev)
     a = torch.empty_like(I)
     g = torch.empty_like(I)
@@ -562,7 +564,9 @@ def run_xc(args, dist, rank, world, local):
         ach = evals * ALG_FLOPS_PER_EVAL / (prof / 1e3) / 1e12
         sweep_rl = {"bound": "alu", "achieved": ach, "peak": peak_max, "unit": "TFLOP/s", "frac": ach / peak_max,
                     "traffic": None,
-                    "kernel": "all profile kernels of the sweep (CUDA events inside the graph), algorithmic flops",
+                    "kernel": "all profile kernels of the sweep (CUDA events on its stream)",
+                    "flops": "algorithmic: every line x grid-point evaluation of the direct sum; the "
+                             "block-interpolated sweep evaluates about one in nine, so the fraction can exceed 1",
                     "peak_basis": f"{nsm} SMs x 128 FP32 lanes x 2 flop x 2070 MHz (max SM clock)",
                     "frac_at_sampled_clock": (ach / (nsm * 128 * 2 * sm_mhz * 1e6 / 1e12)) if sm_mhz else None,
                     "flops_per_eval": ALG_FLOPS_PER_EVAL, "kernel_ms": prof}

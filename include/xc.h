@@ -78,10 +78,10 @@ enum {
 /* xc_load_lines flags */
 enum { XC_ASSUME_SORTED = 1u };
 
-/* xc_opts.flags.  With XC_FP32, Voigt w4, a fixed cut and 16 or more conditions,
- * the far wings (points at least D(l, c) grid steps from a line, D chosen so that
- * the region-I rational equals its three-term series in 1/u to < 2e-7) are summed
- * on the tensor cores as a matrix product (TF32 operands split hi + lo, FP32
+/* xc_opts.flags.  With XC_FP32, Voigt w4, 16 or more conditions and a fixed cut of fewer than
+ * 1024 grid steps, small lists (lines x conditions < 2^19) have the far wings (points at least
+ * D(l, c) grid steps from a line, D chosen so that the region-I rational equals its four-term
+ * series in 1/u to < 2e-7) summed on the tensor cores as a matrix product (TF32 operands, FP32
  * accumulation); XC_OPT_NO_TENSOR_CORES keeps every evaluation on the CUDA cores. */
 enum { XC_OPT_NO_TENSOR_CORES = 1 };
 
@@ -259,11 +259,12 @@ xc_status xc_count_evals(xc_handle *h, const xc_condition *conds, size_t n_cond,
 xc_status xc_cross_section(xc_handle *h, const xc_condition *cond, const xc_grid *grid,
                            const xc_opts *opts, double *sigma_out, int mem, void *stream);
 
-/* n_cond conditions in one persistent launch that shares every staged line
- * across conditions (sigma_out: float64[n_cond][grid->n], condition-major).
- * opts->precision XC_FP32 uses the batched FP32 kernel (window size picked by
- * the autotuner and cached per shape; the sweep is captured once into a CUDA
- * graph and replayed); XC_FP64_PLAIN runs the FP64 kernel per condition. */
+/* n_cond conditions (sigma_out: float64[n_cond][grid->n], condition-major).  Far from its centre
+ * a profile is summed at the Chebyshev nodes of blocks of the grid and the sums are
+ * interpolated to the points (within 2e-8 of each value in FP32, 1e-16 in FP64); XC_FP32 takes
+ * up to four conditions per scan of the lines.  The Vectorized Voigt, a fixed tile shape
+ * (xc_set_tile_shape) and calls whose scratch would not fit run the tiled kernels (FP32: window
+ * size picked by the autotuner and cached per shape, the sweep captured into a CUDA graph). */
 xc_status xc_cross_section_batched(xc_handle *h, const xc_condition *conds, size_t n_cond,
                                    const xc_grid *grid, const xc_opts *opts, double *sigma_out,
                                    int mem, void *stream);
