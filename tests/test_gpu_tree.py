@@ -99,6 +99,22 @@ def test_hotter_conditions_in_a_replayed_graph(eng, xc):  # noqa: F811
     assert close(out.cpu().numpy(), ref) < 2e-5
 
 
+@pytest.mark.parametrize("profile", ["voigt_w4", "lorentz"])
+@pytest.mark.parametrize("n_lines", [3001, 40_001, 40_400, 100_001])
+@pytest.mark.parametrize("n_cond", [5, 16])
+def test_sparse_lists_on_large_outputs(eng, xc, n_cond, n_lines, profile):  # noqa: F811
+    """Either side of the lines a point below which the tiled kernels run (200 and 500 pairs a point)."""
+    L = xs.gen_lines(307, 0, n_lines, 990.0, 11010.0)
+    eng.load_lines(L)
+    eng.set_states(*xs.gen_states(307, 500))
+    grid = xc.make_grid(1000.0, 0.01, 1_000_003)
+    conds = [xc.make_condition(400.0 + 60.0 * i, 0.01 * 1.5 ** i) for i in range(n_cond)]
+    got = eng.cross_section_batched(conds, grid, xc.make_opts(profile, "fp32", 25.0))
+    for c in (0, n_cond - 1):
+        ref = eng.cross_section_batched([conds[c]], grid, xc.make_opts(profile, "fp64", 25.0))
+        assert close(got[c:c + 1], ref) < 2e-5
+
+
 # ------------------------------------------------------------------ FP64
 def binned64(L, Q, T, P, x, step, cut, wm, profile):
     """Binned profiles with one arctangent per node.  (The oracle takes the difference of two, which
