@@ -133,7 +133,7 @@ __global__ void k_line_geom(LinesDev L, size_t n, double nu_A, double step, int6
         }
         double d = (nu - nu_A) * inv_h;
         double fl = floor(d);
-        double flc = fmin(fmax(fl, -1073741824.0), 1073741824.0);
+        double flc = fmin(fmax(fl, kPosMin), kPosMax);
         n_abs[l] = (int)flc;
         f_frac[l] = (float)(d - fl);
         int64_t ka, kb;

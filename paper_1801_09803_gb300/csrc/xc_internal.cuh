@@ -148,6 +148,11 @@ __device__ inline double mixture_gamma64(const LinesDev &L, size_t l, const Cond
     return mixture_gamma64(L, l, c, log(c.T_ref / c.T), c.gamma_scale * (c.P / c.P_ref));
 }
 
+// Integer grid positions of lines are held in 32 bits and clamped to this range.  The FP32 paths
+// take grids of fewer than 2^31 - 2^20 points, so a line right of the clamp does not reach the grid
+// unless its cut is longer than 2^20 steps; lines left of it do not unless theirs is longer than 2^30.
+constexpr double kPosMin = -1073741824.0, kPosMax = 2147483000.0;
+
 // grid point nu_k = nu_A + k * step, rounded exactly as two separate operations
 __device__ inline double grid_x(double nu_A, double step, int64_t k) {
     return __dadd_rn(nu_A, __dmul_rn((double)k, step));

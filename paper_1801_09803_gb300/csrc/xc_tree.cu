@@ -115,7 +115,7 @@ __global__ void __launch_bounds__(256) k_tree_geom(LinesDev L, size_t n, double 
         if (zero_k > 0.0) cut = fmin(cut, zero_k * nu + zero_0);
         const double d = (nu - nu_A) * inv_h;
         const double fl = floor(d);
-        const double flc = fmin(fmax(fl, -1073741824.0), 1073741824.0);
+        const double flc = fmin(fmax(fl, kPosMin), kPosMax);
         const double ta = (nu - cut - nu_A) * inv_h, tb = (nu + cut - nu_A) * inv_h;
         int ka = 1, kb = 0;
         if (fabs(ta - rint(ta)) > eps && fabs(tb - rint(tb)) > eps) {

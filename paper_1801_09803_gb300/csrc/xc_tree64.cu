@@ -70,8 +70,11 @@ __global__ void __launch_bounds__(256) k_t64_geom(const double *__restrict__ nu,
     for (size_t l = (size_t)blockIdx.x * 256 + threadIdx.x; l < n; l += (size_t)gridDim.x * 256) {
         const double v = nu[l];
         double c = cut[l];
-        int4 g = make_int4((int)fmin(fmax(floor((v - nu_A) * inv_h), -1073741824.0), 1073741824.0), 1, 0, 0);
-        if (c >= 0.0 && abs(g.x) < 1073741824) {   // a negative cut: left out by the intensity threshold
+        const double pos = floor((v - nu_A) * inv_h);
+        int4 g = make_int4((int)fmin(fmax(pos, kPosMin), kPosMax), 1, 0, 0);
+        // grids of fewer than 2^30 points and cuts of fewer than 2^20 steps: a line beyond the clamp
+        // reaches no point.  A negative cut: left out by the intensity threshold.
+        if (c >= 0.0 && pos > kPosMin && pos < kPosMax) {
             if (zero_k > 0.0) c = fmin(c, zero_k * al[l] + 2.0 * step);
             int64_t ka = (int64_t)ceil((v - c - nu_A) * inv_h), kb = (int64_t)floor((v + c - nu_A) * inv_h);
             while (__dsub_rn(grid_x(nu_A, step, ka - 1), v) >= -c) --ka;

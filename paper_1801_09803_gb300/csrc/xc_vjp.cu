@@ -636,7 +636,7 @@ __global__ void __launch_bounds__(VT, MIX ? 2 : 3) k_vjp32(Vjp32Params p) {
                 // 2^(-u / a^2) is exactly 0 in FP32 beyond 11.3 a
                 const int r = (int)fminf(ceilf(11.3f * a_h) + 2.f, 1e9f);
                 k0 = max(k0, na - r);
-                k1 = min(k1, na + r);
+                k1 = (int)i64min(k1, (int64_t)na + r);
             } else if (p.gnode) {
                 // The far points on both sides by the nodes of the blocks they fill: a block of
                 // level l when it lies inside the cut and beyond the level's radius (xc_tree.cu).
@@ -648,11 +648,13 @@ __global__ void __launch_bounds__(VT, MIX ? 2 : 3) k_vjp32(Vjp32Params p) {
                               : PROF == XC_VOIGT_GH_BINNED ? 3 + (int)ceilf(am * s_ext)
                                                            : 1;
                 const int core = PROF == XC_VOIGT_W4 ? 2 + (int)ceilf(18.05f * am) : 0;
+                // (the grid ends before 2^30: no block lies right of a line at 2^31 - 2^26 or beyond)
+                const int nar = min(na, 0x7fffffff - (1 << 26));
                 int A[TR_LEVELS], Z[TR_LEVELS];
 #pragma unroll
                 for (int l = 0; l < TR_LEVELS; ++l) {
                     const int D = max(tr_gap(l) + e, core), sh = l == 2 ? 9 : 6 + l;
-                    const int lo = lane >= 5 ? max(ka, na + D + 1) : ka, hi = lane >= 5 ? kb : min(kb, na - D - 1);
+                    const int lo = lane >= 5 ? max(ka, nar + D + 1) : ka, hi = lane >= 5 ? kb : min(kb, na - D - 1);
                     A[l] = (lo + (1 << sh) - 1) >> sh;
                     Z[l] = (hi + 1) >> sh;
                 }
