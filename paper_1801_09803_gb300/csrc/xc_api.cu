@@ -15,6 +15,7 @@
 #include <vector>
 
 #include "xc_internal.cuh"
+#include "xc_route.h"
 #include "xc_batched.cuh"
 
 #include <unistd.h>
@@ -311,7 +312,7 @@ xc_status cross_section_f64(xc_handle *h, const CondDev *dcond, const xc_conditi
     XC_TRY_MEM(h->params.ensure(n * 4 * sizeof(double)));
     // the block-interpolated form (the Vectorized Voigt is not smooth at its split: direct sum),
     // unless its 16 bytes per line do not fit next to a very large list
-    bool tree = tree64_takes(o->profile, *g, o->cutoff, n);
+    bool tree = route_blocks64(o->profile, *g, o->cutoff, n);
     if (tree && (tree64_mat(&h->batched.tree_mat64, s) != cudaSuccess ||
                  h->ranges.ensure(tree64_scratch(*g, o->cutoff, n)) != cudaSuccess)) {
         cudaGetLastError();

@@ -388,9 +388,8 @@ cudaError_t launch_gather_f64(int profile, const double *nu, const double *I, co
                               const int64_t *win_hi, int64_t n_win, double nu_A, double step, int64_t n_pts,
                               const double *ghx, const double *ghw, int ngh, double *sigma, cudaStream_t s,
                               double vv_split = 4.0, int vv_beta = 0);
-// the FP64 cross section with the far field interpolated on blocks (xc_tree64.cu): whether it
-// takes a call, the bytes of device scratch it needs, and the kernels
-bool tree64_takes(int profile, const xc_grid &g, double cutoff, size_t n);
+// the FP64 cross section with the far field interpolated on blocks (xc_tree64.cu), for the calls
+// that route_blocks64 gives it: the bytes of device scratch it needs, and the kernels
 size_t tree64_scratch(const xc_grid &g, double cutoff, size_t n);
 cudaError_t launch_tree64(int profile, const double *nu, const double *I, const double *al, const double *ga,
                           const double *cut, size_t n, double acoef, const xc_grid &g, double cutoff, bool fixed_cut,

@@ -605,11 +605,6 @@ __global__ void __launch_bounds__(128) k_t64_points_w4(T64Params q) {
 // ---------------------------------------------------------------------------
 // host side
 // ---------------------------------------------------------------------------
-bool tree64_takes(int profile, const xc_grid &g, double cutoff, size_t n) {
-    return profile != XC_VOIGT_VV && cutoff / g.step < (double)(1 << 20) && g.n < ((int64_t)1 << 30) &&
-           n < ((size_t)1 << 30);   // beyond, its scratch would crowd out other buffers of the handle
-}
-
 // bytes of scratch behind the int4 geometry of n lines
 static size_t tree64_layout(const xc_grid &g, double cutoff, size_t n, TreeParams *p, size_t *o_cell, size_t *o_nodes) {
     p->n = n;

@@ -1,0 +1,30 @@
+"""Calls at the edges of the routing rules (csrc/xc_route.h), on the device."""
+import numpy as np
+import pytest
+
+import xcsynth as xs
+from test_gpu_parity import eng, metrics, xc  # noqa: F401
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("step", [1e-5, 1e-6, 1e-8, 1e-13, 1e-30])
+def test_fp64_grids_of_fine_steps(eng, xc, oracle_lib, step):  # noqa: F811
+    """From steps the blocks take down to steps below the rounding of the wavenumber, where all points
+    coincide: 1e-12 of the oracle, as the FP64 paths elsewhere (both form nu_A + k step alike).  The
+    oracle's point by point form: its sweep finds a line's range from floor((nu -+ cut - nu_A) / step) to
+    within one point, which does not hold below the rounding."""
+    nu_A, n = 10_000.0, 1500
+    L = xs.gen_lines(309, 0, 40, 9000.0, 11000.0)
+    rng = np.random.default_rng(309)
+    L["nu"] = np.sort(np.concatenate([[nu_A], nu_A + rng.uniform(-600, 2100, 39) * step]))
+    E, g = xs.gen_states(309, 200)
+    eng.load_lines(L)
+    eng.set_states(E, g)
+    cut = 700.0 * step
+    got = eng.cross_section(xc.make_condition(300.0, 1e-9), xc.make_grid(nu_A, step, n), xc.make_opts("voigt_w4", "fp64", cut))
+    Q, dQ = oracle_lib.partition_function(E, g, 300.0)
+    ref = oracle_lib.cross_section_points(L, oracle_lib.make_condition(300.0, 1e-9, Q, dQ), nu_A, step, np.arange(n),
+                                          oracle_lib.make_opts("voigt_w4", cut), nthreads=4)
+    assert metrics(got, ref)[0] < 1e-12

@@ -1,0 +1,57 @@
+"""Which kernels a call runs on (csrc/xc_route.h), compiled for the host: the rules need sizes only."""
+import ctypes as C
+import os
+import shutil
+import subprocess
+
+import numpy as np
+import pytest
+
+ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+CSRC = os.path.join(ROOT, "paper_1801_09803_gb300", "csrc")
+W4, LORENTZ, VV = 2, 1, 7
+
+SHIM = """
+#include "xc_route.h"
+extern "C" int blocks64(int profile, double nu_A, double step, long long n_pts, double cutoff, unsigned long long n) {
+    return xc::route_blocks64(profile, xc_grid{nu_A, step, (int64_t)n_pts}, cutoff, (size_t)n);
+}
+"""
+
+
+@pytest.fixture(scope="module")
+def route(tmp_path_factory):
+    cxx = shutil.which("g++")
+    if not cxx:
+        pytest.skip("no host compiler")
+    d = tmp_path_factory.mktemp("route")
+    (d / "shim.cpp").write_text(SHIM)
+    subprocess.run([cxx, "-std=c++17", "-O1", "-fPIC", "-shared", "-I", CSRC, str(d / "shim.cpp"), "-o", str(d / "r.so")],
+                   check=True)
+    L = C.CDLL(str(d / "r.so"))
+    L.blocks64.argtypes = [C.c_int, C.c_double, C.c_double, C.c_longlong, C.c_double, C.c_ulonglong]
+    return L
+
+
+def test_fp64_blocks_take_ordinary_grids(route):
+    for nu_A, step, n in ((1000.0, 0.01, 200_001), (0.0, 0.01, 1_000_001), (20000.0, 1e-4, 1001), (-5.0, 0.01, 11)):
+        assert route.blocks64(W4, nu_A, step, n, min(25.0, 1e5 * step), 100_000)
+    assert not route.blocks64(VV, 1000.0, 0.01, 1001, 25.0, 1000)
+    assert not route.blocks64(W4, 1000.0, 0.01, 1001, 25.0, 1 << 30)
+    assert not route.blocks64(W4, 1000.0, 0.01, 1 << 30, 25.0, 1000)
+    assert not route.blocks64(W4, 1000.0, 0.01, 1001, 0.01 * 2 ** 20, 1000)
+
+
+def test_fp64_blocks_leave_steps_near_the_rounding_of_the_wavenumber(route):
+    """The first-order term that follows a point's rounding is good to 3 (r / d)^2: every grid that is
+    taken keeps it below 2.3e-16 at the nearest distance of a block, 60 steps."""
+    taken = 0
+    for nu in 10.0 ** np.arange(-2, 6):
+        for step in 10.0 ** np.arange(-30.0, 2.0):
+            r = np.spacing(nu) / 2 / step
+            if route.blocks64(W4, nu, step, 1000, 1000 * step, 1000):
+                taken += 1
+                assert 3 * (r / 60.0) ** 2 < 2.3e-16, (nu, step)
+            else:   # not a line further than it need be
+                assert r > 2.0 ** -23, (nu, step)
+    assert taken > 40
