@@ -621,8 +621,9 @@ __global__ void __launch_bounds__(VT, MIX ? 2 : 3) k_vjp32(Vjp32Params p) {
                     const CondDev cd = p.conds[cc.row];
                     const double nud = p.L.nu[l];
                     const double al = alpha_coef(cd.T, cd.mass_da) * nud;
-                    const double ga = cd.gamma_scale * (double)gref * exp(((double)nT + cd.n_shift) *
-                                                                          log(cd.T_ref / cd.T)) * (cd.P / cd.P_ref);
+                    const double ga = MIX ? mixture_gamma64(p.L, l, cd)
+                                          : cd.gamma_scale * (double)gref * exp(((double)nT + cd.n_shift) *
+                                                                                log(cd.T_ref / cd.T)) * (cd.P / cd.P_ref);
                     line_k_range(nud, fmin(p.width_mult * fmax(al, ga), p.cutoff), p.nu_A, p.step, 1.0 / p.step, p.n_pts, &k0, &k1);
                 }
                 ka = __shfl_sync(0xffffffffu, (int)k0, c);

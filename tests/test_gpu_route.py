@@ -28,3 +28,24 @@ def test_fp64_grids_of_fine_steps(eng, xc, oracle_lib, step):  # noqa: F811
     ref = oracle_lib.cross_section_points(L, oracle_lib.make_condition(300.0, 1e-9, Q, dQ), nu_A, step, np.arange(n),
                                           oracle_lib.make_opts("voigt_w4", cut), nthreads=4)
     assert metrics(got, ref)[0] < 1e-12
+
+
+@pytest.mark.parametrize("profile", ["voigt_w4", "lorentz"])
+def test_adjoint_of_width_limited_cuts_under_a_mixture(eng, xc, profile):  # noqa: F811
+    """The cut follows the mixture's width, not the list's own gamma_ref (here ten times it): FP32 adjoint
+    against the FP64 one, 1e-4 of the largest as in the other adjoint tests."""
+    L = xs.gen_lines(310, 0, 1500, 1000.0, 1060.0)
+    L["gamma_ref"] *= np.float32(10.0)
+    eng.load_lines(L)
+    eng.set_states(*xs.gen_states(310, 500))
+    eng.set_broadening([xc.make_broadener("constant", 0.7, 0.05, 0.6), xc.make_broadener("constant", 0.3, 0.09, 0.4)])
+    conds = [xc.make_condition(T, P) for T, P in ((500.0, 0.2), (900.0, 1.0), (1600.0, 3.0))]
+    n = 4001
+    w = 1e22 * np.random.default_rng(310).uniform(0.5, 1.5, (3, n))
+    grid = xc.make_grid(1010.0, 0.01, n)
+    r32, r64 = (eng.cross_section_vjp_broadening(conds, grid, xc.make_opts(profile, p, 25.0, 100.0), w, 2)
+                for p in ("fp32", "fp64"))
+    eng.set_broadening([])
+    for k in ("dT", "dP", "d_gamma_scale", "d_n_shift", "d_gamma0_broad", "d_n_broad"):
+        a, b = np.asarray(r32[k]), np.asarray(r64[k])
+        assert np.max(np.abs(a - b)) <= 1e-4 * np.max(np.abs(b)), k
