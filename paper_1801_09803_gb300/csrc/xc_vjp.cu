@@ -861,7 +861,7 @@ xc_status vjp_run(BatchedState *st, const VjpArgs &a, int64_t *launches) {
     size_t o_geo = f64 ? 0 : carve(n * 16);
     size_t o_gs = f64 ? 0 : carve(sizeof(GeomStats));
     size_t o_cp = f64 ? 0 : carve((size_t)nc * sizeof(CParam));
-    // block nodes of the far field (FP32, profiles with far wings): 28 floats per 64 points
+    // block nodes of the far field (FP32, profiles with far wings): 208 floats per 512 points
     const bool far = !f64 && a.opts.profile != XC_DOPPLER && a.grid.n < ((int64_t)1 << 30);
     const int nblk512 = far ? (int)((a.grid.n + 511) / 512) : 0;
     const size_t per_cond = (size_t)nblk512 * (128 + 64 + 16);
@@ -929,9 +929,13 @@ xc_status vjp_run(BatchedState *st, const VjpArgs &a, int64_t *launches) {
         if (far && N) {
             const double *mat = nullptr;
             VJ_TRY(tree_mat(st, &mat, s));
-            k_vjp_nodes<<<dim3(nblk512, nc), 128, 0, s>>>(g64, a.grid.n, mat, (float *)(base + o_gn), 0, nblk512 * 128,
-                                                          nblk512 * 192, (int)per_cond);
-            ++*launches;
+            constexpr int kSlice = 65535;   // conditions of a launch: the grid's y limit
+            for (int c0 = 0; c0 < nc; c0 += kSlice) {
+                k_vjp_nodes<<<dim3(nblk512, std::min(kSlice, nc - c0)), 128, 0, s>>>(
+                    g64 + (size_t)c0 * N, a.grid.n, mat, (float *)(base + o_gn) + (size_t)c0 * per_cond, 0, nblk512 * 128,
+                    nblk512 * 192, (int)per_cond);
+                ++*launches;
+            }
         }
         VJ_TRY(launch_fp32_setup(a.L, n, a.conds_dev, nc, a.grid, a.opts.cutoff, geo, gs, cp, s));
         *launches += 2;

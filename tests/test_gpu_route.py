@@ -49,3 +49,19 @@ def test_adjoint_of_width_limited_cuts_under_a_mixture(eng, xc, profile):  # noq
     for k in ("dT", "dP", "d_gamma_scale", "d_n_shift", "d_gamma0_broad", "d_n_broad"):
         a, b = np.asarray(r32[k]), np.asarray(r64[k])
         assert np.max(np.abs(a - b)) <= 1e-4 * np.max(np.abs(b)), k
+
+
+def test_adjoint_of_more_conditions_than_a_grid_dimension(eng, xc):  # noqa: F811
+    """65 536 conditions and more: each condition's gradients as in a call of its own (the FP32 sums of
+    one condition do not depend on the others: equal)."""
+    L = xs.gen_lines(311, 0, 3, 1000.0, 1001.0)
+    eng.load_lines(L)
+    eng.set_states(*xs.gen_states(311, 20))
+    nc, n = 65_600, 130
+    conds = [xc.make_condition(700.0, 0.1 + 1e-4 * i) for i in range(nc)]
+    w = torch.full((nc, n), 1e22, dtype=torch.float64, device="cuda:0")
+    grid, opts = xc.make_grid(1000.0, 0.01, n), xc.make_opts("voigt_w4", "fp32", 25.0)
+    r = eng.cross_section_vjp(conds, grid, opts, w, per_line=False)
+    for i in (0, 65_534, 65_535, 65_536, nc - 1):
+        one = eng.cross_section_vjp([conds[i]], grid, opts, w[i:i + 1], per_line=False)
+        assert float(r["dP"][i]) == float(one["dP"][0]) != 0.0 and float(r["dT"][i]) == float(one["dT"][0]), i
