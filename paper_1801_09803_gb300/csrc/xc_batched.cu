@@ -38,6 +38,7 @@
 
 #include "xc_batched.cuh"
 #include "xc_f32.cuh"
+#include "xc_route.h"
 #include "xc_tcgen05.cuh"
 
 namespace xc {
@@ -1827,38 +1828,11 @@ int grid_size(const Variant *v, int dev, int n_tiles) {
     return std::max(1, std::min(g, n_tiles));
 }
 
-// Autotune: time each candidate variant on a probe (every tile, first 4096 lines)
-// and predict the full run from the measured time per (tile line x condition);
-// the prediction includes the wave quantisation of the tile count.
-// Sparse lists on large outputs: few pairs of a line and a point for each point.  Bringing the node
-// sums to a point costs 16 FP64 operations a condition whatever the list, 118 ps a point, where
-// the tiled kernels need 0.42 ps a pair (0.16 on the tensor cores): 1e6 points, cut 2500 steps, blocks
-// against tiled: 6 conditions, 15 / 100 / 300 pairs a point 844/399, 874/613, 917/1102 us; 24
-// conditions, 15 / 300 / 1000 pairs 2942/911, 3142/1957, 3708/4656 us.  On small outputs launches
-// decide and the blocks are no slower (1e5 points, 6 conditions 188/206 us, 24: 398/376, 405/436).
-// Below 256 steps of cut most pairs are near ones, which cost the same in both.
-bool sparse(const BatchedArgs &a, int nc) {
-    if ((a.opts.profile != XC_VOIGT_W4 && a.opts.profile != XC_LORENTZ) || a.opts.cutoff / a.grid.step < 256.0) return false;
-    const double outputs = (double)a.grid.n * (double)nc;
-    const bool tc = a.allow_tc && a.opts.profile == XC_VOIGT_W4 && a.opts.width_mult <= 0.0 && nc >= 16 &&
-                    !(a.opts.flags & XC_OPT_NO_TENSOR_CORES) && a.grid.n < ((int64_t)1 << 23);
-    const double most = outputs >= 0x1p22 ? (tc ? 500.0 : 200.0) : (outputs >= 0x1p21 ? 50.0 : 0.0);
-    return 2.0 * a.opts.cutoff / a.grid.step * (double)a.n_lines < most * (double)a.grid.n;
+Route32 route_of(const BatchedArgs &a, int nc) {
+    return Route32{a.opts.profile, a.opts.flags, a.opts.cutoff, a.opts.width_mult, a.grid, a.n_lines, nc, a.allow_tc, a.tiled};
 }
 
-// Far wings of the Voigt w4 sweep on the tensor cores: many conditions (the MMA's N is
-// 32, so a handful of conditions would waste it), one fixed cut, grids of < 2^23 points.
-// The block-interpolated sweep (xc_tree.cu) evaluates a ninth of the points at long cuts and is
-// faster at every size measured: 32 conditions x 3e6 lines, cut 1000 steps 23.2 ms against 42.3,
-// 500 steps 20.2 against 35.6, 100 steps 15.7 against 30.2; 15 000 lines 0.2 against 0.9.  This
-// form stays for short cuts and small lists, where xc_last_sweep_kernels and
-// xc_count_far_evals report on it and a call takes about a millisecond either way, and where the
-// tiled kernels run because of a fixed tile shape, a sparse list or for want of memory.
-bool use_tc(const BatchedArgs &a, int nc) {
-    return a.allow_tc && a.opts.profile == XC_VOIGT_W4 && a.opts.width_mult <= 0.0 && nc >= 16 &&
-           !(a.opts.flags & XC_OPT_NO_TENSOR_CORES) && a.grid.n < ((int64_t)1 << 23) &&
-           (a.tiled || sparse(a, nc) || (a.opts.cutoff / a.grid.step < 1024.0 && a.n_lines * (size_t)nc < ((size_t)1 << 19)));
-}
+bool use_tc(const BatchedArgs &a, int nc) { return route_tc32(route_of(a, nc)); }
 
 std::string tuned_key(const BatchedState *st, const BatchedArgs &a, int nc) {
     std::string key = shape_key(a, nc);
@@ -1870,6 +1844,9 @@ std::string tuned_key(const BatchedState *st, const BatchedArgs &a, int nc) {
     return key;
 }
 
+// Autotune: time each candidate variant on a probe (every tile, first 4096 lines)
+// and predict the full run from the measured time per (tile line x condition);
+// the prediction includes the wave quantisation of the tile count.
 xc_status autotune(BatchedState *st, const BatchedArgs &a, int nc, TileCfg *out, int64_t *launches) {
     const std::string key = tuned_key(st, a, nc);
     const bool tc = use_tc(a, nc);
@@ -1985,10 +1962,11 @@ xc_status batched_run(BatchedState *st, const BatchedArgs &args, int64_t *launch
     st->tc_blk_lo = st->tc_blk_hi = nullptr;
     st->tc_n_blk = st->tc_groups = 0;
     if (a.n_lines == 0 || a.n_cond == 0 || a.grid.n == 0) return XC_OK;
-    if (!a.tiled && !sparse(a, a.n_cond) && !use_tc(a, a.n_cond) && tree_takes(a)) {
+    if (route_blocks32(route_of(a, a.n_cond))) {
         // its scratch is larger (32 to 48 bytes per line and condition held): where that does not
         // fit next to a very large list, the tiled kernels below run the call
         const xc_status ts = tree_run(st, a, launches);
+        st->no_room = ts == XC_ENOMEM ? shape_key(a, a.n_cond) : std::string();
         if (ts != XC_ENOMEM) return ts;
         a.tiled = true;
     }
@@ -2090,7 +2068,8 @@ int64_t batched_tc_mma_count(BatchedState *st) {
 
 xc_status batched_count_far(BatchedState *st, const BatchedArgs &args, int64_t *count) {
     BatchedArgs a = args;
-    a.tiled = st->force_R > 0;
+    // as the call itself runs: the last one for want of room in the tiled form, if it was this one
+    a.tiled = st->force_R > 0 || (!st->no_room.empty() && st->no_room == shape_key(a, a.n_cond));
     *count = 0;
     const int nc = a.n_cond;
     if (a.n_lines == 0 || nc == 0 || a.grid.n == 0 || !use_tc(a, nc)) return XC_OK;

@@ -163,6 +163,7 @@ struct BatchedState {
     // the last run's tensor-core work: super-block line ranges (device) and shape
     const unsigned *tc_blk_lo = nullptr, *tc_blk_hi = nullptr;
     int tc_n_blk = 0, tc_groups = 0;
+    std::string no_room;                         // call whose block-interpolated sweep found no room for its scratch
     int force_R = 0, force_CG = 0;               // fixed CUDA-core tile shape (0: autotune)
 };
 
@@ -173,8 +174,7 @@ xc_status batched_run(BatchedState *st, const BatchedArgs &a, int64_t *launches)
 cudaError_t launch_fp32_setup(const LinesDev &L, size_t n, const CondDev *conds, int nc, const xc_grid &grid,
                               double cutoff, int4 *geo, GeomStats *gs, CParam *cp, cudaStream_t s);
 xc_status vjp_run(BatchedState *st, const VjpArgs &a, int64_t *launches);
-// the block-interpolated FP32 sweep (xc_tree.cu): whether it takes a call, and the call
-bool tree_takes(const BatchedArgs &a);
+// the block-interpolated FP32 sweep (xc_tree.cu), for the calls that route_blocks32 gives it
 xc_status tree_run(BatchedState *st, const BatchedArgs &a, int64_t *launches);
 // after the stream has synchronised: XC_ETIMEOUT if the tensor-core kernel reported a
 // wait that ran out (its results are then not valid), else XC_OK

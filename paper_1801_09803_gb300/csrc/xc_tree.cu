@@ -1163,12 +1163,6 @@ constexpr size_t kMaxRecBytes = (size_t)24 << 30;   // profile constants held at
 
 }  // namespace
 
-bool tree_takes(const BatchedArgs &a) {
-    ProfFns f;
-    return fns_of(a.opts.profile, &f) && a.opts.cutoff / a.grid.step < (double)(1 << 20) && a.grid.n < ((int64_t)1 << 30) &&
-           a.n_lines < ((size_t)3 << 29);   // beyond, its scratch would crowd out other buffers of the handle
-}
-
 xc_status tree_run(BatchedState *st, const BatchedArgs &a, int64_t *launches) {
     cudaStream_t s = a.stream;
     const size_t n = a.n_lines;

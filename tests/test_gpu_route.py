@@ -65,3 +65,52 @@ def test_adjoint_of_more_conditions_than_a_grid_dimension(eng, xc):  # noqa: F81
     for i in (0, 65_534, 65_535, 65_536, nc - 1):
         one = eng.cross_section_vjp([conds[i]], grid, opts, w[i:i + 1], per_line=False)
         assert float(r["dP"][i]) == float(one["dP"][0]) != 0.0 and float(r["dT"][i]) == float(one["dT"][0]), i
+
+
+def with_room(room, f):
+    """f() with `room` bytes left free on the device."""
+    torch.cuda.synchronize()
+    torch.cuda.empty_cache()
+    fill = torch.empty(torch.cuda.mem_get_info()[0] - room, dtype=torch.uint8, device="cuda:0")
+    try:
+        return f()
+    finally:
+        del fill
+        torch.cuda.empty_cache()
+
+
+def test_less_room_than_the_blocks_want(xc):
+    """Where the constants of 14 conditions x 1e7 lines (4.5 GB) do not fit, the blocks take four
+    conditions at a time (4, 4, 4, 2), then one, and the tiled kernels run what is left no room for."""
+    n, nc = 10_000_000, 14
+    grid, opts = xc.make_grid(1000.0, 0.01, 50_001), xc.make_opts("voigt_w4", "fp32", 25.0)
+    conds = [xc.make_condition(400.0 + 150.0 * i, 0.01 * 1.6 ** i) for i in range(nc)]
+    out = torch.empty((4, nc, 50_001), dtype=torch.float64, device="cuda:0")
+    ran = []
+    for i, room in enumerate((None, 3 << 30, 1 << 30, 320 << 20)):
+        with xc.Engine(0) as e:
+            e.load_lines(xs.gen_lines_torch(312, 0, n, 990.0, 1510.0, device="cuda:0"))
+            e.set_states(*xs.gen_states(312, 500))
+            call = lambda: e.cross_section_batched(conds, grid, opts, out[i])  # noqa: E731
+            call() if room is None else with_room(room, call)
+            ran.append(e.tuning())
+    assert ["block-interpolated" in r for r in ran] == [True, True, True, False], ran
+    assert [r.split(",")[-1].split()[0] for r in ran[:3]] == ["14", "4", "1"], ran
+    for i in (1, 2, 3):
+        ref = out[0]
+        m = ref > 1e-6 * ref.amax(dim=1, keepdim=True)
+        assert float(((out[i] - ref).abs() / ref)[m].max()) < 2e-5, i
+
+
+def test_more_conditions_than_are_ordered(eng, xc):  # noqa: F811
+    """Above 1024 conditions the sweep leaves them in the caller's order: 2e-5 of FP64."""
+    eng.load_lines(xs.gen_lines(313, 0, 400, 1000.0, 1010.0))
+    eng.set_states(*xs.gen_states(313, 100))
+    conds = [xc.make_condition(300.0 + 2.0 * ((7 * i) % 1100), 0.01 + 0.001 * i) for i in range(1100)]
+    grid = xc.make_grid(1001.0, 0.01, 777)
+    got = eng.cross_section_batched(conds, grid, xc.make_opts("voigt_w4", "fp32", 25.0))
+    assert "block-interpolated" in eng.tuning()
+    for c in (0, 1, 550, 1023, 1024, 1099):
+        ref = eng.cross_section_batched([conds[c]], grid, xc.make_opts("voigt_w4", "fp64", 25.0))[0]
+        m = ref > 1e-6 * ref.max()
+        assert np.max(np.abs(got[c] - ref)[m] / ref[m]) < 2e-5, c

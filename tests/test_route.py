@@ -16,6 +16,13 @@ SHIM = """
 extern "C" int blocks64(int profile, double nu_A, double step, long long n_pts, double cutoff, unsigned long long n) {
     return xc::route_blocks64(profile, xc_grid{nu_A, step, (int64_t)n_pts}, cutoff, (size_t)n);
 }
+// 0: tiled kernels, 1: the same with far wings on the tensor cores, 2: blocks, 3: both rules at once (a fault)
+extern "C" int route32(int profile, int flags, double cutoff, double width_mult, double step, long long n_pts,
+                       unsigned long long n_lines, int n_cond, int allow_tc, int tiled) {
+    const xc::Route32 r{profile, flags, cutoff, width_mult, xc_grid{1000.0, step, (int64_t)n_pts}, (size_t)n_lines,
+                        n_cond, allow_tc != 0, tiled != 0};
+    return 2 * xc::route_blocks32(r) + xc::route_tc32(r);
+}
 """
 
 
@@ -30,7 +37,32 @@ def route(tmp_path_factory):
                    check=True)
     L = C.CDLL(str(d / "r.so"))
     L.blocks64.argtypes = [C.c_int, C.c_double, C.c_double, C.c_longlong, C.c_double, C.c_ulonglong]
+    L.route32.argtypes = [C.c_int, C.c_int, C.c_double, C.c_double, C.c_double, C.c_longlong, C.c_ulonglong, C.c_int,
+                          C.c_int, C.c_int]
     return L
+
+
+TILED, TC, BLOCKS = 0, 1, 2
+
+
+def r32(route, profile=W4, cut=2500.0, wm=0.0, n_pts=1_000_001, n=10_000_000, nc=32, flags=0, allow=1, tiled=0):
+    r = route.route32(profile, flags, cut * 0.01, wm, 0.01, n_pts, n, nc, allow, tiled)
+    assert r != 3
+    return r
+
+
+def test_what_the_blocks_do_not_take_keeps_the_tensor_cores(route):
+    """Every reason that keeps a call from the blocks leaves its far wings on the tensor cores."""
+    assert r32(route) == BLOCKS
+    for kw in (dict(n=3 << 29), dict(n=(3 << 29) + 5, cut=500.0), dict(cut=2.0 ** 20), dict(cut=2.0 ** 21, n=1000, n_pts=4001),
+               dict(tiled=1), dict(n=3000)):
+        assert r32(route, **kw) == TC, kw
+        assert r32(route, nc=15, **{**kw, "tiled": 1}) == TILED
+        assert r32(route, flags=1, **{**kw, "tiled": 1}) == TILED
+        assert r32(route, wm=500.0, **{**kw, "tiled": 1}) == TILED
+        assert r32(route, allow=0, **{**kw, "tiled": 1}) == TILED
+    assert r32(route, n_pts=1 << 30) == TILED        # the tensor-core form itself ends at 2^23 points
+    assert r32(route, profile=VV) == TILED
 
 
 def test_fp64_blocks_take_ordinary_grids(route):
