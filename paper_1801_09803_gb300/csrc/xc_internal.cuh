@@ -137,15 +137,15 @@ __device__ inline double line_strength64(double nu, double elower, double gA, co
 // Lorentz HWHM of line l under the broadener mixture (Sec. "Mixtures of broadeners"):
 // gamma_scale P/P_ref sum_i rho_i gamma_0,i (T_ref/T)^(n_i + n_shift), each term Eq. (e:gamma_L);
 // lnTr = ln(T_ref/T) and pscale = gamma_scale P/P_ref from the caller
-__device__ inline double mixture_gamma64(const LinesDev &L, size_t l, const CondDev &c, double lnTr, double pscale) {
+__device__ inline double mixture_gamma64(const LinesDev &L, size_t l, double n_shift, double lnTr, double pscale) {
     double g = 0.0;
     for (int i = 0; i < L.n_broad; ++i)
-        g += L.bgam[(size_t)i * L.bstride + l] * exp64((L.bn[(size_t)i * L.bstride + l] + c.n_shift) * lnTr);
+        g += L.bgam[(size_t)i * L.bstride + l] * exp64((L.bn[(size_t)i * L.bstride + l] + n_shift) * lnTr);
     return pscale * g;
 }
 
 __device__ inline double mixture_gamma64(const LinesDev &L, size_t l, const CondDev &c) {
-    return mixture_gamma64(L, l, c, log(c.T_ref / c.T), c.gamma_scale * (c.P / c.P_ref));
+    return mixture_gamma64(L, l, c.n_shift, log(c.T_ref / c.T), c.gamma_scale * (c.P / c.P_ref));
 }
 
 // Integer grid positions of lines are held in 32 bits and clamped to this range.  The FP32 paths

@@ -124,7 +124,7 @@ __global__ void __launch_bounds__(256) k_line_params64(LinesDev L, size_t n, con
         double nu = L.nu[l];
         double Il = line_strength64(nu, f2d(L.elower[l]), f2d((float)L.g_up[l]) * f2d(L.A[l]), pre, sel);
         double al = acoef * nu;
-        double ga = L.n_broad > 0 ? mixture_gamma64(L, l, c, lnTr, pscale)
+        double ga = L.n_broad > 0 ? mixture_gamma64(L, l, c.n_shift, lnTr, pscale)
                                   : pscale * f2d(L.gamma_ref[l]) * exp64((f2d(L.n_T[l]) + c.n_shift) * lnTr);
         double cl = line_cut(cut_mode, cutoff, width_mult, al, ga);
         if (Il < 0.0) {   // left out by the intensity threshold: no grid point is within a negative cut
@@ -232,7 +232,7 @@ __global__ void __launch_bounds__(256) k_line_gamma(LinesDev L, size_t n, const 
         const double lnTr = sc[c & 31][0], pscale = sc[c & 31][1];
         float m = 0.f;
         for (size_t l = (size_t)blockIdx.x * blockDim.x + threadIdx.x; l < n; l += (size_t)gridDim.x * blockDim.x) {
-            const float g = (float)mixture_gamma64(L, l, cd, lnTr, pscale);
+            const float g = (float)mixture_gamma64(L, l, cd.n_shift, lnTr, pscale);
             gamma_lc[l * (size_t)nc + c] = g;
             m = fmaxf(m, g);
         }

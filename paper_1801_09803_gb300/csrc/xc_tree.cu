@@ -108,7 +108,7 @@ __global__ void __launch_bounds__(256) k_tree_geom(LinesDev L, size_t n, double 
         const float gr = L.gamma_ref[l], nT = L.n_T[l];
         double cut = cutoff;
         if (width_mult > 0.0) {
-            const double ga = L.n_broad > 0 ? mixture_gamma64(L, l, c, lnTr, c.gamma_scale * gsc)
+            const double ga = L.n_broad > 0 ? mixture_gamma64(L, l, c.n_shift, lnTr, c.gamma_scale * gsc)
                                             : c.gamma_scale * f2d(gr) * exp64((f2d(nT) + c.n_shift) * lnTr) * gsc;
             cut = fmin(width_mult * fmax(ac * nu, ga), cutoff);
         }

@@ -479,7 +479,7 @@ struct Vjp32Params {
     const CParam *cp;                     // this launch's conditions, rows = caller index
     const CondDev *conds;                 // all conditions, caller order
     int nc;                               // conditions in this launch (<= 32)
-    double nu_A, step, cutoff, width_mult;
+    double nu_A, step, inv_step, cutoff, width_mult;
     int64_t n_pts;
     const float *g32;                     // dL/dsigma, [caller row][n_pts]
     double *block_part;                   // [block][nc][4 + 2 nb]
@@ -530,7 +530,8 @@ __global__ void __launch_bounds__(128) k_vjp_nodes(const double *__restrict__ g,
 // (T_ref/T)^(n_i + n_shift), and the adjoint also sums, per broadener, the gradients of a
 // scale on its gamma_0 values (d gamma = gamma_i) and of a shift of its n values
 // (d gamma = gamma_i ln(T_ref/T))
-template <int PROF, bool MIX>
+// WL: width-limited cuts (their code costs the fixed cut's kernel registers that it does not have)
+template <int PROF, bool MIX, bool WL>
 __global__ void __launch_bounds__(VT, MIX ? 2 : 3) k_vjp32(Vjp32Params p) {
     __shared__ double s_part[VW][VMAXC][4];
     __shared__ double s_broad[VW][VMAXC][MIX ? 2 * VMAXB : 1];
@@ -558,15 +559,28 @@ __global__ void __launch_bounds__(VT, MIX ? 2 : 3) k_vjp32(Vjp32Params p) {
     // this lane's condition: FP32 constants, and FP64 accumulators of its four scalars
     const bool mine = lane < nc;
     const CParam cc = p.cp[mine ? lane : 0];
+    // width-limited cuts: FP64 constants of the conditions, formed once (formed for every line from the
+    // condition, their logarithm, root and divisions were most of the kernel at short cuts: 1e6 points,
+    // 3e5 lines, 1 condition, 3.1 ms)
+    __shared__ int2 s_wk[WL ? VW : 1][VMAXC];    // cut ranges of the warp's line
+    __shared__ double s_wl[WL ? VMAXC : 1][5];   // alpha / nu, ln(T_ref/T), gamma_scale, P/P_ref, n_shift
     float invT, dQQ, lnTr, fP, fS;
     {
         const CondDev cd = p.conds[cc.row];
+        if (WL && warp == 0 && mine) {
+            s_wl[lane][0] = alpha_coef(cd.T, cd.mass_da);
+            s_wl[lane][1] = log(cd.T_ref / cd.T);
+            s_wl[lane][2] = cd.gamma_scale;
+            s_wl[lane][3] = cd.P / cd.P_ref;
+            s_wl[lane][4] = cd.n_shift;
+        }
         invT = (float)(1.0 / cd.T);
         dQQ = (float)(cd.dQdT / cd.Q);
         lnTr = (float)log(cd.T_ref / cd.T);
         fP = (float)(cd.gamma_scale / cd.P_ref);     // d(gamma_scale P/P_ref)/dP
         fS = (float)(cd.P / cd.P_ref);               // d(gamma_scale P/P_ref)/d(gamma_scale)
     }
+    if (WL) __syncthreads();
     double accT = 0.0, accP = 0.0, accS = 0.0, accN = 0.0;
     for (size_t l = (size_t)blockIdx.x * VW + warp; l < p.n; l += (size_t)gridDim.x * VW) {
         const float nu = (float)p.L.nu[l];
@@ -610,24 +624,24 @@ __global__ void __launch_bounds__(VT, MIX ? 2 : 3) k_vjp32(Vjp32Params p) {
         const int na = geo.x;
         const float ff = __int_as_float(geo.w);
         int ka = geo.y, kb = geo.z;
+        // lane c: the cut min(cutoff, width_mult max(alpha, gamma)) of its condition, FP64 as in the
+        // forward kernels' geometry
+        if (WL) __syncwarp();   // the last line's ranges are no longer read
+        if (WL && mine) {
+            const double nud = p.L.nu[l], al = s_wl[lane][0] * nud, ns = s_wl[lane][4], lr = s_wl[lane][1];
+            const double ga = MIX ? mixture_gamma64(p.L, l, ns, lr, s_wl[lane][2] * s_wl[lane][3])
+                                  : s_wl[lane][2] * f2d(gref) * exp64((f2d(nT) + ns) * lr) * s_wl[lane][3];
+            int64_t k0, k1;
+            line_k_range(nud, fmin(p.width_mult * fmax(al, ga), p.cutoff), p.nu_A, p.step, p.inv_step, p.n_pts, &k0, &k1);
+            s_wk[warp][lane] = make_int2((int)k0, (int)k1);
+        }
+        if (WL) __syncwarp();
         float SIm = 0.f, Sam = 0.f, Sgm = 0.f;   // lane c: its condition's three sums
         for (int c = 0; c < nc; ++c) {
             const float a_h = __shfl_sync(0xffffffffu, ah, c), g_h = __shfl_sync(0xffffffffu, gh, c);
-            if (p.width_mult > 0.0) {
-                // per-(line, condition) cut min(cutoff, width_mult max(alpha, gamma)), FP64 as in
-                // the forward kernels' geometry
-                int64_t k0 = 1, k1 = 0;
-                if (lane == c) {
-                    const CondDev cd = p.conds[cc.row];
-                    const double nud = p.L.nu[l];
-                    const double al = alpha_coef(cd.T, cd.mass_da) * nud;
-                    const double ga = MIX ? mixture_gamma64(p.L, l, cd)
-                                          : cd.gamma_scale * (double)gref * exp(((double)nT + cd.n_shift) *
-                                                                                log(cd.T_ref / cd.T)) * (cd.P / cd.P_ref);
-                    line_k_range(nud, fmin(p.width_mult * fmax(al, ga), p.cutoff), p.nu_A, p.step, 1.0 / p.step, p.n_pts, &k0, &k1);
-                }
-                ka = __shfl_sync(0xffffffffu, (int)k0, c);
-                kb = __shfl_sync(0xffffffffu, (int)k1, c);
+            if (WL) {
+                ka = s_wk[warp][c].x;
+                kb = s_wk[warp][c].y;
             }
             const float *gc = p.g32 + (size_t)__shfl_sync(0xffffffffu, cc.row, c) * (size_t)p.n_pts;
             KahanF K0, K1, K2, B0, B1, B2;
@@ -649,13 +663,11 @@ __global__ void __launch_bounds__(VT, MIX ? 2 : 3) k_vjp32(Vjp32Params p) {
                               : PROF == XC_VOIGT_GH_BINNED ? 3 + (int)ceilf(am * s_ext)
                                                            : 1;
                 const int core = PROF == XC_VOIGT_W4 ? 2 + (int)ceilf(18.05f * am) : 0;
-                // (the grid ends before 2^30: no block lies right of a line at 2^31 - 2^26 or beyond)
-                const int nar = min(na, 0x7fffffff - (1 << 26));
                 int A[TR_LEVELS], Z[TR_LEVELS];
 #pragma unroll
                 for (int l = 0; l < TR_LEVELS; ++l) {
                     const int D = max(tr_gap(l) + e, core), sh = l == 2 ? 9 : 6 + l;
-                    const int lo = lane >= 5 ? max(ka, nar + D + 1) : ka, hi = lane >= 5 ? kb : min(kb, na - D - 1);
+                    const int lo = lane >= 5 ? max(ka, na + D + 1) : ka, hi = lane >= 5 ? kb : min(kb, na - D - 1);
                     A[l] = (lo + (1 << sh) - 1) >> sh;
                     Z[l] = (hi + 1) >> sh;
                 }
@@ -838,6 +850,14 @@ static VjpFn pick(int prof) {
         }                                                                                       \
     } while (0)
 
+template <int PROF>
+static void launch_vjp32(bool mix, bool wl, int blocks, cudaStream_t s, const Vjp32Params &p) {
+    if (mix && wl) k_vjp32<PROF, true, true><<<blocks, VT, 0, s>>>(p);
+    else if (mix) k_vjp32<PROF, true, false><<<blocks, VT, 0, s>>>(p);
+    else if (wl) k_vjp32<PROF, false, true><<<blocks, VT, 0, s>>>(p);
+    else k_vjp32<PROF, false, false><<<blocks, VT, 0, s>>>(p);
+}
+
 xc_status vjp_run(BatchedState *st, const VjpArgs &a, int64_t *launches) {
     cudaStream_t s = a.stream;
     const int nc = a.n_cond;
@@ -861,8 +881,10 @@ xc_status vjp_run(BatchedState *st, const VjpArgs &a, int64_t *launches) {
     size_t o_geo = f64 ? 0 : carve(n * 16);
     size_t o_gs = f64 ? 0 : carve(sizeof(GeomStats));
     size_t o_cp = f64 ? 0 : carve((size_t)nc * sizeof(CParam));
-    // block nodes of the far field (FP32, profiles with far wings): 208 floats per 512 points
-    const bool far = !f64 && a.opts.profile != XC_DOPPLER && a.grid.n < ((int64_t)1 << 30);
+    // block nodes of the far field (FP32, profiles with far wings): 208 floats per 512 points.  Points
+    // and cuts as for the sweep's blocks: a line whose position is near 2^31 then reaches no point.
+    const bool far = !f64 && a.opts.profile != XC_DOPPLER && a.grid.n < ((int64_t)1 << 30) &&
+                     a.opts.cutoff / a.grid.step < 0x1p20;
     const int nblk512 = far ? (int)((a.grid.n + 511) / 512) : 0;
     const size_t per_cond = (size_t)nblk512 * (128 + 64 + 16);
     size_t o_gn = far ? carve((size_t)nc * per_cond * 4) : 0;
@@ -949,6 +971,7 @@ xc_status vjp_run(BatchedState *st, const VjpArgs &a, int64_t *launches) {
             vp.nc = std::min(VMAXC, nc - c0);
             vp.nu_A = a.grid.nu_A;
             vp.step = a.grid.step;
+            vp.inv_step = 1.0 / a.grid.step;
             vp.cutoff = a.opts.cutoff;
             vp.width_mult = a.opts.width_mult;
             vp.n_pts = a.grid.n;
@@ -966,23 +989,12 @@ xc_status vjp_run(BatchedState *st, const VjpArgs &a, int64_t *launches) {
             vp.node_off[2] = nblk512 * 192;
             vp.nodes_per_cond = (int)per_cond;
             const bool mix = nb > 0;
+            const bool wl = a.opts.width_mult > 0.0;
             switch (a.opts.profile) {
-            case XC_DOPPLER:
-                if (mix) k_vjp32<XC_DOPPLER, true><<<blocks, VT, 0, s>>>(vp);
-                else k_vjp32<XC_DOPPLER, false><<<blocks, VT, 0, s>>>(vp);
-                break;
-            case XC_LORENTZ:
-                if (mix) k_vjp32<XC_LORENTZ, true><<<blocks, VT, 0, s>>>(vp);
-                else k_vjp32<XC_LORENTZ, false><<<blocks, VT, 0, s>>>(vp);
-                break;
-            case XC_VOIGT_GH_BINNED:
-                if (mix) k_vjp32<XC_VOIGT_GH_BINNED, true><<<blocks, VT, 0, s>>>(vp);
-                else k_vjp32<XC_VOIGT_GH_BINNED, false><<<blocks, VT, 0, s>>>(vp);
-                break;
-            default:
-                if (mix) k_vjp32<XC_VOIGT_W4, true><<<blocks, VT, 0, s>>>(vp);
-                else k_vjp32<XC_VOIGT_W4, false><<<blocks, VT, 0, s>>>(vp);
-                break;
+            case XC_DOPPLER: launch_vjp32<XC_DOPPLER>(mix, wl, blocks, s, vp); break;
+            case XC_LORENTZ: launch_vjp32<XC_LORENTZ>(mix, wl, blocks, s, vp); break;
+            case XC_VOIGT_GH_BINNED: launch_vjp32<XC_VOIGT_GH_BINNED>(mix, wl, blocks, s, vp); break;
+            default: launch_vjp32<XC_VOIGT_W4>(mix, wl, blocks, s, vp); break;
             }
             k_vjp_finish<<<(vp.nc * NQ + 3) / 4, 128, 0, s>>>(bp, blocks, vp.nc, NQ, 0, cp + c0, dT, dP, acc);
             *launches += 2;
