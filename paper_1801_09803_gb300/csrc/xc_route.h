@@ -23,11 +23,27 @@ inline bool route_blocks64(int profile, const xc_grid &g, double cutoff, size_t 
            top < g.step * 0x1p32 && cutoff < 1e15;
 }
 
+// A call's cut in grid steps.  Under width-limited cuts the device alone knows them: here that of a
+// line in the middle of the grid with a Lorentz width of 0.07 cm^-1/bar, mean over the conditions --
+// only for the choice between kernels that give the same result.
+inline double route_cut_steps(double cutoff, double width_mult, const xc_grid &g, const xc_condition *c, int n) {
+    if (!(width_mult > 0.0) || !c || n <= 0) return cutoff / g.step;
+    const double nu = fmax(g.nu_A + 0.5 * g.step * (double)g.n, 0.0);
+    double sum = 0.0;
+    for (int i = 0; i < n; ++i) {
+        const double al = 3.581e-7 * nu * sqrt(c[i].T / c[i].mass_da);
+        const double ga = 0.07 * c[i].gamma_scale * (c[i].P / c[i].P_ref) * pow(c[i].T_ref / c[i].T, 0.6);
+        sum += fmin(cutoff, width_mult * fmax(al, ga));
+    }
+    return sum / n / g.step;
+}
+
 // ---- FP32: the block-interpolated sweep (xc_tree.cu), or the tiled kernels with or without the far
 // wings on the tensor cores (xc_batched.cu)
 struct Route32 {
-    int profile, flags;
+    int profile, flags, n_gh;
     double cutoff, width_mult;
+    double cut_steps;   // route_cut_steps
     xc_grid grid;
     size_t n_lines;
     int n_cond;
@@ -35,18 +51,32 @@ struct Route32 {
     bool tiled;      // the tiled kernels whatever the sizes (fixed tile shape, no room for the blocks' scratch)
 };
 
-// Sparse lists on large outputs: few pairs of a line and a point for each point.  Bringing the node
-// sums to a point costs 16 FP64 operations a condition whatever the list, 118 ps a point, where
-// the tiled kernels need 0.42 ps a pair (0.16 on the tensor cores): 1e6 points, cut 2500 steps, blocks
-// against tiled: 6 conditions, 15 / 100 / 300 pairs a point 844/399, 874/613, 917/1102 us; 24
-// conditions, 15 / 300 / 1000 pairs 2942/911, 3142/1957, 3708/4656 us.  On small outputs launches
-// decide and the blocks are no slower (1e5 points, 6 conditions 188/206 us, 24: 398/376, 405/436).
-// Below 256 steps of cut most pairs are near ones, which cost the same in both.
+// Sparse lists on large outputs.  Bringing the node sums to a point costs the blocks 16 FP64 operations a
+// condition whatever the list; the tiled kernels pay for every pair of a line and a point.  Both were
+// timed over 1e5 and 1e6 points x 0.003 to 0.3 lines a point x cuts of 50 to 2500 steps x 1 to 24
+// conditions x fixed and width-limited cuts, and follow
+//     base + a (points x conditions) + b (lines x conditions) + c (pairs)
+// within 10 % (blocks) and 15 to 50 % (tiled, worst where the autotuner picks a slow tile).  Blocks
+// against tiled, ps: a 110-133 / 4-22 (w4 with one condition 127 / 119: a launch for its centre zones),
+// b 24-200 / 70-1260, c 0.02-0.06 / 0.1-3 (20 Gauss-Hermite nodes 0.5-0.9 / 5-23).  The lines below are the
+// differences.  At 1e6 points, 6 conditions, blocks / tiled us: Lorentz 15 pairs a point 886 / 219, 150
+// 930 / 390, 1500 (0.3 lines) 1230 / 2500; w4 15 876 / 461, 150 883 / 685, 1500 1360 / 3900; binned
+// Lorentz 15 871 / 400, 150 880 / 1330.  The Doppler profiles have nothing to bring to the points.
 inline bool route_sparse32(const Route32 &r, bool tc) {
-    if ((r.profile != XC_VOIGT_W4 && r.profile != XC_LORENTZ) || r.cutoff / r.grid.step < 256.0) return false;
-    const double outputs = (double)r.grid.n * (double)r.n_cond;
-    const double most = outputs >= 0x1p22 ? (tc ? 500.0 : 200.0) : (outputs >= 0x1p21 ? 50.0 : 0.0);
-    return 2.0 * r.cutoff / r.grid.step * (double)r.n_lines < most * (double)r.grid.n;
+    const bool wl = r.width_mult > 0.0;               // width-limited: one pass for each condition
+    const double nc = wl ? 1.0 : (double)r.n_cond, gh = r.n_gh / 20.0;
+    double point, line, pair;                         // ps: cost of the blocks, saved by them
+    switch (r.profile) {
+    case XC_VOIGT_W4: point = 100.0 - 92.0 / nc; line = 350.0 + 700.0 / nc; pair = tc ? 0.08 : 0.3; break;
+    case XC_LORENTZ: point = nc > 1.0 ? 125.0 : 104.0; line = 70.0 + 150.0 / nc; pair = nc >= 16.0 ? 0.12 : 0.2; break;
+    case XC_LORENTZ_BINNED: point = 115.0; line = 250.0; pair = 1.5; break;
+    case XC_VOIGT_GH_BINNED: point = 92.0; line = -700.0 * gh; pair = 17.0 * gh; break;
+    case XC_VOIGT_GH_SAMPLED: point = 105.0; line = -130.0 * gh; pair = 5.0 * gh; break;
+    default: return false;
+    }
+    const double base = wl ? 23e6 * r.n_cond : 25e6 + 5e6 * fmin(nc, 24.0);   // shorter launch sequences
+    return base - point * (double)r.grid.n * r.n_cond +
+               (line + pair * 2.0 * r.cut_steps) * (double)r.n_lines * r.n_cond < 0.0;
 }
 
 // Whether the tensor-core kernel can take the far wings of a tiled call: many conditions (the

@@ -114,3 +114,24 @@ def test_more_conditions_than_are_ordered(eng, xc):  # noqa: F811
         ref = eng.cross_section_batched([conds[c]], grid, xc.make_opts("voigt_w4", "fp64", 25.0))[0]
         m = ref > 1e-6 * ref.max()
         assert np.max(np.abs(got[c] - ref)[m] / ref[m]) < 2e-5, c
+
+
+@pytest.mark.parametrize("profile,sparse,dense", [("lorentz", 20_000, 500_000), ("lorentz_binned", 10_000, 200_000),
+                                                  ("voigt_gh_sampled", 2_000, 100_000), ("voigt_w4", 10_000, 400_000)])
+def test_sparse_and_dense_lists_run_their_own_kernels(eng, xc, profile, sparse, dense):  # noqa: F811
+    """Either side of the rule for sparse lists, and both against the general path (a fixed tile shape),
+    2e-5 as between any two FP32 paths.  (FP32 itself is 2.0e-5 from FP64 here: a Lorentz width of 0.07 steps
+    at the sampled Gauss-Hermite nodes, blocks and tiled kernels alike.)"""
+    grid = xc.make_grid(1000.0, 0.01, 500_003)
+    conds = [xc.make_condition(400.0 + 90.0 * i, 0.01 * 1.9 ** i) for i in range(6)]
+    opts = xc.make_opts(profile, "fp32", 5.0)
+    eng.set_states(*xs.gen_states(314, 500))
+    for n, blocks in ((sparse, False), (dense, True)):
+        eng.load_lines(xs.gen_lines(314, 0, n, 995.0, 6005.0))
+        got = eng.cross_section_batched(conds, grid, opts)
+        assert ("block-interpolated" in eng.tuning()) == blocks, (profile, n, eng.tuning())
+        eng.set_tile_shape(8, 1)
+        ref = eng.cross_section_batched(conds, grid, opts)
+        eng.set_tile_shape(0, 0)
+        m = ref > 1e-6 * ref.max(axis=1, keepdims=True)
+        assert np.max(np.abs(got - ref)[m] / ref[m]) < 2e-5, (profile, n)

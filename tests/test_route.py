@@ -9,7 +9,7 @@ import pytest
 
 ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
 CSRC = os.path.join(ROOT, "paper_1801_09803_gb300", "csrc")
-W4, LORENTZ, VV = 2, 1, 7
+DOPPLER, LORENTZ, W4, GH_BINNED, GH_SAMPLED, DOPPLER_BINNED, LORENTZ_BINNED, VV = range(8)
 
 SHIM = """
 #include "xc_route.h"
@@ -19,8 +19,11 @@ extern "C" int blocks64(int profile, double nu_A, double step, long long n_pts, 
 // 0: tiled kernels, 1: the same with far wings on the tensor cores, 2: blocks, 3: both rules at once (a fault)
 extern "C" int route32(int profile, int flags, double cutoff, double width_mult, double step, long long n_pts,
                        unsigned long long n_lines, int n_cond, int allow_tc, int tiled) {
-    const xc::Route32 r{profile, flags, cutoff, width_mult, xc_grid{1000.0, step, (int64_t)n_pts}, (size_t)n_lines,
-                        n_cond, allow_tc != 0, tiled != 0};
+    const xc_grid g{1000.0, step, (int64_t)n_pts};
+    xc_condition c{};
+    c.T = 1000.0, c.P = 0.1, c.mass_da = 18.0, c.T_ref = 296.0, c.P_ref = 1.0, c.gamma_scale = 1.0;
+    const xc::Route32 r{profile, flags, 20, cutoff, width_mult, xc::route_cut_steps(cutoff, width_mult, g, &c, 1), g,
+                        (size_t)n_lines, n_cond, allow_tc != 0, tiled != 0};
     return 2 * xc::route_blocks32(r) + xc::route_tc32(r);
 }
 """
@@ -87,3 +90,49 @@ def test_fp64_blocks_leave_steps_near_the_rounding_of_the_wavenumber(route):
             else:   # not a line further than it need be
                 assert r > 2.0 ** -23, (nu, step)
     assert taken > 40
+
+
+# measured on both sides of the rule (us, blocks and tiled): the faster form is the one chosen
+MEASURED = [
+    # profile, points, lines a point, cut (steps), width multiple, conditions, blocks, tiled
+    (LORENTZ, 1000001, 0.003, 2500, 0, 12, 1696.4, 300.4),
+    (LORENTZ, 1000001, 0.3, 256, 0, 6, 1001.1, 691.5),
+    (LORENTZ, 1000001, 0.003, 256, 0, 2, 344.9, 142.7),
+    (LORENTZ, 100001, 0.3, 256, 500, 12, 855.6, 1361.1),
+    (LORENTZ, 1000001, 0.3, 2500, 0, 12, 2182.7, 4294.7),
+    (LORENTZ, 100001, 0.3, 2500, 500, 1, 127.1, 189.4),
+    (W4, 1000001, 0.03, 2500, 0, 12, 1568.3, 1106.8),
+    (W4, 1000001, 0.03, 50, 0, 6, 853.9, 423.1),
+    (W4, 1000001, 0.03, 50, 0, 4, 573.9, 349.2),
+    (W4, 100001, 0.03, 256, 500, 1, 105.3, 152.3),
+    (W4, 100001, 0.003, 256, 500, 4, 283, 421.9),
+    (W4, 1000001, 0.3, 256, 500, 2, 656, 1425.5),
+    (GH_BINNED, 1000001, 0.003, 50, 0, 6, 864.1, 357.1),
+    (GH_BINNED, 1000001, 0.003, 50, 0, 1, 208.3, 147.6),
+    (GH_BINNED, 1000001, 0.003, 256, 0, 6, 869.7, 481),
+    (GH_BINNED, 1000001, 0.03, 2500, 500, 1, 263.4, 944.9),
+    (GH_BINNED, 1000001, 0.3, 256, 500, 1, 1055, 3129.9),
+    (GH_BINNED, 1000001, 0.03, 256, 0, 1, 243.8, 477.7),
+    (GH_SAMPLED, 1000001, 0.003, 256, 500, 6, 1071.2, 726.4),
+    (GH_SAMPLED, 1000001, 0.003, 50, 0, 6, 860.3, 250.5),
+    (GH_SAMPLED, 1000001, 0.03, 50, 0, 6, 871, 460),
+    (GH_SAMPLED, 100001, 0.03, 2500, 0, 1, 108.8, 498.9),
+    (GH_SAMPLED, 1000001, 0.03, 2500, 0, 1, 265.2, 982.5),
+    (GH_SAMPLED, 100001, 0.3, 256, 500, 1, 160.3, 434.9),
+    (DOPPLER_BINNED, 1000001, 0.03, 2500, 0, 6, 168.1, 3163.1),
+    (DOPPLER_BINNED, 100001, 0.003, 50, 0, 1, 70, 95.9),
+    (DOPPLER_BINNED, 1000001, 0.03, 256, 0, 1, 84.6, 205.2),
+    (LORENTZ_BINNED, 1000001, 0.003, 50, 0, 2, 334.2, 148.7),
+    (LORENTZ_BINNED, 1000001, 0.003, 256, 0, 2, 339.3, 150),
+    (LORENTZ_BINNED, 1000001, 0.03, 256, 0, 4, 604.3, 279.7),
+    (LORENTZ_BINNED, 100001, 0.03, 2500, 0, 2, 112.4, 520.9),
+    (LORENTZ_BINNED, 100001, 0.3, 2500, 500, 6, 545.1, 1304.7),
+    (LORENTZ_BINNED, 100001, 0.03, 256, 500, 24, 1446.2, 1968.3),
+]
+
+
+@pytest.mark.parametrize("row", MEASURED)
+def test_sparse_lists_run_the_faster_form(route, row):
+    profile, n_pts, density, cut, wm, nc, blocks, tiled = row
+    got = r32(route, profile=profile, cut=cut, wm=wm, n_pts=n_pts, n=max(2, int(n_pts * density)), nc=nc)
+    assert (got == BLOCKS) == (blocks < tiled), (got, row)
