@@ -101,6 +101,26 @@ inline bool route_blocks32(const Route32 &r) {
            !(tc && cut < 1024.0 && r.n_lines * (size_t)r.n_cond < ((size_t)1 << 19));
 }
 
+// The FP32 adjoint (xc_vjp.cu): dL/dsigma projected on the block nodes costs 75 ps a point and condition
+// and then saves evaluations of each line's far points.  Timed over the same family: blocks against all
+// points, ps a pair 0.2-0.3 / 0.6 (Lorentz), 2.4 (w4), 24 (20 Gauss-Hermite nodes), and for each line 200, 400
+// and 3000 to 5000 more.  1e6 points, 6 conditions, blocks / points us: w4 15 pairs a point 774 / 624, 150
+// 1178 / 2684; Lorentz 15 758 / 349, 150 1003 / 866, width-limited (500 widths) 15 758 / 309.
+// Points and cuts as for the sweep: a line whose position is near 2^31 then reaches no point.
+inline bool route_adjoint_blocks(int profile, int n_gh, double cutoff, double cut_steps, const xc_grid &g,
+                                 size_t n_lines, int n_cond) {
+    if (profile == XC_DOPPLER || g.n >= ((int64_t)1 << 30) || !(cutoff / g.step < 0x1p20)) return false;
+    double line, pair;   // ps
+    switch (profile) {
+    case XC_LORENTZ: line = 220.0; pair = 0.35; break;
+    case XC_VOIGT_GH_BINNED: line = 250.0 * n_gh; pair = 1.03 * n_gh; break;
+    default: line = 400.0; pair = 2.4; break;
+    }
+    // a warp takes a line through all conditions: below 2000 lines the chip is not full, and the last
+    // line's time is all there is
+    return (pair * 2.0 * cut_steps - line) * fmax((double)n_lines, 2000.0) * n_cond > 1e7 + 75.0 * (double)g.n * n_cond;
+}
+
 // Whatever keeps a call from the blocks, its far wings go to the tensor cores where they can
 inline bool route_tc32(const Route32 &r) { return route_tc_form(r) && !route_blocks32(r); }
 

@@ -44,6 +44,7 @@
 #include <algorithm>
 
 #include "xc_batched.cuh"
+#include "xc_route.h"
 #include "xc_tree.cuh"
 
 namespace xc {
@@ -531,8 +532,10 @@ __global__ void __launch_bounds__(128) k_vjp_nodes(const double *__restrict__ g,
 // scale on its gamma_0 values (d gamma = gamma_i) and of a shift of its n values
 // (d gamma = gamma_i ln(T_ref/T))
 // WL: width-limited cuts (their code costs the fixed cut's kernel registers that it does not have)
-template <int PROF, bool MIX, bool WL>
-__global__ void __launch_bounds__(VT, MIX ? 2 : 3) k_vjp32(Vjp32Params p) {
+// FAR: far points by the block nodes.  Without it (sparse lists, see route_adjoint_blocks) the points of
+// a line are all there is, eight of a lane's in flight at a time.
+template <int PROF, bool MIX, bool WL, bool FAR>
+__global__ void __launch_bounds__(VT, MIX || !FAR ? 2 : 3) k_vjp32(Vjp32Params p) {
     __shared__ double s_part[VW][VMAXC][4];
     __shared__ double s_broad[VW][VMAXC][MIX ? 2 * VMAXB : 1];
     __shared__ float s_gx[PROF == XC_VOIGT_GH_BINNED ? 64 : 1], s_gw[PROF == XC_VOIGT_GH_BINNED ? 64 : 1];
@@ -560,8 +563,8 @@ __global__ void __launch_bounds__(VT, MIX ? 2 : 3) k_vjp32(Vjp32Params p) {
     const bool mine = lane < nc;
     const CParam cc = p.cp[mine ? lane : 0];
     // width-limited cuts: FP64 constants of the conditions, formed once (formed for every line from the
-    // condition, their logarithm, root and divisions were most of the kernel at short cuts: 1e6 points,
-    // 3e5 lines, 1 condition, 3.1 ms)
+    // condition, their logarithm, root and divisions were most of the kernel at short cuts: Lorentz, 1e6
+    // points, 3e5 lines, 1 condition, 500 widths: 3.07 ms, 1.71 now)
     __shared__ int2 s_wk[WL ? VW : 1][VMAXC];    // cut ranges of the warp's line
     __shared__ double s_wl[WL ? VMAXC : 1][5];   // alpha / nu, ln(T_ref/T), gamma_scale, P/P_ref, n_shift
     float invT, dQQ, lnTr, fP, fS;
@@ -652,7 +655,7 @@ __global__ void __launch_bounds__(VT, MIX ? 2 : 3) k_vjp32(Vjp32Params p) {
                 const int r = (int)fminf(ceilf(11.3f * a_h) + 2.f, 1e9f);
                 k0 = max(k0, na - r);
                 k1 = (int)i64min(k1, (int64_t)na + r);
-            } else if (p.gnode) {
+            } else if (FAR) {
                 // The far points on both sides by the nodes of the blocks they fill: a block of
                 // level l when it lies inside the cut and beyond the level's radius (xc_tree.cu).
                 // Lane 5 s + q (s: side) finds segment q of that side: level 0 outside and inside
@@ -707,20 +710,24 @@ __global__ void __launch_bounds__(VT, MIX ? 2 : 3) k_vjp32(Vjp32Params p) {
                 if (hl) k0 = l1;
                 if (hr) k1 = r0 - 1;
             }
+            constexpr int U = FAR || PROF == XC_DOPPLER ? 1 : (PROF == XC_VOIGT_GH_BINNED ? 2 : 8);
             for (int k8 = k0 + lane; k8 <= k1; k8 += 32 * 8) {
                 float q0 = 0.f, q1 = 0.f, q2 = 0.f;
-#pragma unroll 1
+#pragma unroll U
                 for (int j = 0; j < 8; ++j) {
                     const int k = k8 + 32 * j;
-                    if (k > k1) break;
-                    const float d = (float)(k - na) - ff, gk = gc[k];
-                    if (PROF != XC_VOIGT_W4 || d * d >= ln_c.thr2) {
-                        ln_c.add(d, gk, q0, q1, q2);
-                    } else {
-                        const float3 r = w4_band_f32(ln_c.asc * fabsf(d), ln_c.y);
-                        B0.add(gk * r.x);
-                        B1.add(gk * r.z);   // Re(F + t F')
-                        B2.add(gk * r.y);   // Re F'
+                    if (k <= k1) {
+                        const float d = (float)(k - na) - ff, gk = gc[k];
+                        if (PROF != XC_VOIGT_W4 || d * d >= ln_c.thr2) {
+                            ln_c.add(d, gk, q0, q1, q2);
+                        } else {
+                            const float3 r = w4_band_f32(ln_c.asc * fabsf(d), ln_c.y);
+                            B0.add(gk * r.x);
+                            B1.add(gk * r.z);   // Re(F + t F')
+                            B2.add(gk * r.y);   // Re F'
+                        }
+                    } else if (U == 1) {
+                        break;
                     }
                 }
                 K0.add(q0);
@@ -850,12 +857,17 @@ static VjpFn pick(int prof) {
         }                                                                                       \
     } while (0)
 
+template <int PROF, bool FAR>
+static void launch_vjp32(bool mix, bool wl, int blocks, cudaStream_t s, const Vjp32Params &p) {
+    if (mix && wl) k_vjp32<PROF, true, true, FAR><<<blocks, VT, 0, s>>>(p);
+    else if (mix) k_vjp32<PROF, true, false, FAR><<<blocks, VT, 0, s>>>(p);
+    else if (wl) k_vjp32<PROF, false, true, FAR><<<blocks, VT, 0, s>>>(p);
+    else k_vjp32<PROF, false, false, FAR><<<blocks, VT, 0, s>>>(p);
+}
 template <int PROF>
 static void launch_vjp32(bool mix, bool wl, int blocks, cudaStream_t s, const Vjp32Params &p) {
-    if (mix && wl) k_vjp32<PROF, true, true><<<blocks, VT, 0, s>>>(p);
-    else if (mix) k_vjp32<PROF, true, false><<<blocks, VT, 0, s>>>(p);
-    else if (wl) k_vjp32<PROF, false, true><<<blocks, VT, 0, s>>>(p);
-    else k_vjp32<PROF, false, false><<<blocks, VT, 0, s>>>(p);
+    if (p.gnode) launch_vjp32<PROF, PROF != XC_DOPPLER>(mix, wl, blocks, s, p);
+    else launch_vjp32<PROF, false>(mix, wl, blocks, s, p);
 }
 
 xc_status vjp_run(BatchedState *st, const VjpArgs &a, int64_t *launches) {
@@ -881,10 +893,11 @@ xc_status vjp_run(BatchedState *st, const VjpArgs &a, int64_t *launches) {
     size_t o_geo = f64 ? 0 : carve(n * 16);
     size_t o_gs = f64 ? 0 : carve(sizeof(GeomStats));
     size_t o_cp = f64 ? 0 : carve((size_t)nc * sizeof(CParam));
-    // block nodes of the far field (FP32, profiles with far wings): 208 floats per 512 points.  Points
-    // and cuts as for the sweep's blocks: a line whose position is near 2^31 then reaches no point.
-    const bool far = !f64 && a.opts.profile != XC_DOPPLER && a.grid.n < ((int64_t)1 << 30) &&
-                     a.opts.cutoff / a.grid.step < 0x1p20;
+    // block nodes of the far field (FP32, lists that are dense enough): 208 floats per 512 points
+    const bool far = !f64 && n && N &&
+                     route_adjoint_blocks(a.opts.profile, a.opts.n_gh, a.opts.cutoff,
+                                          route_cut_steps(a.opts.cutoff, a.opts.width_mult, a.grid, a.conds_host, nc),
+                                          a.grid, n, nc);
     const int nblk512 = far ? (int)((a.grid.n + 511) / 512) : 0;
     const size_t per_cond = (size_t)nblk512 * (128 + 64 + 16);
     size_t o_gn = far ? carve((size_t)nc * per_cond * 4) : 0;
@@ -948,7 +961,7 @@ xc_status vjp_run(BatchedState *st, const VjpArgs &a, int64_t *launches) {
             k_to_f32<<<nsm * 4, 256, 0, s>>>(g64, g32, (size_t)nc * N);
             ++*launches;
         }
-        if (far && N) {
+        if (far) {
             const double *mat = nullptr;
             VJ_TRY(tree_mat(st, &mat, s));
             constexpr int kSlice = 65535;   // conditions of a launch: the grid's y limit
@@ -983,7 +996,7 @@ xc_status vjp_run(BatchedState *st, const VjpArgs &a, int64_t *launches) {
             vp.ghx = a.ghx;
             vp.ghw = a.ghw;
             vp.ngh = a.opts.n_gh;
-            vp.gnode = far && N ? (const float *)(base + o_gn) : nullptr;
+            vp.gnode = far ? (const float *)(base + o_gn) : nullptr;
             vp.node_off[0] = 0;
             vp.node_off[1] = nblk512 * 128;
             vp.node_off[2] = nblk512 * 192;

@@ -135,3 +135,26 @@ def test_sparse_and_dense_lists_run_their_own_kernels(eng, xc, profile, sparse, 
         eng.set_tile_shape(0, 0)
         m = ref > 1e-6 * ref.max(axis=1, keepdims=True)
         assert np.max(np.abs(got - ref)[m] / ref[m]) < 2e-5, (profile, n)
+
+
+@pytest.mark.parametrize("wm", [0.0, 400.0])
+@pytest.mark.parametrize("profile,n_lines,n,blocks", [
+    ("lorentz", 20_000, 5003, 1), ("lorentz", 300, 200_003, 0), ("voigt_w4", 20_000, 5003, 1),
+    ("voigt_w4", 300, 200_003, 0), ("voigt_gh_binned", 8000, 2003, 1), ("voigt_gh_binned", 20, 200_003, 0)])
+def test_adjoint_of_sparse_and_dense_lists(eng, xc, profile, n_lines, n, blocks, wm):  # noqa: F811
+    """Block nodes and all points, fixed and width-limited cuts, against the FP64 adjoint (1e-4 of the
+    largest, as in the other adjoint tests); the projection on the nodes is one launch more."""
+    L = xs.gen_lines(315, 0, n_lines, 2995.0, 3005.0 + 0.01 * n)
+    eng.load_lines(L)
+    eng.set_states(*xs.gen_states(315, 500))
+    conds = [xc.make_condition(T, P) for T, P in ((500.0, 0.01), (900.0, 0.5), (1600.0, 4.0))]
+    w = 1e22 * np.random.default_rng(315).uniform(0.5, 1.5, (3, n))
+    cut = 25.0 if blocks else 0.5
+    grid = xc.make_grid(3000.0, 0.01, n)
+    for _ in range(2):   # the handle's first call of a Gauss-Hermite profile also makes its nodes
+        r32 = eng.cross_section_vjp(conds, grid, xc.make_opts(profile, "fp32", cut, wm), w)
+    assert eng.last_launch_count() == 7 + blocks
+    r64 = eng.cross_section_vjp(conds, grid, xc.make_opts(profile, "fp64", cut, wm), w)
+    for k in ("dT", "dP", "d_gamma_ref_line", "d_n_line"):
+        a, b = np.asarray(r32[k]), np.asarray(r64[k])
+        assert np.max(np.abs(a - b)) <= 1e-4 * max(np.max(np.abs(b)), 1e-300), k

@@ -26,6 +26,14 @@ extern "C" int route32(int profile, int flags, double cutoff, double width_mult,
                         (size_t)n_lines, n_cond, allow_tc != 0, tiled != 0};
     return 2 * xc::route_blocks32(r) + xc::route_tc32(r);
 }
+extern "C" int adjoint_blocks(int profile, double cutoff, double width_mult, double step, long long n_pts,
+                              unsigned long long n_lines, int n_cond) {
+    const xc_grid g{1000.0, step, (int64_t)n_pts};
+    xc_condition c{};
+    c.T = 1000.0, c.P = 0.1, c.mass_da = 18.0, c.T_ref = 296.0, c.P_ref = 1.0, c.gamma_scale = 1.0;
+    return xc::route_adjoint_blocks(profile, 20, cutoff, xc::route_cut_steps(cutoff, width_mult, g, &c, 1), g,
+                                    (size_t)n_lines, n_cond);
+}
 """
 
 
@@ -42,6 +50,7 @@ def route(tmp_path_factory):
     L.blocks64.argtypes = [C.c_int, C.c_double, C.c_double, C.c_longlong, C.c_double, C.c_ulonglong]
     L.route32.argtypes = [C.c_int, C.c_int, C.c_double, C.c_double, C.c_double, C.c_longlong, C.c_ulonglong, C.c_int,
                           C.c_int, C.c_int]
+    L.adjoint_blocks.argtypes = [C.c_int, C.c_double, C.c_double, C.c_double, C.c_longlong, C.c_ulonglong, C.c_int]
     return L
 
 
@@ -136,3 +145,44 @@ def test_sparse_lists_run_the_faster_form(route, row):
     profile, n_pts, density, cut, wm, nc, blocks, tiled = row
     got = r32(route, profile=profile, cut=cut, wm=wm, n_pts=n_pts, n=max(2, int(n_pts * density)), nc=nc)
     assert (got == BLOCKS) == (blocks < tiled), (got, row)
+
+
+# the adjoint: us with the block nodes and point by point
+MEASURED_ADJOINT = [
+    (LORENTZ, 1000001, 0.003, 256, 0, 6, 723.4, 230),
+    (LORENTZ, 1000001, 0.003, 2500, 500, 3, 470.6, 223.3),
+    (LORENTZ, 1000001, 0.3, 50, 0, 6, 1666, 1011.5),
+    (LORENTZ, 100001, 0.003, 50, 0, 24, 440.6, 217.3),
+    (LORENTZ, 1000001, 0.3, 2500, 0, 1, 952.6, 1381.1),
+    (LORENTZ, 100001, 0.3, 2500, 0, 6, 575.2, 842.2),
+    (W4, 100001, 0.003, 256, 0, 24, 502.3, 326.9),
+    (W4, 1000001, 0.003, 50, 0, 3, 461, 216.6),
+    (W4, 100001, 0.03, 256, 0, 24, 556.1, 410.8),
+    (W4, 1000001, 0.003, 256, 0, 24, 2438.3, 678.7),
+    (W4, 1000001, 0.03, 2500, 0, 1, 382, 631.8),
+    (W4, 100001, 0.03, 2500, 0, 24, 629.9, 1590.9),
+    (W4, 100001, 0.3, 2500, 0, 6, 702.9, 2423.4),
+    (W4, 100001, 0.03, 2500, 0, 3, 252.4, 368),
+    (GH_BINNED, 1000001, 0.003, 50, 0, 6, 797.2, 264.1),
+    (GH_BINNED, 100001, 0.003, 50, 0, 6, 283.4, 205.3),
+    (GH_BINNED, 1000001, 0.003, 256, 0, 6, 918.7, 466.8),
+    (GH_BINNED, 1000001, 0.003, 50, 0, 1, 293.1, 196.7),
+    (GH_BINNED, 100001, 0.3, 2500, 0, 1, 810.6, 3668.3),
+    (GH_BINNED, 100001, 0.03, 2500, 0, 3, 466.5, 1494),
+    (GH_BINNED, 100001, 0.003, 2500, 0, 6, 473.1, 1168.5),
+    (GH_BINNED, 1000001, 0.03, 2500, 500, 1, 717.6, 1029.8),
+]
+
+
+@pytest.mark.parametrize("row", MEASURED_ADJOINT)
+def test_sparse_adjoints_run_the_faster_form(route, row):
+    profile, n_pts, density, cut, wm, nc, blocks, points = row
+    got = route.adjoint_blocks(profile, cut * 0.01, wm, 0.01, n_pts, max(2, int(n_pts * density)), nc)
+    assert bool(got) == (blocks < points), row
+
+
+def test_adjoint_blocks_keep_their_limits(route):
+    assert route.adjoint_blocks(W4, 25.0, 0.0, 0.01, 200_001, 300_000, 4)
+    assert not route.adjoint_blocks(DOPPLER, 25.0, 0.0, 0.01, 200_001, 300_000, 4)
+    assert not route.adjoint_blocks(W4, 25.0, 0.0, 0.01, 1 << 30, 1 << 30, 4)
+    assert not route.adjoint_blocks(W4, 0.01 * 2 ** 20, 0.0, 0.01, 200_001, 300_000, 4)
