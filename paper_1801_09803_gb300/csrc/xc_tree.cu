@@ -694,7 +694,7 @@ __global__ void __launch_bounds__(TR_T) k_tree_points(TreeParams p) {
     if (live) {
         const int p0 = s0 & ~63, p1 = p0 + 63, p1c = min(p1, p.n_pts - 1);
         const int Dp = p.far ? tr_radius(p, p.cp[p.c0 + c].acoef, tr_gap(0), p1) : 0;
-        const Segs sg = tr_point_segs(p, s0, s1, p0, p1, Dp);
+        const Segs sg = tr_point_segs(p, p.far, s0, s1, p0, p1, Dp);
         const float x = (float)lane;
         const f32x2 x2 = pk2(x, x);
         const float4 *recA = p.recA + (size_t)c * p.n;
@@ -884,7 +884,7 @@ __global__ void __launch_bounds__(CG == 1 ? 256 : 128) k_tree_points_w4(TreePara
         const float ac = tr_group_acoef(p, g0, nc);
         const int Dp = tr_radius(p, ac, tr_gap(0), p1);
         const int core = tr_radius(p, ac, -(1 << 28), p1);   // the zones' radius alone
-        const Segs sg = tr_point_segs(p, s0, s1, p0, p1, Dp);
+        const Segs sg = tr_point_segs(p, p.far, s0, s1, p0, p1, Dp);
         const float x = (float)lane;
         const f32x2 x2 = pk2(x, x);
         const unsigned below = (1u << lane) - 1u;

@@ -119,11 +119,12 @@ __device__ __forceinline__ Segs tr_far_segs(const TreeParams &p, int b0, int b1,
     return g;
 }
 
-// Candidate lines of the points s0..s1 inside the level-0 block [p0, p1] of radius Dp
-__device__ __forceinline__ Segs tr_point_segs(const TreeParams &p, int s0, int s1, int p0, int p1, int Dp) {
+// Candidate lines of the points s0..s1 inside the level-0 block [p0, p1] of radius Dp; far: lines that
+// the block takes are left out
+__device__ __forceinline__ Segs tr_point_segs(const TreeParams &p, bool far, int s0, int s1, int p0, int p1, int Dp) {
     const int a = s0 - p.reach, z = s1 + p.reach + 1;
     int e1 = a, s2 = a, e2 = z, s3 = z;
-    if (p.far) {
+    if (far) {
         e1 = max(a, min(p0 - Dp, p1 - p.cover));
         s2 = max(e1, p0 - Dp);
         e2 = min(z, p1 + Dp + 1);

@@ -39,9 +39,27 @@ constexpr int T64_MAT = T64_MAT_DV + T64_M * 128;
 struct T64Params {
     TreeParams t;                 // geo: x = n, y..z = cut range (not clipped to the grid)
     const double *nu, *I, *al, *ga;
+    int *count;                   // lines taken by each block, level 1 first
     float acoef;                  // alpha / nu, rounded up
     int koff;                     // blocks start at multiples of their size minus koff
 };
+
+// Bringing the node sums to a point costs 96 FP64 operations whatever the list.  Points whose blocks
+// took no more than this many lines evaluate them instead (a value takes about 15 operations with
+// the plain Lorentzian and w4's quads, 60 with the binned Lorentzian's arctangent, 20 times that for the
+// Gauss-Hermite sums).  A line that a block takes covers all its points, so every shard of the grid that
+// holds one of them counts the same lines.  1e6 points, 3000 lines, cut 50 and 256 steps, us, direct sum /
+// nodes always / so: Lorentz 95 / 310 / 106 and 128 / 334 / 141, w4 186 / 422 / 215 and 295 / 463 / 271,
+// binned Gauss-Hermite Voigt 932 / 1135 / 908 and 3203 / 3091 / 2835.
+template <int PROF>
+constexpr int t64_few() {
+    return PROF == XC_LORENTZ || PROF == XC_VOIGT_W4 ? 6 : (PROF == XC_LORENTZ_BINNED ? 1 : 0);
+}
+// whether the points of the 128-point block j (parent j / 4) use its nodes
+template <int PROF>
+__device__ __forceinline__ bool t64_far(const T64Params &q, int j) {
+    return q.t.far && q.count[j >> 2] + q.count[q.t.nblk[1] + j] > t64_few<PROF>();
+}
 
 __device__ __forceinline__ double t64_node(int B, int m) {
     return (double)(rintf(64.f * (float)(B - 1) * (1.f - cospif((float)(2 * m + 1) * (1.f / (2 * T64_M))))) * (1.f / 128.f));
@@ -199,7 +217,7 @@ __global__ void __launch_bounds__(32 * T64_NW) k_t64_nodes(T64Params q) {
     const double xl = __dadd_rn(__dadd_rn(__dsub_rn(p.nu_A, __dsub_rn(xh, bb)), __dsub_rn(pr, bb)), pe);
     double *buf = sL[warp];
     double acc = 0.0;
-    int held = 0;
+    int held = 0, taken = 0;
     // lines 0..cnt-1 of the buffer, four to a reciprocal; the last ones (only at the end) singly
     auto quad = [&](int j) {
         double Dn[4], N[4];
@@ -247,6 +265,7 @@ __global__ void __launch_bounds__(32 * T64_NW) k_t64_nodes(T64Params q) {
                     }
                 }
                 held += __popc(m);
+                taken += __popc(m);
                 __syncwarp();
                 if (W4) {
                     int j = 0;
@@ -276,6 +295,7 @@ __global__ void __launch_bounds__(32 * T64_NW) k_t64_nodes(T64Params q) {
         acc = fma(fma(w[3], u, w[4]), t64_rcp(fma(u, u + w[1], w[2])), acc);
     }
     p.nodes[p.node_off[lev] + task * T64_M + lane] = acc;
+    if (lane == 0) q.count[(lev ? 0 : p.nblk[1]) + task] = taken;
 }
 
 // ---------------------------------------------------------------------------
@@ -283,9 +303,9 @@ __global__ void __launch_bounds__(32 * T64_NW) k_t64_nodes(T64Params q) {
 // ---------------------------------------------------------------------------
 // the interpolated far field at point k = s0 + lane added to v, and the output.  j: the
 // 128-point block, o: the point's place in it.
-__device__ __forceinline__ void t64_finish(const T64Params &q, int j, int o, int k, int lane, double v) {
+__device__ __forceinline__ void t64_finish(const T64Params &q, bool far, int j, int o, int k, int lane, double v) {
     const TreeParams &p = q.t;
-    if (p.far) {
+    if (far) {
         const double *up = p.nodes + p.node_off[1] + (j >> 2) * T64_M;
         const double *w = p.mat + T64_MAT_UP + (j & 3) * (T64_M * T64_M) + lane;
         double f = p.nodes[p.node_off[0] + j * T64_M + lane];
@@ -308,10 +328,13 @@ __device__ __forceinline__ void t64_finish(const T64Params &q, int j, int o, int
     if (k >= 0 && k < p.n_pts) p.sigma[k] = v;
 }
 
+// Small CTAs: a value of the binned Gauss-Hermite sum holds a warp for 10 us of its SM's FP64 pipe, so the
+// warps of one crowded stretch of the grid go to several SMs
+constexpr int T64_PW = 2;
 template <int PROF>
-__global__ void __launch_bounds__(TR_T) k_t64_points(T64Params q) {
-    __shared__ double sL[TR_W][32 * 4];
-    __shared__ int2 sR[TR_W][32];
+__global__ void __launch_bounds__(32 * T64_PW) k_t64_points(T64Params q) {
+    __shared__ double sL[T64_PW][32 * 4];
+    __shared__ int2 sR[T64_PW][32];
     __shared__ double sX[64], sW[64];
     const TreeParams &p = q.t;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -322,12 +345,13 @@ __global__ void __launch_bounds__(TR_T) k_t64_points(T64Params q) {
         }
         __syncthreads();
     }
-    const int task = blockIdx.x * TR_W + warp;
+    const int task = blockIdx.x * T64_PW + warp;
     const int s0 = task * 32 - q.koff, s1 = s0 + 31;
     if (s0 >= p.n_pts || s1 < 0) return;
     const int p0 = (task >> 2) * 128 - q.koff, p1 = p0 + 127;
-    const int Dp = p.far ? tr_radius(p, q.acoef, t64_gap(0), p1) : 0;
-    const Segs sg = tr_point_segs(p, s0, s1, p0, p1, Dp);
+    const bool far = t64_far<PROF>(q, task >> 2);
+    const int Dp = far ? tr_radius(p, q.acoef, t64_gap(0), p1) : 0;
+    const Segs sg = tr_point_segs(p, far, s0, s1, p0, p1, Dp);
     const double xk = grid_x(p.nu_A, p.step, s0 + lane);
     double *buf = sL[warp];
     double acc = 0.0;
@@ -339,7 +363,7 @@ __global__ void __launch_bounds__(TR_T) k_t64_points(T64Params q) {
             const unsigned l = i + lane;
             int4 g = make_int4(0, 1, 0, 0);
             if (l < e) g = p.geo[l];
-            const bool ok = g.y <= s1 && g.z >= s0 && g.y <= g.z && !(p.far && tr_takes(g, p0, p1, p1, Dp));
+            const bool ok = g.y <= s1 && g.z >= s0 && g.y <= g.z && !(far && tr_takes(g, p0, p1, p1, Dp));
             const unsigned m = __ballot_sync(0xffffffffu, ok);
             if (!m) continue;
             if (ok) {
@@ -362,7 +386,7 @@ __global__ void __launch_bounds__(TR_T) k_t64_points(T64Params q) {
             __syncwarp();
         }
     }
-    t64_finish(q, task >> 2, (task & 3) * 32 + lane, s0 + lane, lane, acc);
+    t64_finish(q, far, task >> 2, (task & 3) * 32 + lane, s0 + lane, lane, acc);
 }
 
 // Re w in w4's region II, real form (see w4_region2_re)
@@ -427,7 +451,8 @@ __global__ void __launch_bounds__(128) k_t64_points_w4(T64Params q) {
     const int p0 = (task >> 2) * 128 - q.koff, p1 = p0 + 127;
     const int Dp = tr_radius(p, q.acoef, t64_gap(0), p1);
     const int core = tr_radius(p, q.acoef, -(1 << 28), p1) + 1;   // the zones' radius alone
-    const Segs sg = tr_point_segs(p, s0, s1, p0, p1, Dp);
+    const bool far = t64_far<XC_VOIGT_W4>(q, task >> 2);
+    const Segs sg = tr_point_segs(p, far, s0, s1, p0, p1, Dp);
     const double xk = grid_x(p.nu_A, p.step, s0 + lane), x0 = grid_x(p.nu_A, p.step, s0);
     const double inv_h = 1.0 / p.step;
     const unsigned below = (1u << lane) - 1u;
@@ -449,7 +474,7 @@ __global__ void __launch_bounds__(128) k_t64_points_w4(T64Params q) {
             const unsigned l = i + lane;
             int4 g = make_int4(0, 1, 0, 0);
             if (l < e) g = p.geo[l];
-            const bool ok = g.y <= s1 && g.z >= s0 && g.y <= g.z && !tr_takes(g, p0, p1, p1, Dp);
+            const bool ok = g.y <= s1 && g.z >= s0 && g.y <= g.z && !(far && tr_takes(g, p0, p1, p1, Dp));
             if (!__any_sync(0xffffffffu, ok)) continue;
             W4Line w{};
             bool zone = false;
@@ -599,14 +624,15 @@ __global__ void __launch_bounds__(128) k_t64_points_w4(T64Params q) {
         one(j, N, Dn);
         accF = fma(N, t64_rcp(Dn), accF);
     }
-    t64_finish(q, task >> 2, (task & 3) * 32 + lane, s0 + lane, lane, (accF + accZ) + (acc34[0] + acc34[1]));
+    t64_finish(q, far, task >> 2, (task & 3) * 32 + lane, s0 + lane, lane, (accF + accZ) + (acc34[0] + acc34[1]));
 }
 
 // ---------------------------------------------------------------------------
 // host side
 // ---------------------------------------------------------------------------
 // bytes of scratch behind the int4 geometry of n lines
-static size_t tree64_layout(const xc_grid &g, double cutoff, size_t n, TreeParams *p, size_t *o_cell, size_t *o_nodes) {
+static size_t tree64_layout(const xc_grid &g, double cutoff, size_t n, TreeParams *p, size_t *o_cell, size_t *o_nodes,
+                            size_t *o_count) {
     p->n = n;
     p->n_pts = (int)g.n;
     p->nu_A = g.nu_A;
@@ -628,13 +654,14 @@ static size_t tree64_layout(const xc_grid &g, double cutoff, size_t n, TreeParam
     carve(n * sizeof(int4));
     *o_cell = carve((size_t)(p->ncell + 1) * 4);
     *o_nodes = carve((size_t)off * 8);
+    *o_count = carve((size_t)(p->nblk[0] + p->nblk[1]) * 4);
     return o;
 }
 
 size_t tree64_scratch(const xc_grid &g, double cutoff, size_t n) {
     TreeParams p;
-    size_t a, b;
-    return tree64_layout(g, cutoff, n, &p, &a, &b);
+    size_t a, b, c;
+    return tree64_layout(g, cutoff, n, &p, &a, &b, &c);
 }
 
 template <int PROF>
@@ -647,7 +674,7 @@ static void t64_launch(const T64Params &q, int64_t *launches, cudaStream_t s) {
     if (PROF == XC_VOIGT_W4)
         k_t64_points_w4<<<(unsigned)((tasks + 3) / 4), 128, 0, s>>>(q);
     else
-        k_t64_points<PROF><<<(unsigned)((tasks + TR_W - 1) / TR_W), TR_T, 0, s>>>(q);
+        k_t64_points<PROF><<<(unsigned)((tasks + T64_PW - 1) / T64_PW), 32 * T64_PW, 0, s>>>(q);
     *launches += 1;
 }
 
@@ -657,8 +684,8 @@ cudaError_t launch_tree64(int profile, const double *nu, const double *I, const 
                           double *sigma, int64_t *launches, cudaStream_t s) {
     T64Params q;
     TreeParams &p = q.t;
-    size_t o_cell, o_nodes;
-    tree64_layout(g, cutoff, n, &p, &o_cell, &o_nodes);
+    size_t o_cell, o_nodes, o_count;
+    tree64_layout(g, cutoff, n, &p, &o_cell, &o_nodes, &o_count);
     char *b = static_cast<char *>(scratch);
     int4 *geo = reinterpret_cast<int4 *>(b);
     unsigned *cell = reinterpret_cast<unsigned *>(b + o_cell);
@@ -666,6 +693,7 @@ cudaError_t launch_tree64(int profile, const double *nu, const double *I, const 
     p.cell = cell;
     p.mat = mat;
     p.nodes = reinterpret_cast<double *>(b + o_nodes);
+    q.count = reinterpret_cast<int *>(b + o_count);
     p.sigma = sigma;
     p.ghx = ghx;
     p.ghw = ghw;

@@ -158,3 +158,68 @@ def test_adjoint_of_sparse_and_dense_lists(eng, xc, profile, n_lines, n, blocks,
     for k in ("dT", "dP", "d_gamma_ref_line", "d_n_line"):
         a, b = np.asarray(r32[k]), np.asarray(r64[k])
         assert np.max(np.abs(a - b)) <= 1e-4 * max(np.max(np.abs(b)), 1e-300), k
+
+
+@pytest.mark.parametrize("profile", ["voigt_w4", "lorentz", "lorentz_binned", "voigt_gh_binned", "doppler"])
+@pytest.mark.parametrize("n_lines,cut", [(40, 2.0), (150, 4.0), (600, 8.0)])
+def test_sparse_grid_shards_are_bit_exact(eng, xc, profile, n_lines, cut):  # noqa: F811
+    """FP64 lists of 0 to a dozen lines a block, where blocks with few lines are left to the points: a shard
+    of the grid that holds its own lines only decides alike (step 2^-7: exact points)."""
+    from paper_1801_09803_gb300.shard import grid_shard, halo_line_range
+    S = xs.gen_lines(316, 0, n_lines, 990.0, 1075.0)
+    S = {k: v[np.argsort(S["nu"], kind="stable")] for k, v in S.items()}
+    eng.set_states(*xs.gen_states(316, 300))
+    nu_A, step, n, cond = 1000.0, 1.0 / 128.0, 8193, xc.make_condition(900.0, 0.3)
+    opts = xc.make_opts(profile, "fp64", cut)
+    eng.load_lines(S, assume_sorted=True)
+    full = eng.cross_section(cond, xc.make_grid(nu_A, step, n), opts)
+    for world in (3, 7):
+        for r in range(world):
+            k0, k1 = grid_shard(n, world, r)
+            l0, l1 = halo_line_range(S["nu"], nu_A, step, k0, k1, cut)
+            eng.load_lines({k: v[l0:l1] for k, v in S.items()}, assume_sorted=True)
+            part = eng.cross_section(cond, xc.make_grid(nu_A + k0 * step, step, k1 - k0), opts)
+            assert np.array_equal(part, full[k0:k1]), (world, r)
+
+
+@pytest.mark.parametrize("profile,n_gh", [("voigt_gh_sampled", 20), ("voigt_gh_sampled", 7), ("voigt_gh_sampled", 40),
+                                          ("doppler_binned", 20), ("voigt_gh_binned", 7), ("voigt_gh_binned", 40)])
+@pytest.mark.parametrize("n_lines", [30, 1500])
+def test_fp64_blocks_of_the_other_profiles(eng, xc, oracle_lib, profile, n_gh, n_lines):  # noqa: F811
+    """FP64 blocks with other node counts (the outermost node sets the distance a block keeps) and the
+    profiles without a test of their own: 1e-12, as test_fp64_blocks_against_oracle."""
+    L = xs.gen_lines(317, 0, n_lines, 1000.0, 1060.0)
+    E, g = xs.gen_states(317, 500)
+    eng.load_lines(L)
+    eng.set_states(E, g)
+    n = 2049
+    for nu_A, step, cut, wm, T, P in ((1010.003, 0.01, 25.0, 0.0, 900.0, 0.3), (990.0, 0.01, 25.0, 300.0, 2500.0, 10.0)):
+        got = eng.cross_section(xc.make_condition(T, P), xc.make_grid(nu_A, step, n),
+                                xc.make_opts(profile, "fp64", cut, wm, n_gh=n_gh))
+        if profile == "voigt_gh_binned":
+            Q = oracle_lib.partition_function(E, g, T)[0]
+            ref = gh_binned64(L, Q, T, P, nu_A + np.arange(n) * step, step, cut, wm, n_gh)
+        else:
+            Q, dQ = oracle_lib.partition_function(E, g, T)
+            ref = oracle_lib.cross_section(L, oracle_lib.make_condition(T, P, Q, dQ), nu_A, step, n,
+                                           oracle_lib.make_opts(profile, cut, wm, n_gh), nthreads=8)
+        assert metrics(got, ref)[0] < 1e-12, (profile, n_gh, nu_A)
+
+
+def gh_binned64(L, Q, T, P, x, step, cut, wm, n_gh):
+    """The binned Gauss-Hermite Voigt with one arctangent a node (see binned64 in test_gpu_tree)."""
+    c2 = 6.62607015e-34 * 2.99792458e10 / 1.380649e-23
+    nu, f = L["nu"], {k: v.astype(np.float64) for k, v in L.items()}
+    al = nu * np.sqrt(2 * 1.380649e-23 * T * np.log(2) / (18 * 1.66053906660e-27)) / 2.99792458e8
+    ga = f["gamma_ref"] * (296.0 / T) ** f["n_T"] * P
+    S = f["g_up"] * f["A"] / (8 * np.pi * 2.99792458e10 * Q * nu ** 2) * np.exp(-c2 * f["elower"] / T)
+    S = S * -np.expm1(-c2 * nu / T)
+    c = np.minimum(cut, wm * np.maximum(al, ga)) if wm else np.full_like(nu, cut)
+    xj, wj = np.polynomial.hermite.hermgauss(n_gh)
+    out = np.empty_like(x)
+    for k, xk in enumerate(x):
+        D = xk - nu
+        d = D[:, None] - (al / np.sqrt(np.log(2)))[:, None] * xj
+        v = np.arctan2(step * ga[:, None], (d + step / 2) * (d - step / 2) + ga[:, None] ** 2) @ wj
+        out[k] = (S * v)[np.abs(D) <= c].sum() * np.pi ** -1.5 / step
+    return out
