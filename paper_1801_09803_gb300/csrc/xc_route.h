@@ -59,9 +59,10 @@ struct Route32 {
 // within 10 % (blocks) and 15 to 50 % (tiled, worst where the autotuner picks a slow tile).  Blocks
 // against tiled, ps: a 110-133 / 4-22 (w4 with one condition 127 / 119: a launch for its centre zones),
 // b 24-200 / 70-1260, c 0.02-0.06 / 0.1-3 (20 Gauss-Hermite nodes 0.5-0.9 / 5-23).  The lines below are the
-// differences.  At 1e6 points, 6 conditions, blocks / tiled us: Lorentz 15 pairs a point 886 / 219, 150
-// 930 / 390, 1500 (0.3 lines) 1230 / 2500; w4 15 876 / 461, 150 883 / 685, 1500 1360 / 3900; binned
-// Lorentz 15 871 / 400, 150 880 / 1330.  The Doppler profiles have nothing to bring to the points.
+// differences; over 682 calls 10 are more than 5 % off the better form, the worst 20 %.  At 1e6 points, 6
+// conditions, cut 2500 steps, blocks / tiled us: Lorentz 15 pairs a point 886 / 204, 150 928 / 400, 1500
+// 1132 / 2533; w4 836 / 355, 880 / 676, 1375 / 4236; binned Lorentz 861 / 334, 904 / 1171, 1444 / 9031.  The
+// Doppler profiles have nothing to bring to the points.
 inline bool route_sparse32(const Route32 &r, bool tc) {
     const bool wl = r.width_mult > 0.0;               // width-limited: one pass for each condition
     const double nc = wl ? 1.0 : (double)r.n_cond, gh = r.n_gh / 20.0;
@@ -69,12 +70,12 @@ inline bool route_sparse32(const Route32 &r, bool tc) {
     switch (r.profile) {
     case XC_VOIGT_W4: point = 100.0 - 92.0 / nc; line = 350.0 + 700.0 / nc; pair = tc ? 0.08 : 0.3; break;
     case XC_LORENTZ: point = nc > 1.0 ? 125.0 : 104.0; line = 70.0 + 150.0 / nc; pair = nc >= 16.0 ? 0.12 : 0.2; break;
-    case XC_LORENTZ_BINNED: point = 115.0; line = 250.0; pair = 1.5; break;
-    case XC_VOIGT_GH_BINNED: point = 92.0; line = -700.0 * gh; pair = 17.0 * gh; break;
-    case XC_VOIGT_GH_SAMPLED: point = 105.0; line = -130.0 * gh; pair = 5.0 * gh; break;
+    case XC_LORENTZ_BINNED: point = 115.0; line = 250.0; pair = nc >= 8.0 ? 2.5 : 1.5; break;
+    case XC_VOIGT_GH_BINNED: point = 92.0; line = -700.0 * gh; pair = (nc > 1.0 ? 17.0 : 23.0) * gh; break;
+    case XC_VOIGT_GH_SAMPLED: point = 105.0; line = -130.0 * gh; pair = (nc > 1.0 ? 5.0 : 7.0) * gh; break;
     default: return false;
     }
-    const double base = wl ? 23e6 * r.n_cond : 25e6 + 5e6 * fmin(nc, 24.0);   // shorter launch sequences
+    const double base = wl ? 23e6 * r.n_cond : 28e6 + 5e6 * fmin(nc, 24.0);   // shorter launch sequences
     return base - point * (double)r.grid.n * r.n_cond +
                (line + pair * 2.0 * r.cut_steps) * (double)r.n_lines * r.n_cond < 0.0;
 }
@@ -104,8 +105,8 @@ inline bool route_blocks32(const Route32 &r) {
 // The FP32 adjoint (xc_vjp.cu): dL/dsigma projected on the block nodes costs 75 ps a point and condition
 // and then saves evaluations of each line's far points.  Timed over the same family: blocks against all
 // points, ps a pair 0.2-0.3 / 0.6 (Lorentz), 2.4 (w4), 24 (20 Gauss-Hermite nodes), and for each line 200, 400
-// and 3000 to 5000 more.  1e6 points, 6 conditions, blocks / points us: w4 15 pairs a point 774 / 624, 150
-// 1178 / 2684; Lorentz 15 758 / 349, 150 1003 / 866, width-limited (500 widths) 15 758 / 309.
+// and 3000 to 5000 more.  1e6 points, 6 conditions, cut 2500 steps, blocks / points us: w4 15 pairs a point
+// 778 / 581, 150 1178 / 2684; Lorentz 758 / 286, 1024 / 764, width-limited (500 widths) 770 / 250 and 1031 / 502.
 // Points and cuts as for the sweep: a line whose position is near 2^31 then reaches no point.
 inline bool route_adjoint_blocks(int profile, int n_gh, double cutoff, double cut_steps, const xc_grid &g,
                                  size_t n_lines, int n_cond) {
