@@ -1846,6 +1846,23 @@ std::string tuned_key(const BatchedState *st, const BatchedArgs &a, int nc) {
     return key;
 }
 
+// Conditions per tile for sparse lists (8 points a thread; with the far wings on the tensor cores 4, and
+// groups of 8).  The probes of the autotuner time a few hundred us of launches, take 1 to 3 ms of the
+// first call and choose badly there: over 478 sparse calls of 1 to 24 conditions 18 % slower than the
+// best shape in the mean and up to 3.7 times; groups by this rule 3 % and 1.6 times.
+int sparse_cgroup(int profile, bool ext, int nc) {
+    const int pad4 = (nc + 3) / 4 * 4;   // conditions in whole groups of four
+    switch (profile) {
+    case XC_VOIGT_GH_BINNED: return 1;                                 // dear values: no padding
+    case XC_VOIGT_GH_SAMPLED: return 10 * pad4 > 13 * nc ? 1 : 4;
+    case XC_LORENTZ_BINNED: return nc <= 2 ? 1 : 4;
+    default: break;
+    }
+    if (nc == 1) return 1;
+    const bool has8 = profile == XC_LORENTZ || (profile == XC_VOIGT_W4 && !ext);
+    return has8 && (-nc & 7) <= 2 ? 8 : 4;
+}
+
 // Autotune: time each candidate variant on a probe (every tile, first 4096 lines)
 // and predict the full run from the measured time per (tile line x condition);
 // the prediction includes the wave quantisation of the tile count.
@@ -1860,6 +1877,10 @@ xc_status autotune(BatchedState *st, const BatchedArgs &a, int nc, TileCfg *out,
     }
     int dev = 0;
     cudaGetDevice(&dev);
+    // sparse lists take a shape by the number of conditions instead of probes (see sparse_cgroup)
+    const Route32 route = route_of(a, nc);
+    const bool sparse = st->force_R == 0 && !a.tiled && route_sparse32(route, route_tc_form(route));
+    const int sparse_CG = tc ? 8 : sparse_cgroup(a.opts.profile, needs_ext(a), nc);
     std::vector<int> cands;
     // the shape heuristics first; if they leave no variant of this profile (e.g. 5 to 7
     // conditions where only groups of 1, 4 and 16 exist), every admissible shape
@@ -1869,7 +1890,9 @@ xc_status autotune(BatchedState *st, const BatchedArgs &a, int nc, TileCfg *out,
             if (v.profile != a.opts.profile) continue;
             if (v.profile == XC_VOIGT_W4 && v.ext != needs_ext(a)) continue;
             if (a.opts.width_mult > 0.0 && v.CG != 1) continue;  // per-condition cut: one condition per tile
-            if (pass == 0 && a.opts.width_mult <= 0.0 && st->force_R == 0) {
+            if (pass == 0 && sparse && a.opts.width_mult <= 0.0) {
+                if (v.CG != sparse_CG || v.R != (tc ? 4 : 8)) continue;
+            } else if (pass == 0 && a.opts.width_mult <= 0.0 && st->force_R == 0) {
                 if (v.CG > 1 && v.CG > 2 * nc) continue;          // no more than half the group padded
                 if (v.CG < std::min(nc, 8)) continue;              // enough conditions share each staged line
             }
