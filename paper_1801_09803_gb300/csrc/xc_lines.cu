@@ -13,24 +13,27 @@ namespace xc {
 
 // ---------------------------------------------------------------------------
 // Q(T) = sum_n g_n exp(-c2 E_n / T) and dQ/dT = sum_n g_n (c2 E_n / T^2) exp(-c2 E_n / T)
-// A cluster of PF_CL CTAs per temperature: the exponentials are bound by the FP64 pipe (2
-// lanes per cycle and SM), so one CTA's 5000 states took 47 us on one SM.  Each CTA sums
+// A cluster of 8 or 16 CTAs per temperature: the exponentials are bound by the FP64 pipe (2
+// lanes per cycle and SM), so one CTA's 5000 states took 47 us on one SM.  Of 5000 states 8 CTAs take
+// 13.2 us for one temperature and 19.6 for 32, 16 CTAs 14.0 and 26.3; of 1e5 states 64 and 118
+// against 40 and 127.  Clusters of 8 run on any device; of 16 only where a GPC has 16 SMs to give.  Each CTA sums
 // its share of the states by a fixed-order tree; the first adds the others' sums from their
 // shared memory in rank order (deterministic).  tix (may be null): index of the temperature
 // of each condition, whose Q and dQ/dT are then filled in as well.
 // ---------------------------------------------------------------------------
-constexpr int PF_CL = 16;   // 16 is beyond the portable cluster size: allowed explicitly below
+constexpr int PF_CL = 8;         // the portable cluster size
+constexpr int PF_CL_LARGE = 16;  // for many states, where the device has room for such a cluster
 __global__ void __launch_bounds__(256)
     k_partition_function(const double *__restrict__ E, const int32_t *__restrict__ g, size_t n,
                          const double *__restrict__ T, double *Q, double *dQ, CondDev *conds, const int *tix,
                          int n_cond) {
     __shared__ double sq[256], sd[256];
     cooperative_groups::cluster_group cl = cooperative_groups::this_cluster();
-    const int j = blockIdx.x / PF_CL, r = (int)cl.block_rank();
+    const int ncl = (int)cl.num_blocks(), j = blockIdx.x / ncl, r = (int)cl.block_rank();
     const double t = T[j];
     const double a = kC2 / t;
     double q = 0.0, d = 0.0;
-    for (size_t i = threadIdx.x + 256 * (size_t)r; i < n; i += 256 * PF_CL) {
+    for (size_t i = threadIdx.x + 256 * (size_t)r; i < n; i += 256 * (size_t)ncl) {
         const double e = E[i];
         const double gb = (double)g[i] * exp64(-a * e);
         q += gb;
@@ -49,7 +52,7 @@ __global__ void __launch_bounds__(256)
     cl.sync();
     if (r == 0 && threadIdx.x < 32) {
         double sumq = 0.0, sumd = 0.0;
-        for (int k = 0; k < PF_CL; ++k) {
+        for (int k = 0; k < ncl; ++k) {
             sumq += *cl.map_shared_rank(&sq[0], k);
             sumd += *cl.map_shared_rank(&sd[0], k);
         }
@@ -71,19 +74,29 @@ cudaError_t launch_partition_function(const double *E, const int32_t *g, size_t 
                                       double *Q, double *dQ, cudaStream_t s, CondDev *conds, const int *tix,
                                       int n_cond) {
     if (nT <= 0) return cudaSuccess;
-    cudaError_t e = cudaFuncSetAttribute((const void *)k_partition_function,
-                                         cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
-    if (e != cudaSuccess) return e;
     cudaLaunchAttribute at;
     at.id = cudaLaunchAttributeClusterDimension;
-    at.val.clusterDim.x = PF_CL;
     at.val.clusterDim.y = at.val.clusterDim.z = 1;
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)nT * PF_CL);
     cfg.blockDim = dim3(256);
     cfg.stream = s;
     cfg.attrs = &at;
     cfg.numAttrs = 1;
+    auto size = [&](int cl) {
+        at.val.clusterDim.x = cl;
+        cfg.gridDim = dim3((unsigned)nT * cl);
+    };
+    size(PF_CL);
+    if (n >= 32768 && nT <= 8) {
+        int room = 0;
+        size(PF_CL_LARGE);
+        if (cudaFuncSetAttribute((const void *)k_partition_function, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) !=
+                cudaSuccess ||
+            cudaOccupancyMaxActiveClusters(&room, k_partition_function, &cfg) != cudaSuccess || room < 1) {
+            cudaGetLastError();
+            size(PF_CL);
+        }
+    }
     return cudaLaunchKernelEx(&cfg, k_partition_function, E, g, n, T, Q, dQ, conds, tix, n_cond);
 }
 

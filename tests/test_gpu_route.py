@@ -223,3 +223,16 @@ def gh_binned64(L, Q, T, P, x, step, cut, wm, n_gh):
         v = np.arctan2(step * ga[:, None], (d + step / 2) * (d - step / 2) + ga[:, None] ** 2) @ wj
         out[k] = (S * v)[np.abs(D) <= c].sum() * np.pi ** -1.5 / step
     return out
+
+
+@pytest.mark.parametrize("n", [1, 7, 255, 2049, 32_767, 32_768, 200_001])
+@pytest.mark.parametrize("nT", [1, 9])
+def test_partition_function_of_many_states(xc, oracle_lib, n, nT):
+    """Clusters of 8 and of 16 CTAs, shares that are empty or ragged: Q and dQ/dT to 1e-13 of the oracle
+    (sums of positive terms in another order, exponentials to an ulp)."""
+    E, g = xs.gen_states(318, n)
+    T = np.linspace(200.0, 3000.0, nT)
+    Q, dQ = xc.partition_function(E, g, T)
+    for t, q, d in zip(T, Q, dQ):
+        rq, rd = oracle_lib.partition_function(E, g, t)
+        assert abs(q - rq) <= 1e-13 * rq and abs(d - rd) <= 1e-13 * max(abs(rd), 1e-300), (n, t)
