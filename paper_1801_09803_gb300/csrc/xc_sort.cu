@@ -5,8 +5,8 @@
 // wavenumbers keep their input order) carries a 32-bit index payload, and a
 // gather pass then reorders every field.  Digit positions where all keys share
 // one digit value are skipped (decided once from a global histogram), and of the
-// rest only the highest five are sorted by passes: the short runs of keys that
-// agree in them are then sorted in place (by every digit if a run is long).
+// rest only the highest five are sorted by passes: the runs of keys that agree in
+// them are then sorted in place.
 //
 // Per pass: (1) per-tile digit histograms, (2) digit totals and exclusive scan
 // into per-(digit, tile) output offsets, (3) a stable scatter where each warp
@@ -339,16 +339,17 @@ __global__ void k_gather_recs(const LineRec *__restrict__ rec, size_t n, const u
 
 // Sorts by the whole key inside runs of equal high parts (key >> shift), which the radix passes
 // left in input order: the thread at a run's first key sorts it in place (stable insertion).
-// A run longer than RS_RUN raises flag bit 4, and the caller sorts by every digit instead.
+// Runs of more than RS_RUN keys go on a list for k_rs_sort_run (their first keys, at most n /
+// RS_RUN of them, and their number).
 constexpr int RS_RUN = 64;
-__global__ void k_rs_finish_runs(uint64_t *keys, uint32_t *vals, size_t n, int shift, int *flag) {
+__global__ void k_rs_finish_runs(uint64_t *keys, uint32_t *vals, size_t n, int shift, uint32_t *count, uint32_t *list) {
     for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i + 1 < n; i += (size_t)gridDim.x * blockDim.x) {
         const uint64_t top = keys[i] >> shift;
         if ((keys[i + 1] >> shift) != top || (i > 0 && (keys[i - 1] >> shift) == top)) continue;
         size_t e = i + 2;
         while (e < n && e - i <= RS_RUN && (keys[e] >> shift) == top) ++e;
         if (e - i > RS_RUN) {
-            atomicOr(flag, 4);
+            list[atomicAdd(count, 1u)] = (uint32_t)i;
             continue;
         }
         for (size_t a = i + 1; a < e; ++a) {
@@ -362,6 +363,70 @@ __global__ void k_rs_finish_runs(uint64_t *keys, uint32_t *vals, size_t n, int s
             keys[b] = k;
             vals[b] = v;
         }
+    }
+}
+
+// Long runs (band heads of large lists, repeated wavenumbers), one CTA each.  A run already in order --
+// equal keys -- is only read; others of up to RS_BIG keys are sorted in shared memory by key and place
+// (bitonic, so stable).  A longer one that is out of order, or too long to look through, raises flag
+// bit 4: the caller sorts the list by every digit.
+constexpr int RS_BIG = 2048, RS_LONG = 65536;
+__global__ void __launch_bounds__(256) k_rs_sort_run(uint64_t *keys, uint32_t *vals, size_t n, int shift,
+                                                     const uint32_t *count, const uint32_t *list, int *flag) {
+    __shared__ uint64_t sk[RS_BIG];
+    __shared__ uint32_t sv[RS_BIG];
+    __shared__ uint16_t sp[RS_BIG];   // place in the run
+    const int tid = threadIdx.x;
+    const uint32_t runs = *count;
+    for (uint32_t q = blockIdx.x; q < runs; q += gridDim.x) {
+        const size_t i = list[q];
+        const uint64_t top = keys[i] >> shift;
+        // length, and whether the run is in order
+        size_t len = 0;
+        bool bad = false;
+        for (bool more = true; more; len += more ? 256 : 0) {
+            const size_t j = i + len + tid;
+            const bool in = j < n && (keys[j] >> shift) == top;
+            bad |= in && j > i && keys[j - 1] > keys[j];
+            const int m = __syncthreads_count(in);
+            if (m < 256) {
+                len += m;
+                more = false;
+            } else if (len >= RS_LONG) {
+                more = false;
+            }
+        }
+        if (!__syncthreads_or(bad || len >= RS_LONG)) continue;
+        if (len > RS_BIG) {
+            if (tid == 0) atomicOr(flag, 4);
+            continue;
+        }
+        int P = 128;
+        while (P < (int)len) P <<= 1;
+        for (int j = tid; j < P; j += 256) {
+            sk[j] = j < (int)len ? keys[i + j] : ~0ull;
+            sv[j] = j < (int)len ? vals[i + j] : 0u;
+            sp[j] = (uint16_t)j;
+        }
+        __syncthreads();
+        for (int k = 2; k <= P; k <<= 1)
+            for (int j = k >> 1; j > 0; j >>= 1) {
+                for (int t = tid; t < P / 2; t += 256) {
+                    const int a = 2 * j * (t / j) + t % j, b = a + j;
+                    const bool up = (a & k) == 0, gt = sk[a] > sk[b] || (sk[a] == sk[b] && sp[a] > sp[b]);
+                    if (gt == up) {
+                        const uint64_t tk = sk[a]; sk[a] = sk[b]; sk[b] = tk;
+                        const uint32_t tv = sv[a]; sv[a] = sv[b]; sv[b] = tv;
+                        const uint16_t tp = sp[a]; sp[a] = sp[b]; sp[b] = tp;
+                    }
+                }
+                __syncthreads();
+            }
+        for (int j = tid; j < (int)len; j += 256) {
+            keys[i + j] = sk[j];
+            vals[i + j] = sv[j];
+        }
+        __syncthreads();
     }
 }
 
@@ -393,9 +458,10 @@ cudaError_t launch_sort_lines(const LinesDev &in, size_t n, bool assume_sorted, 
                               uint32_t *perm, int *d_flag, cudaStream_t s, cudaEvent_t *ev, int64_t *launches,
                               bool *bad_input, bool *unsorted) {
     cudaError_t e;
+    int h_flag = 0;
     *bad_input = false;
     *unsorted = false;
-    if ((e = cudaMemsetAsync(d_flag, 0, sizeof(int), s)) != cudaSuccess) return e;
+    if ((e = cudaMemsetAsync(d_flag, 0, 2 * sizeof(int), s)) != cudaSuccess) return e;
     if (ev) cudaEventRecord(ev[0], s);
     if (assume_sorted) {
         k_copy_sorted<<<grid_for(n), 256, 0, s>>>(in, n, nu, elower, A, gref, nT, g, j, perm, d_flag);
@@ -409,6 +475,9 @@ cudaError_t launch_sort_lines(const LinesDev &in, size_t n, bool assume_sorted, 
             cudaEventRecord(ev[1], s);
             cudaEventRecord(ev[2], s);
         }
+        if ((e = cudaGetLastError()) != cudaSuccess) return e;
+        if ((e = cudaMemcpyAsync(&h_flag, d_flag, sizeof(int), cudaMemcpyDeviceToHost, s)) != cudaSuccess) return e;
+        if ((e = cudaStreamSynchronize(s)) != cudaSuccess) return e;
     } else {
         const uint32_t n_tiles = (uint32_t)((n + RS_TILE - 1) / RS_TILE);
         // scratch: keys x2 (8 B), vals x2 (4 B), tile hist (256 x n_tiles), totals, global hist
@@ -426,26 +495,25 @@ cudaError_t launch_sort_lines(const LinesDev &in, size_t n, bool assume_sorted, 
         // packed records for the gather, where 32 bytes per line are to be had
         if (tmp[5].ensure(n * sizeof(LineRec)) != cudaSuccess) cudaGetLastError();
         LineRec *rec = tmp[5].as<LineRec>();
-        bool whole = false;
+        k_make_keys<<<grid_for(n), 256, 0, s>>>(in, n, k0, v0, rec, d_flag);
+        if ((e = cudaMemsetAsync(ghist, 0, 8 * 256 * 8, s)) != cudaSuccess) return e;
+        k_rs_global_hist<<<grid_for(n, 4), 256, 0, s>>>(k0, n, ghist);
+        *launches += 2;
+        unsigned long long h_g[8 * 256];
+        if ((e = cudaMemcpyAsync(h_g, ghist, sizeof(h_g), cudaMemcpyDeviceToHost, s)) != cudaSuccess) return e;
+        if ((e = cudaStreamSynchronize(s)) != cudaSuccess) return e;
+        int digit[8], nd = 0;
+        for (int d = 0; d < 8; ++d) {
+            bool trivial = false;
+            for (int b = 0; b < 256; ++b)
+                if (h_g[d * 256 + b] == (unsigned long long)n) trivial = true;
+            if (!trivial) digit[nd++] = d;
+        }
+        // The highest RS_DIGITS digits decide the order of all but a few lines (28 mantissa
+        // bits where the wavenumbers span several powers of two: 3e-5 cm^-1 at 10^4 cm^-1);
+        // the runs they leave are sorted in place.  Three passes of eight fewer.
+        int first = nd <= RS_DIGITS ? 0 : nd - RS_DIGITS;
         for (;;) {
-            k_make_keys<<<grid_for(n), 256, 0, s>>>(in, n, k0, v0, rec, d_flag);
-            if ((e = cudaMemsetAsync(ghist, 0, 8 * 256 * 8, s)) != cudaSuccess) return e;
-            k_rs_global_hist<<<grid_for(n, 4), 256, 0, s>>>(k0, n, ghist);
-            *launches += 2;
-            unsigned long long h_g[8 * 256];
-            if ((e = cudaMemcpyAsync(h_g, ghist, sizeof(h_g), cudaMemcpyDeviceToHost, s)) != cudaSuccess) return e;
-            if ((e = cudaStreamSynchronize(s)) != cudaSuccess) return e;
-            int digit[8], nd = 0;
-            for (int d = 0; d < 8; ++d) {
-                bool trivial = false;
-                for (int b = 0; b < 256; ++b)
-                    if (h_g[d * 256 + b] == (unsigned long long)n) trivial = true;
-                if (!trivial) digit[nd++] = d;
-            }
-            // The highest RS_DIGITS digits decide the order of all but a few lines (28 mantissa
-            // bits where the wavenumbers span several powers of two: 3e-5 cm^-1 at 10^4 cm^-1);
-            // the runs they leave are sorted in place.  Three passes of eight fewer.
-            const int first = whole || nd <= RS_DIGITS ? 0 : nd - RS_DIGITS;
             for (int q = first; q < nd; ++q) {
                 const int shift = 8 * digit[q];
                 k_rs_tile_hist<<<n_tiles, RS_THREADS, 0, s>>>(k0, n, shift, hist, n_tiles);
@@ -457,8 +525,12 @@ cudaError_t launch_sort_lines(const LinesDev &in, size_t n, bool assume_sorted, 
                 uint32_t *tv = v0; v0 = v1; v1 = tv;
             }
             if (first > 0) {
-                k_rs_finish_runs<<<grid_for(n, 16), 256, 0, s>>>(k0, v0, n, 8 * digit[first], d_flag);
-                ++*launches;
+                // the other key buffer is free: the long runs' list; their number beside the flag
+                uint32_t *list = reinterpret_cast<uint32_t *>(k1), *count = reinterpret_cast<uint32_t *>(d_flag + 1);
+                const int shift = 8 * digit[first];
+                k_rs_finish_runs<<<grid_for(n, 16), 256, 0, s>>>(k0, v0, n, shift, count, list);
+                k_rs_sort_run<<<152 * 4, 256, 0, s>>>(k0, v0, n, shift, count, list, d_flag);
+                *launches += 2;
             }
             if ((e = cudaGetLastError()) != cudaSuccess) return e;
             if (ev) cudaEventRecord(ev[1], s);
@@ -469,18 +541,13 @@ cudaError_t launch_sort_lines(const LinesDev &in, size_t n, bool assume_sorted, 
                 k_gather_lines<<<grid_for(n), 256, 0, s>>>(in, n, k0, v0, nu, elower, A, gref, nT, g, j);
             ++*launches;
             if (ev) cudaEventRecord(ev[2], s);
-            if (first == 0) break;
-            int f = 0;
-            if ((e = cudaMemcpyAsync(&f, d_flag, sizeof(int), cudaMemcpyDeviceToHost, s)) != cudaSuccess) return e;
+            // the flag with the gather already on its way: a list that needs another round gathers twice
+            if ((e = cudaMemcpyAsync(&h_flag, d_flag, sizeof(int), cudaMemcpyDeviceToHost, s)) != cudaSuccess) return e;
             if ((e = cudaStreamSynchronize(s)) != cudaSuccess) return e;
-            if (!(f & 4)) break;
-            whole = true;   // a long run: once more, by every digit
+            if (first == 0 || !(h_flag & 4)) break;
+            first = 0;   // once more, by every digit: equal keys are in input order here too
         }
     }
-    if ((e = cudaGetLastError()) != cudaSuccess) return e;
-    int h_flag = 0;
-    if ((e = cudaMemcpyAsync(&h_flag, d_flag, sizeof(int), cudaMemcpyDeviceToHost, s)) != cudaSuccess) return e;
-    if ((e = cudaStreamSynchronize(s)) != cudaSuccess) return e;
     // the packed records of a very large list are given back
     if (tmp[5].bytes > ((size_t)4 << 30)) tmp[5].release();
     *bad_input = (h_flag & 1) != 0;

@@ -236,3 +236,29 @@ def test_partition_function_of_many_states(xc, oracle_lib, n, nT):
     for t, q, d in zip(T, Q, dQ):
         rq, rd = oracle_lib.partition_function(E, g, t)
         assert abs(q - rq) <= 1e-13 * rq and abs(d - rd) <= 1e-13 * max(abs(rd), 1e-300), (n, t)
+
+
+# ------------------------------------------------------------------ sort: runs of keys that agree in their high digits
+@pytest.mark.parametrize("lengths,equal", [((2, 63, 64, 65, 66, 127, 128, 129, 255, 256, 257, 1000, 2047, 2048), False),
+                                           ((100, 2049), False), ((300,) * 700, False), ((65, 2048, 5000, 40_000), True),
+                                           ((70_000,), True), ((66_000,), False)])
+def test_sort_of_long_runs(eng, xc, lengths, equal):  # noqa: F811
+    """Runs at the limits of the forms that finish them (64 keys by a thread, 2048 by a CTA, longer by every
+    digit), out of order or all equal, between lines of their own: the stable order, bit for bit."""
+    rng = np.random.default_rng(len(lengths) + sum(lengths))
+    n = sum(lengths) + 20_000
+    L = xs.gen_lines(319, 0, n, 1.0, 9000.0)
+    nu, at = L["nu"], 20_000
+    nu[:20_000] = np.sort(rng.uniform(1.0, 9000.0, 20_000))
+    for i, m in enumerate(lengths):
+        low = np.zeros(m) if equal else rng.integers(0, 2 ** 20, m) * 2.0 ** -40
+        nu[at:at + m] = 2048.0 + 4.0 * i + low      # 2^-40 of 2048..8191: below the 28 leading mantissa bits
+        at += m
+    p = rng.permutation(n)
+    L = {k: v[p] for k, v in L.items()}
+    eng.load_lines(L)
+    order = np.argsort(L["nu"], kind="stable")
+    assert np.array_equal(eng.get_permutation(), order.astype(np.uint32))
+    got = eng.get_lines()
+    for k in L:
+        assert np.array_equal(got[k], L[k][order]), k
