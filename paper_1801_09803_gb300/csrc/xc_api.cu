@@ -881,6 +881,7 @@ xc_status xc_cross_section_batched(xc_handle *h, const xc_condition *conds, size
         if (opts->profile == XC_VOIGT_W4) h->kernel_ms[2] = h->last_ms[ST_RANGES];
         cudaGetLastError();
     }
+    batched_trim(&h->batched);
     return XC_OK;
 }
 
@@ -1026,7 +1027,9 @@ xc_status xc_count_far_evals(xc_handle *h, const xc_condition *conds, size_t n_c
     a.grid = *grid;
     a.opts = *opts;
     a.stream = s;
-    return batched_count_far(&h->batched, a, count_out);
+    st = batched_count_far(&h->batched, a, count_out);
+    if (!st) batched_trim(&h->batched);   // (it has synchronised)
+    return st;
 }
 
 xc_status xc_set_tile_shape(xc_handle *h, int R, int CG) {

@@ -2130,6 +2130,14 @@ xc_status batched_count_far(BatchedState *st, const BatchedArgs &args, int64_t *
     return XC_OK;
 }
 
+void batched_trim(BatchedState *st) {
+    if (st->tiles.bytes <= kMaxKeptBytes) return;
+    st->tiles.release();
+    st->tc_status = nullptr;   // these lie in it
+    st->tc_blk_lo = st->tc_blk_hi = nullptr;
+    st->tc_n_blk = st->tc_groups = 0;
+}
+
 void batched_invalidate(BatchedState *st) {
     for (auto &kv : st->graphs) {
         if (kv.second.exec) cudaGraphExecDestroy(kv.second.exec);

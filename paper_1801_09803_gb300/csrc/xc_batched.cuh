@@ -185,6 +185,10 @@ int64_t batched_tc_mma_count(BatchedState *st);
 // (line, grid point, condition) evaluations the tensor-core far-wing kernel takes in a
 // batched call with these arguments (0 when that kernel would not run); synchronises
 xc_status batched_count_far(BatchedState *st, const BatchedArgs &a, int64_t *count);
+// after a call's stream has synchronised and its counters are read: scratch above kMaxKeptBytes is given back,
+// so that what a handle keeps between calls is bounded whatever the lists it has seen (1e9 lines want 48 GB)
+constexpr size_t kMaxKeptBytes = (size_t)16 << 30;
+void batched_trim(BatchedState *st);
 void batched_invalidate(BatchedState *st);
 void batched_release(BatchedState *st);
 

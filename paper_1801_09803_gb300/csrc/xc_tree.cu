@@ -1159,7 +1159,9 @@ int warps_per_task(int64_t tasks, int most = TR_W) {
     return w;
 }
 
-constexpr size_t kMaxRecBytes = (size_t)24 << 30;   // profile constants held at a time
+// Profile constants held at a time: 32 conditions of 1e7 lines, four of 1e8.  (More buys nothing: a pass
+// over the lines for four conditions is far longer than its launches.)
+constexpr size_t kMaxRecBytes = (size_t)12 << 30;
 
 }  // namespace
 

@@ -262,3 +262,21 @@ def test_sort_of_long_runs(eng, xc, lengths, equal):  # noqa: F811
     got = eng.get_lines()
     for k in L:
         assert np.array_equal(got[k], L[k][order]), k
+
+
+def test_scratch_of_a_large_list_is_given_back(xc):
+    """4e8 lines want 19 GB of scratch for one condition: after the call the handle keeps none of it, and the
+    next call of the same shape gives the same bits."""
+    n = 400_000_000
+    with xc.Engine(0) as e:
+        e.load_lines(xs.gen_lines_torch(320, 0, n, 990.0, 3010.0, device="cuda:0"))
+        e.set_states(*xs.gen_states(320, 100))
+        torch.cuda.synchronize()
+        torch.cuda.empty_cache()
+        call = lambda: e.cross_section_batched([xc.make_condition(900.0, 0.1)], xc.make_grid(2000.0, 0.01, 501),  # noqa: E731
+                                               xc.make_opts("voigt_w4", "fp32", 1.0))
+        free = torch.cuda.mem_get_info()[0]
+        a = call()
+        assert "block-interpolated" in e.tuning()
+        assert free - torch.cuda.mem_get_info()[0] < 1 << 30
+        assert np.array_equal(a, call()) and a.min() > 0
