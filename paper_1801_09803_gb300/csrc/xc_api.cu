@@ -125,6 +125,16 @@ struct DeviceGuard {
     }
 };
 
+// A call that fails waits for what it has launched: the handle's buffers and constants may be used by the
+// next call on another stream.
+struct Settle {
+    cudaStream_t s;
+    bool done = false;
+    ~Settle() {
+        if (!done) cudaStreamSynchronize(s);
+    }
+};
+
 inline cudaStream_t S(void *s) { return static_cast<cudaStream_t>(s); }
 
 void stage_begin(xc_handle *h, int st, cudaStream_t s) {
@@ -815,6 +825,7 @@ xc_status xc_cross_section_batched(xc_handle *h, const xc_condition *conds, size
     bool anyQ = false;
     for (size_t c = 0; c < n_cond; ++c) anyQ |= conds[c].Q <= 0.0;
     used[ST_Q] = anyQ;
+    Settle settle{s};
     CondDev *dc = nullptr;
     if ((st = resolve_conds(h, conds, n_cond, s, &dc))) return st;
     if (opts->precision == XC_FP64_PLAIN || h->n_lines == 0) {
@@ -882,6 +893,7 @@ xc_status xc_cross_section_batched(xc_handle *h, const xc_condition *conds, size
         cudaGetLastError();
     }
     batched_trim(&h->batched);
+    settle.done = true;
     return XC_OK;
 }
 
@@ -917,6 +929,7 @@ static xc_status vjp_common(xc_handle *h, const xc_condition *conds, size_t n_co
     a.grid = *grid;
     a.opts = *opts;
     a.stream = s;
+    Settle settle{s};
     CondDev *dc = nullptr;
     if (n_cond) {
         if ((st = resolve_conds(h, conds, n_cond, s, &dc))) return st;
@@ -948,6 +961,7 @@ static xc_status vjp_common(xc_handle *h, const xc_condition *conds, size_t n_co
     used[ST_VJP] = true;
     XC_TRY(cudaStreamSynchronize(s));
     collect_timing(h, used);
+    settle.done = true;
     return XC_OK;
 }
 

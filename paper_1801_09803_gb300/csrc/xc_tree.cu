@@ -30,6 +30,7 @@
 
 #include "xc_batched.cuh"
 #include "xc_f32.cuh"
+#include "xc_once.h"
 #include "xc_tree.cuh"
 
 namespace xc {
@@ -262,19 +263,12 @@ cudaError_t launch_fp32_setup(const LinesDev &L, size_t n, const CondDev *conds,
     return cudaGetLastError();
 }
 
-// the handle's interpolation matrices (constants), made by its first call that needs them; that
-// call synchronises its stream before it returns
+// the handle's interpolation matrices (constants), made by its first call that needs them
 cudaError_t tree_mat(BatchedState *st, const double **mat, cudaStream_t s) {
+    const cudaError_t e = make_once(st->tree_mat, TR_MAT * sizeof(double),
+                                    [&] { return launch_tree_mat(st->tree_mat.as<double>(), s); });
     *mat = st->tree_mat.as<double>();
-    if (*mat) return cudaSuccess;
-    cudaError_t e = st->tree_mat.ensure(TR_MAT * sizeof(double));
-    if (e == cudaSuccess) e = launch_tree_mat(st->tree_mat.as<double>(), s);
-    if (e != cudaSuccess) {
-        st->tree_mat.release();
-        return e;
-    }
-    *mat = st->tree_mat.as<double>();
-    return cudaSuccess;
+    return e;
 }
 
 cudaError_t launch_tree_mat(double *mat, cudaStream_t s) {

@@ -23,6 +23,7 @@
 #include <algorithm>
 
 #include "xc_internal.cuh"
+#include "xc_once.h"
 #include "xc_profile64.cuh"
 #include "xc_tree.cuh"
 
@@ -138,14 +139,12 @@ __global__ void __launch_bounds__(64) k_t64_mat(double *mat) {
     }
 }
 
-// the handle's interpolation matrices (constants), made by its first call that needs them; that
-// call synchronises its stream before it returns
+// the handle's interpolation matrices (constants), made by its first call that needs them
 cudaError_t tree64_mat(DevBuf *buf, cudaStream_t s) {
-    if (buf->p) return cudaSuccess;
-    const cudaError_t e = buf->ensure((size_t)T64_MAT * sizeof(double));
-    if (e != cudaSuccess) return e;
-    k_t64_mat<<<(T64_MAT_DV + 63) / 64, 64, 0, s>>>(buf->as<double>());
-    return cudaGetLastError();
+    return make_once(*buf, (size_t)T64_MAT * sizeof(double), [&] {
+        k_t64_mat<<<(T64_MAT_DV + 63) / 64, 64, 0, s>>>(buf->as<double>());
+        return cudaGetLastError();
+    });
 }
 
 // w4 region I in u = D^2: I V = P (u + C) / (u^2 + E u + C^2), with s = alpha^2 / ln 2,
