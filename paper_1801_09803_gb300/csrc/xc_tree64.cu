@@ -167,14 +167,6 @@ __device__ __forceinline__ W4Line t64_line(const T64Params &p, size_t l) {
     return w;
 }
 
-// 1/d to a last-place error: the hardware's approximation (2^-20 or better) and two Newton steps
-__device__ __forceinline__ double t64_rcp(double d) {
-    double r;
-    asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(d));
-    r = fma(r, fma(-d, r, 1.0), r);
-    return fma(r, fma(-d, r, 1.0), r);
-}
-
 // ---------------------------------------------------------------------------
 // nodes: a warp owns a block, a lane a node
 // ---------------------------------------------------------------------------
@@ -229,7 +221,7 @@ __global__ void __launch_bounds__(32 * T64_NW) k_t64_nodes(T64Params q) {
         }
         const double D01 = Dn[0] * Dn[1], D23 = Dn[2] * Dn[3];
         const double N01 = fma(N[0], Dn[1], N[1] * Dn[0]), N23 = fma(N[2], Dn[3], N[3] * Dn[2]);
-        acc = fma(fma(N01, D23, N23 * D01), t64_rcp(D01 * D23), acc);
+        acc = fma(fma(N01, D23, N23 * D01), rcp64(D01 * D23), acc);
     };
 #pragma unroll 1
     for (int k = 0; k < 4; ++k) {
@@ -291,7 +283,7 @@ __global__ void __launch_bounds__(32 * T64_NW) k_t64_nodes(T64Params q) {
     for (int j = 0; W4 && j < held; ++j) {
         const double *w = buf + 5 * j;
         const double d = (xh - w[0]) + xl, u = d * d;
-        acc = fma(fma(w[3], u, w[4]), t64_rcp(fma(u, u + w[1], w[2])), acc);
+        acc = fma(fma(w[3], u, w[4]), rcp64(fma(u, u + w[1], w[2])), acc);
     }
     p.nodes[p.node_off[lev] + task * T64_M + lane] = acc;
     if (lane == 0) q.count[(lev ? 0 : p.nblk[1]) + task] = taken;
@@ -396,7 +388,7 @@ __device__ __forceinline__ double t64_region2(double X, double y, double Y) {
     const double Z = X + Y, t1 = Z - Q1, t2 = Z - Q2;
     const double D1 = fma(t1, t1, 4.0 * Q1 * Y), D2 = fma(t2, t2, 4.0 * Q2 * Y);
     const double N1 = A1 * (Z + Q1), N2 = A2 * (Z + Q2);
-    return y * fma(N1, D2, N2 * D1) * t64_rcp(D1 * D2);
+    return y * fma(N1, D2, N2 * D1) * rcp64(D1 * D2);
 }
 
 // region III: real coefficients, so two operations each by division through (z - t)(z - conj t)
@@ -411,7 +403,7 @@ __device__ __forceinline__ double t64_region3(double x, double y) {
     const double d1 = fma(r, d2, fma(-s, d3, 38.82363));
     const double Nr = fma(y, n1, fma(-s, n2, 16.4955)), Dr = fma(y, d1, fma(-s, d2, 16.4955));
     const double Ni = x * n1, Di = x * d1;
-    return fma(Nr, Dr, Ni * Di) * t64_rcp(fma(Dr, Dr, Di * Di));
+    return fma(Nr, Dr, Ni * Di) * rcp64(fma(Dr, Dr, Di * Di));
 }
 
 // region IV, real part only (no sine)
@@ -422,7 +414,7 @@ __device__ __forceinline__ double t64_region4(double x, double y) {
     const Z N = 36183.31 + m * (3321.9905 + m * (1540.787 + m * (219.0313 + m * (35.76683 + m * (1.320522 + 0.56419 * m)))));
     const Z D = 32066.6 + m * (24322.84 + m * (9022.228 + m * (2186.181 + m * (364.2191 + m * (61.57037 +
                 m * (1.841439 + m))))));
-    const double d = t64_rcp(D.re * D.re + D.im * D.im);
+    const double d = rcp64(D.re * D.re + D.im * D.im);
     const double rr = (N.re * D.re + N.im * D.im) * d, ri = (N.im * D.re - N.re * D.im) * d;
     return exp64(ur) * cos(ui) - (y * rr + x * ri);   // t = y - i x
 }
@@ -561,7 +553,7 @@ __global__ void __launch_bounds__(128) k_t64_points_w4(T64Params q) {
                 for (int j = 0; j < 4; ++j) one(j4 + j, N[j], Dn[j]);
                 const double D01 = Dn[0] * Dn[1], D23 = Dn[2] * Dn[3];
                 const double N01 = fma(N[0], Dn[1], N[1] * Dn[0]), N23 = fma(N[2], Dn[3], N[3] * Dn[2]);
-                accF = fma(fma(N01, D23, N23 * D01), t64_rcp(D01 * D23), accF);
+                accF = fma(fma(N01, D23, N23 * D01), rcp64(D01 * D23), accF);
             }
             if (j4) {   // the lines left over move to the front
                 const int rest = held - j4;
@@ -581,7 +573,7 @@ __global__ void __launch_bounds__(128) k_t64_points_w4(T64Params q) {
                 double v = 0.0;
                 if (__any_sync(0xffffffffu, in && !first)) v = b[7] * t64_region2(x * x, y, y * y);
                 if (__any_sync(0xffffffffu, in && first)) {
-                    const double v1 = fma(b[3], u, b[4]) * t64_rcp(fma(u, u + b[1], b[2]));
+                    const double v1 = fma(b[3], u, b[4]) * rcp64(fma(u, u + b[1], b[2]));
                     v = first ? v1 : v;
                 }
                 if (in) accZ += v;
@@ -621,7 +613,7 @@ __global__ void __launch_bounds__(128) k_t64_points_w4(T64Params q) {
     for (int j = 0; j < held; ++j) {
         double N, Dn;
         one(j, N, Dn);
-        accF = fma(N, t64_rcp(Dn), accF);
+        accF = fma(N, rcp64(Dn), accF);
     }
     t64_finish(q, far, task >> 2, (task & 3) * 32 + lane, s0 + lane, lane, (accF + accZ) + (acc34[0] + acc34[1]));
 }

@@ -280,3 +280,30 @@ def test_scratch_of_a_large_list_is_given_back(xc):
         assert "block-interpolated" in e.tuning()
         assert free - torch.cuda.mem_get_info()[0] < 1 << 30
         assert np.array_equal(a, call()) and a.min() > 0
+
+
+def test_tensor_core_far_wings_of_long_cuts(eng, xc):  # noqa: F811
+    """At cuts the blocks take by themselves a fixed tile shape still runs the far wings on the tensor cores:
+    against the tiled form without them and against the blocks (2e-5 as between any two FP32 paths)."""
+    L = xs.gen_lines(321, 0, 30_000, 1000.0, 1100.0)
+    eng.load_lines(L)
+    eng.set_states(*xs.gen_states(321, 500))
+    conds = [xc.make_condition(300.0 + 60.0 * i, 1e-3 * 1.33 ** i) for i in range(32)]
+    grid = xc.make_grid(1000.0, 0.01, 10_001)
+    blocks = eng.cross_section_batched(conds, grid, xc.make_opts("voigt_w4", "fp32", 25.0))
+    assert "block-interpolated" in eng.tuning()
+    eng.set_timing(True)
+    eng.set_tile_shape(4, 16)
+    try:
+        tc = eng.cross_section_batched(conds, grid, xc.make_opts("voigt_w4", "fp32", 25.0))
+        far_ms, _, _, mma = eng.sweep_kernels()
+        far = eng.count_far_evals(conds, grid, xc.make_opts("voigt_w4", "fp32", 25.0))
+        cores = eng.cross_section_batched(conds, grid, xc.make_opts("voigt_w4", "fp32", 25.0, tensor_cores=False))
+        assert eng.sweep_kernels()[3] == 0
+    finally:
+        eng.set_tile_shape(0, 0)
+        eng.set_timing(False)
+    assert mma > 0 and far > 0 and far_ms > 0
+    for ref in (cores, blocks):
+        m = ref > 1e-6 * ref.max(axis=1, keepdims=True)
+        assert np.max(np.abs(tc - ref)[m] / ref[m]) < 2e-5
