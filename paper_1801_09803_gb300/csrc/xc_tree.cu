@@ -276,13 +276,15 @@ cudaError_t launch_tree_mat(double *mat, cudaStream_t s) {
     return cudaGetLastError();
 }
 
-// profile constants of every (condition, line) of the group
+// profile constants of the group's conditions, for the lines that can reach the grid (a contiguous range of
+// the sorted list: 32 conditions of a 301-point Lorentz window in 1e7 lines 2.55 ms with all lines', 0.69 so)
 template <int PROF, bool EXT>
 __global__ void __launch_bounds__(256) k_tree_recs(TreeParams p, float4 *recA, float4 *recB) {
     const int c = blockIdx.y;
     const CParam cp = p.cp[p.c0 + c];
     const float h = (float)p.step;
-    for (size_t l = (size_t)blockIdx.x * 256 + threadIdx.x; l < p.n; l += (size_t)gridDim.x * 256) {
+    const size_t l1 = tr_upper(p, p.n_pts + p.reach + 1);
+    for (size_t l = tr_lower(p, -p.reach) + (size_t)blockIdx.x * 256 + threadIdx.x; l < l1; l += (size_t)gridDim.x * 256) {
         float4 A, B = make_float4(0.f, 0.f, 0.f, -1.f), S;
         float t2;
         line_consts<PROF, EXT>(p.L, l, cp, h, p.inv_h, &A, &B, &t2, &S);

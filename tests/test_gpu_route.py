@@ -307,3 +307,22 @@ def test_tensor_core_far_wings_of_long_cuts(eng, xc):  # noqa: F811
     for ref in (cores, blocks):
         m = ref > 1e-6 * ref.max(axis=1, keepdims=True)
         assert np.max(np.abs(tc - ref)[m] / ref[m]) < 2e-5
+
+
+@pytest.mark.parametrize("profile", ["voigt_w4", "lorentz", "doppler_binned", "voigt_gh_binned"])
+@pytest.mark.parametrize("cut,wm", [(0.3, 0.0), (25.0, 0.0), (25.0, 300.0)])
+def test_windows_inside_a_long_list(eng, xc, profile, cut, wm):  # noqa: F811
+    """A narrow grid in a list that reaches far beyond it on both sides, and at either end of the list:
+    constants are made for the lines in reach only (2e-5 of the general path)."""
+    eng.load_lines(xs.gen_lines(322, 0, 60_000, 1000.0, 2000.0))
+    eng.set_states(*xs.gen_states(322, 300))
+    conds = [xc.make_condition(T, P) for T, P in ((400.0, 0.01), (1200.0, 0.5), (2600.0, 3.0))]
+    for nu_A in (900.0, 974.5, 1000.0, 1500.37, 1999.0, 2030.0):
+        grid, opts = xc.make_grid(nu_A, 0.01, 333), xc.make_opts(profile, "fp32", cut, wm)
+        got = eng.cross_section_batched(conds, grid, opts)
+        assert "block-interpolated" in eng.tuning()
+        eng.set_tile_shape(8, 1)
+        ref = eng.cross_section_batched(conds, grid, opts)
+        eng.set_tile_shape(0, 0)
+        m = ref > 1e-6 * ref.max(axis=1, keepdims=True)
+        assert not m.any() or np.max(np.abs(got - ref)[m] / ref[m]) < 2e-5, nu_A
