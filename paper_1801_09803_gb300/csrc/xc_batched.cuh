@@ -147,7 +147,8 @@ struct GraphEntry {
 };
 
 struct BatchedState {
-    DevBuf tiles;      // tile table (window, group, line range, cost order)
+    DevBuf tiles;      // tile table (window, group, line range, cost order); the blocks' scratch
+    size_t tiles_need = 0;   // bytes of it that the last call used
     DevBuf cparams;    // per-condition constants
     DevBuf counter;    // work-queue counter
     DevBuf vjp_buf;    // adjoint scratch
@@ -185,10 +186,11 @@ int64_t batched_tc_mma_count(BatchedState *st);
 // (line, grid point, condition) evaluations the tensor-core far-wing kernel takes in a
 // batched call with these arguments (0 when that kernel would not run); synchronises
 xc_status batched_count_far(BatchedState *st, const BatchedArgs &a, int64_t *count);
-// after a call's stream has synchronised and its counters are read: scratch above kMaxKeptBytes is given back,
-// so that what a handle keeps between calls is bounded whatever the lists it has seen (1e9 lines want 48 GB)
+// Scratch above kMaxKeptBytes (1e9 lines want 48 GB) stays with its handle only while calls use most of it:
+// it is given back when a call has needed less than half of it, and when a list is loaded.  (After every call
+// it would cost 0.5 ms a GB: 4 % of a call on 1e9 lines.)  The stream has synchronised, counters are read.
 constexpr size_t kMaxKeptBytes = (size_t)16 << 30;
-void batched_trim(BatchedState *st);
+void batched_trim(BatchedState *st, bool loading = false);
 void batched_invalidate(BatchedState *st);
 void batched_release(BatchedState *st);
 

@@ -1155,9 +1155,10 @@ int warps_per_task(int64_t tasks, int most = TR_W) {
     return w;
 }
 
-// Profile constants held at a time: 32 conditions of 1e7 lines, four of 1e8.  (More buys nothing: a pass
-// over the lines for four conditions is far longer than its launches.)
-constexpr size_t kMaxRecBytes = (size_t)12 << 30;
+// Profile constants held at a time: 32 conditions of 1e7 lines, eight of 1e8 (four, 12 GB: 1067 ms for 32
+// conditions instead of 1041), and no more than half of what the device has free, so that a neighbour
+// in the process finds room.
+constexpr size_t kMaxRecBytes = (size_t)24 << 30;
 
 }  // namespace
 
@@ -1222,6 +1223,12 @@ xc_status tree_run(BatchedState *st, const BatchedArgs &a, int64_t *launches) {
     }
     p.nodes_per_cond = off;
 
+    const size_t rec = n * (w4 ? 32 : 16);
+    if ((size_t)cg * rec > st->tiles.bytes) {
+        size_t room = 0, total = 0;
+        if (cudaMemGetInfo(&room, &total) != cudaSuccess) cudaGetLastError();
+        else cg = (int)std::min<size_t>((size_t)cg, std::max<size_t>(1, (room + st->tiles.bytes) / 2 / rec));
+    }
     if (cg < nc_pass && cg > 4) cg &= ~3;   // whole groups of four
     size_t o = 0, o_gs, o_cp, o_cell, o_nodes, o_geo, o_A, o_B, o_keep = 0, o_glc = 0;
     auto carve = [&](size_t bytes) { size_t r = o; o += (bytes + 255) & ~size_t(255); return r; };
@@ -1242,6 +1249,7 @@ xc_status tree_run(BatchedState *st, const BatchedArgs &a, int64_t *launches) {
             continue;
         }
         TR_TRY(e);   // out of memory here: the caller falls back to the tiled kernels
+        st->tiles_need = o;
         break;
     }
     char *b = st->tiles.as<char>();

@@ -410,6 +410,8 @@ __device__ __forceinline__ F2 f2_scale(F2 a, float k) {
 __device__ __forceinline__ F2 f2_of(const KahanF &k) { return F2{k.s, -k.c}; }
 
 // Sums of one line and condition over grid points or block nodes, without their constant
+// (q1 and q2 hold terms that fall as the fourth power of the distance: interpolated from 16 nodes these are
+// good to 2.3e-6 of the value at a block's far end, 1.2e-7 of the near end's; q0's to 1.4e-8)
 // factors, and the profile's constants in grid units.
 template <int PROF>
 struct VjpLine {

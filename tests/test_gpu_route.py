@@ -265,21 +265,30 @@ def test_sort_of_long_runs(eng, xc, lengths, equal):  # noqa: F811
 
 
 def test_scratch_of_a_large_list_is_given_back(xc):
-    """4e8 lines want 19 GB of scratch for one condition: after the call the handle keeps none of it, and the
-    next call of the same shape gives the same bits."""
+    """4e8 lines want 19 GB of scratch for one condition: it stays while calls need it, and goes when a call needs
+    less than half of it or a list is loaded; the same call then gives the same bits."""
     n = 400_000_000
     with xc.Engine(0) as e:
         e.load_lines(xs.gen_lines_torch(320, 0, n, 990.0, 3010.0, device="cuda:0"))
         e.set_states(*xs.gen_states(320, 100))
         torch.cuda.synchronize()
         torch.cuda.empty_cache()
-        call = lambda: e.cross_section_batched([xc.make_condition(900.0, 0.1)], xc.make_grid(2000.0, 0.01, 501),  # noqa: E731
-                                               xc.make_opts("voigt_w4", "fp32", 1.0))
+
+        def call(profile="voigt_w4"):
+            out = e.cross_section_batched([xc.make_condition(900.0, 0.1)], xc.make_grid(2000.0, 0.01, 501),
+                                          xc.make_opts(profile, "fp32", 1.0))
+            return out, free - torch.cuda.mem_get_info()[0]
         free = torch.cuda.mem_get_info()[0]
-        a = call()
-        assert "block-interpolated" in e.tuning()
+        a, held = call()
+        assert "block-interpolated" in e.tuning() and held > 17 << 30
+        b, held = call()
+        assert np.array_equal(a, b) and a.min() > 0 and held > 17 << 30
+        e.set_tile_shape(8, 1)       # 16 bytes a line
+        assert call()[1] < 1 << 30
+        e.set_tile_shape(0, 0)
+        assert np.array_equal(a, call()[0])
+        e.load_lines(xs.gen_lines(320, 0, 1000, 990.0, 3010.0))
         assert free - torch.cuda.mem_get_info()[0] < 1 << 30
-        assert np.array_equal(a, call()) and a.min() > 0
 
 
 def test_tensor_core_far_wings_of_long_cuts(eng, xc):  # noqa: F811
