@@ -78,11 +78,11 @@ enum {
 /* xc_load_lines flags */
 enum { XC_ASSUME_SORTED = 1u };
 
-/* xc_opts.flags.  With XC_FP32, Voigt w4, 16 or more conditions and a fixed cut of fewer than
- * 1024 grid steps, small lists (lines x conditions < 2^19) have the far wings (points at least
- * D(l, c) grid steps from a line, D chosen so that the region-I rational equals its four-term
- * series in 1/u to < 2e-7) summed on the tensor cores as a matrix product (TF32 operands, FP32
- * accumulation); XC_OPT_NO_TENSOR_CORES keeps every evaluation on the CUDA cores. */
+/* xc_opts.flags.  With XC_FP32, Voigt w4, 16 or more conditions, a fixed cut and fewer than 2^23
+ * grid points, a call that runs the tiled kernels (see xc_cross_section_batched) has the far wings
+ * (points at least D(l, c) grid steps from a line, D chosen so that the region-I rational equals its
+ * four-term series in 1/u to < 2e-7) summed on the tensor cores as a matrix product (TF32 operands,
+ * FP32 accumulation); XC_OPT_NO_TENSOR_CORES keeps every evaluation on the CUDA cores. */
 enum { XC_OPT_NO_TENSOR_CORES = 1 };
 
 /* xc_opts.quantity: what each line contributes, times its profile */
@@ -261,10 +261,14 @@ xc_status xc_cross_section(xc_handle *h, const xc_condition *cond, const xc_grid
 
 /* n_cond conditions (sigma_out: float64[n_cond][grid->n], condition-major).  Far from its centre
  * a profile is summed at the Chebyshev nodes of blocks of the grid and the sums are
- * interpolated to the points (within 2e-8 of each value in FP32, 1e-16 in FP64); XC_FP32 takes
- * up to four conditions per scan of the lines.  The Vectorized Voigt, a fixed tile shape
- * (xc_set_tile_shape) and calls whose scratch would not fit run the tiled kernels (FP32: window
- * size picked by the autotuner and cached per shape, the sweep captured into a CUDA graph). */
+ * interpolated to the points (truncation within 2e-8 of each value in FP32, 1e-16 in FP64, where
+ * rounding adds about 1e-15 of a single line's value); the FP32 Voigt w4 takes up to four conditions per
+ * scan of the lines.  FP32 calls that run the tiled kernels instead: the Vectorized Voigt, a fixed tile
+ * shape (xc_set_tile_shape), lists that are sparse for the grid and conditions, with 16 or more
+ * conditions also short cuts (< 1024 steps) of small lists (lines x conditions < 2^19), cuts of 2^20
+ * steps and more, 2^30 points and more, 1.6e9 lines and more, and calls whose scratch would not fit.
+ * Tiled: window size by rule (sparse lists) or by the autotuner, cached per shape; a fixed cut's sweep is
+ * captured into a CUDA graph.  Scratch above 16 GB is given back when the call has finished. */
 xc_status xc_cross_section_batched(xc_handle *h, const xc_condition *conds, size_t n_cond,
                                    const xc_grid *grid, const xc_opts *opts, double *sigma_out,
                                    int mem, void *stream);
