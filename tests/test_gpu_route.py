@@ -335,3 +335,26 @@ def test_windows_inside_a_long_list(eng, xc, profile, cut, wm):  # noqa: F811
         eng.set_tile_shape(0, 0)
         m = ref > 1e-6 * ref.max(axis=1, keepdims=True)
         assert not m.any() or np.max(np.abs(got - ref)[m] / ref[m]) < 2e-5, nu_A
+
+
+@pytest.mark.parametrize("wm", [0.0, 300.0])
+@pytest.mark.parametrize("profile,n_lines,n", [("voigt_w4", 15_000, 4003), ("lorentz", 15_000, 4003),
+                                               ("voigt_gh_binned", 3000, 2003), ("voigt_w4", 200, 150_003),
+                                               ("doppler", 3000, 2003)])
+def test_adjoint_under_a_mixture_sparse_and_dense(eng, xc, profile, n_lines, n, wm):  # noqa: F811
+    """The mixture's adjoint kernels with and without blocks, fixed and width-limited cuts, 35 conditions (two
+    launches): FP32 against FP64, 1e-4 of the largest."""
+    eng.load_lines(xs.gen_lines(323, 0, n_lines, 2995.0, 3005.0 + 0.01 * n))
+    eng.set_states(*xs.gen_states(323, 300))
+    eng.set_broadening([xc.make_broadener("constant", 0.6, 0.05, 0.6), xc.make_broadener("constant", 0.4, 0.09, 0.4)])
+    conds = [xc.make_condition(500.0 + 30.0 * i, 0.02 * 1.1 ** i) for i in range(35)]
+    w = 1e22 * np.random.default_rng(323).uniform(0.5, 1.5, (35, n))
+    grid = xc.make_grid(3000.0, 0.01, n)
+    try:
+        r32, r64 = (eng.cross_section_vjp_broadening(conds, grid, xc.make_opts(profile, p, 5.0, wm), w, 2)
+                    for p in ("fp32", "fp64"))
+    finally:
+        eng.set_broadening([])
+    for k in ("dT", "dP", "d_gamma_scale", "d_n_shift", "d_gamma0_broad", "d_n_broad"):
+        a, b = np.asarray(r32[k]), np.asarray(r64[k])
+        assert np.max(np.abs(a - b)) <= 1e-4 * max(np.max(np.abs(b)), 1e-300), k
