@@ -152,7 +152,8 @@ __device__ inline void gh_binned_deriv64(double D, double h, double al, double g
     for (int j = 0; j < n; ++j) {
         const double xs = x[j] / kSqrtLn2;
         const double sp = D + 0.5 * h - al * xs, sm = sp - h;
-        const double iQ = 1.0 / ((sp * sp + g2) * (sm * sm + g2));
+        // (gamma = 0, a bin's edge exactly on a node: the derivatives have a pole there, taken as 0)
+        const double Q = (sp * sp + g2) * (sm * sm + g2), iQ = Q > 0.0 ? 1.0 / Q : 0.0;
         v += w[j] * atan2(ga * h, g2 + sp * sm);
         dg += w[j] * h * (sp * sm - g2) * iQ;
         da += w[j] * xs * ga * h * (sp + sm) * iQ;
@@ -452,7 +453,8 @@ struct VjpLine {
             float v = 0.f, da = 0.f, dg = 0.f;
             for (int m = 0; m < ngh; ++m) {
                 const float sp = fmaf(-a_h, gx[m], d), sm = sp - 1.f;
-                const float iQ = rcp_approx(fmaf(sp, sp, g2) * fmaf(sm, sm, g2));
+                const float Q = fmaf(sp, sp, g2) * fmaf(sm, sm, g2);
+                const float iQ = Q > 1e-37f ? rcp_approx(Q) : 0.f;   // a pole at gamma = 0 (see gh_binned_deriv64)
                 v = fmaf(gw[m], atan2_ypos(g_h, fmaf(sp, sm, g2)), v);
                 dg = fmaf(gw[m], fmaf(sp, sm, -g2) * iQ, dg);
                 da = fmaf(gw[m] * gx[m], (sp + sm) * iQ, da);

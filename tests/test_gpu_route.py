@@ -358,3 +358,30 @@ def test_adjoint_under_a_mixture_sparse_and_dense(eng, xc, profile, n_lines, n, 
     for k in ("dT", "dP", "d_gamma_scale", "d_n_shift", "d_gamma0_broad", "d_n_broad"):
         a, b = np.asarray(r32[k]), np.asarray(r64[k])
         assert np.max(np.abs(a - b)) <= 1e-4 * max(np.max(np.abs(b)), 1e-300), k
+
+
+@pytest.mark.parametrize("precision", ["fp32", "fp64"])
+def test_gauss_hermite_adjoint_without_pressure(eng, xc, precision):  # noqa: F811
+    """P = 0: no Lorentz width, and the derivatives of a bin whose edge lies exactly on a node have a pole
+    (a line halfway between two grid points of a binary step, one node): finite, and the neighbours' values
+    against the direct formula 1 / (s+ s-) (1e-5 FP32, 1e-12 FP64)."""
+    L = xs.gen_lines(324, 0, 1, 1000.0, 1001.0)
+    step, n, i0 = 1.0 / 128.0, 41, 20
+    L["nu"][:] = 1000.0 + (i0 + 0.5) * step
+    E, g = xs.gen_states(324, 20)
+    eng.load_lines(L)
+    eng.set_states(E, g)
+    w = np.full((1, n), 1e22)
+    cond = [xc.make_condition(296.0, 0.0)]
+    r = eng.cross_section_vjp(cond, xc.make_grid(1000.0, step, n), xc.make_opts("voigt_gh_binned", precision, 25.0, n_gh=1), w)
+    assert all(np.all(np.isfinite(np.asarray(v))) for v in r.values())
+    sp = np.arange(n) - (i0 + 0.5) + 0.5
+    sm = sp - 1.0
+    ok = sp * sm != 0
+    # dL/dP = I gamma_ref sum w / (h^2 pi) / (s+ s-), one node of weight sqrt(pi)
+    Q = xc.partition_function(E, g, [296.0])[0][0]
+    c2, f = 1.4387768775039338, {k: float(v[0]) for k, v in L.items()}
+    S = f["g_up"] * f["A"] / (8 * np.pi * 2.99792458e10 * Q * f["nu"] ** 2) * np.exp(-c2 * f["elower"] / 296.0)
+    S *= -np.expm1(-c2 * f["nu"] / 296.0)
+    ref = S * f["gamma_ref"] * 1e22 / np.pi / step ** 2 * np.sum(1.0 / (sp * sm)[ok])
+    assert abs(float(r["dP"][0]) - ref) <= (1e-5 if precision == "fp32" else 1e-12) * abs(ref)
