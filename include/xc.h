@@ -269,7 +269,7 @@ xc_status xc_cross_section(xc_handle *h, const xc_condition *cond, const xc_grid
  * steps and more, 2^30 points and more, 1.6e9 lines and more, and calls whose scratch would not fit.
  * Tiled: window size by rule (sparse lists) or by the autotuner, cached per shape; a fixed cut's sweep is
  * captured into a CUDA graph.  Scratch above 16 GB is given back after a call that needs less than half
- * of it, and by xc_load_lines. */
+ * of it, and by xc_load_lines of a list of less than half the lines. */
 xc_status xc_cross_section_batched(xc_handle *h, const xc_condition *conds, size_t n_cond,
                                    const xc_grid *grid, const xc_opts *opts, double *sigma_out,
                                    int mem, void *stream);

@@ -475,7 +475,7 @@ xc_status xc_load_lines(xc_handle *h, const xc_lines *L, size_t n, unsigned flag
     }
     h->n_lines = 0;
     h->n_broad = 0;   // a broadener mixture belongs to the lines it was set for
-    batched_trim(&h->batched, true);
+    if (2 * n < h->batched.tiles_lines) batched_trim(&h->batched, true);
     // graphs and tuning stay valid: they key on shapes and buffer addresses, and read the
     // line data when replayed
     if (n == 0) return XC_OK;

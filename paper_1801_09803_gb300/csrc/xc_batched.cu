@@ -1539,6 +1539,7 @@ xc_status make_plan(BatchedState *st, const BatchedArgs &a, const Variant *v, in
     }
     BT_TRY(st->tiles.ensure(off));
     st->tiles_need = off;
+    st->tiles_lines = n;
     char *b = st->tiles.as<char>();
     pl->n_abs = (int *)(b + o_n);
     pl->f = (float *)(b + o_f);
@@ -2131,8 +2132,8 @@ xc_status batched_count_far(BatchedState *st, const BatchedArgs &args, int64_t *
     return XC_OK;
 }
 
-void batched_trim(BatchedState *st, bool loading) {
-    if (st->tiles.bytes <= kMaxKeptBytes || (!loading && st->tiles_need > st->tiles.bytes / 2)) return;
+void batched_trim(BatchedState *st, bool smaller_list) {
+    if (st->tiles.bytes <= kMaxKeptBytes || (!smaller_list && st->tiles_need > st->tiles.bytes / 2)) return;
     st->tiles.release();
     st->tc_status = nullptr;   // these lie in it
     st->tc_blk_lo = st->tc_blk_hi = nullptr;

@@ -149,6 +149,7 @@ struct GraphEntry {
 struct BatchedState {
     DevBuf tiles;      // tile table (window, group, line range, cost order); the blocks' scratch
     size_t tiles_need = 0;   // bytes of it that the last call used
+    size_t tiles_lines = 0;  // ... and that call's lines
     DevBuf cparams;    // per-condition constants
     DevBuf counter;    // work-queue counter
     DevBuf vjp_buf;    // adjoint scratch
@@ -187,10 +188,11 @@ int64_t batched_tc_mma_count(BatchedState *st);
 // batched call with these arguments (0 when that kernel would not run); synchronises
 xc_status batched_count_far(BatchedState *st, const BatchedArgs &a, int64_t *count);
 // Scratch above kMaxKeptBytes (1e9 lines want 48 GB) stays with its handle only while calls use most of it:
-// it is given back when a call has needed less than half of it, and when a list is loaded.  (After every call
-// it would cost 0.5 ms a GB: 4 % of a call on 1e9 lines.)  The stream has synchronised, counters are read.
+// it is given back when a call has needed less than half of it, and when a list of less than half the lines
+// is loaded.  (After every call, or at every load, it would cost 0.5 ms a GB: 4 % of a call on 1e9 lines, 1.4 %
+// of loading and sweeping 1e8 lines.)  The stream has synchronised, counters are read.
 constexpr size_t kMaxKeptBytes = (size_t)16 << 30;
-void batched_trim(BatchedState *st, bool loading = false);
+void batched_trim(BatchedState *st, bool smaller_list = false);
 void batched_invalidate(BatchedState *st);
 void batched_release(BatchedState *st);
 

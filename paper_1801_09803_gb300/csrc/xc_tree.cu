@@ -1224,7 +1224,7 @@ xc_status tree_run(BatchedState *st, const BatchedArgs &a, int64_t *launches) {
     p.nodes_per_cond = off;
 
     const size_t rec = n * (w4 ? 32 : 16);
-    if ((size_t)cg * rec > st->tiles.bytes) {
+    if ((size_t)cg * rec > std::max(st->tiles.bytes, (size_t)1 << 30)) {   // (the question takes 25 us)
         size_t room = 0, total = 0;
         if (cudaMemGetInfo(&room, &total) != cudaSuccess) cudaGetLastError();
         else cg = (int)std::min<size_t>((size_t)cg, std::max<size_t>(1, (room + st->tiles.bytes) / 2 / rec));
@@ -1250,6 +1250,7 @@ xc_status tree_run(BatchedState *st, const BatchedArgs &a, int64_t *launches) {
         }
         TR_TRY(e);   // out of memory here: the caller falls back to the tiled kernels
         st->tiles_need = o;
+        st->tiles_lines = n;
         break;
     }
     char *b = st->tiles.as<char>();
