@@ -57,6 +57,7 @@ using namespace xc;
 struct xc_handle {
     int device = 0;
     size_t n_lines = 0, cap_lines = 0;
+    double nu_range[2] = {-1.0, -1.0};   // first and last wavenumber, when a call has asked (see lines_in_reach)
     double *nu = nullptr;
     float *elower = nullptr, *A = nullptr, *gamma_ref = nullptr, *n_T = nullptr;
     int16_t *g_up = nullptr, *j_lo = nullptr;
@@ -158,6 +159,25 @@ void collect_timing(xc_handle *h, const bool *used) {
         if (cudaEventElapsedTime(&ms, h->ev[2 * i], h->ev[2 * i + 1]) == cudaSuccess) h->last_ms[i] = ms;
         else cudaGetLastError();
     }
+}
+
+// About how many lines reach the grid, for the choice of FP32 kernels.  Where outputs are few (2^20) the
+// choice does not hang on it, and the list's ends need not be fetched; once per list otherwise.
+double lines_in_reach(xc_handle *h, const xc_grid *g, double cutoff, size_t n_cond, cudaStream_t s) {
+    const size_t n = h->n_lines;
+    if (n == 0 || (double)n_cond * (double)g->n < 0x1p20) return (double)n;
+    if (h->nu_range[0] < 0.0) {
+        double r[2];
+        if (cudaMemcpyAsync(&r[0], h->nu, 8, cudaMemcpyDeviceToHost, s) != cudaSuccess ||
+            cudaMemcpyAsync(&r[1], h->nu + n - 1, 8, cudaMemcpyDeviceToHost, s) != cudaSuccess ||
+            cudaStreamSynchronize(s) != cudaSuccess) {
+            cudaGetLastError();
+            return (double)n;
+        }
+        h->nu_range[0] = r[0];
+        h->nu_range[1] = r[1];
+    }
+    return route_reach(n, h->nu_range[0], h->nu_range[1], *g, cutoff);
 }
 
 xc_status check_handle(const xc_handle *h) {
@@ -476,6 +496,7 @@ xc_status xc_load_lines(xc_handle *h, const xc_lines *L, size_t n, unsigned flag
     h->n_lines = 0;
     h->n_broad = 0;   // a broadener mixture belongs to the lines it was set for
     if (2 * n < h->batched.tiles_lines) batched_trim(&h->batched, true);
+    h->nu_range[0] = h->nu_range[1] = -1.0;
     // graphs and tuning stay valid: they key on shapes and buffer addresses, and read the
     // line data when replayed
     if (n == 0) return XC_OK;
@@ -838,6 +859,7 @@ xc_status xc_cross_section_batched(xc_handle *h, const xc_condition *conds, size
         BatchedArgs a;
         a.L = lines_of(h);
         a.n_lines = h->n_lines;
+        a.reach = lines_in_reach(h, grid, opts->cutoff, n_cond, s);
         a.conds_dev = dc;
         a.conds_host = conds;
         a.n_cond = (int)n_cond;
@@ -926,6 +948,7 @@ static xc_status vjp_common(xc_handle *h, const xc_condition *conds, size_t n_co
     VjpArgs a;
     a.L = lines_of(h);
     a.n_lines = h->n_lines;
+    a.reach = lines_in_reach(h, grid, opts->cutoff, n_cond, s);
     a.n_cond = (int)n_cond;
     a.grid = *grid;
     a.opts = *opts;
@@ -1036,6 +1059,7 @@ xc_status xc_count_far_evals(xc_handle *h, const xc_condition *conds, size_t n_c
     BatchedArgs a;
     a.L = lines_of(h);
     a.n_lines = h->n_lines;
+    a.reach = lines_in_reach(h, grid, opts->cutoff, n_cond, s);
     a.conds_dev = dc;
     a.conds_host = conds;
     a.n_cond = (int)n_cond;

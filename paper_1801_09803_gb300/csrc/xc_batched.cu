@@ -1833,7 +1833,7 @@ int grid_size(const Variant *v, int dev, int n_tiles) {
 Route32 route_of(const BatchedArgs &a, int nc) {
     const double cut = route_cut_steps(a.opts.cutoff, a.opts.width_mult, a.grid, a.conds_host, nc);
     return Route32{a.opts.profile, a.opts.flags, a.opts.n_gh, a.opts.cutoff, a.opts.width_mult, cut, a.grid,
-                   a.n_lines, nc, a.allow_tc, a.tiled};
+                   a.n_lines, a.reach, nc, a.allow_tc, a.tiled};
 }
 
 bool use_tc(const BatchedArgs &a, int nc) { return route_tc32(route_of(a, nc)); }

@@ -96,6 +96,7 @@ __device__ __forceinline__ void line_widths(float nu, float gref, float nT, cons
 struct BatchedArgs {
     LinesDev L{};
     size_t n_lines = 0;
+    double reach = 0.0;                     // lines that reach the grid, about (route_reach)
     const CondDev *conds_dev = nullptr;     // resolved conditions (Q filled) on the device
     const xc_condition *conds_host = nullptr;
     int n_cond = 0;
@@ -117,6 +118,7 @@ struct BatchedArgs {
 struct VjpArgs {
     LinesDev L{};
     size_t n_lines = 0;
+    double reach = 0.0;
     const CondDev *conds_dev = nullptr;
     const xc_condition *conds_host = nullptr;
     int n_cond = 0;

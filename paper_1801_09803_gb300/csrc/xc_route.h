@@ -38,6 +38,12 @@ inline double route_cut_steps(double cutoff, double width_mult, const xc_grid &g
     return sum / n / g.step;
 }
 
+// Lines of a list over [lo, hi] (spread evenly) whose cuts can reach the grid -- for the same choice
+inline double route_reach(size_t n, double lo, double hi, const xc_grid &g, double cutoff) {
+    const double a = fmax(lo, g.nu_A - cutoff), b = fmin(hi, g.nu_A + g.step * (double)g.n + cutoff);
+    return hi > lo ? (double)n * fmin(1.0, fmax(b - a, 0.0) / (hi - lo)) : (double)n;
+}
+
 // ---- FP32: the block-interpolated sweep (xc_tree.cu), or the tiled kernels with or without the far
 // wings on the tensor cores (xc_batched.cu)
 struct Route32 {
@@ -46,6 +52,7 @@ struct Route32 {
     double cut_steps;   // route_cut_steps
     xc_grid grid;
     size_t n_lines;
+    double reach;       // route_reach
     int n_cond;
     bool allow_tc;   // far wings may use the tensor-core kernel
     bool tiled;      // the tiled kernels whatever the sizes (fixed tile shape, no room for the blocks' scratch)
@@ -77,7 +84,7 @@ inline bool route_sparse32(const Route32 &r, bool tc) {
     }
     const double base = wl ? 23e6 * r.n_cond : 28e6 + 5e6 * fmin(nc, 24.0);   // shorter launch sequences
     return base - point * (double)r.grid.n * r.n_cond +
-               (line + pair * 2.0 * r.cut_steps) * (double)r.n_lines * r.n_cond < 0.0;
+               (line + pair * 2.0 * r.cut_steps) * r.reach * r.n_cond < 0.0;
 }
 
 // Whether the tensor-core kernel can take the far wings of a tiled call: many conditions (the
@@ -109,7 +116,7 @@ inline bool route_blocks32(const Route32 &r) {
 // 778 / 581, 150 1178 / 2684; Lorentz 758 / 286, 1024 / 764, width-limited (500 widths) 770 / 250 and 1031 / 502.
 // Points and cuts as for the sweep: a line whose position is near 2^31 then reaches no point.
 inline bool route_adjoint_blocks(int profile, int n_gh, double cutoff, double cut_steps, const xc_grid &g,
-                                 size_t n_lines, int n_cond) {
+                                 double reach, int n_cond) {
     if (profile == XC_DOPPLER || g.n >= ((int64_t)1 << 30) || !(cutoff / g.step < 0x1p20)) return false;
     double line, pair;   // ps
     switch (profile) {
@@ -119,7 +126,7 @@ inline bool route_adjoint_blocks(int profile, int n_gh, double cutoff, double cu
     }
     // a warp takes a line through all conditions: below 2000 lines the chip is not full, and the last
     // line's time is all there is
-    return (pair * 2.0 * cut_steps - line) * fmax((double)n_lines, 2000.0) * n_cond > 1e7 + 75.0 * (double)g.n * n_cond;
+    return (pair * 2.0 * cut_steps - line) * fmax(reach, 2000.0) * n_cond > 1e7 + 75.0 * (double)g.n * n_cond;
 }
 
 // Whatever keeps a call from the blocks, its far wings go to the tensor cores where they can

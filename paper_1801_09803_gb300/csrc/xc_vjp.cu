@@ -901,7 +901,7 @@ xc_status vjp_run(BatchedState *st, const VjpArgs &a, int64_t *launches) {
     const bool far = !f64 && n && N &&
                      route_adjoint_blocks(a.opts.profile, a.opts.n_gh, a.opts.cutoff,
                                           route_cut_steps(a.opts.cutoff, a.opts.width_mult, a.grid, a.conds_host, nc),
-                                          a.grid, n, nc);
+                                          a.grid, a.reach, nc);
     const int nblk512 = far ? (int)((a.grid.n + 511) / 512) : 0;
     const size_t per_cond = (size_t)nblk512 * (128 + 64 + 16);
     size_t o_gn = far ? carve((size_t)nc * per_cond * 4) : 0;

@@ -385,3 +385,20 @@ def test_gauss_hermite_adjoint_without_pressure(eng, xc, precision):  # noqa: F8
     S *= -np.expm1(-c2 * f["nu"] / 296.0)
     ref = S * f["gamma_ref"] * 1e22 / np.pi / step ** 2 * np.sum(1.0 / (sp * sm)[ok])
     assert abs(float(r["dP"][0]) - ref) <= (1e-5 if precision == "fp32" else 1e-12) * abs(ref)
+
+
+def test_the_rule_counts_the_lines_in_reach(eng, xc):  # noqa: F811
+    """A list twenty times wider than the grid is as sparse there as its part in reach; a list of the same
+    length loaded afterwards over the grid alone is not."""
+    grid, opts = xc.make_grid(5000.0, 0.01, 100_001), xc.make_opts("lorentz", "fp32", 25.0)
+    conds = [xc.make_condition(400.0 + 60.0 * i, 0.01 * 1.3 ** i) for i in range(24)]
+    eng.set_states(*xs.gen_states(325, 300))
+    for lo, hi, blocks in ((0.0, 20_000.0, False), (4990.0, 6010.0, True)):
+        eng.load_lines(xs.gen_lines(325, 0, 150_000, lo, hi))
+        got = eng.cross_section_batched(conds, grid, opts)
+        assert ("block-interpolated" in eng.tuning()) == blocks
+        eng.set_tile_shape(8, 1)
+        ref = eng.cross_section_batched(conds, grid, opts)
+        eng.set_tile_shape(0, 0)
+        m = ref > 1e-6 * ref.max(axis=1, keepdims=True)
+        assert np.max(np.abs(got - ref)[m] / ref[m]) < 2e-5

@@ -23,7 +23,7 @@ extern "C" int route32(int profile, int flags, double cutoff, double width_mult,
     xc_condition c{};
     c.T = 1000.0, c.P = 0.1, c.mass_da = 18.0, c.T_ref = 296.0, c.P_ref = 1.0, c.gamma_scale = 1.0;
     const xc::Route32 r{profile, flags, 20, cutoff, width_mult, xc::route_cut_steps(cutoff, width_mult, g, &c, 1), g,
-                        (size_t)n_lines, n_cond, allow_tc != 0, tiled != 0};
+                        (size_t)n_lines, (double)n_lines, n_cond, allow_tc != 0, tiled != 0};
     return 2 * xc::route_blocks32(r) + xc::route_tc32(r);
 }
 extern "C" int adjoint_blocks(int profile, double cutoff, double width_mult, double step, long long n_pts,
@@ -32,7 +32,10 @@ extern "C" int adjoint_blocks(int profile, double cutoff, double width_mult, dou
     xc_condition c{};
     c.T = 1000.0, c.P = 0.1, c.mass_da = 18.0, c.T_ref = 296.0, c.P_ref = 1.0, c.gamma_scale = 1.0;
     return xc::route_adjoint_blocks(profile, 20, cutoff, xc::route_cut_steps(cutoff, width_mult, g, &c, 1), g,
-                                    (size_t)n_lines, n_cond);
+                                    (double)n_lines, n_cond);
+}
+extern "C" double reach(unsigned long long n, double lo, double hi, double nu_A, double step, long long n_pts, double cutoff) {
+    return xc::route_reach((size_t)n, lo, hi, xc_grid{nu_A, step, (int64_t)n_pts}, cutoff);
 }
 """
 
@@ -50,6 +53,8 @@ def route(tmp_path_factory):
     L.blocks64.argtypes = [C.c_int, C.c_double, C.c_double, C.c_longlong, C.c_double, C.c_ulonglong]
     L.route32.argtypes = [C.c_int, C.c_int, C.c_double, C.c_double, C.c_double, C.c_longlong, C.c_ulonglong, C.c_int,
                           C.c_int, C.c_int]
+    L.reach.argtypes = [C.c_ulonglong, C.c_double, C.c_double, C.c_double, C.c_double, C.c_longlong, C.c_double]
+    L.reach.restype = C.c_double
     L.adjoint_blocks.argtypes = [C.c_int, C.c_double, C.c_double, C.c_double, C.c_longlong, C.c_ulonglong, C.c_int]
     return L
 
@@ -186,3 +191,13 @@ def test_adjoint_blocks_keep_their_limits(route):
     assert not route.adjoint_blocks(DOPPLER, 25.0, 0.0, 0.01, 200_001, 300_000, 4)
     assert not route.adjoint_blocks(W4, 25.0, 0.0, 0.01, 1 << 30, 1 << 30, 4)
     assert not route.adjoint_blocks(W4, 0.01 * 2 ** 20, 0.0, 0.01, 200_001, 300_000, 4)
+
+
+def test_lines_in_reach(route):
+    r = route.reach
+    assert r(1000, 0.0, 10_000.0, 5000.0, 0.01, 100_000, 0.0) == pytest.approx(100.0)
+    assert r(1000, 0.0, 10_000.0, 5000.0, 0.01, 100_000, 500.0) == pytest.approx(200.0)
+    assert r(1000, 0.0, 10_000.0, 9900.0, 0.01, 100_000, 25.0) == pytest.approx(12.5)
+    assert r(1000, 100.0, 200.0, 0.0, 0.01, 100_000, 25.0) == 1000.0     # the grid covers the list
+    assert r(1000, 100.0, 200.0, 500.0, 0.01, 1000, 25.0) == 0.0
+    assert r(7, 100.0, 100.0, 50.0, 0.01, 10_000, 25.0) == 7.0           # one wavenumber
