@@ -284,7 +284,8 @@ __global__ void __launch_bounds__(256) k_tree_recs(TreeParams p, float4 *recA, f
     const CParam cp = p.cp[p.c0 + c];
     const float h = (float)p.step;
     const size_t l1 = tr_upper(p, p.n_pts + p.reach + 1);
-    for (size_t l = tr_lower(p, -p.reach) + (size_t)blockIdx.x * 256 + threadIdx.x; l < l1; l += (size_t)gridDim.x * 256) {
+    const size_t l0 = tr_lower(p, -p.reach) & ~63u;   // whole sectors for a warp
+    for (size_t l = l0 + (size_t)blockIdx.x * 256 + threadIdx.x; l < l1; l += (size_t)gridDim.x * 256) {
         float4 A, B = make_float4(0.f, 0.f, 0.f, -1.f), S;
         float t2;
         line_consts<PROF, EXT>(p.L, l, cp, h, p.inv_h, &A, &B, &t2, &S);
@@ -1268,7 +1269,7 @@ xc_status tree_run(BatchedState *st, const BatchedArgs &a, int64_t *launches) {
     p.recA = recA;
     p.recB = recB;
     p.nodes = (double *)(b + o_nodes);
-    const unsigned lb = (unsigned)std::max<size_t>(1, std::min<size_t>((n + 255) / 256, 152 * 16));
+    const unsigned lb = (unsigned)std::max<size_t>(1, std::min<size_t>((n + 255) / 256, 152 * 8));
 
     const double eps = geom_eps(a.grid, a.opts.cutoff);
     if (a.timing) TR_TRY(cudaEventRecord(a.ev_begin, s));
